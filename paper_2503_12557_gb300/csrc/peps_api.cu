@@ -1018,7 +1018,7 @@ static peps_status ensure_minsr(peps_handle* h, int Ns, long long Np) {
   return PEPS_OK;
 }
 
-// MinSR scratch slots (h->cnt, 16 doubles): 0 factor breakdown (int), 2 weight sum, 3 FP64
+// MinSR scratch slots (h->cnt, 16 doubles): 0 factor breakdown (int), 3 FP64
 // fallback flag of the mixed solve (int), 4 tensor-core Gram wait timeout (int), 6-7 residual
 // norms, 8-9 Jacobi rotation counters (unsigned long long)
 
@@ -1115,7 +1115,6 @@ extern "C" peps_status minsr_step(peps_handle* h, const void* O_dev, const doubl
   if (ps != PEPS_OK) return ps;
   cudaStream_t s = (cudaStream_t)stream;
   const int n = Ns + (Ns & 1);
-  double* wsum = h->cnt + 2;
   int* gerr = (int*)(h->cnt + 4);
   int ts = tstart(h, TC_MINSR, s);
   CK(cudaMemsetAsync(h->ebar, 0, sizeof(double) * n, s), "memset");
@@ -1124,16 +1123,16 @@ extern "C" peps_status minsr_step(peps_handle* h, const void* O_dev, const doubl
     using T = decltype(z);
     using R = typename Scal<T>::R;
     if constexpr (Scal<T>::complex) {
-      const cudaError_t e1 = launch_center_cplx<R>((const R*)O_dev, w_dev, Ns_c, Np_c, h->Obar, wsum, s);
+      const cudaError_t e1 = launch_center_cplx<R>((const R*)O_dev, w_dev, Ns_c, Np_c, h->Obar, h->xv, h->yv, s);
       return e1 != cudaSuccess ? e1 : launch_center_e_cplx(eloc_dev, w_dev, Ns_c, h->ebar, s);
     } else {
-      const cudaError_t e1 = launch_center<T>((const T*)O_dev, w_dev, Ns, Np, h->mean, h->Obar, wsum, s);
+      const cudaError_t e1 = launch_center<T>((const T*)O_dev, w_dev, Ns, Np, h->mean, h->Obar, h->xv, h->yv, s);
       return e1 != cudaSuccess ? e1 : launch_center_e(eloc_dev, w_dev, Ns, h->ebar, s);
     }
   });
   if (e != cudaSuccess) return cuda_fail(h, e, "centre O and E_loc");
   CK(cudaMemsetAsync(h->Tm, 0, sizeof(double) * (size_t)n * n, s), "memset");
-  tstop(h, ts, s, (w_dev ? 3 : 2) + 2);
+  tstop(h, ts, s, 3 + 2);
   if ((ps = minsr_gram_into(h, h->Obar, Ns, Np, h->Tm, n, rcond > 0.0, s)) != PEPS_OK) return ps;
   if ((ps = minsr_solve_core(h, Ns, lambda, rcond, info_dev, s)) != PEPS_OK) return ps;
   ts = tstart(h, TC_MINSR, s);

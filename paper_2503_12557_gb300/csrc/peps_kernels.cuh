@@ -205,15 +205,15 @@ cudaError_t launch_minsr_finish(double* info, const int* gram_err, double* dthet
 // ---- MinSR (FP64)
 // column means m_k = sum_S w_S O_{S,k} (w normalised), and Obar = sqrt(w)(O - m) written as
 // double (Ns x Np)
-// (wsum_dev: one device double of scratch for the weight sum, used when w is not NULL)
+// (wn, sw: Ns device doubles of scratch each)
 template <typename TO>
-cudaError_t launch_center(const TO* O, const double* w, int Ns, long long Np, double* mean, double* Obar,
-                          double* wsum_dev, cudaStream_t s);
+cudaError_t launch_center(const TO* O, const double* w, int Ns, long long Np, double* mean, double* Obar, double* wn,
+                          double* sw, cudaStream_t s);
 cudaError_t launch_center_e(const double* eloc, const double* w, int Ns, double* ebar, cudaStream_t s);
 // complex O (Ns x Np (re, im) pairs of TO): the real embedding W (2Ns x 2Np), [Re ebar; Im ebar]
 // (2Ns), and dtheta back from [Re; Im] (2Np) to Np (re, im) pairs
 template <typename TO>
-cudaError_t launch_center_cplx(const TO* O, const double* w, int Ns, long long Np, double* W, double* wsum_dev,
+cudaError_t launch_center_cplx(const TO* O, const double* w, int Ns, long long Np, double* W, double* wn, double* sw,
                                cudaStream_t s);
 cudaError_t launch_center_e_cplx(const double* eloc, const double* w, int Ns, double* ebar2, cudaStream_t s);
 cudaError_t launch_unembed(const double* d2, long long Np, double* dtheta, cudaStream_t s);

@@ -9,20 +9,66 @@ namespace cg = cooperative_groups;
 namespace peps {
 
 // ---- centring: mean_k = sum_S w_S O_{S,k}; Obar_{S,k} = sqrt(w_S) (O_{S,k} - mean_k)
-// The weight sum is read from the device (written by k_wsum), so that no host round trip
-// separates the two launches.
+// Column kernels: a CTA of 32 x 32 threads owns 32 adjacent columns and its 32 warps share the rows
+// (a warp reads one row's 32 columns), so that N_p columns keep N_p threads x 32 in flight; the
+// warps' sums meet in shared memory in a fixed order.  One thread per column, as before, left
+// 85 CTAs walking 4096 rows alone with a weight division per entry: 8.3 ms for the centring of
+// 4096 x 21 632 FP32 entries and 1.6 ms for Obar^T x, against 0.2 and 0.1 ms of HBM time; now
+// FP64 issue is the limit (a conversion, a multiply-add, a subtraction and a product per entry):
+// the whole MinSR step went from 127.1 to 118.4 ms there, from 10.26 to 8.28 ms at 1000 x 3528
+// FP64 entries.
+constexpr int CC = 32;
+__device__ __forceinline__ double col_reduce(double v, double (&red)[CC][CC + 1]) {
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  __syncthreads();
+  red[ty][tx] = v;
+  __syncthreads();
+  if (ty == 0) {
+#pragma unroll 8
+    for (int i = 1; i < CC; ++i) v += red[i][tx];
+    red[0][tx] = v;
+  }
+  __syncthreads();
+  return red[0][tx];
+}
+static inline int col_grid(long long Np) {
+  const long long b = (Np + CC - 1) / CC;
+  return (int)(b < 1 ? 1 : (b < (1ll << 30) ? b : (1ll << 30)));
+}
+
+// wn = w / sum(w) (1 / Ns without weights) and sw = sqrt(wn) of every sample, computed once
+// instead of once per column; every CTA sums the weights itself, in the same order
+__global__ void __launch_bounds__(256) k_wprep(const double* __restrict__ w, int Ns, double* wn, double* sw) {
+  __shared__ double red[33];
+  double ws = 0.0;
+  if (w) {
+    for (int i = threadIdx.x; i < Ns; i += 256) ws += w[i];
+    ws = block_sum(ws, red);
+  }
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < Ns; i += gridDim.x * 256) {
+    const double v = w ? w[i] / ws : 1.0 / Ns;
+    wn[i] = v;
+    sw[i] = sqrt(v);
+  }
+}
+
 template <typename TO>
-__global__ void k_center(const TO* __restrict__ O, const double* __restrict__ w, int Ns, long long Np,
-                         const double* __restrict__ wsum_dev, double* mean, double* Obar) {
-  const double wsum = w ? *wsum_dev : 1.0;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < Np; k += (long long)gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(CC* CC) k_center(const TO* __restrict__ O, const double* __restrict__ wn,
+                                                   const double* __restrict__ sw, int Ns, long long Np, double* mean,
+                                                   double* Obar) {
+  __shared__ double red[CC][CC + 1];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (long long cb = blockIdx.x; cb * CC < Np; cb += gridDim.x) {
+    const long long k = cb * CC + tx;
+    const bool in = k < Np;
     double m = 0.0;
-    for (int s = 0; s < Ns; ++s) m += (w ? w[s] / wsum : 1.0 / Ns) * (double)O[(size_t)s * Np + k];
-    mean[k] = m;
-    for (int s = 0; s < Ns; ++s) {
-      const double sw = sqrt(w ? w[s] / wsum : 1.0 / Ns);
-      Obar[(size_t)s * Np + k] = sw * ((double)O[(size_t)s * Np + k] - m);
-    }
+#pragma unroll 4
+    for (int s = ty; s < Ns; s += CC) m = fma(wn[s], in ? (double)O[(size_t)s * Np + k] : 0.0, m);
+    m = col_reduce(m, red);
+    if (ty == 0 && in) mean[k] = m;
+#pragma unroll 4
+    for (int s = ty; s < Ns; s += CC)
+      if (in) Obar[(size_t)s * Np + k] = sw[s] * ((double)O[(size_t)s * Np + k] - m);
   }
 }
 
@@ -32,21 +78,27 @@ __global__ void k_center(const TO* __restrict__ O, const double* __restrict__ w,
 // W^T [Re x; Im x] = [Re(Obar^H x); Im(Obar^H x)]: the real pipeline on (W, [Re ebar; Im ebar])
 // returns [Re dtheta; Im dtheta].  O: Ns x Np (re, im) pairs of TO.
 template <typename TO>
-__global__ void k_center_cplx(const TO* __restrict__ O, const double* __restrict__ w, int Ns, long long Np,
-                              const double* __restrict__ wsum_dev, double* W) {
-  const double wsum = w ? *wsum_dev : 1.0;
+__global__ void __launch_bounds__(CC* CC) k_center_cplx(const TO* __restrict__ O, const double* __restrict__ wn,
+                                                        const double* __restrict__ sw, int Ns, long long Np, double* W) {
+  __shared__ double red[CC][CC + 1];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const long long Np2 = 2 * Np;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < Np; k += (long long)gridDim.x * blockDim.x) {
+  for (long long cb = blockIdx.x; cb * CC < Np; cb += gridDim.x) {
+    const long long k = cb * CC + tx;
+    const bool in = k < Np;
     double mr = 0.0, mi = 0.0;
-    for (int s = 0; s < Ns; ++s) {
-      const double ws = w ? w[s] / wsum : 1.0 / Ns;
-      mr += ws * (double)O[2 * ((size_t)s * Np + k)];
-      mi += ws * (double)O[2 * ((size_t)s * Np + k) + 1];
+#pragma unroll 2
+    for (int s = ty; s < Ns; s += CC) {
+      const size_t o = 2 * ((size_t)s * Np + (in ? k : 0));
+      mr = fma(wn[s], (double)O[o], mr);
+      mi = fma(wn[s], (double)O[o + 1], mi);
     }
-    for (int s = 0; s < Ns; ++s) {
-      const double sw = sqrt(w ? w[s] / wsum : 1.0 / Ns);
-      const double re = sw * ((double)O[2 * ((size_t)s * Np + k)] - mr);
-      const double im = sw * ((double)O[2 * ((size_t)s * Np + k) + 1] - mi);
+    mr = col_reduce(mr, red);
+    mi = col_reduce(mi, red);
+    if (!in) continue;  // (every thread of the CTA has passed the last barrier of this trip)
+    for (int s = ty; s < Ns; s += CC) {
+      const size_t o = 2 * ((size_t)s * Np + k);
+      const double re = sw[s] * ((double)O[o] - mr), im = sw[s] * ((double)O[o + 1] - mi);
       W[(size_t)s * Np2 + k] = re;
       W[(size_t)s * Np2 + Np + k] = -im;
       W[(size_t)(Ns + s) * Np2 + k] = im;
@@ -83,14 +135,6 @@ __global__ void k_unembed(const double* d2, long long Np, double* dtheta) {
   }
 }
 
-__global__ void k_wsum(const double* w, int Ns, double* out) {
-  __shared__ double red[33];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < Ns; i += blockDim.x) s += w[i];
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) *out = s;
-}
-
 // ebar_S = sqrt(w_S) (Re E_loc(S) - sum_S' w_S' Re E_loc(S')); eloc is (re, im) interleaved
 __global__ void k_center_e(const double* eloc, const double* w, int Ns, double* ebar) {
   __shared__ double red[33];
@@ -113,12 +157,18 @@ __global__ void k_center_e(const double* eloc, const double* w, int Ns, double* 
 // sums[k] = sum_S w_S O_{S,k} (k < Np), sums[Np] = sum_S w_S, sums[Np + 1] = sum_S w_S Re E_loc(S)
 // (w NULL: every w_S = 1)
 template <typename TO>
-__global__ void k_colsum(const TO* __restrict__ O, const double* __restrict__ w, int Ns, long long Np,
-                         double* __restrict__ sums) {
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < Np; k += (long long)gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(CC* CC) k_colsum(const TO* __restrict__ O, const double* __restrict__ w, int Ns,
+                                                   long long Np, double* __restrict__ sums) {
+  __shared__ double red[CC][CC + 1];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (long long cb = blockIdx.x; cb * CC < Np; cb += gridDim.x) {
+    const long long k = cb * CC + tx;
+    const bool in = k < Np;
     double m = 0.0;
-    for (int s = 0; s < Ns; ++s) m += (w ? w[s] : 1.0) * (double)O[(size_t)s * Np + k];
-    sums[k] = m;
+#pragma unroll 4
+    for (int s = ty; s < Ns; s += CC) m = fma(w ? w[s] : 1.0, in ? (double)O[(size_t)s * Np + k] : 0.0, m);
+    m = col_reduce(m, red);
+    if (ty == 0 && in) sums[k] = m;
   }
 }
 
@@ -138,14 +188,24 @@ __global__ void k_wsums(const double* __restrict__ w, const double* __restrict__
 // Obar_{S,k} = sqrt(w_S / W) (O_{S,k} - g_k / W), ebar_S = sqrt(w_S / W) (Re E_loc(S) - g_E / W) with
 // the global sums g (layout of k_colsum / k_wsums: Np column sums, W, g_E)
 template <typename TO>
-__global__ void k_center_global(const TO* __restrict__ O, const double* __restrict__ w, int Ns, long long Np,
-                                const double* __restrict__ g, double* __restrict__ Obar) {
+__global__ void __launch_bounds__(CC* CC) k_center_global(const TO* __restrict__ O, const double* __restrict__ w, int Ns,
+                                                          long long Np, const double* __restrict__ g,
+                                                          double* __restrict__ Obar) {
+  __shared__ double sw[CC * CC];  // sqrt(w_S / W) of 1024 rows at a time
   const double W = g[Np];
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < Np; k += (long long)gridDim.x * blockDim.x) {
-    const double m = g[k] / W;
-    for (int s = 0; s < Ns; ++s) {
-      const double sw = sqrt((w ? w[s] : 1.0) / W);
-      Obar[(size_t)s * Np + k] = sw * ((double)O[(size_t)s * Np + k] - m);
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (long long cb = blockIdx.x; cb * CC < Np; cb += gridDim.x) {
+    const long long k = cb * CC + tx;
+    const bool in = k < Np;
+    const double m = in ? g[k] / W : 0.0;
+    for (int s0 = 0; s0 < Ns; s0 += CC * CC) {
+      __syncthreads();
+      if (s0 + (int)threadIdx.x < Ns) sw[threadIdx.x] = sqrt((w ? w[s0 + threadIdx.x] : 1.0) / W);
+      __syncthreads();
+      const int ns = min(Ns - s0, CC * CC);
+#pragma unroll 4
+      for (int s = ty; s < ns; s += CC)
+        if (in) Obar[(size_t)(s0 + s) * Np + k] = sw[s] * ((double)O[(size_t)(s0 + s) * Np + k] - m);
     }
   }
 }
@@ -160,8 +220,7 @@ __global__ void k_center_e_global(const double* __restrict__ eloc, const double*
 template <typename TO>
 cudaError_t launch_partial_sums(const TO* O, const double* w, const double* eloc, int Ns, long long Np, double* sums,
                                 cudaStream_t s) {
-  const long long blocks = (Np + 255) / 256;
-  k_colsum<TO><<<(int)(blocks < 4096 ? (blocks > 0 ? blocks : 1) : 4096), 256, 0, s>>>(O, w, Ns, Np, sums);
+  k_colsum<TO><<<col_grid(Np), CC * CC, 0, s>>>(O, w, Ns, Np, sums);
   k_wsums<<<1, 1024, 0, s>>>(w, eloc, Ns, sums + Np);
   return cudaGetLastError();
 }
@@ -173,8 +232,7 @@ template cudaError_t launch_partial_sums<float>(const float*, const double*, con
 template <typename TO>
 cudaError_t launch_center_global(const TO* O, const double* w, const double* eloc, int Ns, long long Np,
                                  const double* g, double* Obar, double* ebar, cudaStream_t s) {
-  const long long blocks = (Np + 255) / 256;
-  k_center_global<TO><<<(int)(blocks < 4096 ? (blocks > 0 ? blocks : 1) : 4096), 256, 0, s>>>(O, w, Ns, Np, g, Obar);
+  k_center_global<TO><<<col_grid(Np), CC * CC, 0, s>>>(O, w, Ns, Np, g, Obar);
   k_center_e_global<<<(Ns + 255) / 256 > 0 ? (Ns + 255) / 256 : 1, 256, 0, s>>>(eloc, w, Ns, Np, g, ebar);
   return cudaGetLastError();
 }
@@ -400,41 +458,44 @@ __global__ void k_v_y(const double* V, const double* y, int n, double* x) {
   }
 }
 
-__global__ void k_obar_t_x(const double* __restrict__ Ob, const double* __restrict__ x, int Ns, long long Np,
-                           double tau, double* dtheta) {
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < Np; k += (long long)gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int i = 0; i < Ns; ++i) s += Ob[(size_t)i * Np + k] * x[i];
-    dtheta[k] = -tau * s;
+__global__ void __launch_bounds__(CC* CC) k_obar_t_x(const double* __restrict__ Ob, const double* __restrict__ x, int Ns,
+                                                     long long Np, double tau, double* dtheta) {
+  __shared__ double red[CC][CC + 1];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (long long cb = blockIdx.x; cb * CC < Np; cb += gridDim.x) {
+    const long long k = cb * CC + tx;
+    double v = 0.0;
+#pragma unroll 4
+    for (int i = ty; i < Ns; i += CC) v = fma(k < Np ? Ob[(size_t)i * Np + k] : 0.0, x[i], v);
+    v = col_reduce(v, red);
+    if (ty == 0 && k < Np) dtheta[k] = -tau * v;
   }
 }
 
 // ---- host wrappers
-// wsum_dev: one device double for the weight sum (used only when w is not NULL)
+// wn, sw: Ns doubles of scratch each (the normalised weights and their square roots)
 template <typename TO>
-cudaError_t launch_center(const TO* O, const double* w, int Ns, long long Np, double* mean, double* Obar,
-                          double* wsum_dev, cudaStream_t s) {
-  if (w) k_wsum<<<1, 256, 0, s>>>(w, Ns, wsum_dev);
-  const long long blocks = (Np + 255) / 256;
-  k_center<TO><<<(int)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(O, w, Ns, Np, wsum_dev, mean, Obar);
+cudaError_t launch_center(const TO* O, const double* w, int Ns, long long Np, double* mean, double* Obar, double* wn,
+                          double* sw, cudaStream_t s) {
+  k_wprep<<<(Ns + 255) / 256, 256, 0, s>>>(w, Ns, wn, sw);
+  k_center<TO><<<col_grid(Np), CC * CC, 0, s>>>(O, wn, sw, Ns, Np, mean, Obar);
   return cudaGetLastError();
 }
 template cudaError_t launch_center<double>(const double*, const double*, int, long long, double*, double*, double*,
-                                           cudaStream_t);
-template cudaError_t launch_center<float>(const float*, const double*, int, long long, double*, double*, double*,
+                                           double*, cudaStream_t);
+template cudaError_t launch_center<float>(const float*, const double*, int, long long, double*, double*, double*, double*,
                                           cudaStream_t);
 
 template <typename TO>
-cudaError_t launch_center_cplx(const TO* O, const double* w, int Ns, long long Np, double* W, double* wsum_dev,
+cudaError_t launch_center_cplx(const TO* O, const double* w, int Ns, long long Np, double* W, double* wn, double* sw,
                                cudaStream_t s) {
-  if (w) k_wsum<<<1, 256, 0, s>>>(w, Ns, wsum_dev);
-  const long long blocks = (Np + 255) / 256;
-  k_center_cplx<TO><<<(int)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(O, w, Ns, Np, wsum_dev, W);
+  k_wprep<<<(Ns + 255) / 256, 256, 0, s>>>(w, Ns, wn, sw);
+  k_center_cplx<TO><<<col_grid(Np), CC * CC, 0, s>>>(O, wn, sw, Ns, Np, W);
   return cudaGetLastError();
 }
-template cudaError_t launch_center_cplx<double>(const double*, const double*, int, long long, double*, double*,
+template cudaError_t launch_center_cplx<double>(const double*, const double*, int, long long, double*, double*, double*,
                                                 cudaStream_t);
-template cudaError_t launch_center_cplx<float>(const float*, const double*, int, long long, double*, double*,
+template cudaError_t launch_center_cplx<float>(const float*, const double*, int, long long, double*, double*, double*,
                                                cudaStream_t);
 
 cudaError_t launch_center_e_cplx(const double* eloc, const double* w, int Ns, double* ebar2, cudaStream_t s) {
@@ -570,8 +631,7 @@ cudaError_t launch_minsr_apply(const double* A, const double* V, const double* e
 
 cudaError_t launch_obar_t_x(const double* Obar, const double* x, int Ns, long long Np, double tau, double* dtheta,
                             cudaStream_t s) {
-  const long long blocks = (Np + 255) / 256;
-  k_obar_t_x<<<(int)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(Obar, x, Ns, Np, tau, dtheta);
+  k_obar_t_x<<<col_grid(Np), CC * CC, 0, s>>>(Obar, x, Ns, Np, tau, dtheta);
   return cudaGetLastError();
 }
 
