@@ -52,8 +52,8 @@ def _args():
                     help="MinSR Cholesky: float-float factor + FP64 refinement (FP32 default), FP64 "
                          "(FP64 default), or FP32 factor + FP64 refinement")
     ap.add_argument("--gram", default=None, choices=["ff", "fp64", "bf16"],
-                    help="MinSR Gram of the step: float-float on the FP32 pipes (default with --prec fp32), "
-                         "FP64 (default with --prec fp64), or split-BF16 tcgen05")
+                    help="MinSR Gram of the step: FP64 accuracy from digits on the tensor cores (ff and fp64 "
+                         "alike, the default), or split-BF16 tcgen05")
     return ap.parse_args()
 
 
@@ -398,13 +398,12 @@ def run_gpu(a):
     dom = max(flops, key=lambda k: ms_cls.get(k, 0.0))
     dom_launch_ms = ms_cls[dom] / max(1, launches[dom])
     achieved = flops[dom] / max(1, launches[dom]) / (dom_launch_ms / 1e3) / 1e12
-    # a Gram-dominated step: FP64 FMA peak, FP32 pipe peak (float-float) or the BF16 tensor peak
-    gram_peak = {0: fp64_peak, 1: peaks.get("bf16_tflops", 1900.0), 2: fp32_peak}[gram]
+    gram_peak = peaks.get("bf16_tflops", 1900.0)  # every Gram mode runs on the BF16 tensor cores
     peak = gram_peak if dom == "minsr_gram" else alu_peak
     sampler_name = ("sampler call of alternating sweeps (k_env one-side pass where a sweep needs one, then "
                     "k_sweep_moves and k_env_row per row)" if prec == P.PREC_FP32 else "k_sample")
     roof = {"kernel": {"env": "k_env", "sample": sampler_name, "row": "k_row", "pair": "k_pair",
-                       "minsr_gram": "k_gram"}[dom],
+                       "minsr_gram": "k_gram_sl"}[dom],
             "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             # per launch, as achieved: the call's bytes spread over the launches the call made
             "traffic": (None if _measured_traffic(dom, ns, a.sweeps, prec) is None else
@@ -423,8 +422,7 @@ def run_gpu(a):
             "warmup": a.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f32" if prec == P.PREC_FP32 else "f64", "data": "synthetic",
             "config": _config(w, ns, a.sweeps), "step_ms": step_ms, "minsr_step_s": minsr_s,
-            "minsr": {"gram": {0: "FP64 CUDA cores", 1: "split-BF16 tcgen05",
-                               2: "float-float pairs on the FP32 pipes"}[gram],
+            "minsr": {"gram": "split-BF16 tcgen05" if gram == 1 else "FP64 accuracy, 7 BF16 digits on tcgen05",
                       "solve": {0: "FP64 Cholesky", 1: "FP32 Cholesky + FP64 refinement",
                                 2: "float-float Cholesky + FP64 refinement"}[solve],
                       "sharded_over_processes": world > 1,
@@ -645,12 +643,11 @@ def run_learned(a):
 
 def run_gram(a):
     """MinSR step on a synthetic O (N_s x N_p, entries N(0,1) plus a 0.1 column offset so that
-    centring matters) with the FP64 CUDA-core Gram, the split-BF16 tcgen05 Gram and the float-float
-    Gram on the FP32 pipes; reports each Gram's time, its pipe rate (3 BF16 products, 13 FP32
-    operations per algorithmic multiply-add) and the relative difference of each dtheta from the
-    FP64 one."""
+    centring matters) with the FP64-accurate digit Gram and the split-BF16 Gram; reports each
+    Gram's time, its tensor rate (28 or 3 BF16 products per algorithmic multiply-add) and the
+    relative difference of the split-BF16 dtheta from the other."""
     import torch
-    from paper_2503_12557_gb300 import build, inputs as I, peps as P
+    from paper_2503_12557_gb300 import build, costmodel, inputs as I, peps as P
     build.build()
     ns = a.ns or 16384
     lat = I.Lattice(14, 14, 2, 4)  # N_p = 80 000, the smallest square open lattice above 73 728
@@ -658,7 +655,7 @@ def run_gram(a):
     out = {"mode": "gram", "ns": ns}
     res = {}
     g = torch.Generator(device="cuda").manual_seed(5005)
-    for gram, tag in ((1, "tcgen05_split_bf16"), (2, "float_float_fp32"), (0, "fp64_cuda_cores")):
+    for gram, tag in ((1, "tcgen05_split_bf16"), (0, "tcgen05_fp64_digits")):
         h = P.PEPS(lat.Lx, lat.Ly, 2, lat.D, lat.D, prec=P.PREC_FP64, max_samples=2, gram=gram)
         out["np"] = h.Np
         g.manual_seed(5005)
@@ -666,7 +663,7 @@ def run_gram(a):
         O += 0.1 * torch.randn(h.Np, dtype=torch.float64, device="cuda", generator=g)
         e = torch.zeros(ns, 2, dtype=torch.float64, device="cuda")
         e[:, 0] = torch.randn(ns, dtype=torch.float64, device="cuda", generator=g) - 3.0
-        reps = 1 if gram == 0 else 3
+        reps = 3
         h.minsr_step(O, e, lam=1.0, tau=0.1)  # warm-up (allocations)
         h.timing(True)
         for _ in range(reps):
@@ -678,24 +675,17 @@ def run_gram(a):
         mac = ns * (ns + 1) / 2 * h.Np  # algorithmic multiply-adds of one triangle
         r = {"gram_ms": gram_ms, "solve_ms": ms["minsr_eig"] / reps, "step_s": sum(ms.values()) / reps / 1e3,
              "lambda": 1.0, "warning": h.last_warning}
-        if gram == 1:
-            tflops = 3 * 2 * mac / (gram_ms / 1e3) / 1e12
-            r["tensor_tflops_bf16"] = tflops
-            r["roofline"] = {"bound": "tensor", "achieved": tflops, "peak": peaks.get("bf16_tflops", 1900.0),
-                             "unit": "TFLOP/s", "frac": tflops / peaks.get("bf16_tflops", 1900.0)}
-        elif gram == 2:
-            r["fp32_pipe_tflops"] = 13 * 2 * mac / (gram_ms / 1e3) / 1e12
-            r["fp32_pipe_frac_of_measured_fma_peak"] = r["fp32_pipe_tflops"] / P.probe_fma(False)
-        else:
-            r["fp64_tflops"] = 2 * mac / (gram_ms / 1e3) / 1e12
+        tflops = costmodel.GRAM_PIPE_OPS[gram] * 2 * mac / (gram_ms / 1e3) / 1e12
+        r["tensor_tflops_bf16"] = tflops
+        r["roofline"] = {"bound": "tensor", "achieved": tflops, "peak": peaks.get("bf16_tflops", 1900.0),
+                         "unit": "TFLOP/s", "frac": tflops / peaks.get("bf16_tflops", 1900.0)}
         res[tag] = dth
         out[tag] = r
         del O
         h.close()
         torch.cuda.empty_cache()
-    for tag in ("tcgen05_split_bf16", "float_float_fp32"):
-        d = res[tag] - res["fp64_cuda_cores"]
-        out[tag]["dtheta_rel_diff"] = float(d.norm() / res["fp64_cuda_cores"].norm())
+    d = res["tcgen05_split_bf16"] - res["tcgen05_fp64_digits"]
+    out["tcgen05_split_bf16"]["dtheta_rel_diff"] = float(d.norm() / res["tcgen05_fp64_digits"].norm())
     print(json.dumps(out), flush=True)
 
 

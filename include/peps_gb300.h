@@ -79,9 +79,8 @@ enum {
 /* Arithmetic of the contraction kernels.  FP64: every step in double.  FP32: the environment,
  * truncation and sandwich arithmetic in float, logarithms and E_loc accumulated in double.
  * MIXED: the reduced-precision preset of the whole step: the FP32 contraction kernels (CUDA
- * cores; logarithms, E_loc and O's scale in double), the MinSR Gram as float-float pairs on the
- * FP32 pipes (cfg.gram == 0 becomes 2; 1 keeps the split-BF16 tensor-core Gram) and the solve as
- * a float-float Cholesky with FP64 refinement and an FP64 fallback (cfg.solve becomes 2); the
+ * cores; logarithms, E_loc and O's scale in double), the MinSR Gram at FP64 accuracy (cfg.gram == 0
+ * becomes 2; 1 keeps the split-BF16 tensor-core Gram) and the solve as a float-float Cholesky with FP64 refinement and an FP64 fallback (cfg.solve becomes 2); the
  * handle then reports FP32 (its O is float). */
 typedef enum { PEPS_PREC_FP64 = 0, PEPS_PREC_FP32 = 1, PEPS_PREC_MIXED = 2 } peps_prec;
 
@@ -94,12 +93,11 @@ typedef struct {
     int chi;      /* boundary-MPS bond dimension D_c (paper's notation), D <= chi <= 64      */
     int prec;     /* peps_prec                                                               */
     int max_samples; /* largest Ns any later call may pass (sizes the environment store)     */
-    int gram;     /* MinSR Gram matrix: 0 = FP64 on CUDA cores; 1 = split BF16 on the tcgen05
-                     tensor cores (Obar = hi + lo, T ~ hi hi^T + hi lo^T + lo hi^T, FP32
-                     accumulation; about 1e-5 relative error per entry); 2 = float-float on
-                     the FP32 pipes (Obar = hi + lo in floats, exact hi products by FMA plus the
-                     cross terms, sums kept as float pairs; about 48 significant bits, for
-                     GPUs whose FP64 rate is a small fraction of their FP32 rate)          */
+    int gram;     /* MinSR Gram matrix: 0 or 2 = FP64 accuracy (each row of Obar as seven signed
+                     8-bit digits of a fixed-point number, the digit products exact on the
+                     tcgen05 tensor cores and summed in 64-bit integers); 1 = split BF16 on the
+                     tcgen05 tensor cores (Obar = hi + lo, T ~ hi hi^T + hi lo^T + lo hi^T, FP32
+                     accumulation; about 1e-5 relative error per entry)                     */
     int solve;    /* MinSR solve when rcond == 0: 0 = FP64 Cholesky; 1 = FP32 Cholesky of
                      T + lambda followed by 4 steps of iterative refinement with FP64 residuals
                      (info[1] reports the final relative residual); 2 = float-float Cholesky
@@ -309,8 +307,8 @@ peps_status peps_local_energy_bound(peps_handle* h, const peps_hamiltonian* H, c
  * lambda is not positive definite in floating point even in FP64 (lambda far below the
  * rounding error of T, e.g. a split-BF16 Gram of badly scaled O), info[0] = -1, dtheta_dev is
  * set to zero and the status word gets PEPS_SW_MINSR_BREAKDOWN (peps_last_status then returns
- * PEPS_W_NUMERIC).  Needs lambda > 0 or rcond > 0.  The Gram matrix is FP64 (cfg.gram == 0), split
- * BF16 on the tensor cores (cfg.gram == 1) or float-float on the FP32 pipes (cfg.gram == 2);
+ * PEPS_W_NUMERIC).  Needs lambda > 0 or rcond > 0.  The Gram matrix has FP64 accuracy
+ * (cfg.gram == 0 or 2) or is split BF16 (cfg.gram == 1), both on the tensor cores;
  * the factorisation is FP64, FP32 or float-float (cfg.solve), the eigendecomposition FP64, the
  * residuals of the refinement FP64.  The call is
  * asynchronous like every other (no host round trip: the mixed solve's FP64 fallback and the

@@ -87,16 +87,15 @@ def sample_flops(Lx, Ly, chi, D, nchains, nsweeps, sweeps, rotations, move="exch
 
 
 def gram_flops(ns, npar):
-    """k_gram computes the lower-triangle 64x64 tiles in full: about (Ns^2/2 + 32 Ns) Np MACs."""
-    nt = (ns + 63) // 64
-    return 2.0 * (nt * (nt + 1) // 2) * 64 * 64 * npar
+    """The Gram kernels compute the lower-triangle 128x128 tiles in full: about
+    (Ns^2/2 + 64 Ns) Np MACs."""
+    nt = (ns + 127) // 128
+    return 2.0 * (nt * (nt + 1) // 2) * 128 * 128 * npar
 
 
-# pipe operations per algorithmic multiply-add of each Gram kernel, counted as flops (2 per
-# issued FMA-pipe operation, so that the figure compares with the FMA peaks): FP64 one FMA;
-# split-BF16 three tensor products; float-float 13 FP32 operations (product and its FMA error,
-# the two cross terms, Knuth's two-sum, three adds into the low word)
-GRAM_PIPE_OPS = {0: 1, 1: 3, 2: 13}
+# BF16 tensor products per algorithmic multiply-add of each Gram kernel: 28 digit products at FP64
+# accuracy (0, 2), three for split BF16 (1)
+GRAM_PIPE_OPS = {0: 28, 1: 3, 2: 28}
 
 
 def gram_pipe_flops(ns, npar, gram):

@@ -92,8 +92,9 @@ struct peps_handle {
   // learned-proposal workspace (allocated on first use)
   uint8_t* lp_Sp = nullptr;
   double *lp_l0 = nullptr, *lp_l1 = nullptr, *lp_aux = nullptr;
-  // split-BF16 operands of the tensor-core Gram
+  // operands of the tensor-core Gram: split BF16 (gram = 1), or the digits (g_hi, g_bytes)
   void *g_hi = nullptr, *g_lo = nullptr;
+  size_t g_bytes = 0;
   // status word (device): OR of the per-sample status bits and the MinSR flags since the last
   // peps_last_status
   int* sword = nullptr;
@@ -1005,12 +1006,15 @@ static peps_status ensure_minsr(peps_handle* h, int Ns, long long Np) {
       h_malloc(h, (void**)&h->ebar, sizeof(double) * n) != cudaSuccess || h_malloc(h, (void**)&h->yv, sizeof(double) * n) != cudaSuccess ||
       h_malloc(h, (void**)&h->xv, sizeof(double) * n) != cudaSuccess || h_malloc(h, (void**)&h->cnt, sizeof(double) * 16) != cudaSuccess)
     return fail(h, PEPS_E_WORKSPACE, "MinSR workspace allocation failed");
-  if (h->cfg.gram == 1 || h->cfg.gram == 2) {
-    if (h->g_hi) { h_free(h, h->g_hi); h->g_hi = nullptr; }
-    if (h->g_lo) { h_free(h, h->g_lo); h->g_lo = nullptr; }
-    const size_t e = (h->cfg.gram == 1) ? (size_t)gram_tc_pad_rows(Ns) * (size_t)gram_tc_pad_k(h->Np) * 2
-                                        : (size_t)n * (size_t)Np * sizeof(float);  // the capacity, n rows
+  if (h->g_hi) { h_free(h, h->g_hi); h->g_hi = nullptr; }
+  if (h->g_lo) { h_free(h, h->g_lo); h->g_lo = nullptr; }
+  if (h->cfg.gram == 1) {
+    const size_t e = (size_t)gram_tc_pad_rows(Ns) * (size_t)gram_tc_pad_k(h->Np) * 2;
     if (h_malloc(h, (void**)&h->g_hi, e) != cudaSuccess || h_malloc(h, (void**)&h->g_lo, e) != cudaSuccess)
+      return fail(h, PEPS_E_WORKSPACE, "Gram workspace allocation failed");
+  } else {
+    h->g_bytes = gram_sl_bytes(n, Np);  // the capacity, n rows
+    if (h_malloc(h, (void**)&h->g_hi, h->g_bytes) != cudaSuccess)
       return fail(h, PEPS_E_WORKSPACE, "Gram workspace allocation failed");
   }
   h->ms_cap = n;
@@ -1030,12 +1034,10 @@ static peps_status minsr_gram_into(peps_handle* h, const double* A, int Ns, long
   if (h->cfg.gram == 1) {
     CK(launch_gram_tc(A, Ns, K, h->g_hi, h->g_lo, T, ld, mirror, gerr, s), "tensor-core Gram");
     tstop(h, ts, s, mirror ? 3 : 2);
-  } else if (h->cfg.gram == 2) {
-    CK(launch_gram_ff(A, Ns, K, (float*)h->g_hi, (float*)h->g_lo, T, ld, s), "float-float Gram");
-    tstop(h, ts, s, 2);
   } else {
-    CK(launch_gram(A, Ns, K, T, ld, s), "Gram");
-    tstop(h, ts, s);
+    long long nl = 0;
+    CK(launch_gram_sl(A, Ns, K, h->g_hi, h->g_bytes, T, ld, gerr, s, &nl), "Gram");
+    tstop(h, ts, s, nl);
   }
   return PEPS_OK;
 }
@@ -1140,7 +1142,7 @@ extern "C" peps_status minsr_step(peps_handle* h, const void* O_dev, const doubl
   if (cx) CK(launch_unembed(h->mean, Np_c, dtheta_dev, s), "dtheta");
   // a breakdown or a Gram timeout zeroes dtheta on the device and is reported through the
   // status word (peps_last_status)
-  CK(launch_minsr_finish(info_dev, h->cfg.gram == 1 ? gerr : nullptr, dtheta_dev, cx ? 2 * Np_c : Np, cx ? 1 : 0,
+  CK(launch_minsr_finish(info_dev, gerr, dtheta_dev, cx ? 2 * Np_c : Np, cx ? 1 : 0,
                          rcond > 0.0 ? 0 : 1, h->sword, s),
      "MinSR finish");
   tstop(h, ts, s, cx ? 4 : 3);
@@ -1200,7 +1202,7 @@ extern "C" peps_status minsr_gram(peps_handle* h, const double* A_dev, int Ns, l
   CK(cudaMemsetAsync(T_dev, 0, sizeof(double) * (size_t)Ns * Ns, s), "memset");
   if (K == 0) return PEPS_OK;
   if ((ps = minsr_gram_into(h, A_dev, Ns, K, T_dev, Ns, true, s)) != PEPS_OK) return ps;
-  if (h->cfg.gram == 1) CK(launch_flag_or(gerr, PEPS_SW_GRAM_TIMEOUT, h->sword, s), "status word");
+  CK(launch_flag_or(gerr, PEPS_SW_GRAM_TIMEOUT, h->sword, s), "status word");
   return PEPS_OK;
 }
 

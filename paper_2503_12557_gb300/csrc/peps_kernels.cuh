@@ -225,10 +225,13 @@ cudaError_t launch_partial_sums(const TO* O, const double* w, const double* eloc
 template <typename TO>
 cudaError_t launch_center_global(const TO* O, const double* w, const double* eloc, int Ns, long long Np,
                                  const double* g, double* Obar, double* ebar, cudaStream_t s);
-cudaError_t launch_gram(const double* Obar, int Ns, long long Np, double* Tm, int ld, cudaStream_t s);
-// float-float Gram on the FP32 pipes (hi, lo: Ns x Np floats of scratch)
-cudaError_t launch_gram_ff(const double* Obar, int Ns, long long Np, float* hi, float* lo, double* Tm, int ld,
-                           cudaStream_t s);
+// T = A A^T (Ns x Ns, both triangles; its lower triangle zero on entry, leading dimension ld) at
+// FP64 accuracy from BF16 digits on the tensor cores (peps_gram_sl.cu).  ws: scratch of at least
+// the digits of 32 columns, gram_sl_bytes(Ns, K) for the fewest launches; err: device int, set to 1
+// when a pipeline wait timed out; *launches = kernels launched.
+size_t gram_sl_bytes(int Ns, long long K);
+cudaError_t launch_gram_sl(const double* A, int Ns, long long K, void* ws, size_t ws_bytes, double* Tm, int ld, int* err,
+                           cudaStream_t s, long long* launches);
 // cyclic Jacobi eigendecomposition of the symmetric n x n matrix A (overwritten by its
 // diagonal form), V accumulates the rotations, *info_sweeps (device) = sweeps used or -1 at the
 // limit; one cooperative launch (hbuf: n x n scratch, cs: n doubles of scratch, cnt: 2 device

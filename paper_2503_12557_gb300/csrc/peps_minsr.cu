@@ -241,52 +241,6 @@ template cudaError_t launch_center_global<double>(const double*, const double*, 
 template cudaError_t launch_center_global<float>(const float*, const double*, const double*, int, long long,
                                                  const double*, double*, double*, cudaStream_t);
 
-// ---- Gram T = Obar Obar^T, 64 x 64 output tiles, K staged through shared memory in chunks
-// of 16; only tiles with ti >= tj are computed, the upper triangle is mirrored.
-constexpr int GT = 64, GK = 16;
-__global__ void __launch_bounds__(256) k_gram(const double* __restrict__ Ob, int Ns, long long Np, double* Tm, int ld) {
-  __shared__ double As[GK][GT + 1], Bs[GK][GT + 1];
-  const int nt = (Ns + GT - 1) / GT;
-  // linear index over lower-triangle tiles
-  int t = blockIdx.x, ti = 0;
-  while (t >= ti + 1) { t -= ti + 1; ++ti; }
-  const int tj = t;
-  if (ti >= nt) return;
-  const int r0 = ti * GT, c0 = tj * GT;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;  // each thread: 4 x 4 outputs
-  double acc[4][4] = {};
-  for (long long k0 = 0; k0 < Np; k0 += GK) {
-    for (int o = threadIdx.x; o < GK * GT; o += blockDim.x) {
-      const int kk = o % GK, rr = o / GK;
-      const long long k = k0 + kk;
-      As[kk][rr] = (r0 + rr < Ns && k < Np) ? Ob[(size_t)(r0 + rr) * Np + k] : 0.0;
-      Bs[kk][rr] = (c0 + rr < Ns && k < Np) ? Ob[(size_t)(c0 + rr) * Np + k] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < GK; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = As[kk][ty * 4 + i]; b[i] = Bs[kk][tx * 4 + i]; }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int r = r0 + ty * 4 + i, c = c0 + tx * 4 + j;
-      if (r < Ns && c < Ns) {
-        Tm[(size_t)r * ld + c] = acc[i][j];
-        Tm[(size_t)c * ld + r] = acc[i][j];
-      }
-    }
-}
-
 // ---- cyclic Jacobi, parallel round-robin ordering.  One launch per round: every thread owns
 // one 2x2 block (pair I, pair J) of the old matrix and writes the rotated block into the new
 // one; rotation parameters are recomputed from the old diagonal blocks (classical two-sided
@@ -514,113 +468,6 @@ cudaError_t launch_center_e(const double* eloc, const double* w, int Ns, double*
   return cudaGetLastError();
 }
 
-// ---- float-float ("double-single") Gram on the FP32 pipes
-// Obar split once into hi = float(x), lo = float(x - hi) (x = hi + lo to about 48 bits).
-__global__ void k_split_ff(const double* __restrict__ x, size_t n, float* __restrict__ hi, float* __restrict__ lo) {
-  for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < n; o += (size_t)gridDim.x * blockDim.x) {
-    const double v = x[o];
-    const float h = __double2float_rn(v);
-    hi[o] = h;
-    lo[o] = __double2float_rn(v - (double)h);
-  }
-}
-
-// T = Obar Obar^T from the float pairs: each product a b with a = ah + al, b = bh + bl is taken
-// as p + e + c, p = ah bh rounded, e = fma(ah, bh, -p) its exact error, c = ah bl + al bh (al bl,
-// about 2^-48 of the product, dropped); the running sum is a float pair (sh, sl): sh + p by
-// Knuth's two-sum, its error and e + c into sl, renormalised after every GK k-steps; the result
-// is sh + sl in double.  The error-free steps use the _rn intrinsics so that no multiply and add
-// are fused.  Same lower-triangle 64 x 64 tiling as k_gram.
-__global__ void __launch_bounds__(256) k_gram_ff(const float* __restrict__ Oh, const float* __restrict__ Ol, int Ns,
-                                                 long long Np, double* Tm, int ld) {
-  __shared__ float Ah[GK][GT + 1], Al[GK][GT + 1], Bh[GK][GT + 1], Bl[GK][GT + 1];
-  const int nt = (Ns + GT - 1) / GT;
-  int t = blockIdx.x, ti = 0;
-  while (t >= ti + 1) { t -= ti + 1; ++ti; }
-  const int tj = t;
-  if (ti >= nt) return;
-  const int r0 = ti * GT, c0 = tj * GT;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  float sh[4][4], sl[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) { sh[i][j] = 0.f; sl[i][j] = 0.f; }
-  for (long long k0 = 0; k0 < Np; k0 += GK) {
-    for (int o = threadIdx.x; o < GK * GT; o += blockDim.x) {
-      const int kk = o % GK, rr = o / GK;
-      const long long k = k0 + kk;
-      const bool ra = (r0 + rr < Ns && k < Np), rb = (c0 + rr < Ns && k < Np);
-      Ah[kk][rr] = ra ? Oh[(size_t)(r0 + rr) * Np + k] : 0.f;
-      Al[kk][rr] = ra ? Ol[(size_t)(r0 + rr) * Np + k] : 0.f;
-      Bh[kk][rr] = rb ? Oh[(size_t)(c0 + rr) * Np + k] : 0.f;
-      Bl[kk][rr] = rb ? Ol[(size_t)(c0 + rr) * Np + k] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < GK; ++kk) {
-      float ah[4], al[4], bh[4], bl[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        ah[i] = Ah[kk][ty * 4 + i]; al[i] = Al[kk][ty * 4 + i];
-        bh[i] = Bh[kk][tx * 4 + i]; bl[i] = Bl[kk][tx * 4 + i];
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float p = __fmul_rn(ah[i], bh[j]);
-          const float e = __fmaf_rn(ah[i], bh[j], -p);
-          const float c = __fmaf_rn(ah[i], bl[j], __fmul_rn(al[i], bh[j]));
-          const float s0 = __fadd_rn(sh[i][j], p);
-          const float bb = __fsub_rn(s0, sh[i][j]);
-          const float er = __fadd_rn(__fsub_rn(sh[i][j], __fsub_rn(s0, bb)), __fsub_rn(p, bb));
-          sh[i][j] = s0;
-          sl[i][j] = __fadd_rn(sl[i][j], __fadd_rn(er, __fadd_rn(e, c)));
-        }
-    }
-    // renormalise the pairs (fast two-sum: |sh| >= |sl|)
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float s0 = __fadd_rn(sh[i][j], sl[i][j]);
-        sl[i][j] = __fsub_rn(sl[i][j], __fsub_rn(s0, sh[i][j]));
-        sh[i][j] = s0;
-      }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int r = r0 + ty * 4 + i, c = c0 + tx * 4 + j;
-      // the cross terms make the pair (r, c) and (c, r) round differently: only the lower
-      // entry's thread writes both (a diagonal tile would otherwise race on them)
-      if (r < Ns && c < Ns && c <= r) {
-        const double v = (double)sh[i][j] + (double)sl[i][j];
-        Tm[(size_t)r * ld + c] = v;
-        Tm[(size_t)c * ld + r] = v;
-      }
-    }
-}
-
-cudaError_t launch_gram_ff(const double* Obar, int Ns, long long Np, float* hi, float* lo, double* Tm, int ld,
-                           cudaStream_t s) {
-  const size_t n = (size_t)Ns * (size_t)Np;
-  k_split_ff<<<1216, 256, 0, s>>>(Obar, n, hi, lo);
-  const int nt = (Ns + GT - 1) / GT;
-  k_gram_ff<<<nt * (nt + 1) / 2, 256, 0, s>>>(hi, lo, Ns, Np, Tm, ld);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gram(const double* Obar, int Ns, long long Np, double* Tm, int ld, cudaStream_t s) {
-  const int nt = (Ns + GT - 1) / GT;
-  const int ntiles = nt * (nt + 1) / 2;
-  k_gram<<<ntiles, 256, 0, s>>>(Obar, Ns, Np, Tm, ld);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_minsr_apply(const double* A, const double* V, const double* ebar, int n, int nreal, double lambda,
                                double rcond, double* y, double* x, double* info, cudaStream_t s) {
   k_minsr_scalars<<<1, 1024, 0, s>>>(A, n, nreal, rcond, info);
@@ -812,8 +659,8 @@ __global__ void __launch_bounds__(256) k_chol_update(T* A, int n, int k0, const 
 // The same trailing update on the float-float factor: the panel's columns as float pairs, each
 // product a b = (ah + al)(bh + bl) taken as p + e + c (p = ah bh rounded, e its exact error by
 // fma, c = ah bl + al bh; al bl, about 2^-48 of the product, dropped) and summed into a float
-// pair by Knuth's two-sum, as the float-float Gram does; the pair is then subtracted from A_ij
-// with one more two-sum and stored renormalised.
+// pair by Knuth's two-sum; the pair is then subtracted from A_ij with one more two-sum and stored
+// renormalised.
 constexpr int UK = 32;  // panel columns staged per pass (four UK x CB float tiles: 33 KB)
 __global__ void __launch_bounds__(256) k_chol_update_ff(float* Ah, float* Al, int n, int k0, const int* gate) {
   if (gate && !*gate) return;
@@ -1160,8 +1007,8 @@ long long chol_solve_mixed(double* A, float* A32, int n, int nreal, double lambd
   return launches;
 }
 
-// ---- float-float factor (solve = 2): T + lambda split into float pairs (about 48 bits, the
-// precision of the float-float Gram that usually produced T), the trailing updates on the FP32
+// ---- float-float factor (solve = 2): T + lambda split into float pairs (about 48 bits), the
+// trailing updates on the FP32
 // pipes (k_chol_update_ff), the diagonal blocks and panels in FP64 through the pair accessor,
 // then `iters` steps of refinement with FP64 residuals as in the FP32 mixed solve.  On this part
 // FP64 runs at 1/64 of the FP32 rate, so the factor's n^3/6 multiply-adds cost several times
