@@ -49,7 +49,7 @@ def _args():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--solve", default=None, choices=["ff", "fp64", "fp32"],
-                    help="MinSR Cholesky: float-float factor + FP64 refinement (FP32 default), FP64 "
+                    help="MinSR Cholesky: FP64 factor + refinement (ff, the FP32 default), FP64 "
                          "(FP64 default), or FP32 factor + FP64 refinement")
     ap.add_argument("--gram", default=None, choices=["ff", "fp64", "bf16"],
                     help="MinSR Gram of the step: FP64 accuracy from digits on the tensor cores (ff and fp64 "
@@ -424,7 +424,7 @@ def run_gpu(a):
             "config": _config(w, ns, a.sweeps), "step_ms": step_ms, "minsr_step_s": minsr_s,
             "minsr": {"gram": "split-BF16 tcgen05" if gram == 1 else "FP64 accuracy, 7 BF16 digits on tcgen05",
                       "solve": {0: "FP64 Cholesky", 1: "FP32 Cholesky + FP64 refinement",
-                                2: "float-float Cholesky + FP64 refinement"}[solve],
+                                2: "FP64 Cholesky + refinement"}[solve],
                       "sharded_over_processes": world > 1,
                       "gram_ms": ms_cls["minsr_gram"] / a.steps, "solve_ms": ms_cls["minsr_eig"] / a.steps,
                       "gram_tflops_algorithmic": (flops["minsr_gram"] / a.steps /

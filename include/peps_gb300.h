@@ -80,8 +80,8 @@ enum {
  * truncation and sandwich arithmetic in float, logarithms and E_loc accumulated in double.
  * MIXED: the reduced-precision preset of the whole step: the FP32 contraction kernels (CUDA
  * cores; logarithms, E_loc and O's scale in double), the MinSR Gram at FP64 accuracy (cfg.gram == 0
- * becomes 2; 1 keeps the split-BF16 tensor-core Gram) and the solve as a float-float Cholesky with FP64 refinement and an FP64 fallback (cfg.solve becomes 2); the
- * handle then reports FP32 (its O is float). */
+ * becomes 2; 1 keeps the split-BF16 tensor-core Gram) and the solve as an FP64 Cholesky with
+ * FP64 refinement (cfg.solve becomes 2); the handle then reports FP32 (its O is float). */
 typedef enum { PEPS_PREC_FP64 = 0, PEPS_PREC_FP32 = 1, PEPS_PREC_MIXED = 2 } peps_prec;
 
 typedef enum { PEPS_MOVE_EXCHANGE = 0, PEPS_MOVE_FLIP = 1 } peps_move;
@@ -100,11 +100,8 @@ typedef struct {
                      accumulation; about 1e-5 relative error per entry)                     */
     int solve;    /* MinSR solve when rcond == 0: 0 = FP64 Cholesky; 1 = FP32 Cholesky of
                      T + lambda followed by 4 steps of iterative refinement with FP64 residuals
-                     (info[1] reports the final relative residual); 2 = float-float Cholesky
-                     (T + lambda as float pairs of about 48 bits, the trailing updates on the
-                     FP32 pipes, diagonal blocks and panels in FP64) followed by 2 steps of
-                     refinement with FP64 residuals: the FP64 factor's work at a fraction of
-                     its time on GPUs whose FP64 rate is a small fraction of their FP32 rate;
+                     (info[1] reports the final relative residual); 2 = FP64 Cholesky of a copy
+                     of T + lambda followed by 2 steps of refinement with FP64 residuals;
                      3 = FP64 Cholesky when rcond == 0, and the tridiagonal eigen route (see
                      minsr_step) instead of the cyclic Jacobi when rcond > 0 */
     int cplx;     /* 0 = real PEPS; 1 = complex PEPS: theta is N_p (re, im) pairs of doubles,
@@ -302,14 +299,13 @@ peps_status peps_local_energy_bound(peps_handle* h, const peps_hamiltonian* H, c
  * with cfg.solve == 0, info = (Ns, |ebar - (T + lambda) x| / |ebar|, refinement steps, -1)
  * with cfg.solve == 1, where refinement steps = 0 means that the FP32 factor failed or the
  * refined residual stayed above 1e-10 and the FP64 factorisation was used instead; the same
- * with cfg.solve == 2, where the FP64 factorisation replaces the float-float one only when the
- * latter breaks down (a pivot that is not positive).  When T +
+ * with cfg.solve == 2, whose factor is FP64 to begin with.  When T +
  * lambda is not positive definite in floating point even in FP64 (lambda far below the
  * rounding error of T, e.g. a split-BF16 Gram of badly scaled O), info[0] = -1, dtheta_dev is
  * set to zero and the status word gets PEPS_SW_MINSR_BREAKDOWN (peps_last_status then returns
  * PEPS_W_NUMERIC).  Needs lambda > 0 or rcond > 0.  The Gram matrix has FP64 accuracy
  * (cfg.gram == 0 or 2) or is split BF16 (cfg.gram == 1), both on the tensor cores;
- * the factorisation is FP64, FP32 or float-float (cfg.solve), the eigendecomposition FP64, the
+ * the factorisation is FP64 or FP32 (cfg.solve), the eigendecomposition FP64, the
  * residuals of the refinement FP64.  The call is
  * asynchronous like every other (no host round trip: the mixed solve's FP64 fallback and the
  * zeroing of dtheta on a breakdown are decided on the device; rcond > 0 runs the whole cyclic

@@ -81,6 +81,7 @@ struct peps_handle {
   long long ms_np = 0;
   double *Obar = nullptr, *Tm = nullptr, *Vm = nullptr, *Hm = nullptr, *mean = nullptr, *ebar = nullptr,
          *yv = nullptr, *xv = nullptr, *cnt = nullptr;
+  void* cw = nullptr;    // FP64 Cholesky: digits, inverted diagonal blocks (chol64_ws_bytes)
   double* td = nullptr;  // tridiagonal eigen route: vectors and partial sums (td_workspace_doubles)
   // timing: event pairs per kernel class, recorded on the call's stream when enabled
   bool timing = false;
@@ -397,8 +398,8 @@ extern "C" peps_status peps_create_ex(peps_handle** out, const peps_config* cfg,
     return PEPS_E_SHAPE;
   if (c.prec != PEPS_PREC_FP64 && c.prec != PEPS_PREC_FP32 && c.prec != PEPS_PREC_MIXED) return PEPS_E_ARG;
   if (c.prec == PEPS_PREC_MIXED) {
-    // the mixed-precision preset: the FP32 contraction kernels, a float-float Gram unless the
-    // caller asked for the tensor-core one, and the float-float Cholesky with FP64 refinement
+    // the mixed-precision preset: the FP32 contraction kernels, the FP64-accurate Gram unless the
+    // caller asked for the split-BF16 one, and the Cholesky with FP64 refinement
     c.prec = PEPS_PREC_FP32;
     if (c.gram == 0) c.gram = 2;
     c.solve = 2;
@@ -469,7 +470,7 @@ extern "C" peps_status peps_destroy(peps_handle* h) {
   if (!h) return PEPS_E_ARG;
   void* ptrs[] = {h->Tpad, h->site_off, h->envs, h->logs, h->wdisc, h->rowout, h->pairout, h->status_tmp,
                   h->gscratch, h->d_tinfo, h->d_ab, h->d_eh, h->d_rowoff, h->d_pairoff, h->d_pij, h->d_pv,
-                  h->d_onsite, h->Obar, h->Tm, h->Vm, h->Hm, h->mean, h->ebar, h->yv, h->xv, h->cnt, h->td, h->ctr,
+                  h->d_onsite, h->Obar, h->Tm, h->Vm, h->Hm, h->mean, h->ebar, h->yv, h->xv, h->cnt, h->td, h->cw, h->ctr,
                   h->lp_Sp, h->lp_l0, h->lp_l1, h->lp_aux, h->g_hi, h->g_lo, h->bout, h->DL, h->dl_work,
                   h->dl_status, h->dscratch, h->ustat, h->sword};
   for (void* p : ptrs)
@@ -1006,6 +1007,9 @@ static peps_status ensure_minsr(peps_handle* h, int Ns, long long Np) {
       h_malloc(h, (void**)&h->ebar, sizeof(double) * n) != cudaSuccess || h_malloc(h, (void**)&h->yv, sizeof(double) * n) != cudaSuccess ||
       h_malloc(h, (void**)&h->xv, sizeof(double) * n) != cudaSuccess || h_malloc(h, (void**)&h->cnt, sizeof(double) * 16) != cudaSuccess)
     return fail(h, PEPS_E_WORKSPACE, "MinSR workspace allocation failed");
+  if (h->cw) { h_free(h, h->cw); h->cw = nullptr; }
+  if (h_malloc(h, &h->cw, chol64_ws_bytes(n)) != cudaSuccess)
+    return fail(h, PEPS_E_WORKSPACE, "MinSR workspace allocation failed");
   if (h->g_hi) { h_free(h, h->g_hi); h->g_hi = nullptr; }
   if (h->g_lo) { h_free(h, h->g_lo); h->g_lo = nullptr; }
   if (h->cfg.gram == 1) {
@@ -1074,18 +1078,22 @@ static peps_status minsr_solve_core(peps_handle* h, int Ns, double lambda, doubl
     const int ts = tstart(h, TC_EIG, s);
     long long nl = 0;
     if (h->cfg.solve == 1 || h->cfg.solve == 2) {
+      // the refinement's residuals read the whole of T: its upper triangle from the lower one
+      // (the split-BF16 Gram and a caller's T may leave it unset)
+      CK(launch_mirror_lower(h->Tm, n, s), "mirror");
       // h->Hm: the residual norms' block partials at its start, the solves' vector from n on;
-      // h->Vm (n x n doubles) holds the FP32 factor, or the float-float factor's two n x n halves
-      if (h->cfg.solve == 1)
-        nl = chol_solve_mixed(h->Tm, (float*)h->Vm, n, Ns, lambda, h->ebar, h->xv, h->yv, h->cnt + 6, h->Hm, 4,
-                              (int*)h->cnt, info_dev, need64, h->Hm + n, s, &e);
-      else
-        nl = chol_solve_ff(h->Tm, (float*)h->Vm, (float*)h->Vm + (size_t)n * n, n, Ns, lambda, h->ebar, h->xv, h->yv,
-                           h->cnt + 6, h->Hm, 2, (int*)h->cnt, info_dev, need64, h->Hm + n, s, &e);
-      if (e != cudaSuccess) return cuda_fail(h, e, "Cholesky");
-      nl += chol_solve(h->Tm, n, Ns, lambda, h->ebar, h->xv, (int*)h->cnt, info_dev, need64, h->yv, s, &e);
+      // h->Vm (n x n doubles) holds the factor
+      if (h->cfg.solve == 1) {
+        nl = 1 + chol_solve_mixed(h->Tm, (float*)h->Vm, n, Ns, lambda, h->ebar, h->xv, h->yv, h->cnt + 6, h->Hm, 4,
+                                  (int*)h->cnt, info_dev, need64, h->Hm + n, s, &e);
+        if (e != cudaSuccess) return cuda_fail(h, e, "Cholesky");
+        nl += chol_solve(h->Tm, n, Ns, lambda, h->ebar, h->xv, (int*)h->cnt, info_dev, need64, h->yv, h->cw, s, &e);
+      } else {
+        nl = 1 + chol_solve_refined(h->Tm, h->Vm, n, Ns, lambda, h->ebar, h->xv, h->yv, h->cnt + 6, h->Hm, 2,
+                                    (int*)h->cnt, info_dev, h->Hm + n, h->cw, s, &e);
+      }
     } else {
-      nl = chol_solve(h->Tm, n, Ns, lambda, h->ebar, h->xv, (int*)h->cnt, info_dev, nullptr, h->yv, s, &e);
+      nl = chol_solve(h->Tm, n, Ns, lambda, h->ebar, h->xv, (int*)h->cnt, info_dev, nullptr, h->yv, h->cw, s, &e);
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "Cholesky");
     tstop(h, ts, s, nl);

@@ -27,22 +27,12 @@
 #include <cuda_bf16.h>
 
 #include "peps_kernels.cuh"
-#include "peps_tma.cuh"
+#include "peps_slices.cuh"
 
 namespace peps {
 namespace {
 
-constexpr int NS = 7;                        // digits
-constexpr int SM_ = 128;                     // tile rows and columns
-constexpr int CK = 32;                       // columns of Obar per stage (64 bytes: one 64B-swizzle row)
-constexpr int SSTAGES = 2;
-constexpr int STILE = SM_ * CK * 2;          // 8 KB: one digit of one row block
-constexpr int SOPND = NS * STILE;            // 56 KB
-constexpr int SSTAGE = 2 * SOPND;            // 112 KB
-constexpr int EPI_WARPS = 8;
-constexpr int SL_THREADS = (EPI_WARPS + 2) * 32;
 constexpr int F_MAX = 52, F_MIN = 38;        // range of f
-constexpr int ROW_NONFINITE = -1;
 
 // f and the extra row exponent t (t > 0 only when the largest scaled squared row norm exceeds
 // 2^23, i.e. beyond 8 million columns) from nmax, the largest sum_k (x_k / 2^e)^2 of any row.
@@ -114,76 +104,13 @@ __global__ void __launch_bounds__(256) k_slice_digits(const double* __restrict__
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const unsigned long long b = (E >= 0 && kb + j < kw) ? x[j] : 0ull;
-      const int ex = (int)(b >> 52) & 0x7ff;
-      const int sh = E + t - max(ex, 1);
-      unsigned long long m = (b & 0xfffffffffffffull) | (ex ? 0x10000000000000ull : 0ull);
-      m <<= 2;  // below 2^55
-      if (sh > 0) m = sh < 60 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
-      long long q = (b >> 63) ? -(long long)m : (long long)m;
-#pragma unroll
-      for (int p = NS - 1; p >= 0; --p) {
-        const int d = p ? (int)(signed char)(q & 0xff) : (int)q;
-        if (p) q = (q - d) >> 8;
-        const uint32_t h = (uint32_t)__bfloat16_as_ushort(__int2bfloat16_rn(d));
-        if (j & 1) w[p][j >> 1] |= h << 16;
-        else w[p][j >> 1] = h;
-      }
+      put_digits(fixed_point(b, E + t), j, w);
     }
 #pragma unroll
     for (int p = 0; p < NS; ++p)
       *reinterpret_cast<uint4*>(D + p * plane + (size_t)r * Kpad + kb) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
   }
 }
-
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
-          smem_u32(dst)),
-      "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
-      : "memory");
-}
-
-// K-major operand tile of 128 rows x 32 bf16 in the 64-byte swizzle: 8-row groups 512 bytes apart
-// (stride byte offset), layout code 4 at bits [61, 64); the other fields as for 128 bytes.
-__device__ __forceinline__ uint64_t desc64(uint32_t addr) {
-  return (uint64_t)((addr >> 4) & 0x3FFF) | (1ull << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
-}
-constexpr uint32_t SL_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(SM_ >> 3) << 17) | ((uint32_t)(SM_ >> 4) << 24);
-__device__ __forceinline__ void mma_sl(uint32_t tmem, uint64_t a, uint64_t b, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(SL_IDESC), "r"(acc));
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// bounded wait that also gives up when another role of the CTA has failed
-__device__ __forceinline__ bool wait_ok(uint64_t* bar, uint32_t parity, int* failed) {
-  if (mbar_try(bar, parity)) return true;
-  unsigned long long t0, t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
-  do {
-    if (mbar_try(bar, parity)) return true;
-    if (*(volatile int*)failed) return false;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  } while (t - t0 < 1000000000ull);  // one second; a unit takes microseconds
-  atomicExch(failed, 1);
-  return false;
-}
-// 16 accumulator columns of this warp's 32 tensor-memory lanes
-__device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&v)[16]) {
-  uint32_t u[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), "=r"(u[8]),
-        "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
-      : "r"(addr));
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(u[i]);
-}
-__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// integer of an exact FP32 integer |v| <= 2^22
-__device__ __forceinline__ int f2i_exact(float v) { return __float_as_int(__fadd_rn(v, 12582912.f)) - 0x4B400000; }
 
 // One CTA per (tile, K part): a 128 x 128 tile on or below the diagonal over the chunks [c0, c1).
 // Warp 8 loads (two TMA boxes of 32 columns x 128 rows x 7 digits per chunk, double buffered),

@@ -219,12 +219,12 @@ cudaError_t launch_gram_tc(const double* Obar, int Ns, long long Np, void* hi, v
   if (e != cudaSuccess) return e;
   k_gram_tc<<<ntile * (ntile + 1) / 2, 128, smem, s>>>(mh, ml, ntile, nk, Ns, Tm, ld, err);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (mirror) {
-    dim3 grid((ld + 31) / 32, (ld + 31) / 32), block(32, 8);
-    k_mirror_lower<<<grid, block, 0, s>>>(Tm, ld);
-    e = cudaGetLastError();
-  }
-  return e;
+  return mirror ? launch_mirror_lower(Tm, ld, s) : cudaSuccess;
+}
+
+cudaError_t launch_mirror_lower(double* T, int n, cudaStream_t s) {
+  k_mirror_lower<<<dim3((n + 31) / 32, (n + 31) / 32), dim3(32, 8), 0, s>>>(T, n);
+  return cudaGetLastError();
 }
 
 }  // namespace peps

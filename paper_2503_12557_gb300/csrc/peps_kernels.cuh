@@ -252,25 +252,29 @@ cudaError_t td_pinv_apply(double* A, int ld, int N, const double* ebar, double l
                           cudaStream_t s, long long* launches);
 cudaError_t launch_obar_t_x(const double* Obar, const double* x, int Ns, long long Np, double tau, double* dtheta,
                             cudaStream_t s);
-// x = (A + lambda I)^-1 ebar by blocked Cholesky (A overwritten by its factor); returns launches
-// gate (device flag, may be NULL): every launch does nothing while *gate == 0 (the FP64
-// fallback of the mixed solve, decided on the device); a gated run sets info[2] = 0;
-// scratch: n doubles (the triangular solves' intermediate vector)
+// r = b - (A + lambda) x for the full symmetric A (part: 2 (n + 7) / 8 doubles of scratch; rn, may
+// be NULL: |r|^2 and |b|^2); returns launches
+long long launch_residual(const double* A, int n, int nreal, double lambda, const double* b, const double* x, double* r,
+                          double* part, double* rn, cudaStream_t s);
+// x = (A + lambda I)^-1 ebar by blocked FP64 Cholesky (peps_chol.cu; n even, A's lower triangle
+// overwritten by its factor); returns launches.  gate (device flag, may be NULL): every launch does
+// nothing while *gate == 0 (the FP64 fallback of the mixed solve, decided on the device); a gated
+// run sets info[2] = 0; scratch: n doubles; ws: chol64_ws_bytes(n) bytes
+size_t chol64_ws_bytes(int n);
 long long chol_solve(double* A, int n, int nreal, double lambda, const double* ebar, double* x, int* bad,
-                     double* info, const int* gate, double* scratch, cudaStream_t s, cudaError_t* err);
-// the same solve with an FP32 factor (A32: n x n floats, A kept and mirrored to full) and
-// `iters` refinement steps with FP64 residuals (r: n doubles, rn: 2 doubles, part: 2 (n + 7) / 8
-// doubles of scratch, scratch: n doubles);
-// info = (Ns or -1, relative residual, iters, -); *need64 (device) = 1 when the FP64
-// factorisation must replace it (factor breakdown or relative residual above 1e-10)
+                     double* info, const int* gate, double* scratch, void* ws, cudaStream_t s, cudaError_t* err);
+// the same factor of a copy F (n x n doubles) of A + lambda (A full and kept), then `iters`
+// refinement steps with FP64 residuals (r: n doubles, rn: 2 doubles, part as launch_residual);
+// info = (Ns or -1, relative residual, iters, -)
+long long chol_solve_refined(double* A, double* F, int n, int nreal, double lambda, const double* ebar, double* x,
+                             double* r, double* rn, double* part, int iters, int* bad, double* info, double* scratch,
+                             void* ws, cudaStream_t s, cudaError_t* err);
+// the refined solve with an FP32 factor (A32: n x n floats; A full and kept);
+// *need64 (device) = 1 when the FP64 factorisation must replace it (factor breakdown or relative
+// residual above 1e-10)
 long long chol_solve_mixed(double* A, float* A32, int n, int nreal, double lambda, const double* ebar, double* x,
                            double* r, double* rn, double* part, int iters, int* bad, double* info, int* need64,
                            double* scratch, cudaStream_t s, cudaError_t* err);
-// the same with the float-float factor (Fh, Fl: n x n floats each); *need64 = 1 only when the
-// pair factorisation broke down; info = (Ns or -1, relative residual after refinement, iters, -)
-long long chol_solve_ff(double* A, float* Fh, float* Fl, int n, int nreal, double lambda, const double* ebar, double* x,
-                        double* r, double* rn, double* part, int iters, int* bad, double* info, int* need64,
-                        double* scratch, cudaStream_t s, cudaError_t* err);
 // ---- learned proposal (peps_proposal.cu)
 size_t prop_smem_bytes(int Lx, int Ly, int C, int act_bytes, bool train);
 cudaError_t launch_prop_logits(int Lx, int Ly, int C, int wprec, const void* w, const uint8_t* S, int Ns, double* logits,
@@ -290,6 +294,8 @@ int gram_tc_pad_rows(int Ns);
 long long gram_tc_pad_k(long long Np);
 cudaError_t launch_gram_tc(const double* Obar, int Ns, long long Np, void* hi, void* lo, double* Tm, int ld, bool mirror,
                            int* err, cudaStream_t s);
+// upper triangle of T (n x n) from the lower one
+cudaError_t launch_mirror_lower(double* T, int n, cudaStream_t s);
 // y += x (n doubles)
 cudaError_t launch_axpy(double* y, const double* x, long long n, cudaStream_t s);
 
