@@ -33,7 +33,6 @@ struct peps_handle {
   std::vector<long long> site_off_h;
   void* envs = nullptr;
   double* logs = nullptr;
-  float* wdisc = nullptr;
   double* rowout = nullptr;
   double* pairout = nullptr;
   int* status_tmp = nullptr;
@@ -447,7 +446,6 @@ extern "C" peps_status peps_create_ex(peps_handle** out, const peps_config* cfg,
   const size_t envb = (size_t)c.max_samples * 2 * c.Lx * c.Ly * g.se * h->esz;
   if (h_malloc(h, (void**)&h->envs, envb) != cudaSuccess) return bad(PEPS_E_WORKSPACE, "environment store");
   if (h_malloc(h, (void**)&h->logs, sizeof(double) * (size_t)c.max_samples * 2 * c.Lx) != cudaSuccess) return bad(PEPS_E_WORKSPACE, "logs");
-  if (h_malloc(h, (void**)&h->wdisc, sizeof(float) * (size_t)c.max_samples) != cudaSuccess) return bad(PEPS_E_WORKSPACE, "wdisc");
   if (h_malloc(h, (void**)&h->rowout, sizeof(double) * 4 * (size_t)c.max_samples * c.Lx) != cudaSuccess) return bad(PEPS_E_WORKSPACE, "rowout");
   if (h_malloc(h, (void**)&h->pairout, sizeof(double) * 4 * (size_t)c.max_samples * c.Lx) != cudaSuccess) return bad(PEPS_E_WORKSPACE, "pairout");
   if (h_malloc(h, (void**)&h->status_tmp, sizeof(int) * (size_t)c.max_samples) != cudaSuccess) return bad(PEPS_E_WORKSPACE, "status");
@@ -468,7 +466,7 @@ extern "C" peps_status peps_create_ex(peps_handle** out, const peps_config* cfg,
 
 extern "C" peps_status peps_destroy(peps_handle* h) {
   if (!h) return PEPS_E_ARG;
-  void* ptrs[] = {h->Tpad, h->site_off, h->envs, h->logs, h->wdisc, h->rowout, h->pairout, h->status_tmp,
+  void* ptrs[] = {h->Tpad, h->site_off, h->envs, h->logs, h->rowout, h->pairout, h->status_tmp,
                   h->gscratch, h->d_tinfo, h->d_ab, h->d_eh, h->d_rowoff, h->d_pairoff, h->d_pij, h->d_pv,
                   h->d_onsite, h->Obar, h->Tm, h->Vm, h->Hm, h->mean, h->ebar, h->yv, h->xv, h->cnt, h->td, h->cw, h->ctr,
                   h->lp_Sp, h->lp_l0, h->lp_l1, h->lp_aux, h->g_hi, h->g_lo, h->bout, h->DL, h->dl_work,
@@ -652,7 +650,6 @@ static peps_status run_eval(peps_handle* h, const peps_hamiltonian* H, const uin
                      h->rs_gen == h->param_gen && !(h->rs_up && sides == 1);
   if (reuse) CK(cudaMemcpyAsync(st, h->ustat, sizeof(int) * Ns, cudaMemcpyDeviceToDevice, s), "copy status");
   else CK(cudaMemsetAsync(st, 0, sizeof(int) * Ns, s), "memset status");
-  CK(cudaMemsetAsync(h->wdisc, 0, sizeof(float) * Ns, s), "memset wdisc");
   if (Ns == 0) return PEPS_OK;
   if (reuse) sides = (sides == 3) ? (h->rs_up ? 1 : 2) : 0;
   else h->rs_gen = -1;  // the store's upper rows now belong to this batch
@@ -674,7 +671,7 @@ static peps_status run_eval(peps_handle* h, const peps_hamiltonian* H, const uin
   if (sides != 0) {
     ts = tstart(h, TC_ENV, s);
     CK(launch_env<T>(g, ke.p, std::min(ke.grid, Ns * (sides == 3 ? 2 : 1)), ke.smem, (const T*)h->Tpad, S, Ns, sides,
-                     (T*)h->envs, h->logs, st, h->wdisc, s), "env kernel");
+                     (T*)h->envs, h->logs, st, s), "env kernel");
     tstop(h, ts, s);
   }
   const KPlan& kr = h->kp[1];
@@ -892,7 +889,6 @@ extern "C" peps_status peps_local_energy_bound(peps_handle* h, const peps_hamilt
   cudaStream_t s = (cudaStream_t)stream;
   int* st = status_dev ? (int*)status_dev : h->status_tmp;
   CK(cudaMemsetAsync(st, 0, sizeof(int) * Ns, s), "memset status");
-  CK(cudaMemsetAsync(h->wdisc, 0, sizeof(float) * Ns, s), "memset wdisc");
   if (Ns == 0) return PEPS_OK;
   peps_status ps = set_hamiltonian(h, H, s);
   if (ps != PEPS_OK) return ps;
@@ -912,7 +908,7 @@ extern "C" peps_status peps_local_energy_bound(peps_handle* h, const peps_hamilt
   cudaError_t e = dispatch_elem(h, [&](auto z) {
     using T = decltype(z);
     return launch_env<T>(h->g, ke.p, std::min(ke.grid, Ns * 2), ke.smem, (const T*)h->Tpad, S_dev, Ns, 3, (T*)h->envs,
-                         h->logs, st, h->wdisc, s);
+                         h->logs, st, s);
   });
   if (e != cudaSuccess) return cuda_fail(h, e, "env kernel");
   tstop(h, ts, s);
@@ -1414,7 +1410,6 @@ struct BatchGroup {
   int ninst = 0;
   long long nitems = 0;
   std::vector<int*> status;
-  std::vector<float*> wdisc;
   std::vector<int> ns;
   std::vector<int*> sword;
 };
@@ -1442,7 +1437,6 @@ static peps_status batch_prepare(peps_batch* b, const peps_batch_item* items, co
     q.S = it.S_dev;
     q.envs = (T*)h->envs;
     q.logs = h->logs;
-    q.wdisc = h->wdisc;
     q.O = (T*)it.O_dev;
     q.site_off = h->site_off;
     q.Np = h->Np;
@@ -1461,7 +1455,6 @@ static peps_status batch_prepare(peps_batch* b, const peps_batch_item* items, co
     q.item0 = item0;
     item0 += it.Ns;
     grp->status.push_back(q.status);
-    grp->wdisc.push_back(q.wdisc);
     grp->ns.push_back(it.Ns);
     grp->sword.push_back(h->sword);
   }
@@ -1519,8 +1512,7 @@ template <typename T>
 static peps_status batch_record(peps_batch* b, const BatchGroup& grp, cudaStream_t s) {
   if (cudaMemsetAsync(b->next + grp.elem, 0, sizeof(unsigned long long), s) != cudaSuccess) return PEPS_E_CUDA;
   for (int k = 0; k < grp.ninst; ++k)
-    if (cudaMemsetAsync(grp.status[k], 0, sizeof(int) * grp.ns[k], s) != cudaSuccess ||
-        cudaMemsetAsync(grp.wdisc[k], 0, sizeof(float) * grp.ns[k], s) != cudaSuccess)
+    if (cudaMemsetAsync(grp.status[k], 0, sizeof(int) * grp.ns[k], s) != cudaSuccess)
       return PEPS_E_CUDA;
   if (launch_batch<T>((const BatchInst<T>*)b->inst_dev[grp.elem], grp.ninst, grp.nitems, b->next + grp.elem, grp.grid,
                       grp.smem, s) != cudaSuccess)

@@ -122,16 +122,7 @@ __global__ void __launch_bounds__(NTHREADS) k_dl_env(G g, int chid, const T* __r
       __syncthreads();
       const int sweeps = hestenes_rows<T, 0>(w.X, mX, Lr, LX, &flag, nullptr, red, sig);
       if (sweeps < 0 && tid == 0) st |= ST_NOCONV;
-      {
-        const int lane = tid & 31, warp = tid >> 5, nw = NT >> 5;
-        for (int p = warp; p < mX; p += nw) {
-          RT s = 0;
-          for (int i = lane; i < Lr; i += 32) s += abs2_(w.X[(size_t)p * LX + i]);
-          s = warp_sum(s);
-          if (lane == 0) sig[p] = sqrt(s);
-        }
-      }
-      __syncthreads();
+      // hestenes_rows left the singular values in sig
       // stable descending ranks (NaN below every number)
       for (int p = tid; p < mX; p += NT) {
         const RT sp = sig[p];
@@ -225,7 +216,6 @@ __global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_direct(G g, P
   T* LC = (T*)buf_ptr(plan, B_LW2, smem, gbase);   // d candidates + the running left partial
   double* red = w.red;
   __shared__ int st, flag;
-  __shared__ float wd;
   __shared__ double pw[8];
   __shared__ int pick;
   const int tid = threadIdx.x, NT = blockDim.x;
@@ -237,7 +227,7 @@ __global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_direct(G g, P
   // register-tile edge of the large contractions (complex double: smaller, to stay in registers)
   constexpr int TE = sizeof(T) >= 16 ? 4 : 8;
   for (int c = blockIdx.x; c < Ns; c += gridDim.x) {
-    if (tid == 0) { st = 0; wd = 0.f; }
+    if (tid == 0) st = 0;
     // E^u[-1]: the trivial row
     for (int k = 0; k < Ly; ++k) blk_unit(EU + (size_t)k * g.se, g.se);
     __syncthreads();
@@ -357,7 +347,7 @@ __global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_direct(G g, P
       if (x < Lx - 1) {
         T* out = EU + (size_t)(cur ^ 1) * rowsz;
         if (x == 0) env_first_row(g, out, Tpad, 0, Sl, false, w.A, w.Z, red, &st);
-        else env_row_step(g, Eu, out, Tpad, x, Sl + (size_t)x * Ly, false, w, &st, &wd, &flag);
+        else env_row_step(g, Eu, out, Tpad, x, Sl + (size_t)x * Ly, false, w, &st, &flag);
         cur ^= 1;
         __syncthreads();
       }

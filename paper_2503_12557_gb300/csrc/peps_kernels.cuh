@@ -44,7 +44,6 @@ struct BatchInst {
   const uint8_t* S;
   T* envs;
   double* logs;
-  float* wdisc;
   T* O;                     // may be null
   const long long* site_off;
   long long Np;
@@ -70,7 +69,7 @@ cudaError_t kattr_batch(size_t set_bytes, int* occ, size_t occ_smem);
 
 template <typename T>
 cudaError_t launch_env(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
-                       int sides, T* envs, double* logs, int* status, float* wdisc, cudaStream_t s);
+                       int sides, T* envs, double* logs, int* status, cudaStream_t s);
 template <typename T>
 cudaError_t launch_row(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
                        int x_lo, int x_hi, const T* envs, const double* logs, T* O, const long long* site_off,

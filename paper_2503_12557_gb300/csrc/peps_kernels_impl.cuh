@@ -40,7 +40,7 @@ __device__ RowWork<T> carve_row(const Plan& p, char* smem, char* gbase) {
 // Upper environments E^u[-1..Lx-2] of configuration Ss into env (one sample's store).
 template <typename T, typename G>
 __device__ void build_upper(const G& g, const T* Tpad, const uint8_t* Ss, T* env, double* logs,
-                            const RowWork<T>& w, int* st, float* wd, int* flag) {
+                            const RowWork<T>& w, int* st, int* flag) {
   const size_t row = (size_t)g.Ly * g.se;
   // trivial E^u[-1], and the trivial E^l[Lx] that closes psi_top = E^u[Lx-2] . T_proj[Lx-1]
   T* trivial = env + (size_t)slot_up(g, -1) * row;
@@ -51,12 +51,13 @@ __device__ void build_upper(const G& g, const T* Tpad, const uint8_t* Ss, T* env
   }
   if (threadIdx.x == 0) { logs[slot_up(g, -1)] = 0.0; logs[slot_lo(g, g.Lx)] = 0.0; }
   __syncthreads();
-  double lg = env_first_row(g, env + (size_t)slot_up(g, 0) * row, Tpad, 0, Ss, false, w.A, w.Z, w.red, st);
-  if (threadIdx.x == 0) logs[slot_up(g, 0)] = lg;
+  Scaled f = env_first_row(g, env + (size_t)slot_up(g, 0) * row, Tpad, 0, Ss, false, w.A, w.Z, w.red, st);
+  double lg = 0.0;
+  if (threadIdx.x == 0) logs[slot_up(g, 0)] = lg = sc_log(f);
   for (int x = 1; x <= g.Lx - 2; ++x) {
-    lg += env_row_step(g, env + (size_t)slot_up(g, x - 1) * row, env + (size_t)slot_up(g, x) * row, Tpad, x,
-                       Ss + (size_t)x * g.Ly, false, w, st, wd, flag);
-    if (threadIdx.x == 0) logs[slot_up(g, x)] = lg;
+    f = env_row_step(g, env + (size_t)slot_up(g, x - 1) * row, env + (size_t)slot_up(g, x) * row, Tpad, x,
+                       Ss + (size_t)x * g.Ly, false, w, st, flag);
+    if (threadIdx.x == 0) logs[slot_up(g, x)] = lg += sc_log(f);
   }
   __syncthreads();
 }
@@ -64,19 +65,20 @@ __device__ void build_upper(const G& g, const T* Tpad, const uint8_t* Ss, T* env
 // Lower environments E^l[2..Lx] (and E^l[1] when full) of configuration Ss.
 template <typename T, typename G>
 __device__ void build_lower(const G& g, const T* Tpad, const uint8_t* Ss, T* env, double* logs,
-                            const RowWork<T>& w, int* st, float* wd, int* flag, int xmin) {
+                            const RowWork<T>& w, int* st, int* flag, int xmin) {
   const size_t row = (size_t)g.Ly * g.se;
   T* trivial = env + (size_t)slot_lo(g, g.Lx) * row;
   for (int k = 0; k < g.Ly; ++k) blk_unit(trivial + (size_t)k * g.se, g.se);
   if (threadIdx.x == 0) logs[slot_lo(g, g.Lx)] = 0.0;
   __syncthreads();
-  double lg = env_first_row(g, env + (size_t)slot_lo(g, g.Lx - 1) * row, Tpad, g.Lx - 1,
-                            Ss + (size_t)(g.Lx - 1) * g.Ly, true, w.A, w.Z, w.red, st);
-  if (threadIdx.x == 0) logs[slot_lo(g, g.Lx - 1)] = lg;
+  Scaled f = env_first_row(g, env + (size_t)slot_lo(g, g.Lx - 1) * row, Tpad, g.Lx - 1,
+                           Ss + (size_t)(g.Lx - 1) * g.Ly, true, w.A, w.Z, w.red, st);
+  double lg = 0.0;
+  if (threadIdx.x == 0) logs[slot_lo(g, g.Lx - 1)] = lg = sc_log(f);
   for (int x = g.Lx - 2; x >= xmin; --x) {
-    lg += env_row_step(g, env + (size_t)slot_lo(g, x + 1) * row, env + (size_t)slot_lo(g, x) * row, Tpad, x,
-                       Ss + (size_t)x * g.Ly, true, w, st, wd, flag);
-    if (threadIdx.x == 0) logs[slot_lo(g, x)] = lg;
+    f = env_row_step(g, env + (size_t)slot_lo(g, x + 1) * row, env + (size_t)slot_lo(g, x) * row, Tpad, x,
+                       Ss + (size_t)x * g.Ly, true, w, st, flag);
+    if (threadIdx.x == 0) logs[slot_lo(g, x)] = lg += sc_log(f);
   }
   __syncthreads();
 }
@@ -85,20 +87,18 @@ __device__ void build_lower(const G& g, const T* Tpad, const uint8_t* Ss, T* env
 template <typename T, typename G>
 __device__ __forceinline__ void env_item(const G g, const RowWork<T>& w, const T* __restrict__ Tpad,
                                          const uint8_t* __restrict__ S,
-                         int smp, int side, T* envs, double* logs, int* status, float* wdisc) {
+                         int smp, int side, T* envs, double* logs, int* status) {
   __shared__ int st, flag;
-  __shared__ float wd;
   const int N = g.Lx * g.Ly;
-  if (threadIdx.x == 0) { st = 0; wd = 0.f; }
+  if (threadIdx.x == 0) st = 0;
   __syncthreads();
   T* env = envs + (size_t)smp * env_sample_elems(g);
   double* lg = logs + (size_t)smp * 2 * g.Lx;
   const uint8_t* Ss = S + (size_t)smp * N;
-  if (side == 0) build_upper(g, Tpad, Ss, env, lg, w, &st, &wd, &flag);
-  else build_lower(g, Tpad, Ss, env, lg, w, &st, &wd, &flag, 1);
+  if (side == 0) build_upper(g, Tpad, Ss, env, lg, w, &st, &flag);
+  else build_lower(g, Tpad, Ss, env, lg, w, &st, &flag, 1);
   if (threadIdx.x == 0) {
     if (st) atomicOr(status + smp, st);
-    if (wdisc) atomicMax((int*)(wdisc + smp), __float_as_int(wd));  // wd >= 0: int order = float order
   }
   __syncthreads();
 }
@@ -106,14 +106,14 @@ __device__ __forceinline__ void env_item(const G g, const RowWork<T>& w, const T
 template <typename T, typename G>
 __global__ void __launch_bounds__(NTHREADS, EnvBlocks<T>::value) k_env(G g, Plan plan, const T* __restrict__ Tpad,
                                                   const uint8_t* __restrict__ S, int Ns, int sides, T* envs,
-                                                  double* logs, int* status, float* wdisc) {
+                                                  double* logs, int* status) {
   extern __shared__ __align__(16) char smem[];
   RowWork<T> w = carve_row<T>(plan, smem, plan.gbase);
   const int nside = (sides == 3) ? 2 : 1;
   for (int item = blockIdx.x; item < Ns * nside; item += gridDim.x) {
     const int smp = item / nside;
     const int side = (sides == 3) ? (item % nside) : (sides == 1 ? 0 : 1);
-    env_item(g, w, Tpad, S, smp, side, envs, logs, status, wdisc);
+    env_item(g, w, Tpad, S, smp, side, envs, logs, status);
   }
 }
 
@@ -163,7 +163,8 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
   T* LW = (T*)buf_ptr(plan, B_LW, smem, gbase);
   T* LW2 = (T*)buf_ptr(plan, B_LW2, smem, gbase);
   double* red = (double*)buf_ptr(plan, B_RED, smem, gbase);
-  __shared__ double logL[MAX_LY + 1], logR[MAX_LY + 1];
+  __shared__ Scaled logL[MAX_LY + 1], logR[MAX_LY + 1];  // factors taken out of the partials
+  __shared__ dz fO;
   __shared__ int st;
   const int N = g.Lx * g.Ly, Ly = g.Ly, se = g.se;
   const size_t rowsz = (size_t)Ly * se;
@@ -175,7 +176,7 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
   if (threadIdx.x == 0) st = 0;
   // right partials R[Ly] = unit, R[y] = R[y+1] absorbed over column y
   blk_unit(RP + (size_t)Ly * se, se);
-  if (threadIdx.x == 0) logR[Ly] = 0.0;
+  if (threadIdx.x == 0) logR[Ly] = sc_one();
   __syncthreads();
   for (int y = Ly - 1; y >= 0; --y) {
     blk_copy(eu, EU + (size_t)y * se, se);
@@ -183,12 +184,12 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
     load_A(A, Tpad, g, x * Ly + y, Ss[x * Ly + y], false);
     __syncthreads();
     absorb1_right(g, RP + (size_t)(y + 1) * se, eu, A, el, t1, t2, RP + (size_t)y * se);
-    const double l = blk_normalize(RP + (size_t)y * se, se, red, &st);
-    if (threadIdx.x == 0) logR[y] = logR[y + 1] + l;
+    const double l = (double)blk_normalize(RP + (size_t)y * se, se, red, &st);
+    if (threadIdx.x == 0) logR[y] = sc_mul(logR[y + 1], l);
   }
   // left partials
   blk_unit(LP, se);
-  if (threadIdx.x == 0) logL[0] = 0.0;
+  if (threadIdx.x == 0) logL[0] = sc_one();
   __syncthreads();
   for (int y = 0; y < Ly; ++y) {
     blk_copy(eu, EU + (size_t)y * se, se);
@@ -196,13 +197,13 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
     load_A(A, Tpad, g, x * Ly + y, Ss[x * Ly + y], false);
     __syncthreads();
     absorb1(g, LP + (size_t)y * se, eu, A, el, t1, t2, LP + (size_t)(y + 1) * se);
-    const double l = blk_normalize(LP + (size_t)(y + 1) * se, se, red, &st);
-    if (threadIdx.x == 0) logL[y + 1] = logL[y] + l;
+    const double l = (double)blk_normalize(LP + (size_t)(y + 1) * se, se, red, &st);
+    if (threadIdx.x == 0) logL[y + 1] = sc_mul(logL[y], l);
   }
   __syncthreads();
   const T val = LP[(size_t)Ly * se];
-  const double lpsi_norm = logL[Ly];
-  const double env_log = lg[slot_up(g, x - 1)] + lg[slot_lo(g, x + 1)];
+  // 1 / psi_x without its scale, in thread 0
+  const dz ival = threadIdx.x == 0 ? dz_div(dz{1.0, 0.0}, to_dz(val)) : dz{0.0, 0.0};
   // ---- log-derivatives of row x
   if (O != nullptr) {
     for (int y = 0; y < Ly; ++y) {
@@ -216,23 +217,29 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
       }
       __syncthreads();
       site_env1(g, LP + (size_t)y * se, eu, LW2, RP + (size_t)(y + 1) * se, t1, t2, A);
-      const double sc = exp(logL[y] + logR[y + 1] - lpsi_norm);
+      if (threadIdx.x == 0) {
+        const double sc = sc_ratio(sc_mul(logL[y], logR[y + 1]), logL[Ly]);
+        fO = dz{ival.re * sc, ival.im * sc};
+      }
       int Dl, Du, Dr, Dd;
       site_dims(g, x, y, &Dl, &Du, &Dr, &Dd);
       const int blk = Dl * Du * Dr * Dd;
       const int s_here = Ss[site];
       T* Orow = O + (size_t)smp * Np + site_off[site];
       const int D = g.D;
-      for (int o = threadIdx.x; o < g.d * blk; o += blockDim.x) {
-        const int s = o / blk, c = o % blk;
-        const int dd = c % Dd, r = (c / Dd) % Dr, u = (c / (Dd * Dr)) % Du, l = c / (Dd * Dr * Du);
-        T v = T(0);
-        if (s == s_here) {
-          const dz e = to_dz(A[((l * D + u) * D + r) * D + dd]);
-          v = from_dz<T>(dz_div(dz{e.re * sc, e.im * sc}, to_dz(val)));
+      __syncthreads();
+      const dz f = fO;
+      for (int s = 0; s < g.d; ++s)
+        for (int c = threadIdx.x; c < blk; c += blockDim.x) {
+          T v = T(0);
+          if (s == s_here) {
+            const int dd = c % Dd, r = (c / Dd) % Dr, u = (c / (Dd * Dr)) % Du, l = c / (Dd * Dr * Du);
+            const T a = A[((l * D + u) * D + r) * D + dd];
+            if constexpr (Scal<T>::complex) v = from_dz<T>(dz_mul(to_dz(a), f));
+            else v = (T)((double)a * f.re);
+          }
+          Orow[s * blk + c] = v;
         }
-        Orow[o] = v;
-      }
       __syncthreads();
     }
   }
@@ -249,7 +256,7 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
         if (b == a) { ere += hr; eim += hi; continue; }
         const int y0 = ti[TI_Y0], w = ti[TI_W];
         blk_copy(LW, LP + (size_t)y0 * se, se);
-        double lw = logL[y0];
+        Scaled lw = logL[y0];  // carried in thread 0
         __syncthreads();
         for (int c = y0; c < y0 + w; ++c) {
           const int site = x * Ly + c;
@@ -258,16 +265,18 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
           load_A(A, Tpad, g, site, state_after(ti, site, Ss, b, g.d), false);
           __syncthreads();
           absorb1(g, LW, eu, A, el, t1, t2, LW2);
-          lw += blk_normalize(LW2, se, red, &st);
+          const double l = (double)blk_normalize(LW2, se, red, &st);
+          if (threadIdx.x == 0) lw = sc_mul(lw, l);
           blk_copy(LW, LW2, se);
           __syncthreads();
         }
         const T v = blk_dot(LW, RP + (size_t)(y0 + w) * se, se, red);
-        lw += logR[y0 + w];
-        const dz q = dz_div(to_dz(v), to_dz(val));
-        const double f = exp(lw - lpsi_norm);
-        ere += (hr * q.re - hi * q.im) * f;
-        eim += (hr * q.im + hi * q.re) * f;
+        if (threadIdx.x == 0) {
+          const dz q = dz_mul(to_dz(v), ival);
+          const double f = sc_ratio(sc_mul(lw, logR[y0 + w]), logL[Ly]);
+          ere += (hr * q.re - hi * q.im) * f;
+          eim += (hr * q.im + hi * q.re) * f;
+        }
       }
     }
   }
@@ -275,7 +284,7 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
     double* out = rowout + ((size_t)smp * g.Lx + x) * 4;
     const dz vz = to_dz(val);
     const double av = dz_abs(vz);
-    out[0] = (av > 0.0) ? log(av) + lpsi_norm + env_log : -INFINITY;
+    out[0] = (av > 0.0) ? sc_log(sc_mul(logL[Ly], av)) + lg[slot_up(g, x - 1)] + lg[slot_lo(g, x + 1)] : -INFINITY;
     out[1] = (vz.im == 0.0) ? ((vz.re < 0.0) ? 3.141592653589793 : 0.0) : atan2(vz.im, vz.re);
     out[2] = ere;
     out[3] = eim;
@@ -316,7 +325,7 @@ __device__ __forceinline__ void pair_item(const G g, const Plan plan, char* smem
   T* LW = (T*)buf_ptr(plan, B_LW, smem, gbase);
   T* LW2 = (T*)buf_ptr(plan, B_LW2, smem, gbase);
   double* red = (double*)buf_ptr(plan, B_RED, smem, gbase);
-  __shared__ double logL[MAX_LY + 1], logR[MAX_LY + 1];
+  __shared__ Scaled logL[MAX_LY + 1], logR[MAX_LY + 1];  // factors taken out of the partials
   __shared__ int st;
   const int N = g.Lx * g.Ly, Ly = g.Ly, se = g.se, s2 = g.s2;
   const size_t rowsz = (size_t)Ly * se;
@@ -334,7 +343,7 @@ __device__ __forceinline__ void pair_item(const G g, const Plan plan, char* smem
   const T* EL = env + (size_t)slot_lo(g, x + 2) * rowsz;
   if (threadIdx.x == 0) st = 0;
   blk_unit(RP + (size_t)Ly * s2, s2);
-  if (threadIdx.x == 0) logR[Ly] = 0.0;
+  if (threadIdx.x == 0) logR[Ly] = sc_one();
   __syncthreads();
   for (int y = Ly - 1; y >= 0; --y) {
     blk_copy(eu, EU + (size_t)y * se, se);
@@ -343,11 +352,11 @@ __device__ __forceinline__ void pair_item(const G g, const Plan plan, char* smem
     load_A(A2, Tpad, g, (x + 1) * Ly + y, Ss[(x + 1) * Ly + y], false);
     __syncthreads();
     absorb2_right(g, RP + (size_t)(y + 1) * s2, eu, A1, A2, el, t1, t2, RP + (size_t)y * s2, plan.cx);
-    const double l = blk_normalize(RP + (size_t)y * s2, s2, red, &st);
-    if (threadIdx.x == 0) logR[y] = logR[y + 1] + l;
+    const double l = (double)blk_normalize(RP + (size_t)y * s2, s2, red, &st);
+    if (threadIdx.x == 0) logR[y] = sc_mul(logR[y + 1], l);
   }
   blk_unit(LP, s2);
-  if (threadIdx.x == 0) logL[0] = 0.0;
+  if (threadIdx.x == 0) logL[0] = sc_one();
   __syncthreads();
   // the left partials are only needed up to the last window start; build them all
   for (int y = 0; y < Ly; ++y) {
@@ -357,12 +366,12 @@ __device__ __forceinline__ void pair_item(const G g, const Plan plan, char* smem
     load_A(A2, Tpad, g, (x + 1) * Ly + y, Ss[(x + 1) * Ly + y], false);
     __syncthreads();
     absorb2(g, LP + (size_t)y * s2, eu, A1, A2, el, t1, t2, LP + (size_t)(y + 1) * s2, plan.cx);
-    const double l = blk_normalize(LP + (size_t)(y + 1) * s2, s2, red, &st);
-    if (threadIdx.x == 0) logL[y + 1] = logL[y] + l;
+    const double l = (double)blk_normalize(LP + (size_t)(y + 1) * s2, s2, red, &st);
+    if (threadIdx.x == 0) logL[y + 1] = sc_mul(logL[y], l);
   }
   __syncthreads();
   const T val = LP[(size_t)Ly * s2];
-  const double lpsi_norm = logL[Ly];
+  const dz ival = threadIdx.x == 0 ? dz_div(dz{1.0, 0.0}, to_dz(val)) : dz{0.0, 0.0};
   double ere = 0.0, eim = 0.0;
   for (int ti_ = tt.pair_off[x]; ti_ < tt.pair_off[x + 1]; ++ti_) {
     const int* ti = tt.tinfo + (size_t)ti_ * TI_N;
@@ -374,7 +383,7 @@ __device__ __forceinline__ void pair_item(const G g, const Plan plan, char* smem
       if (b == a) { ere += hr; eim += hi; continue; }
       const int y0 = ti[TI_Y0], w = ti[TI_W];
       blk_copy(LW, LP + (size_t)y0 * s2, s2);
-      double lw = logL[y0];
+      Scaled lw = logL[y0];  // carried in thread 0
       __syncthreads();
       for (int c = y0; c < y0 + w; ++c) {
         blk_copy(eu, EU + (size_t)c * se, se);
@@ -383,16 +392,18 @@ __device__ __forceinline__ void pair_item(const G g, const Plan plan, char* smem
         load_A(A2, Tpad, g, (x + 1) * Ly + c, state_after(ti, (x + 1) * Ly + c, Ss, b, g.d), false);
         __syncthreads();
         absorb2(g, LW, eu, A1, A2, el, t1, t2, LW2, plan.cx);
-        lw += blk_normalize(LW2, s2, red, &st);
+        const double l = (double)blk_normalize(LW2, s2, red, &st);
+        if (threadIdx.x == 0) lw = sc_mul(lw, l);
         blk_copy(LW, LW2, s2);
         __syncthreads();
       }
       const T v = blk_dot(LW, RP + (size_t)(y0 + w) * s2, s2, red);
-      lw += logR[y0 + w];
-      const dz q = dz_div(to_dz(v), to_dz(val));
-      const double f = exp(lw - lpsi_norm);
-      ere += (hr * q.re - hi * q.im) * f;
-      eim += (hr * q.im + hi * q.re) * f;
+      if (threadIdx.x == 0) {
+        const dz q = dz_mul(to_dz(v), ival);
+        const double f = sc_ratio(sc_mul(lw, logR[y0 + w]), logL[Ly]);
+        ere += (hr * q.re - hi * q.im) * f;
+        eim += (hr * q.im + hi * q.re) * f;
+      }
     }
   }
   if (threadIdx.x == 0) {
@@ -553,8 +564,8 @@ template <typename T, typename G>
 __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, const T* Tpad, uint8_t* Sl,
                           const T* env, int x, int up, int move, unsigned slot0, unsigned long long sweep_id, int c,
                           unsigned long long seed, long long* acc, int* st) {
-  __shared__ double logR[MAX_LY + 1];
-  __shared__ double logLc, lcur;
+  __shared__ Scaled logR[MAX_LY + 1];   // factors taken out of the partials
+  __shared__ Scaled logLc, lcur;        // of the running left partial; |psi| of the configuration
   __shared__ int accept_flag;
   const int Ly = g.Ly, Lx = g.Lx, se = g.se, s2 = g.s2;
   const size_t rowsz = (size_t)Ly * se;
@@ -568,7 +579,7 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
     const T* EU = env + (size_t)slot_up(g, x - 1) * rowsz;
     const T* EL = env + (size_t)slot_lo(g, x + 1) * rowsz;
     blk_unit(RP + (size_t)Ly * se, se);
-    if (threadIdx.x == 0) logR[Ly] = 0.0;
+    if (threadIdx.x == 0) logR[Ly] = sc_one();
     __syncthreads();
     for (int y = Ly - 1; y >= 0; --y) {
       blk_copy(eu, EU + (size_t)y * se, se);
@@ -576,20 +587,18 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
       load_A(A1, Tpad, g, x * Ly + y, Sl[x * Ly + y], false);
       __syncthreads();
       absorb1_right(g, RP + (size_t)(y + 1) * se, eu, A1, el, t1, t2, RP + (size_t)y * se);
-      const double l = blk_normalize(RP + (size_t)y * se, se, red, st);
-      if (threadIdx.x == 0) logR[y] = logR[y + 1] + l;
+      const double l = (double)blk_normalize(RP + (size_t)y * se, se, red, st);
+      if (threadIdx.x == 0) logR[y] = sc_mul(logR[y + 1], l);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      const double v = dz_abs(to_dz(RP[0]));
-      lcur = (v != 0.0) ? log(v) + logR[0] : -INFINITY;
-      logLc = 0.0;
+      lcur = sc_mul(logR[0], dz_abs(to_dz(RP[0])));
+      logLc = sc_one();
     }
     blk_unit(LC, se);
     __syncthreads();
     for (int y = 0; y < nmv; ++y) {
-      const double u = uniform53(slot, (uint32_t)sweep_id, (uint32_t)c, 0u, seed);
-      ++slot;
+      const unsigned my_slot = slot++;
       const int i0 = x * Ly + y, i1 = i0 + 1;
       const bool possible = (move == 0) ? (Sl[i0] != Sl[i1]) : true;
       int taken = 0;
@@ -597,7 +606,8 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
         // the window: LC with column y in its proposed state (LW2, kept: it is the next LC if
         // the move is accepted), then for an exchange column y+1 as well (LW)
         const int w_ = (move == 0) ? 2 : 1;
-        double lw = logLc, l0 = 0.0;
+        Scaled lw = sc_one();  // in thread 0
+        double l0 = 0.0;
         for (int cc = 0; cc < w_; ++cc) {
           const int site = i0 + cc;
           int s_new;
@@ -609,19 +619,20 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
           __syncthreads();
           if (cc == 0) {
             absorb1(g, LC, eu, A1, el, t1, t2, LW2);
-            l0 = blk_normalize(LW2, se, red, st);
-            lw += l0;
+            l0 = (double)blk_normalize(LW2, se, red, st);
+            if (threadIdx.x == 0) lw = sc_mul(logLc, l0);
           } else {
             absorb1(g, LW2, eu, A1, el, t1, t2, LW);
-            lw += blk_normalize(LW, se, red, st);
+            const double l = (double)blk_normalize(LW, se, red, st);
+            if (threadIdx.x == 0) lw = sc_mul(lw, l);
           }
           __syncthreads();
         }
         const T v = blk_dot(w_ == 2 ? LW : LW2, RP + (size_t)(y + w_) * se, se, red);
         if (threadIdx.x == 0) {
-          const double av = dz_abs(to_dz(v));
-          const double l1 = (av != 0.0) ? log(av) + lw + logR[y + w_] : -INFINITY;
-          accept_flag = (isfinite(l1) && u < exp(2.0 * (l1 - lcur))) ? 1 : 0;
+          const double u = uniform53(my_slot, (uint32_t)sweep_id, (uint32_t)c, 0u, seed);
+          const Scaled l1 = sc_mul(sc_mul(lw, logR[y + w_]), dz_abs(to_dz(v)));
+          accept_flag = sc_accept(u, l1, lcur) ? 1 : 0;
           if (accept_flag) {
             lcur = l1;
             if (move == 0) { const uint8_t tmp = Sl[i0]; Sl[i0] = Sl[i1]; Sl[i1] = tmp; }
@@ -634,7 +645,7 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
         if (taken) {
           // column y now holds the proposed state: the new LC is the window's first column
           blk_copy(LC, LW2, se);
-          if (threadIdx.x == 0) logLc += l0;
+          if (threadIdx.x == 0) logLc = sc_mul(logLc, l0);
           __syncthreads();
         }
       }
@@ -644,9 +655,9 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
         load_A(A1, Tpad, g, x * Ly + y, Sl[x * Ly + y], false);
         __syncthreads();
         absorb1(g, LC, eu, A1, el, t1, t2, LW2);
-        const double l = blk_normalize(LW2, se, red, st);
+        const double l = (double)blk_normalize(LW2, se, red, st);
         blk_copy(LC, LW2, se);
-        if (threadIdx.x == 0) logLc += l;
+        if (threadIdx.x == 0) logLc = sc_mul(logLc, l);
         __syncthreads();
       }
     }
@@ -657,7 +668,7 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
     const T* EU = env + (size_t)slot_up(g, xt - 1) * rowsz;
     const T* EL2 = env + (size_t)slot_lo(g, xt + 2) * rowsz;
     blk_unit(RP + (size_t)Ly * s2, s2);
-    if (threadIdx.x == 0) logR[Ly] = 0.0;
+    if (threadIdx.x == 0) logR[Ly] = sc_one();
     __syncthreads();
     for (int y = Ly - 1; y >= 0; --y) {
       blk_copy(eu, EU + (size_t)y * se, se);
@@ -666,20 +677,18 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
       load_A(A2, Tpad, g, (xt + 1) * Ly + y, Sl[(xt + 1) * Ly + y], false);
       __syncthreads();
       absorb2_right(g, RP + (size_t)(y + 1) * s2, eu, A1, A2, el, t1, t2, RP + (size_t)y * s2, plan.cx);
-      const double l = blk_normalize(RP + (size_t)y * s2, s2, red, st);
-      if (threadIdx.x == 0) logR[y] = logR[y + 1] + l;
+      const double l = (double)blk_normalize(RP + (size_t)y * s2, s2, red, st);
+      if (threadIdx.x == 0) logR[y] = sc_mul(logR[y + 1], l);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      const double v = dz_abs(to_dz(RP[0]));
-      lcur = (v != 0.0) ? log(v) + logR[0] : -INFINITY;
-      logLc = 0.0;
+      lcur = sc_mul(logR[0], dz_abs(to_dz(RP[0])));
+      logLc = sc_one();
     }
     blk_unit(LC, s2);
     __syncthreads();
     for (int y = 0; y < Ly; ++y) {
-      const double u = uniform53(slot, (uint32_t)sweep_id, (uint32_t)c, 0u, seed);
-      ++slot;
+      const unsigned my_slot = slot++;
       const int i0 = xt * Ly + y, i1 = (xt + 1) * Ly + y;
       blk_copy(eu, EU + (size_t)y * se, se);
       blk_copy(el, EL2 + (size_t)y * se, se);
@@ -689,13 +698,12 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
         load_A(A2, Tpad, g, i1, Sl[i0], false);
         __syncthreads();
         absorb2(g, LC, eu, A1, A2, el, t1, t2, LW2, plan.cx);
-        const double l0 = blk_normalize(LW2, s2, red, st);
-        const double lw = logLc + l0;
+        const double l0 = (double)blk_normalize(LW2, s2, red, st);
         const T v = blk_dot(LW2, RP + (size_t)(y + 1) * s2, s2, red);
         if (threadIdx.x == 0) {
-          const double av = dz_abs(to_dz(v));
-          const double l1 = (av != 0.0) ? log(av) + lw + logR[y + 1] : -INFINITY;
-          accept_flag = (isfinite(l1) && u < exp(2.0 * (l1 - lcur))) ? 1 : 0;
+          const double u = uniform53(my_slot, (uint32_t)sweep_id, (uint32_t)c, 0u, seed);
+          const Scaled l1 = sc_mul(sc_mul(sc_mul(logLc, l0), logR[y + 1]), dz_abs(to_dz(v)));
+          accept_flag = sc_accept(u, l1, lcur) ? 1 : 0;
           if (accept_flag) {
             lcur = l1;
             const uint8_t tmp = Sl[i0]; Sl[i0] = Sl[i1]; Sl[i1] = tmp;
@@ -707,7 +715,7 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
         if (taken) {
           // the proposal's window is the new LC
           blk_copy(LC, LW2, s2);
-          if (threadIdx.x == 0) logLc += l0;
+          if (threadIdx.x == 0) logLc = sc_mul(logLc, l0);
           __syncthreads();
         }
       }
@@ -716,9 +724,9 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
         load_A(A2, Tpad, g, i1, Sl[i1], false);
         __syncthreads();
         absorb2(g, LC, eu, A1, A2, el, t1, t2, LW2, plan.cx);
-        const double l = blk_normalize(LW2, s2, red, st);
+        const double l = (double)blk_normalize(LW2, s2, red, st);
         blk_copy(LC, LW2, s2);
-        if (threadIdx.x == 0) logLc += l;
+        if (threadIdx.x == 0) logLc = sc_mul(logLc, l);
         __syncthreads();
       }
     }
@@ -785,31 +793,33 @@ __global__ void __launch_bounds__(NTHREADS, EnvBlocks<T>::value) k_env_row(G g, 
   char* gbase = plan.gbase;
   RowWork<T> w = carve_row<T>(plan, smem, gbase);
   __shared__ int st, flag;
-  __shared__ float wd;
   const int N = g.Lx * g.Ly;
   const size_t rowsz = (size_t)g.Ly * g.se;
   for (int c = blockIdx.x; c < Ns; c += gridDim.x) {
-    if (threadIdx.x == 0) { st = 0; wd = 0.f; }
+    if (threadIdx.x == 0) st = 0;
     __syncthreads();
     T* env = envs + (size_t)c * env_sample_elems(g);
     double* lg = logs + (size_t)c * 2 * g.Lx;
     const uint8_t* Ss = S + (size_t)c * N;
-    double l;
+    Scaled l;
+    double l0 = 0.0;  // the row before's logarithm, in thread 0
     int slot;
     if (!lower) {
       slot = slot_up(g, x);
+      if (threadIdx.x == 0 && x > 0) l0 = lg[slot_up(g, x - 1)];
       if (x == 0) l = env_first_row(g, env + (size_t)slot * rowsz, Tpad, 0, Ss, false, w.A, w.Z, w.red, &st);
-      else l = lg[slot_up(g, x - 1)] + env_row_step(g, env + (size_t)slot_up(g, x - 1) * rowsz, env + (size_t)slot * rowsz,
-                                                    Tpad, x, Ss + (size_t)x * g.Ly, false, w, &st, &wd, &flag);
+      else l = env_row_step(g, env + (size_t)slot_up(g, x - 1) * rowsz, env + (size_t)slot * rowsz, Tpad, x,
+                            Ss + (size_t)x * g.Ly, false, w, &st, &flag);
     } else {
       slot = slot_lo(g, x);
+      if (threadIdx.x == 0 && x < g.Lx - 1) l0 = lg[slot_lo(g, x + 1)];
       if (x == g.Lx - 1)
         l = env_first_row(g, env + (size_t)slot * rowsz, Tpad, x, Ss + (size_t)x * g.Ly, true, w.A, w.Z, w.red, &st);
-      else l = lg[slot_lo(g, x + 1)] + env_row_step(g, env + (size_t)slot_lo(g, x + 1) * rowsz, env + (size_t)slot * rowsz,
-                                                    Tpad, x, Ss + (size_t)x * g.Ly, true, w, &st, &wd, &flag);
+      else l = env_row_step(g, env + (size_t)slot_lo(g, x + 1) * rowsz, env + (size_t)slot * rowsz, Tpad, x,
+                            Ss + (size_t)x * g.Ly, true, w, &st, &flag);
     }
     if (threadIdx.x == 0) {
-      lg[slot] = l;
+      lg[slot] = l0 + sc_log(l);
       if (st) atomicOr(status + c, st);
       if (st && ustat) atomicOr(ustat + c, st);
     }
@@ -835,13 +845,12 @@ __global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_sample(G g, P
   const MoveBufs<T> b = carve_moves<T>(plan, smem, gbase);
   uint8_t* Sl = (uint8_t*)buf_ptr(plan, B_S, smem, gbase);
   __shared__ int st, flag;
-  __shared__ float wd;
   const int N = g.Lx * g.Ly, Ly = g.Ly, Lx = g.Lx;
   const size_t rowsz = (size_t)Ly * g.se;
   for (int c = blockIdx.x; c < Ns; c += gridDim.x) {
     uint8_t* Sg = S + (size_t)c * N;
     for (int i = threadIdx.x; i < N; i += blockDim.x) Sl[i] = Sg[i];
-    if (threadIdx.x == 0) { st = 0; wd = 0.f; }
+    if (threadIdx.x == 0) st = 0;
     long long acc = 0;
     T* env = envs + (size_t)c * env_sample_elems(g);
     double* lg = logs + (size_t)c * 2 * Lx;
@@ -850,34 +859,34 @@ __global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_sample(G g, P
       const unsigned long long sweep_id = sweep0 + (unsigned long long)t;
       const int up = (int)(sweep_id & 1ull);
       if (!up) {
-        build_lower(g, Tpad, Sl, env, lg, w, &st, &wd, &flag, 1);
+        build_lower(g, Tpad, Sl, env, lg, w, &st, &flag, 1);
         sweep_trivial_row(g, env, lg, 0);
         __syncthreads();
         for (int x = 0; x < Lx; ++x) {
           row_moves(g, plan, b, Tpad, Sl, env, x, 0, move, sweep_slot0(g, x, 0, move), sweep_id, c, seed, &acc, &st);
           if (x < Lx - 1) {
             const size_t sl = (size_t)slot_up(g, x) * rowsz;
-            double l;
+            Scaled l;
             if (x == 0) l = env_first_row(g, env + sl, Tpad, 0, Sl, false, w.A, w.Z, w.red, &st);
-            else l = lg[slot_up(g, x - 1)] + env_row_step(g, env + (size_t)slot_up(g, x - 1) * rowsz, env + sl, Tpad, x,
-                                                           Sl + (size_t)x * Ly, false, w, &st, &wd, &flag);
-            if (threadIdx.x == 0) lg[slot_up(g, x)] = l;
+            else l = env_row_step(g, env + (size_t)slot_up(g, x - 1) * rowsz, env + sl, Tpad, x,
+                                  Sl + (size_t)x * Ly, false, w, &st, &flag);
+            if (threadIdx.x == 0) lg[slot_up(g, x)] = (x == 0 ? 0.0 : lg[slot_up(g, x - 1)]) + sc_log(l);
             __syncthreads();
           }
         }
       } else {
-        if (t == 0) build_upper(g, Tpad, Sl, env, lg, w, &st, &wd, &flag);
+        if (t == 0) build_upper(g, Tpad, Sl, env, lg, w, &st, &flag);
         sweep_trivial_row(g, env, lg, 1);
         __syncthreads();
         for (int x = Lx - 1; x >= 0; --x) {
           row_moves(g, plan, b, Tpad, Sl, env, x, 1, move, sweep_slot0(g, x, 1, move), sweep_id, c, seed, &acc, &st);
           if (x > 0) {
             const size_t sl = (size_t)slot_lo(g, x) * rowsz;
-            double l;
+            Scaled l;
             if (x == Lx - 1) l = env_first_row(g, env + sl, Tpad, x, Sl + (size_t)x * Ly, true, w.A, w.Z, w.red, &st);
-            else l = lg[slot_lo(g, x + 1)] + env_row_step(g, env + (size_t)slot_lo(g, x + 1) * rowsz, env + sl, Tpad, x,
-                                                           Sl + (size_t)x * Ly, true, w, &st, &wd, &flag);
-            if (threadIdx.x == 0) lg[slot_lo(g, x)] = l;
+            else l = env_row_step(g, env + (size_t)slot_lo(g, x + 1) * rowsz, env + sl, Tpad, x,
+                                  Sl + (size_t)x * Ly, true, w, &st, &flag);
+            if (threadIdx.x == 0) lg[slot_lo(g, x)] = (x == Lx - 1 ? 0.0 : lg[slot_lo(g, x + 1)]) + sc_log(l);
             __syncthreads();
           }
         }
@@ -916,7 +925,6 @@ __global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_bound(G g, Pl
   T* tb = (T*)buf_ptr(plan, B_LW2, smem, gbase);   // chi D chi
   T* Lb2 = Lb + (size_t)g.chi * g.chi;
   __shared__ int st, flag;
-  __shared__ float wd;
   const int N = g.Lx * g.Ly, Ly = g.Ly, Lx = g.Lx;
   const size_t rowsz = (size_t)Ly * g.se;
   const int nt = tt.nterm > 0 ? tt.nterm : 1;
@@ -926,10 +934,11 @@ __global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_bound(G g, Pl
     const uint8_t* Ss = S + (size_t)smp * N;
     const T* env = envs + (size_t)smp * env_sample_elems(g);
     const double* lg = logs + (size_t)smp * 2 * Lx;
-    if (threadIdx.x == 0) { st = 0; wd = 0.f; }
+    if (threadIdx.x == 0) st = 0;
     __syncthreads();
-    double l0 = lg[su] + lg[sl];
-    const dz z0 = to_dz(mps_overlap(g, env + (size_t)su * rowsz, env + (size_t)sl * rowsz, Lb, Lb2, tb, w.red, &st, &l0));
+    Scaled f0 = sc_one();
+    const dz z0 = to_dz(mps_overlap(g, env + (size_t)su * rowsz, env + (size_t)sl * rowsz, Lb, Lb2, tb, w.red, &st, &f0));
+    const double l0 = threadIdx.x == 0 ? lg[su] + lg[sl] + sc_log(f0) : 0.0;
     double ere = 0.0, eim = 0.0;
     if (t < tt.nterm) {
       const int* ti = tt.tinfo + (size_t)t * TI_N;
@@ -956,8 +965,10 @@ __global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_bound(G g, Pl
           lu = lg[slot_up(g, rlo - 1)];
           for (int r = rlo; r < cut; ++r) {
             T* out = EUb + (size_t)((r - rlo) & 1) * rowsz;
-            if (r == 0) lu = env_first_row(g, out, Tpad, 0, Sl, false, w.A, w.Z, w.red, &st);
-            else lu += env_row_step(g, prev, out, Tpad, r, Sl + (size_t)r * Ly, false, w, &st, &wd, &flag);
+            Scaled f;
+            if (r == 0) f = env_first_row(g, out, Tpad, 0, Sl, false, w.A, w.Z, w.red, &st);
+            else f = env_row_step(g, prev, out, Tpad, r, Sl + (size_t)r * Ly, false, w, &st, &flag);
+            if (threadIdx.x == 0) lu = (r == 0 ? 0.0 : lu) + sc_log(f);
             prev = out;
           }
           EU = prev;
@@ -969,15 +980,18 @@ __global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_bound(G g, Pl
           ll = lg[slot_lo(g, rhi + 1)];
           for (int r = rhi; r >= cut; --r) {
             T* out = ELb + (size_t)((rhi - r) & 1) * rowsz;
-            if (r == Lx - 1) ll = env_first_row(g, out, Tpad, Lx - 1, Sl + (size_t)(Lx - 1) * Ly, true, w.A, w.Z, w.red, &st);
-            else ll += env_row_step(g, prev, out, Tpad, r, Sl + (size_t)r * Ly, true, w, &st, &wd, &flag);
+            Scaled f;
+            if (r == Lx - 1) f = env_first_row(g, out, Tpad, Lx - 1, Sl + (size_t)(Lx - 1) * Ly, true, w.A, w.Z, w.red, &st);
+            else f = env_row_step(g, prev, out, Tpad, r, Sl + (size_t)r * Ly, true, w, &st, &flag);
+            if (threadIdx.x == 0) ll = (r == Lx - 1 ? 0.0 : ll) + sc_log(f);
             prev = out;
           }
           EL = prev;
         }
-        double l1 = lu + ll;
-        const dz z1 = to_dz(mps_overlap(g, EU, EL, Lb, Lb2, tb, w.red, &st, &l1));
-        if (z1.re != 0.0 || z1.im != 0.0) {
+        Scaled f1 = sc_one();
+        const dz z1 = to_dz(mps_overlap(g, EU, EL, Lb, Lb2, tb, w.red, &st, &f1));
+        if (threadIdx.x == 0 && (z1.re != 0.0 || z1.im != 0.0)) {
+          const double l1 = lu + ll + sc_log(f1);
           const dz q = dz_div(z1, z0);
           const double f = exp(l1 - l0);
           ere += (hr * q.re - hi * q.im) * f;
@@ -1064,15 +1078,15 @@ static cudaError_t with_geo_for(const Geo& g, F&& f) {
 // instances first; each CTA takes the next item with one atomic and runs that sample's whole
 // evaluation with the same device functions as the per-handle kernels (so the results are bit
 // for bit theirs): the environment sides, the one-row sandwiches of every row needed, the two-row
-// sandwiches, and the combine.  The caller zeroes *next and every instance's status and wdisc.
+// sandwiches, and the combine.  The caller zeroes *next and every instance's status.
 // the three phases as separate functions: their register allocations stay separate instead of
 // one inlined body holding every phase's live ranges
 // (an instance whose (chi, D) has a compiled specialisation runs it, as the per-handle kernels do)
 template <typename T, typename G>
 __device__ __noinline__ void batch_env(const BatchInst<T>& b, G g, char* smem, int smp) {
   RowWork<T> w = carve_row<T>(b.pe, smem, b.pe.gbase);
-  env_item(g, w, b.Tpad, b.S, smp, 0, b.envs, b.logs, b.status, b.wdisc);
-  if (b.sides == 3) env_item(g, w, b.Tpad, b.S, smp, 1, b.envs, b.logs, b.status, b.wdisc);
+  env_item(g, w, b.Tpad, b.S, smp, 0, b.envs, b.logs, b.status);
+  if (b.sides == 3) env_item(g, w, b.Tpad, b.S, smp, 1, b.envs, b.logs, b.status);
 }
 template <typename T, typename G>
 __device__ __noinline__ void batch_row(const BatchInst<T>& b, G g, char* smem, int smp, int x) {
@@ -1142,16 +1156,16 @@ cudaError_t kattr_batch(size_t set_bytes, int* occ, size_t occ_smem) {
 #ifdef PEPS_PART_ENV
 template <typename T>
 cudaError_t launch_env(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
-                       int sides, T* envs, double* logs, int* status, float* wdisc, cudaStream_t s) {
+                       int sides, T* envs, double* logs, int* status, cudaStream_t s) {
   return with_geo_for<T>(g, [&](auto gg) {
-    k_env<T, decltype(gg)><<<grid, NTHREADS, smem, s>>>(gg, p, Tpad, S, Ns, sides, envs, logs, status, wdisc);
+    k_env<T, decltype(gg)><<<grid, NTHREADS, smem, s>>>(gg, p, Tpad, S, Ns, sides, envs, logs, status);
     return cudaGetLastError();
   });
 }
 PEPS_KATTR(kattr_env, k_env)
 #define PEPS_INST_ENV(T)                                                                                          \
   template cudaError_t launch_env<T>(const Geo&, const Plan&, int, size_t, const T*, const uint8_t*, int, int, T*, \
-                                     double*, int*, float*, cudaStream_t);                                        \
+                                     double*, int*, cudaStream_t);                                        \
   template cudaError_t kattr_env<T>(const Geo&, size_t, int*, size_t);
 #endif
 
@@ -1209,7 +1223,7 @@ cudaError_t launch_sample(const Geo& g, const Plan& p, int grid, size_t smem, co
         const int up = (int)(sid & 1ull);
         int* us = (t == nsweeps - 1) ? ustat : nullptr;
         if (!up) {
-          k_env<T, GG><<<grid_e, NTHREADS, smem_e, s>>>(gg, pe, Tpad, S, Ns, 2, envs, logs, status, nullptr);
+          k_env<T, GG><<<grid_e, NTHREADS, smem_e, s>>>(gg, pe, Tpad, S, Ns, 2, envs, logs, status);
           for (int x = 0; x < g.Lx; ++x) {
             k_sweep_moves<T, GG><<<grid, NTHREADS, smem, s>>>(gg, p, Tpad, S, Ns, move, x, 0, seed, sid, envs, logs,
                                                               accepted, status);
@@ -1218,7 +1232,7 @@ cudaError_t launch_sample(const Geo& g, const Plan& p, int grid, size_t smem, co
           }
         } else {
           // the previous sweep of this call left the upper environments of these configurations
-          if (t == 0) k_env<T, GG><<<grid_e, NTHREADS, smem_e, s>>>(gg, pe, Tpad, S, Ns, 1, envs, logs, status, nullptr);
+          if (t == 0) k_env<T, GG><<<grid_e, NTHREADS, smem_e, s>>>(gg, pe, Tpad, S, Ns, 1, envs, logs, status);
           for (int x = g.Lx - 1; x >= 0; --x) {
             k_sweep_moves<T, GG><<<grid, NTHREADS, smem, s>>>(gg, p, Tpad, S, Ns, move, x, 1, seed, sid, envs, logs,
                                                               accepted, status);

@@ -102,7 +102,6 @@ peps_status run(const peps_config& c, const double* theta, const uint8_t* S, int
   T* envs = (T*)take((size_t)Ns * 2 * g.Lx * Ly * g.se * E);
   double* logs = (double*)take(sizeof(double) * (size_t)Ns * 2 * g.Lx);
   double* rowout = (double*)take(sizeof(double) * 4 * (size_t)Ns * g.Lx);
-  float* wdisc = (float*)take(sizeof(float) * (size_t)Ns);
   int* st_own = (int*)take(sizeof(int) * (size_t)Ns);
   if (off > kNoAllocBytes) return PEPS_E_CAPACITY;
   // the kernels loop over samples with a grid stride, so fewer CTAs give the same results;
@@ -118,10 +117,9 @@ peps_status run(const peps_config& c, const double* theta, const uint8_t* S, int
   int* st = status ? (int*)status : st_own;
   // what the kernels accumulate into must start at zero
   if (cudaMemsetAsync(st, 0, sizeof(int) * (size_t)Ns, s) != cudaSuccess) return PEPS_E_CUDA;
-  if (cudaMemsetAsync(wdisc, 0, sizeof(float) * (size_t)Ns, s) != cudaSuccess) return PEPS_E_CUDA;
   k_noalloc_site_offsets<<<1, 32, 0, s>>>(g.Lx, g.Ly, g.d, g.D, site_off);
   if (launch_pad<T>(g, theta, site_off, Tpad, s) != cudaSuccess) return PEPS_E_CUDA;
-  if (launch_env<T>(g, pe, grid, 0, Tpad, S, Ns, 1, envs, logs, st, wdisc, s) != cudaSuccess) return PEPS_E_CUDA;
+  if (launch_env<T>(g, pe, grid, 0, Tpad, S, Ns, 1, envs, logs, st, s) != cudaSuccess) return PEPS_E_CUDA;
   TermTab none{};
   if (launch_row<T>(g, pr, grid, 0, Tpad, S, Ns, g.Lx - 1, g.Lx, envs, logs, (T*)nullptr, site_off, 0, none, rowout,
                     st, s) != cudaSuccess)

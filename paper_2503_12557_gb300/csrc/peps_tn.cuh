@@ -190,36 +190,44 @@ __device__ __forceinline__ T warp_max(T v) {
   return v;
 }
 
-// red: at least 33 doubles of shared (or global) scratch.  All threads get the result.
+// red: at least 33 doubles of shared (or global) scratch.  All threads get the result.  In FP32
+// every warp adds the warps' sums itself, by the butterfly that the first warp used (the same
+// bits), and nothing passes through doubles: GB300's FP64 pipes, which also convert, take 64
+// cycles per warp instruction.
 template <typename T>
 __device__ T block_sum(T v, double* red) {
   v = warp_sum(v);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (l == 0) red[w] = (double)v;
-  __syncthreads();
-  if (w == 0) {
-    T t = (l < nw) ? (T)red[l] : T(0);
-    t = warp_sum(t);
-    if (l == 0) red[32] = (double)t;
+  if constexpr (sizeof(T) == 4) {
+    T* r = reinterpret_cast<T*>(red);
+    __syncthreads();
+    if (l == 0) r[w] = v;
+    __syncthreads();
+    return warp_sum(l < nw ? r[l] : T(0));
+  } else {
+    __syncthreads();
+    if (l == 0) red[w] = (double)v;
+    __syncthreads();
+    if (w == 0) {
+      T t = (l < nw) ? (T)red[l] : T(0);
+      t = warp_sum(t);
+      if (l == 0) red[32] = (double)t;
+    }
+    __syncthreads();
+    return (T)red[32];
   }
-  __syncthreads();
-  return (T)red[32];
 }
 template <typename T>
 __device__ T block_max(T v, double* red) {
   v = warp_max(v);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
+  T* r = reinterpret_cast<T*>(red);
   __syncthreads();
-  if (l == 0) red[w] = (double)v;
+  if (l == 0) r[w] = v;
   __syncthreads();
-  if (w == 0) {
-    T t = (l < nw) ? (T)red[l] : T(0);
-    t = warp_max(t);
-    if (l == 0) red[32] = (double)t;
-  }
-  __syncthreads();
-  return (T)red[32];
+  T m = r[0];
+  for (int i = 1; i < nw; ++i) m = fmax(m, r[i]);
+  return m;
 }
 
 template <typename R>
@@ -229,9 +237,16 @@ __device__ cplx<R> block_sum(cplx<R> v, double* red) {
   return cplx<R>(re, im);
 }
 
+// 16 bytes at a time when both ends and the length allow it
 template <typename T>
 __device__ void blk_copy(T* dst, const T* src, int n) {
-  for (int o = threadIdx.x; o < n; o += blockDim.x) dst[o] = src[o];
+  constexpr int V = 16 / sizeof(T) > 0 ? 16 / sizeof(T) : 1;
+  if (V > 1 && n % V == 0 && (((uintptr_t)dst | (uintptr_t)src) & 15) == 0) {
+    for (int o = threadIdx.x; o < n / V; o += blockDim.x)
+      reinterpret_cast<uint4*>(dst)[o] = reinterpret_cast<const uint4*>(src)[o];
+  } else {
+    for (int o = threadIdx.x; o < n; o += blockDim.x) dst[o] = src[o];
+  }
 }
 template <typename T>
 __device__ void blk_fill(T* dst, T v, int n) {
@@ -243,28 +258,79 @@ __device__ void blk_unit(T* dst, int n) {
   for (int o = threadIdx.x; o < n; o += blockDim.x) dst[o] = (o == 0) ? T(1) : T(0);
 }
 
-// Divide v[0..n) by its largest modulus; returns ln(max) (or -inf with ZERO_NORM / NONFINITE
-// set in *st when the maximum is 0 or not finite).  Ends with a barrier.
+// A positive number m 2^e, 1 <= m < 2, or 0 (also for a factor that was zero or not finite, whose
+// logarithm counts as -inf).  The factors that the normalisations take out are multiplied up in
+// this form by one thread and turned into a logarithm once per row or item: a logarithm per
+// normalisation, in every warp, was about 6000 cycles of an SM's FP64 pipes each, most of the
+// sandwich kernels' time in FP32.
+struct Scaled {
+  double m;
+  int e;
+};
+__device__ __forceinline__ Scaled sc_one() { return Scaled{1.0, 0}; }
+__device__ __forceinline__ Scaled sc_norm(double m, int e) {
+  if (m < 2.2250738585072014e-308) {  // subnormal, zero or negative
+    m *= 18446744073709551616.0;
+    e -= 64;
+  }
+  const long long b = __double_as_longlong(m);
+  const int ex = (int)(b >> 52) & 0x7ff;
+  if (!(m > 0.0) || ex == 0x7ff) return Scaled{0.0, 0};
+  return Scaled{__longlong_as_double((b & 0x000fffffffffffffll) | 0x3ff0000000000000ll), e + ex - 1023};
+}
+__device__ __forceinline__ Scaled sc_mul(const Scaled& a, double f) { return sc_norm(a.m * f, a.e); }
+__device__ __forceinline__ Scaled sc_mul(const Scaled& a, const Scaled& b) { return sc_norm(a.m * b.m, a.e + b.e); }
+// (not inlined: the environments a sampler leaves behind and those of an evaluation have to get the
+// same bits from every kernel that takes the logarithm)
+static __device__ __noinline__ double sc_log(Scaled a) {
+  return a.m > 0.0 ? __fma_rn((double)a.e, 0.6931471805599453, log(a.m)) : -INFINITY;
+}
+// a / b (inf or NaN when b is 0)
+__device__ __forceinline__ double sc_ratio(const Scaled& a, const Scaled& b) { return scalbn(a.m / b.m, a.e - b.e); }
+// u < (a / b)^2 for a finite, nonzero a (b = 0: true), without division or transcendentals
+__device__ __forceinline__ bool sc_accept(double u, const Scaled& a, const Scaled& b) {
+  if (!(a.m > 0.0)) return false;
+  int k = 2 * (a.e - b.e);
+  k = k > 1000 ? 1000 : (k < -1000 ? -1000 : k);
+  return u * b.m * b.m < a.m * a.m * __longlong_as_double((long long)(k + 1023) << 52);
+}
+
+// Divide v[0..n) by its largest modulus (double: by the power of two below it, which changes no
+// mantissa and needs no division); returns what it was divided by (the same in every thread), or
+// 0 with ZERO_NORM / NONFINITE set in *st when the maximum is 0 or not finite.  Called with v
+// complete behind a barrier; ends with a barrier.
 template <typename T>
-__device__ double blk_normalize(T* v, int n, double* red, int* st) {
+__device__ typename Scal<T>::R blk_normalize(T* v, int n, double* red, int* st) {
   using R = typename Scal<T>::R;
   R m = 0;
   for (int o = threadIdx.x; o < n; o += blockDim.x) m = fmax(m, abs_(v[o]));
-  m = block_max(m, red);
-  if (!(m < INFINITY)) {  // NaN or Inf
-    if (threadIdx.x == 0) *st |= ST_NONFINITE;
+  m = warp_max(m);
+  const int nw = blockDim.x >> 5;
+  R* r = reinterpret_cast<R*>(red);
+  if ((threadIdx.x & 31) == 0) r[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = r[0];
+  for (int i = 1; i < nw; ++i) m = fmax(m, r[i]);
+  if (!(m < INFINITY) || m == R(0)) {  // NaN, Inf or zero
+    if (threadIdx.x == 0) *st |= (m == R(0)) ? ST_ZERO_NORM : ST_NONFINITE;
     __syncthreads();
-    return -INFINITY;
+    return R(0);
   }
-  if (m == R(0)) {
-    if (threadIdx.x == 0) *st |= ST_ZERO_NORM;
-    __syncthreads();
-    return -INFINITY;
+  R inv;
+  if constexpr (sizeof(R) == 8) {
+    const long long ex = (__double_as_longlong(m) >> 52) & 0x7ff;
+    if (ex > 0 && ex < 2046) {
+      m = __longlong_as_double(ex << 52);
+      inv = __longlong_as_double((2046 - ex) << 52);
+    } else {
+      inv = R(1) / m;
+    }
+  } else {
+    inv = R(1) / m;
   }
-  const R inv = R(1) / m;
   for (int o = threadIdx.x; o < n; o += blockDim.x) v[o] *= inv;
   __syncthreads();
-  return log((double)m);
+  return m;
 }
 
 // Projected PEPS tensor of site `site` with local state s, as A[l][u][r][d] (swap_ud: as
@@ -569,12 +635,20 @@ __device__ void qr_keep_r(T* Z, int m, int nc, T* R, T* taus, int ldr) {
   if constexpr (Scal<T>::complex) {
     qr_keep_r_smem(Z, m, nc, R, taus, ldr);
   } else if constexpr (MC > 0) {
-    // the register form is compiled for up to MC rows and runs on the m <= MC rows given
+    // the register form is compiled for up to MC rows and runs on the m <= MC rows given, the
+    // sites near the open edge on a shorter one (rows past m are zeros that change no sum)
     constexpr int RPL = (MC + 31) / 32;
+    if constexpr (RPL <= 8) {
+      if (m <= 32) return qr_keep_r_reg<T, 1>(Z, m, nc, R, taus, ldr);
+      if (m <= 64) return qr_keep_r_reg<T, 2>(Z, m, nc, R, taus, ldr);
+    }
     if constexpr (RPL <= 24) qr_keep_r_reg<T, RPL>(Z, m, nc, R, taus, ldr);
     else qr_keep_r_smem(Z, m, nc, R, taus, ldr);
   } else {
-    if (m <= 256) qr_keep_r_reg<T, 8>(Z, m, nc, R, taus, ldr);
+    if (m <= 32) qr_keep_r_reg<T, 1>(Z, m, nc, R, taus, ldr);
+    else if (m <= 64) qr_keep_r_reg<T, 2>(Z, m, nc, R, taus, ldr);
+    else if (m <= 128) qr_keep_r_reg<T, 4>(Z, m, nc, R, taus, ldr);
+    else if (m <= 256) qr_keep_r_reg<T, 8>(Z, m, nc, R, taus, ldr);
     else if (m <= 768) qr_keep_r_reg<T, 24>(Z, m, nc, R, taus, ldr);
     else qr_keep_r_smem(Z, m, nc, R, taus, ldr);
   }
@@ -605,16 +679,20 @@ template <> __device__ __forceinline__ float jacobi_tol_r<float>(int L) { return
 
 // Rows whose squared norm is at most `tiny` are numerically zero singular values: the Jacobi
 // sweeps never rotate them against the others, so they are not orthogonal to the kept
-// directions and must not enter the kept basis.  Set them to exactly zero.  Ends with a barrier.
+// directions and must not enter the kept basis.  Set them to exactly zero.  sig[p] = the norm of
+// row p, the singular value.  Ends with a barrier.
 template <typename T>
-__device__ void zero_tiny_rows(T* X, int m, int L, int ldx, typename Scal<T>::R tiny) {
+__device__ void zero_tiny_rows(T* X, int m, int L, int ldx, typename Scal<T>::R tiny, typename Scal<T>::R* sig) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int p = warp; p < m; p += nw) {
     typename Scal<T>::R s = 0;
     for (int i = lane; i < L; i += 32) s += abs2_(X[(size_t)p * ldx + i]);
     s = warp_sum(s);
-    if (s <= tiny)
+    if (s <= tiny) {
       for (int i = lane; i < L; i += 32) X[(size_t)p * ldx + i] = T(0);
+      s = 0;
+    }
+    if (lane == 0) sig[p] = sqrt(s);
   }
   __syncthreads();
 }
@@ -626,7 +704,7 @@ __device__ void zero_tiny_rows(T* X, int m, int L, int ldx, typename Scal<T>::R 
 // the first sweep in which no pair had a relative dot product of sqrt(tol) or more: by the
 // quadratic convergence of cyclic Jacobi, that sweep's rotations leave dot products of order tol,
 // so the next sweep would rotate nothing.  On return the rows are sigma_i v_i^T with v_i the
-// right singular vectors of the input.
+// right singular vectors of the input, and nrm[p] = sigma_p (zero for the rows set to zero).
 //   Each warp treats four pairs at once (eight lanes per pair).  The squared row norms live in
 //   nrm[] (m entries): exact at the start of every sweep, and within a sweep updated after a
 //   rotation by Rutishauser's formulas a' = a - t g, b' = b + t g (g the pair's dot product), so
@@ -706,13 +784,13 @@ __device__ int hestenes_rows_smem(T* X, int m, int L, int ldx, int* flag, unsign
     const int any = *flag;
     __syncthreads();
     if (!(any & 2)) {
-      zero_tiny_rows(X, m, L, ldx, tiny);
+      zero_tiny_rows(X, m, L, ldx, tiny, nrm);
       if (ctr && nrot) atomicAdd(ctr + 1, nrot);
       if (ctr && threadIdx.x == 0) { atomicAdd(ctr + 0, (unsigned long long)(sweep + 1)); atomicAdd(ctr + 2, 1ull); }
       return sweep + 1;
     }
   }
-  zero_tiny_rows(X, m, L, ldx, tiny);
+  zero_tiny_rows(X, m, L, ldx, tiny, nrm);
   if (ctr && nrot) atomicAdd(ctr + 1, nrot);
   if (ctr && threadIdx.x == 0) { atomicAdd(ctr + 0, (unsigned long long)JacobiTol<R>::sweeps); atomicAdd(ctr + 2, 1ull); }
   return -1;
@@ -726,8 +804,11 @@ __device__ int hestenes_rows_smem(T* X, int m, int L, int ldx, int* flag, unsign
 // is set when the pair's relative dot product |c| / sqrt(a b) is at least `stop`.
 __device__ __forceinline__ void jac_params(double a, double b, double c, double tol, double tiny, double stop,
                                            double& cs, double& sn, double& tc, int& big) {
-  if (c != 0.0 && a > tiny && b > tiny && fabs(c) > tol * sqrt(a * b)) {
-    if (fabs(c) >= stop * sqrt(a * b)) big = 1;
+  // |c| > tol sqrt(a b) as c^2 > tol^2 a b: most pairs fail it, and a square root is a dozen FP64
+  // instructions of 64 cycles each (a, b > tiny keep the squares of what matters in range)
+  const double ab = a * b, c2 = c * c;
+  if (c2 > tol * tol * ab && a > tiny && b > tiny) {
+    if (c2 >= stop * stop * ab) big = 1;
     const double zeta = (b - a) / (2.0 * c);
     const double t = (fabs(zeta) > 1e15) ? 0.5 / zeta : copysign(1.0, zeta) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
     cs = 1.0 / sqrt(1.0 + t * t);
@@ -904,13 +985,13 @@ __device__ __noinline__ int hestenes_rows_grp(T* X, int m, int L, int ldx, int* 
     const int any = *flag;
     __syncthreads();
     if (!(any & 2)) {
-      zero_tiny_rows(X, m, L, ldx, tiny);
+      zero_tiny_rows(X, m, L, ldx, tiny, nrm);
       if (ctr && nrot) atomicAdd(ctr + 1, nrot);
       if (ctr && threadIdx.x == 0) { atomicAdd(ctr + 0, (unsigned long long)(sweep + 1)); atomicAdd(ctr + 2, 1ull); }
       return sweep + 1;
     }
   }
-  zero_tiny_rows(X, m, L, ldx, tiny);
+  zero_tiny_rows(X, m, L, ldx, tiny, nrm);
   if (ctr && nrot) atomicAdd(ctr + 1, nrot);
   if (ctr && threadIdx.x == 0) { atomicAdd(ctr + 0, (unsigned long long)JacobiTol<T>::sweeps); atomicAdd(ctr + 2, 1ull); }
   return -1;
@@ -929,6 +1010,10 @@ __device__ int hestenes_rows(T* X, int m, int L, int ldx, int* flag, unsigned lo
     if constexpr (E8 <= 16) return hestenes_rows_grp<T, E8>(X, m, LC, ldx, flag, ctr, red, nrm);
     else return hestenes_rows_smem(X, m, LC, ldx, flag, ctr, red, nrm);
   } else {
+    // (elements past L are zeros that change no sum: the smallest register form that holds a row)
+    if (L <= 8) return hestenes_rows_grp<T, 1>(X, m, L, ldx, flag, ctr, red, nrm);
+    if (L <= 16) return hestenes_rows_grp<T, 2>(X, m, L, ldx, flag, ctr, red, nrm);
+    if (L <= 32) return hestenes_rows_grp<T, 4>(X, m, L, ldx, flag, ctr, red, nrm);
     if (L <= 64) return hestenes_rows_grp<T, 8>(X, m, L, ldx, flag, ctr, red, nrm);
     if (L <= 128) return hestenes_rows_grp<T, 16>(X, m, L, ldx, flag, ctr, red, nrm);
     return hestenes_rows_smem(X, m, L, ldx, flag, ctr, red, nrm);
@@ -1027,12 +1112,10 @@ __device__ __forceinline__ void blk_gemm(const T* __restrict__ A, const T* __res
 // One row step of the boundary MPS: Eout = normalise(truncate_chi(Eprev o T_proj[row])).
 //   Eprev, Eout: Ly environment sites (chi x D x chi each), may be global memory.
 //   Srow: the Ly local states of the applied row; lower: lower-environment orientation.
-// Returns the sum of the Ly log factors; *st collects status bits; *wdisc the largest
-// discarded weight (sum of discarded sigma^2 over sum of sigma^2) of any cut.
+// Returns the product of the Ly normalisation factors (in thread 0); *st collects status bits.
 template <typename T, typename G>
-__device__ double env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpad, int row,
-                               const uint8_t* Srow, bool lower, const RowWork<T>& w, int* st,
-                               float* wdisc, int* flag) {
+__device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpad, int row,
+                               const uint8_t* Srow, bool lower, const RowWork<T>& w, int* st, int* flag) {
   const int chi = g.chi, D = g.D, n = g.n, Ly = g.Ly;
   const int tid = threadIdx.x, NT = blockDim.x;
   const int Lr = D * chi;           // row length of X, Y (open leg x truncated bond)
@@ -1043,11 +1126,13 @@ __device__ double env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
   // rows, all of them first in its (i, d) row order.  The products and the QR run on those rows
   // alone (Z stored compactly with ld rk D); the dropped rows are exact zeros that would leave
   // every reflector, and so R, unchanged.
-  blk_unit(w.R, n * n);
+  blk_unit(w.R, n);  // row 0; the later rows of R are read only where a QR wrote them
   __shared__ int rks_s[MAX_LY];  // rks_s[k]: nonzero rows of R_{k-1}
   __syncthreads();
   int rk = 1;
+  __shared__ int ncz_s, bx_s;
   for (int k = 0; k + 1 < Ly; ++k) {
+    if (tid == 0) { ncz_s = 0; bx_s = 0; }
     blk_copy(w.E, Eprev + (size_t)k * g.se, g.se);
     load_A(w.A, Tpad, g, row * Ly + k, Srow[k], lower);
     __syncthreads();
@@ -1071,26 +1156,32 @@ __device__ double env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
     // the columns (b, r) of Z with b at or beyond the bond of E's site k are exact zeros (E's
     // bonds are padded to chi with zeros; the first row has bond D, a truncation keeps at most
     // chi): find the nonzero prefix and factor only it (a zero column leaves every reflector
-    // unchanged and is a zero column of R); R's rank, hence the next rk, is at most that width
-    __shared__ int ncz_s;
-    if (tid == 0) ncz_s = 0;
-    __syncthreads();
+    // unchanged and is a zero column of R); R's rank, hence the next rk, is at most that width.
+    // The bond comes from E, so that only Z's columns from its last index down are looked at.
     {
-      int last = 0;
-      for (int o = tid; o < mZ * n; o += NT)
-        if (w.Z[o] != T(0)) last = max(last, o / mZ + 1);  // NaN compares unequal: kept
-      last = __reduce_max_sync(0xffffffffu, (unsigned)last);
-      if ((tid & 31) == 0 && last) atomicMax(&ncz_s, last);
+      int bx = 0;
+      for (int o = tid; o < g.se; o += NT)
+        if (w.E[o] != T(0)) bx = max(bx, o % chi + 1);  // NaN compares unequal: kept
+      bx = (int)__reduce_max_sync(0xffffffffu, (unsigned)bx);
+      if ((tid & 31) == 0 && bx) atomicMax(&bx_s, bx);
+      __syncthreads();
+      for (int c1 = bx_s * D; c1 > 0; c1 -= D) {
+        int last = 0;
+        for (int o = (c1 - D) * mZ + tid; o < c1 * mZ; o += NT)
+          if (w.Z[o] != T(0)) last = max(last, o / mZ + 1);
+        last = (int)__reduce_max_sync(0xffffffffu, (unsigned)last);
+        if ((tid & 31) == 0 && last) atomicMax(&ncz_s, last);
+        if (__syncthreads_or(last)) break;
+      }
     }
-    __syncthreads();
     const int ncz = ncz_s;
     qr_keep_r<T, GeoMz<G>::value>(w.Z, mZ, ncz, w.R, w.sig, n);
-    blk_copy(w.Rhist + (size_t)k * n * n, w.R, n * n);
     if (tid == 0) rks_s[k] = rk;
-    __syncthreads();
     rk = (mZ < ncz) ? mZ : ncz;
     if (rk > n) rk = n;
     if (rk < 1) rk = 1;
+    blk_copy(w.Rhist + (size_t)k * n * n, w.R, rk * n);
+    __syncthreads();
   }
   if (tid == 0) rks_s[Ly - 1] = rk;  // the rows of R_{Ly-2}, the right pass's first cut
   __syncthreads();
@@ -1104,12 +1195,11 @@ __device__ double env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
   T* Y = P + (size_t)chi * D * D * chi;    // n x Lr   (ld LY)
   T* X = Y + (size_t)n * LY;               // mX x Lr  (ld LX)
   T* Vt = X + (size_t)mX * LX;             // chi x Lr (ld LY)
-  T* Cn = Vt + (size_t)chi * LY;           // n x chi
-  T* Bs = Cn + (size_t)n * chi;            // chi x D x chi (site being written)
+  T* Bs = Vt + (size_t)chi * LY;           // chi x D x chi (the first site)
   // C_{Ly-1}[(b,r)][c] = delta_{(b,r),0} delta_{c,0}
   blk_unit(w.C, n * chi);
   __syncthreads();
-  double logsum = 0.0;
+  Scaled lg = sc_one();
   for (int k = Ly - 1; k >= 0; --k) {
     blk_copy(w.E, Eprev + (size_t)k * g.se, g.se);
     load_A(w.A, Tpad, g, row * Ly + k, Srow[k], lower);
@@ -1130,7 +1220,8 @@ __device__ double env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
         Bs[o] = s;
       }
       __syncthreads();
-      logsum += blk_normalize(Bs, g.se, w.red, st);
+      const double f = (double)blk_normalize(Bs, g.se, w.red, st);
+      if (tid == 0) lg = sc_mul(lg, f);
       blk_copy(Eout, Bs, g.se);
       __syncthreads();
       break;
@@ -1188,32 +1279,30 @@ __device__ double env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
     // rotation would touch)
     int mJ = rks_s[k] < n ? rks_s[k] : n;  // nonzero rows of R_{k-1} (k >= 1 here)
     mJ += (mJ & 1);
-    const int sweeps = hestenes_rows<T, GeoLr<G>::value>(X, mJ < mX ? mJ : mX, Lr, LX, flag, w.ctr, w.red, sig);
+    if (mJ > mX) mJ = mX;
+    const int sweeps = hestenes_rows<T, GeoLr<G>::value>(X, mJ, Lr, LX, flag, w.ctr, w.red, sig);
     if (sweeps < 0 && tid == 0) *st |= ST_NOCONV;
-    // singular values = row norms
-    {
-      const int lane = tid & 31, warp = tid >> 5, nw = NT >> 5;
-      for (int p = warp; p < mX; p += nw) {
-        RT s = 0;
-        for (int i = lane; i < Lr; i += 32) s += abs2_(X[(size_t)p * LX + i]);
-        s = warp_sum(s);
-        if (lane == 0) sig[p] = sqrt(s);
-      }
-    }
+    // singular values: hestenes_rows left those of its rows in sig, the other rows are zero
+    for (int p = mJ + tid; p < mX; p += NT) sig[p] = RT(0);
     __syncthreads();
     // stable descending rank; the first chi ranks are kept.  A NaN singular value (non-finite
     // input) ranks below every number, so that the ranks stay a permutation and every kept
     // index is valid; the sample is flagged.
-    for (int p = tid; p < mX; p += NT) {
-      const RT sp = sig[p];
+    // Four threads count for a row.
+    for (int p0 = 0; p0 < mX; p0 += NT >> 2) {
+      const int p = p0 + (tid >> 2);
+      const RT sp = sig[p < mX ? p : 0];
       const RT kp = (sp == sp) ? sp : RT(-1);
-      if (!(sp == sp) || isinf(sp)) atomicOr(st, (int)ST_NONFINITE);
       int rk = 0;
-      for (int q = 0; q < mX; ++q) {
+      for (int q = tid & 3; q < mX; q += 4) {
         const RT sq = sig[q];
         const RT kq = (sq == sq) ? sq : RT(-1);
         rk += (kq > kp) || (kq == kp && q < p);
       }
+      rk += __shfl_xor_sync(0xffffffffu, rk, 1);
+      rk += __shfl_xor_sync(0xffffffffu, rk, 2);
+      if (p >= mX || (tid & 3) != 0) continue;
+      if (!(sp == sp) || isinf(sp)) atomicOr(st, (int)ST_NONFINITE);
       w.sel[mX + p] = rk;          // rank of row p
       if (rk < chi) w.sel[rk] = p; // row holding rank rk
       if (rk == chi - 1) sig[mX + 0] = sp;  // sigma_(chi-1)
@@ -1253,45 +1342,22 @@ __device__ double env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
         }
         nkeep = kc;
       }
-      // discarded weight and near-degenerate cut at the chosen boundary (the oracle's rule)
-      RT tot = 0, dis = 0;
-      for (int p = tid; p < mX; p += NT) {
-        const RT s2 = sig[p] * sig[p];
-        tot += s2;
-        if (w.sel[mX + p] >= nkeep) dis += s2;
-      }
-      tot = block_sum(tot, w.red);
-      dis = block_sum(dis, w.red);
+      // near-degenerate cut at the chosen boundary (the oracle's rule)
       if (tid == 0 && nkeep < mX) {
         const RT s0 = sig[mX + 2], sk = sig[w.sel[nkeep - 1]];
         const RT sd = (nkeep < chi) ? sig[w.sel[nkeep]] : sig[mX + 1];
         if (s0 > RT(0) && (sk - sd) < RT(1e-8) * s0 && sd > RT(1e-12) * s0) *st |= ST_NEAR_DEGENERATE;
-        if (tot > RT(0)) {
-          const float wd = (float)(dis / tot);
-          if (wd > *wdisc) *wdisc = wd;
-        }
       }
-      __syncthreads();
     } else if (mX > chi) {
-      // discarded weight and near-degenerate cut (same rule as the oracle)
-      RT tot = 0, dis = 0;
-      for (int p = tid; p < mX; p += NT) {
-        const RT s2 = sig[p] * sig[p];
-        tot += s2;
-        if (w.sel[mX + p] >= chi) dis += s2;
-      }
-      tot = block_sum(tot, w.red);
-      dis = block_sum(dis, w.red);
+      // near-degenerate cut (same rule as the oracle)
       if (tid == 0) {
         const RT s0 = sig[mX + 2], sk = sig[mX + 0], sd = sig[mX + 1];
         if (s0 > RT(0) && (sk - sd) < RT(1e-8) * s0 && sd > RT(1e-12) * s0) *st |= ST_NEAR_DEGENERATE;
-        if (tot > RT(0)) {
-          const float wd = (float)(dis / tot);
-          if (wd > *wdisc) *wdisc = wd;
-        }
       }
     }
-    // Vt[c'][q] = X[sel(c')][q] / sigma  (the rows of V^H); rows from nkeep on are zero
+    // Vt[c'][q] = X[sel(c')][q] / sigma  (the rows of V^H); rows from nkeep on are zero.  Its
+    // largest modulus normalises the new site B[c'][d][c] = Vt[c'][(d, c)] on the way out.
+    RT vm = 0;
     for (int o = tid; o < chi * Lr; o += NT) {
       const int q = o % Lr, cp = o / Lr;
       T v = 0;
@@ -1301,34 +1367,50 @@ __device__ double env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
         if (s > RT(0)) v = X[(size_t)p * LX + q] * (RT(1) / s);
       }
       Vt[(size_t)cp * LY + q] = v;
+      vm = fmax(vm, abs_(v));
     }
+    vm = warp_max(vm);
+    RT* rmax = reinterpret_cast<RT*>(w.red);
+    if ((tid & 31) == 0) rmax[tid >> 5] = vm;
     __syncthreads();
-    // C_{k-1} = Y V: C[j][c'] = sum_q Y[j][q] conj(Vt[c'][q]);  new site B[c'][d][c] = Vt[c'][(d,c)]
-    for (int o = tid; o < n * chi; o += NT) {
-      const int cp = o % chi, j = o / chi;
-      const T* Yr = Y + (size_t)j * LY;
-      const T* Vr = Vt + (size_t)cp * LY;
-      T s = 0;
-      for (int q = 0; q < Lr; ++q) s = mad(s, Yr[q], conj_(Vr[q]));
-      Cn[o] = s;
+    vm = rmax[0];
+    for (int i = 1; i < (NT >> 5); ++i) vm = fmax(vm, rmax[i]);
+    RT inv = RT(1);
+    if (!(vm < INFINITY) || vm == RT(0)) {
+      if (tid == 0) { *st |= (vm == RT(0)) ? ST_ZERO_NORM : ST_NONFINITE; lg.m = 0.0; }
+    } else {
+      inv = RT(1) / vm;
+      if (tid == 0) lg = sc_mul(lg, (double)vm);
     }
-    for (int o = tid; o < g.se; o += NT) Bs[o] = Vt[(size_t)(o / Lr) * LY + o % Lr];  // [c'][d][c]
-    __syncthreads();
-    logsum += blk_normalize(Bs, g.se, w.red, st);
-    blk_copy(Eout + (size_t)k * g.se, Bs, g.se);
-    blk_copy(w.C, Cn, n * chi);
-    __syncthreads();
+    T* Ek = Eout + (size_t)k * g.se;
+    for (int o = tid; o < g.se; o += NT) Ek[o] = Vt[(size_t)(o / Lr) * LY + o % Lr] * inv;
+    // C_{k-1} = Y V: C[j][c'] = sum_q Y[j][q] conj(Vt[c'][q])   (C_k was last read by P)
+    if constexpr (Scal<T>::complex) {
+      for (int o = tid; o < n * chi; o += NT) {
+        const int cp = o % chi, j = o / chi;
+        const T* Yr = Y + (size_t)j * LY;
+        const T* Vr = Vt + (size_t)cp * LY;
+        T s = 0;
+        for (int q = 0; q < Lr; ++q) s = mad(s, Yr[q], conj_(Vr[q]));
+        w.C[o] = s;
+      }
+      __syncthreads();
+    } else {
+      blk_gemm<2, 2>(Y, Vt, w.C, n, chi, Lr, 1, 1, 0, 1, 0, [=](int m) { return Off2{m * LY, m * chi}; },
+                     [=](int nn) { return Off2{nn * LY, nn}; });
+    }
   }
-  return logsum;
+  return lg;
 }
 
 // First environment row: row 0 read as an MPS (upper side, e[a=l][p=d][b=r] = A[l][0][r][d])
-// or row Lx-1 (lower side, e[l][u][r] = A[l][u][r][0]); every site normalised.
+// or row Lx-1 (lower side, e[l][u][r] = A[l][u][r][0]); every site normalised.  Returns the product
+// of the factors (in thread 0).
 template <typename T, typename G>
-__device__ double env_first_row(const G& g, T* Eout, const T* Tpad, int row, const uint8_t* Srow,
+__device__ Scaled env_first_row(const G& g, T* Eout, const T* Tpad, int row, const uint8_t* Srow,
                                 bool lower, T* Abuf, T* Bs, double* red, int* st) {
   const int chi = g.chi, D = g.D;
-  double logsum = 0.0;
+  Scaled lg = sc_one();
   for (int k = 0; k < g.Ly; ++k) {
     load_A(Abuf, Tpad, g, row * g.Ly + k, Srow[k], lower);
     __syncthreads();
@@ -1338,11 +1420,12 @@ __device__ double env_first_row(const G& g, T* Eout, const T* Tpad, int row, con
       Bs[o] = (a < D && b < D) ? Abuf[((a * D + 0) * D + b) * D + p] : T(0);
     }
     __syncthreads();
-    logsum += blk_normalize(Bs, g.se, red, st);
+    const double f = (double)blk_normalize(Bs, g.se, red, st);
+    if (threadIdx.x == 0) lg = sc_mul(lg, f);
     blk_copy(Eout + (size_t)k * g.se, Bs, g.se);
     __syncthreads();
   }
-  return logsum;
+  return lg;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1513,11 +1596,10 @@ __device__ T blk_dot(const T* a, const T* b, int n, double* red) {
 // psi_i = E^u[i] . E^l[i+1] of the variational-bound estimator): the plain contraction (no
 // conjugation) over the shared physical legs, column by column from the left,
 //   L'[x][z] = sum_{a, b, p} L[a][b] eu[a][p][x] el[b][p][z],
-// each partial divided by its largest modulus, the log factors added to *lg (the same value
-// in every thread).  Lb, Lb2: chi^2 elements; tb: chi D chi.  Returns the last partial.
+// each partial divided by its largest modulus, the factors multiplied into *lg (in thread 0).  Lb, Lb2: chi^2 elements; tb: chi D chi.  Returns the last partial.
 template <typename T, typename G>
 __device__ T mps_overlap(const G& g, const T* EU, const T* EL, T* Lb, T* Lb2, T* tb, double* red, int* st,
-                         double* lg) {
+                         Scaled* lg) {
   const int chi = g.chi, cd = g.chi * g.D, cc = g.chi * g.chi;
   blk_unit(Lb, cc);
   __syncthreads();
@@ -1540,7 +1622,8 @@ __device__ T mps_overlap(const G& g, const T* EU, const T* EL, T* Lb, T* Lb2, T*
       Lb2[o] = acc;
     }
     __syncthreads();
-    *lg += blk_normalize(Lb2, cc, red, st);
+    const double f = (double)blk_normalize(Lb2, cc, red, st);
+    if (threadIdx.x == 0) *lg = sc_mul(*lg, f);
     blk_copy(Lb, Lb2, cc);
     __syncthreads();
   }
