@@ -221,18 +221,18 @@ static void place_overlay(Plan& p, size_t& smem, size_t budget, const std::vecto
   p.gstride = gl;
 }
 
-// Default shared-memory budget per CTA: FP64 one CTA per SM (the FP64 pipe is the limit), FP32
-// two CTAs per SM.
 // Default shared-memory budget per CTA and kernel class (0 env, 1 row, 2 pair, 3 sampler): FP64
-// one CTA per SM (the FP64 pipe is the limit); FP32 three CTAs per SM (72 KB each, the larger
-// buffers in the L2-resident arena) for the environment, one-row and sampler kernels (the
-// sampler's moves and row steps run as separate launches in FP32), two for the two-row kernel.
+// one CTA of 256 threads per SM (the FP64 pipe is the limit; smaller CTAs share the SM's memory);
+// FP32 three CTAs per SM (72 KB each, the larger buffers in the L2-resident arena) for the
+// environment, one-row and sampler kernels (the sampler's moves and row steps run as separate
+// launches in FP32), two for the two-row kernel; complex FP32 two for every kernel.
 static size_t default_budget(const peps_handle* h, int cls) {
-  if (h->esz >= 8) return 210 * 1024;
-  return (cls == 2) ? 110 * 1024 : 72 * 1024;
+  const bool f64 = h->cfg.prec == PEPS_PREC_FP64;
+  if (f64) return (210 * 1024) / (NTHREADS / cta_threads(8, h->g.n));
+  return (cls == 2 || h->cfg.cplx) ? 110 * 1024 : 72 * 1024;
 }
 // budget of the bound and direct-sampling plans (compiled for two CTAs per SM in FP32)
-static size_t wide_budget(const peps_handle* h) { return (h->esz >= 8) ? 210 * 1024 : 110 * 1024; }
+static size_t wide_budget(const peps_handle* h) { return h->cfg.prec == PEPS_PREC_FP64 ? 210 * 1024 : 110 * 1024; }
 
 static void plan_all(peps_handle* h) {
   const Geo& g = h->g;

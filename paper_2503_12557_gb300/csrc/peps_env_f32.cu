@@ -4,4 +4,5 @@
 
 namespace peps {
 PEPS_INST_ENV(float)
+PEPS_INST_ENV_ROW(float)
 }  // namespace peps

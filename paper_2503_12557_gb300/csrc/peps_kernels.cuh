@@ -4,13 +4,26 @@
 
 namespace peps {
 
-constexpr int NTHREADS = 256;
-// resident blocks per SM the sampler, bound and direct-sampling kernels are compiled for: two in
-// FP32 (about 100 KB of shared memory each), one in FP64 (about 200 KB)
-template <typename T> struct MinBlocks { static constexpr int value = sizeof(T) == 4 ? 2 : 1; };
+constexpr int NTHREADS = 256;  // the most threads of a contraction kernel's CTA
+// resident blocks per SM of 256 threads the sampler, bound and direct-sampling kernels are compiled
+// for: two in FP32, real (about 100 KB of shared memory each) or complex, one in FP64 (200 KB)
+template <typename T> struct MinBlocks { static constexpr int value = sizeof(typename Scal<T>::R) == 4 ? 2 : 1; };
 // the environment kernel in FP32: three blocks per SM (80 registers; measured 10 % faster than
-// two at 8x8, D = 4, chi = 16, where the sampler, which also runs the sandwiches, is 9 % slower)
-template <typename T> struct EnvBlocks { static constexpr int value = sizeof(T) == 4 ? 3 : 1; };
+// two at 8x8, D = 4, chi = 16, where the sampler, which also runs the sandwiches, is 9 % slower);
+// complex FP32 two (5x5, D = 3, chi = 9, 152 samples: 6.65 ms at one per SM, 4.36 ms at two)
+template <typename T> struct EnvBlocks {
+  static constexpr int value = sizeof(T) == 4 ? 3 : (sizeof(typename Scal<T>::R) == 4 ? 2 : 1);
+};
+// Threads of a contraction kernel's CTA.  A CTA works on one sample, and the matrices of a small
+// bond (n = chi D) do not give 256 threads work, while whatever every warp repeats costs per warp:
+// 64 threads for n <= 16 (in FP64, where a kernel uses 255 registers, four samples then share an SM
+// instead of one) and, in FP64, 128 for n <= 32.  Measured, with one output per thread in the FP64
+// products (evaluation, one GB300, before -> after): 4x4, D = 2, chi = 4, 256 samples FP64
+// 3.52 -> 0.61 ms; n <= 32 flip chains 6x6, D = 3, chi = 9 FP64 18.6 -> 15.5 ms.
+inline int cta_threads(int esz_real, int n) {
+  if (n <= 16) return 64;
+  return (n <= 32 && esz_real == 8) ? 128 : NTHREADS;
+}
 
 // term record (ints): number of sites, the sites, window (first row, first column, width,
 // two-row flag) and the entry range
@@ -70,6 +83,10 @@ cudaError_t kattr_batch(size_t set_bytes, int* occ, size_t occ_smem);
 template <typename T>
 cudaError_t launch_env(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
                        int sides, T* envs, double* logs, int* status, cudaStream_t s);
+// one environment row of every chain (the FP32 sampler's row steps, on the environment plan)
+template <typename T>
+cudaError_t launch_env_row(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
+                           int x, int lower, T* envs, double* logs, int* status, int* ustat, cudaStream_t s);
 template <typename T>
 cudaError_t launch_row(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
                        int x_lo, int x_hi, const T* envs, const double* logs, T* O, const long long* site_off,

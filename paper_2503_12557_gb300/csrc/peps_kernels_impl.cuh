@@ -1066,7 +1066,7 @@ static cudaError_t with_geo_for(const Geo& g, F&& f) {
       using GG = decltype(gg);                                                                                   \
       cudaError_t e = cudaSuccess;                                                                               \
       if (set_bytes) e = cudaFuncSetAttribute(KERNEL<T, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)set_bytes); \
-      if (e == cudaSuccess && occ) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, KERNEL<T, GG>, NTHREADS, occ_smem); \
+      if (e == cudaSuccess && occ) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, KERNEL<T, GG>, cta_threads(sizeof(typename Scal<T>::R), g.n), occ_smem); \
       return e;                                                                                                  \
     });                                                                                                          \
   }
@@ -1158,11 +1158,32 @@ template <typename T>
 cudaError_t launch_env(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
                        int sides, T* envs, double* logs, int* status, cudaStream_t s) {
   return with_geo_for<T>(g, [&](auto gg) {
-    k_env<T, decltype(gg)><<<grid, NTHREADS, smem, s>>>(gg, p, Tpad, S, Ns, sides, envs, logs, status);
+    k_env<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n), smem, s>>>(gg, p, Tpad, S, Ns, sides, envs, logs, status);
     return cudaGetLastError();
   });
 }
-PEPS_KATTR(kattr_env, k_env)
+template <typename T>
+cudaError_t launch_env_row(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
+                           int x, int lower, T* envs, double* logs, int* status, int* ustat, cudaStream_t s) {
+  return with_geo_for<T>(g, [&](auto gg) {
+    k_env_row<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n), smem, s>>>(
+        gg, p, Tpad, S, Ns, x, lower, envs, logs, status, ustat);
+    return cudaGetLastError();
+  });
+}
+PEPS_KATTR(kattr_env_only, k_env)
+PEPS_KATTR(kattr_env_row, k_env_row)
+// k_env and, in FP32, the sampler's k_env_row, which runs on the same plan
+template <typename T>
+cudaError_t kattr_env(const Geo& g, size_t set_bytes, int* occ, size_t occ_smem) {
+  cudaError_t e = cudaSuccess;
+  if constexpr (sizeof(T) == 4)
+    if (set_bytes) e = kattr_env_row<T>(g, set_bytes, nullptr, 0);
+  return e == cudaSuccess ? kattr_env_only<T>(g, set_bytes, occ, occ_smem) : e;
+}
+#define PEPS_INST_ENV_ROW(T)                                                                                      \
+  template cudaError_t launch_env_row<T>(const Geo&, const Plan&, int, size_t, const T*, const uint8_t*, int, int, int, T*, \
+                                         double*, int*, int*, cudaStream_t);
 #define PEPS_INST_ENV(T)                                                                                          \
   template cudaError_t launch_env<T>(const Geo&, const Plan&, int, size_t, const T*, const uint8_t*, int, int, T*, \
                                      double*, int*, cudaStream_t);                                        \
@@ -1175,7 +1196,7 @@ cudaError_t launch_row(const Geo& g, const Plan& p, int grid, size_t smem, const
                        int x_lo, int x_hi, const T* envs, const double* logs, T* O, const long long* site_off,
                        long long Np, const TermTab& tt, double* rowout, int* status, cudaStream_t s) {
   return with_geo_for<T>(g, [&](auto gg) {
-    k_row<T, decltype(gg)><<<grid, NTHREADS, smem, s>>>(gg, p, Tpad, S, Ns, x_lo, x_hi, envs, logs, O, site_off, Np,
+    k_row<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n), smem, s>>>(gg, p, Tpad, S, Ns, x_lo, x_hi, envs, logs, O, site_off, Np,
                                                         tt, rowout, status);
     return cudaGetLastError();
   });
@@ -1184,7 +1205,7 @@ template <typename T>
 cudaError_t launch_pair(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
                         const T* envs, const double* logs, const TermTab& tt, double* pairout, int* status, cudaStream_t s) {
   return with_geo_for<T>(g, [&](auto gg) {
-    k_pair<T, decltype(gg)><<<grid, NTHREADS, smem, s>>>(gg, p, Tpad, S, Ns, envs, logs, tt, pairout, status);
+    k_pair<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n), smem, s>>>(gg, p, Tpad, S, Ns, envs, logs, tt, pairout, status);
     return cudaGetLastError();
   });
 }
@@ -1215,60 +1236,48 @@ cudaError_t launch_sample(const Geo& g, const Plan& p, int grid, size_t smem, co
                           size_t smem_e, const T* Tpad, uint8_t* S, int Ns, int move, int nsweeps,
                           unsigned long long seed, unsigned long long sweep0, T* envs, double* logs,
                           long long* accepted, int* status, int* ustat, cudaStream_t s) {
+  const int nt = cta_threads(sizeof(typename Scal<T>::R), g.n);
   return with_geo_for<T>(g, [&](auto gg) {
     using GG = decltype(gg);
     if constexpr (sizeof(T) == 4) {
+      cudaError_t e = cudaSuccess;
       for (int t = 0; t < nsweeps; ++t) {
         const unsigned long long sid = sweep0 + t;
         const int up = (int)(sid & 1ull);
         int* us = (t == nsweeps - 1) ? ustat : nullptr;
-        if (!up) {
-          k_env<T, GG><<<grid_e, NTHREADS, smem_e, s>>>(gg, pe, Tpad, S, Ns, 2, envs, logs, status);
-          for (int x = 0; x < g.Lx; ++x) {
-            k_sweep_moves<T, GG><<<grid, NTHREADS, smem, s>>>(gg, p, Tpad, S, Ns, move, x, 0, seed, sid, envs, logs,
-                                                              accepted, status);
-            if (x < g.Lx - 1)
-              k_env_row<T, GG><<<grid_e, NTHREADS, smem_e, s>>>(gg, pe, Tpad, S, Ns, x, 0, envs, logs, status, us);
-          }
-        } else {
-          // the previous sweep of this call left the upper environments of these configurations
-          if (t == 0) k_env<T, GG><<<grid_e, NTHREADS, smem_e, s>>>(gg, pe, Tpad, S, Ns, 1, envs, logs, status);
-          for (int x = g.Lx - 1; x >= 0; --x) {
-            k_sweep_moves<T, GG><<<grid, NTHREADS, smem, s>>>(gg, p, Tpad, S, Ns, move, x, 1, seed, sid, envs, logs,
-                                                              accepted, status);
-            if (x > 0)
-              k_env_row<T, GG><<<grid_e, NTHREADS, smem_e, s>>>(gg, pe, Tpad, S, Ns, x, 1, envs, logs, status, us);
-          }
+        // a downward sweep starts from the lower environments of its configurations; an upward one
+        // from the upper ones, which the previous sweep of this call left
+        if (!up || t == 0) {
+          if ((e = launch_env<T>(g, pe, grid_e, smem_e, Tpad, S, Ns, up ? 1 : 2, envs, logs, status, s)) != cudaSuccess) return e;
+        }
+        for (int i = 0; i < g.Lx; ++i) {
+          const int x = up ? g.Lx - 1 - i : i;
+          k_sweep_moves<T, GG><<<grid, nt, smem, s>>>(gg, p, Tpad, S, Ns, move, x, up, seed, sid, envs, logs, accepted,
+                                                      status);
+          if (i < g.Lx - 1 &&
+              (e = launch_env_row<T>(g, pe, grid_e, smem_e, Tpad, S, Ns, x, up, envs, logs, status, us, s)) != cudaSuccess)
+            return e;
         }
       }
     } else {
-      k_sample<T, GG><<<grid, NTHREADS, smem, s>>>(gg, p, Tpad, S, Ns, move, nsweeps, seed, sweep0, envs, logs,
-                                                   accepted, status);
+      k_sample<T, GG><<<grid, nt, smem, s>>>(gg, p, Tpad, S, Ns, move, nsweeps, seed, sweep0, envs, logs, accepted, status);
     }
     return cudaGetLastError();
   });
 }
 template <typename T>
 cudaError_t kattr_sample(const Geo& g, size_t set_bytes, int* occ, size_t occ_smem) {
+  const int nt = cta_threads(sizeof(typename Scal<T>::R), g.n);
   return with_geo_for<T>(g, [&](auto gg) {
     using GG = decltype(gg);
-    cudaError_t e = cudaSuccess;
-    if (set_bytes) {
-      e = cudaFuncSetAttribute(k_sample<T, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)set_bytes);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_sweep_moves<T, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)set_bytes);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_env_row<T, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)set_bytes);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_env<T, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)set_bytes);
-    }
-    if (e == cudaSuccess && occ) {
-      if constexpr (sizeof(T) == 4)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k_sweep_moves<T, GG>, NTHREADS, occ_smem);
-      else
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k_sample<T, GG>, NTHREADS, occ_smem);
-    }
-    return e;
+    auto kernel = [&](auto* k) {
+      cudaError_t e = cudaSuccess;
+      if (set_bytes) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)set_bytes);
+      if (e == cudaSuccess && occ) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, nt, occ_smem);
+      return e;
+    };
+    if constexpr (sizeof(T) == 4) return kernel(&k_sweep_moves<T, GG>);
+    else return kernel(&k_sample<T, GG>);
   });
 }
 #define PEPS_INST_SAMPLE(T)                                                                                       \
@@ -1284,7 +1293,7 @@ cudaError_t launch_bound(const Geo& g, const Plan& p, int grid, size_t smem, con
                          int cut, const T* envs, const double* logs, const TermTab& tt, double* bout, double* logabs,
                          double* phase, int* status, cudaStream_t s) {
   return with_geo_for<T>(g, [&](auto gg) {
-    k_bound<T, decltype(gg)><<<grid, NTHREADS, smem, s>>>(gg, p, Tpad, S, Ns, cut, envs, logs, tt, bout, logabs, phase,
+    k_bound<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n), smem, s>>>(gg, p, Tpad, S, Ns, cut, envs, logs, tt, bout, logabs, phase,
                                                           status);
     return cudaGetLastError();
   });

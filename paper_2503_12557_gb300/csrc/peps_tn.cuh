@@ -99,6 +99,22 @@ template <> __device__ __forceinline__ cplx<double> from_dz<cplx<double>>(dz a) 
 __device__ __forceinline__ float re_(float x) { return x; }
 __device__ __forceinline__ double re_(double x) { return x; }
 template <typename R> __device__ __forceinline__ R re_(const cplx<R>& z) { return z.re; }
+// x != 0 (NaN counts as nonzero); doubles by their bits, off the FP64 pipe
+__device__ __forceinline__ bool nonzero_(float x) { return x != 0.f; }
+__device__ __forceinline__ bool nonzero_(double x) { return (__double_as_longlong(x) << 1) != 0; }
+template <typename R> __device__ __forceinline__ bool nonzero_(const cplx<R>& z) { return nonzero_(z.re) || nonzero_(z.im); }
+// Keys of non-negative numbers as integers of the same order (NaN: -1, below every number)
+__device__ __forceinline__ int order_key(float x) { return x == x ? __float_as_int(x) : -1; }
+__device__ __forceinline__ long long order_key(double x) {
+  const long long b = __double_as_longlong(x);
+  return b <= 0x7ff0000000000000ll ? b : -1;
+}
+// max of non-negative numbers, a NaN left out as fmax does; doubles by their bits
+__device__ __forceinline__ float max_(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double max_(double a, double b) {
+  const long long x = order_key(a), y = order_key(b), m = x > y ? x : y;
+  return __longlong_as_double(m > 0 ? m : 0);
+}
 // 1 / z
 __device__ __forceinline__ float inv_(float x) { return 1.f / x; }
 __device__ __forceinline__ double inv_(double x) { return 1.0 / x; }
@@ -303,15 +319,16 @@ template <typename T>
 __device__ typename Scal<T>::R blk_normalize(T* v, int n, double* red, int* st) {
   using R = typename Scal<T>::R;
   R m = 0;
-  for (int o = threadIdx.x; o < n; o += blockDim.x) m = fmax(m, abs_(v[o]));
-  m = warp_max(m);
+  for (int o = threadIdx.x; o < n; o += blockDim.x) m = max_(m, abs_(v[o]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max_(m, __shfl_xor_sync(0xffffffffu, m, o));
   const int nw = blockDim.x >> 5;
   R* r = reinterpret_cast<R*>(red);
   if ((threadIdx.x & 31) == 0) r[threadIdx.x >> 5] = m;
   __syncthreads();
   m = r[0];
-  for (int i = 1; i < nw; ++i) m = fmax(m, r[i]);
-  if (!(m < INFINITY) || m == R(0)) {  // NaN, Inf or zero
+  for (int i = 1; i < nw; ++i) m = max_(m, r[i]);
+  if (!(m < INFINITY) || m == R(0)) {  // Inf or zero
     if (threadIdx.x == 0) *st |= (m == R(0)) ? ST_ZERO_NORM : ST_NONFINITE;
     __syncthreads();
     return R(0);
@@ -425,6 +442,38 @@ __device__ void qr_keep_r_smem(T* Z, int m, int nc, T* R, T* taus, int ldr) {
   __syncthreads();
 }
 
+// beta, tau and the scale 1 / (alpha - beta) of xLARFG's reflector for a real column with head
+// alpha and squared tail norm sigma > 0.  Double: one reciprocal square root and one reciprocal,
+// each a single-precision start and two Newton steps, where sqrt and two divisions would be
+// about 70 instructions of 64 cycles on the FP64 pipes (tau = 1 + |alpha| / norm).
+__device__ __forceinline__ void reflector(float alpha, float sigma, float& beta, float& tau, float& sc) {
+  const float nrm = sqrt(alpha * alpha + sigma);
+  beta = (alpha >= 0.f) ? -nrm : nrm;
+  tau = (beta - alpha) / beta;
+  sc = 1.f / (alpha - beta);
+}
+__device__ __forceinline__ void reflector(double alpha, double sigma, double& beta, double& tau, double& sc) {
+  const double n2 = fma(alpha, alpha, sigma);
+  if (n2 > 1e-30 && n2 < 1e30) {
+    double y = (double)rsqrtf((float)n2);
+    const double h = -0.5 * n2;
+    y = y * fma(h, y * y, 1.5);
+    y = y * fma(h, y * y, 1.5);
+    const double nrm = n2 * y, aa = fabs(alpha), d = aa + nrm;
+    tau = fma(aa, y, 1.0);
+    double r = (double)__frcp_rn((float)d);
+    r = fma(r, fma(-d, r, 1.0), r);
+    r = fma(r, fma(-d, r, 1.0), r);
+    beta = (alpha >= 0.0) ? -nrm : nrm;
+    sc = (alpha >= 0.0) ? r : -r;
+  } else {
+    const double nrm = sqrt(n2);
+    beta = (alpha >= 0.0) ? -nrm : nrm;
+    tau = (beta - alpha) / beta;
+    sc = 1.0 / (alpha - beta);
+  }
+}
+
 // Panel of QB columns (j0 .. j0+pb-1) factored by one warp with the columns in registers
 // (element i = lane + 32 r, m <= 32 RPL): per column one warp reduction for the norm and one
 // independent reduction per remaining panel column, no shared-memory round trips.
@@ -453,10 +502,8 @@ __device__ __forceinline__ void qr_panel_reg(T* Z, int m, int j0, int pb, T* tau
       const T alpha = __shfl_sync(0xffffffffu, aj, j & 31);
       T tau = 0, beta = alpha;
       if (sigma != T(0)) {
-        const T nrm = sqrt(alpha * alpha + sigma);
-        beta = (alpha >= T(0)) ? -nrm : nrm;
-        tau = (beta - alpha) / beta;
-        const T sc = T(1) / (alpha - beta);
+        T sc;
+        reflector(alpha, sigma, beta, tau, sc);
 #pragma unroll
         for (int r = 0; r < RPL; ++r)
           if (lane + 32 * r > j) zp[jj][r] *= sc;
@@ -510,7 +557,9 @@ template <typename T, int RPL>
 __device__ __noinline__ void qr_keep_r_reg(T* Z, int m, int nc, T* R, T* taus, int ldr) {
   // FP32 with 256 rows: panels of four columns, whose register panel (4 x 8 values a lane)
   // fits the environment kernels' 80 registers; eight columns spilled there
-  constexpr int QB = (RPL == 8 && sizeof(T) == 4) ? 4 : 8;
+  // (FP64: two columns, since a warp alone has only its sub-partition's FP64 pipe, a quarter of the
+  // SM's, and the trailing columns are spread over all four)
+  constexpr int QB = sizeof(T) == 8 ? 2 : (RPL == 8 ? 4 : 8);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int steps = (m < nc) ? m : nc;
   for (int j0 = 0; j0 < steps; j0 += QB) {
@@ -528,10 +577,8 @@ __device__ __noinline__ void qr_keep_r_reg(T* Z, int m, int nc, T* R, T* taus, i
           const T alpha = zj[j];
           T tau = 0, beta = alpha;
           if (sigma != T(0)) {
-            const T nrm = sqrt(alpha * alpha + sigma);
-            beta = (alpha >= T(0)) ? -nrm : nrm;
-            tau = (beta - alpha) / beta;
-            const T sc = T(1) / (alpha - beta);
+            T sc;
+            reflector(alpha, sigma, beta, tau, sc);
             for (int i = j + 1 + lane; i < m; i += 32) zj[i] *= sc;
           }
           __syncwarp();
@@ -1057,7 +1104,7 @@ struct Off2 {
   int a, c;
 };
 template <int RM, int RN, typename T, class FM, class FN>
-__device__ __forceinline__ void blk_gemm(const T* __restrict__ A, const T* __restrict__ B, T* __restrict__ C, int M,
+__device__ __forceinline__ void blk_gemm_tile(const T* __restrict__ A, const T* __restrict__ B, T* __restrict__ C, int M,
                                          int N, int K1, int K2, int sa1, int sa2, int sb1, int sb2, FM fm, FN fn) {
   const int tm = (M + RM - 1) / RM, tn = (N + RN - 1) / RN;
   for (int t = threadIdx.x; t < tm * tn; t += blockDim.x) {
@@ -1106,6 +1153,14 @@ __device__ __forceinline__ void blk_gemm(const T* __restrict__ A, const T* __res
         if (mv[i] && nv[j]) C[co[i] + cn[j]] = acc[i][j];
   }
   __syncthreads();
+}
+// In FP64 one output per thread: a multiply-add holds its SM sub-partition for 64 cycles, so that
+// operand loads are free beside it and what counts is to have all four sub-partitions busy.
+template <int RM, int RN, typename T, class FM, class FN>
+__device__ __forceinline__ void blk_gemm(const T* __restrict__ A, const T* __restrict__ B, T* __restrict__ C, int M,
+                                         int N, int K1, int K2, int sa1, int sa2, int sb1, int sb2, FM fm, FN fn) {
+  constexpr bool f64 = sizeof(typename Scal<T>::R) == 8;
+  blk_gemm_tile<f64 ? 1 : RM, f64 ? 1 : RN>(A, B, C, M, N, K1, K2, sa1, sa2, sb1, sb2, fm, fn);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1161,14 +1216,14 @@ __device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
     {
       int bx = 0;
       for (int o = tid; o < g.se; o += NT)
-        if (w.E[o] != T(0)) bx = max(bx, o % chi + 1);  // NaN compares unequal: kept
+        if (nonzero_(w.E[o])) bx = max(bx, o % chi + 1);
       bx = (int)__reduce_max_sync(0xffffffffu, (unsigned)bx);
       if ((tid & 31) == 0 && bx) atomicMax(&bx_s, bx);
       __syncthreads();
       for (int c1 = bx_s * D; c1 > 0; c1 -= D) {
         int last = 0;
         for (int o = (c1 - D) * mZ + tid; o < c1 * mZ; o += NT)
-          if (w.Z[o] != T(0)) last = max(last, o / mZ + 1);
+          if (nonzero_(w.Z[o])) last = max(last, o / mZ + 1);
         last = (int)__reduce_max_sync(0xffffffffu, (unsigned)last);
         if ((tid & 31) == 0 && last) atomicMax(&ncz_s, last);
         if (__syncthreads_or(last)) break;
@@ -1239,7 +1294,16 @@ __device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
     // triangular (explicit zeros below the diagonal) its sums start at j = 8b: the terms skipped
     // are exact zeros and the others are added in the same order as the full product.  Rows from
     // rkx on are zero.
-    {
+    if constexpr (sizeof(typename Scal<T>::R) == 8) {
+      for (int o = tid; o < mX * Lr; o += NT) {  // one output per thread, as in blk_gemm
+        const int q = o % Lr, i = o / Lr;
+        T acc = T(0);
+        if (i < rkx)
+          for (int j = i; j < n; ++j) acc = mad(acc, Y[(size_t)j * LY + q], w.R[(size_t)i * n + j]);
+        X[(size_t)i * LX + q] = acc;
+      }
+      __syncthreads();
+    } else {
       const int nbk = (rkx + 7) / 8, tmq = (Lr + 1) / 2;
       for (int t = tid; t < tmq * nbk; t += NT) {
         const int ti = t % tmq, b = t / tmq;
@@ -1292,11 +1356,10 @@ __device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
     for (int p0 = 0; p0 < mX; p0 += NT >> 2) {
       const int p = p0 + (tid >> 2);
       const RT sp = sig[p < mX ? p : 0];
-      const RT kp = (sp == sp) ? sp : RT(-1);
+      const auto kp = order_key(sp);
       int rk = 0;
       for (int q = tid & 3; q < mX; q += 4) {
-        const RT sq = sig[q];
-        const RT kq = (sq == sq) ? sq : RT(-1);
+        const auto kq = order_key(sig[q]);
         rk += (kq > kp) || (kq == kp && q < p);
       }
       rk += __shfl_xor_sync(0xffffffffu, rk, 1);
@@ -1367,14 +1430,15 @@ __device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
         if (s > RT(0)) v = X[(size_t)p * LX + q] * (RT(1) / s);
       }
       Vt[(size_t)cp * LY + q] = v;
-      vm = fmax(vm, abs_(v));
+      vm = max_(vm, abs_(v));
     }
-    vm = warp_max(vm);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) vm = max_(vm, __shfl_xor_sync(0xffffffffu, vm, o));
     RT* rmax = reinterpret_cast<RT*>(w.red);
     if ((tid & 31) == 0) rmax[tid >> 5] = vm;
     __syncthreads();
     vm = rmax[0];
-    for (int i = 1; i < (NT >> 5); ++i) vm = fmax(vm, rmax[i]);
+    for (int i = 1; i < (NT >> 5); ++i) vm = max_(vm, rmax[i]);
     RT inv = RT(1);
     if (!(vm < INFINITY) || vm == RT(0)) {
       if (tid == 0) { *st |= (vm == RT(0)) ? ST_ZERO_NORM : ST_NONFINITE; lg.m = 0.0; }
@@ -1458,8 +1522,8 @@ __device__ BondExt bond_ext(const G& g, const T* eu, const T* el) {
   int ea = 0, ex = 0, eb = 0, ez = 0;
   for (int o = threadIdx.x; o < g.se; o += blockDim.x) {
     const int a = o / Dc + 1, x = o % chi + 1;
-    if (eu[o] != T(0)) { ea = max(ea, a); ex = max(ex, x); }
-    if (el[o] != T(0)) { eb = max(eb, a); ez = max(ez, x); }
+    if (nonzero_(eu[o])) { ea = max(ea, a); ex = max(ex, x); }
+    if (nonzero_(el[o])) { eb = max(eb, a); ez = max(ez, x); }
   }
   const unsigned full = 0xffffffffu;
   ea = (int)__reduce_max_sync(full, (unsigned)ea);
@@ -1584,11 +1648,23 @@ __device__ void site_env1(const G& g, const T* L, const T* eu, const T* elT, con
                  [=](int n) { return Off2{(n / D) * D * S1 + (n % D) * S1, ((n % D) * D + n / D) * D * D}; });
 }
 
+// sum_i a_i b_i, summed as 256 threads do it whatever the CTA's size (a smaller CTA's threads stand
+// in for several), so that the result does not depend on the launch shape.
 template <typename T>
 __device__ T blk_dot(const T* a, const T* b, int n, double* red) {
-  T s = 0;
-  for (int o = threadIdx.x; o < n; o += blockDim.x) s += a[o] * b[o];
-  return block_sum(s, red);
+  const int l = threadIdx.x & 31;
+  T* r = reinterpret_cast<T*>(red);
+  __syncthreads();
+  for (int w = threadIdx.x >> 5; w < 8; w += blockDim.x >> 5) {
+    T s = 0;
+    if (w * 32 < n) {
+      for (int o = w * 32 + l; o < n; o += 256) s += a[o] * b[o];
+      s = warp_sum(s);
+    }
+    if (l == 0) r[w] = s;
+  }
+  __syncthreads();
+  return warp_sum(l < 8 ? r[l] : T(0));
 }
 
 // ------------------------------------------------------------------------------------------
