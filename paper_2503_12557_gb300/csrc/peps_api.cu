@@ -221,20 +221,30 @@ static void place_overlay(Plan& p, size_t& smem, size_t budget, const std::vecto
   p.gstride = gl;
 }
 
-// Default shared-memory budget per CTA and kernel class (0 env, 1 row, 2 pair, 3 sampler): FP64
-// one CTA of 256 threads per SM (the FP64 pipe is the limit; smaller CTAs share the SM's memory);
-// FP32 three CTAs per SM (72 KB each, the larger buffers in the L2-resident arena) for the
-// environment, one-row and sampler kernels (the sampler's moves and row steps run as separate
+// Default shared-memory budget per CTA of 256 threads and kernel class (0 env, 1 row, 2 pair, 3
+// sampler); what does not fit is in the L2-resident arena.  FP64: one CTA of 256 threads per SM (the
+// FP64 pipe is the limit; smaller CTAs share the SM's memory); FP32 three CTAs per SM (72 KB each) for
+// the environment, one-row and sampler kernels (the sampler's moves and row steps run as separate
 // launches in FP32), two for the two-row kernel; complex FP32 two for every kernel.
 static size_t default_budget(const peps_handle* h, int cls) {
   const bool f64 = h->cfg.prec == PEPS_PREC_FP64;
-  if (f64) return (210 * 1024) / (NTHREADS / cta_threads(8, h->g.n));
+  if (f64) return (210 * 1024) / (NTHREADS / cta_threads(8, h->g.n, 1));
   return (cls == 2 || h->cfg.cplx) ? 110 * 1024 : 72 * 1024;
+}
+// Parts a budget is shared in: FP32 beyond n = 16, where the handle's batch gives more than three items
+// per SM, two CTAs of half the size and threads (cta_threads), the moves of more than six chains per SM
+// four of a quarter.
+static size_t budget_parts(const peps_handle* h, int cls) {
+  const long long per[4] = {2, h->g.Lx, h->g.Lx - 1, 1};
+  const long long items = (long long)h->cfg.max_samples * per[cls];
+  if (h->cfg.prec == PEPS_PREC_FP64 || h->g.n <= 16 || items <= 3 * N_SM) return 1;
+  return cls == 3 && !h->cfg.cplx && items > 6 * N_SM ? 4 : 2;
 }
 // budget of the bound and direct-sampling plans (compiled for two CTAs per SM in FP32)
 static size_t wide_budget(const peps_handle* h) { return h->cfg.prec == PEPS_PREC_FP64 ? 210 * 1024 : 110 * 1024; }
 
-static void plan_all(peps_handle* h) {
+// (split: at the budgets' parts; a batch's CTAs take them whole)
+static void plan_all(peps_handle* h, bool split = true) {
   const Geo& g = h->g;
   const size_t E = h->esz;
   const int n = g.n, chi = g.chi, D = g.D, Ly = g.Ly;
@@ -242,7 +252,8 @@ static void plan_all(peps_handle* h) {
   const int Lr = D * chi;
   for (int i = 0; i < 4; ++i)
     if (h->budget[i] == 0) h->budget[i] = default_budget(h, i);
-  size_t budget = h->budget[0];
+  auto part = [&](int cls) { return h->budget[cls] / (split ? budget_parts(h, cls) : 1); };
+  size_t budget = part(0);
   int ci = std::min(n, 8);
   const size_t zsz = env_z_elems(chi, D);
   // one-row / two-row temporaries
@@ -257,7 +268,7 @@ static void plan_all(peps_handle* h) {
     k.p.cx = cx;
     std::vector<std::pair<int, size_t>> b = {
         {B_RED, 40 * 8}, {B_SIG, (mX + 4) * E}, {B_SEL, 2 * mX * 4}, {B_A, (size_t)g.sT * E}, {B_E, (size_t)g.se * E},
-        {B_C, (size_t)n * chi * E}, {B_W, env_w_elems(chi, D, ci) * E}, {B_R, (size_t)n * n * E}, {B_Z, zsz * E},
+        {B_C, (size_t)n * chi * E}, {B_W, env_w_elems(chi, D, ci) * E}, {B_ZS, (size_t)env_zs_elems(chi, D) * E}, {B_R, (size_t)n * n * E}, {B_Z, zsz * E},
         {B_RHIST, (size_t)std::max(1, Ly - 1) * n * n * E}};
     place(k.p, k.smem, budget, b);
   }
@@ -269,14 +280,14 @@ static void plan_all(peps_handle* h) {
     k.p.cx = cx;
     std::vector<std::pair<int, size_t>> b = {
         {B_RED, 40 * 8}, {B_SIG, (mX + 4) * E}, {B_SEL, 2 * mX * 4}, {B_A, (size_t)g.sT * E}, {B_E, (size_t)g.se * E},
-        {B_C, (size_t)n * chi * E}, {B_W, env_w_elems(chi, D, ci) * E}, {B_R, (size_t)n * n * E}, {B_Z, zsz * E},
+        {B_C, (size_t)n * chi * E}, {B_W, env_w_elems(chi, D, ci) * E}, {B_ZS, (size_t)env_zs_elems(chi, D) * E}, {B_R, (size_t)n * n * E}, {B_Z, zsz * E},
         {B_RHIST, (size_t)std::max(1, Ly - 1) * n * n * E}, {B_S, (size_t)g.Lx * g.Ly},
         {B_LW, (size_t)2 * chi * chi * E}, {B_LW2, (size_t)g.se * E}, {B_LP, (size_t)2 * Ly * g.se * E},
         {B_RP, (size_t)2 * Ly * g.se * E}};
     place(k.p, k.smem, wide_budget(h), b);
   }
   // row plan
-  budget = h->budget[1];
+  budget = part(1);
   {
     KPlan& k = h->kp[1];
     k.p.ci = ci;
@@ -288,7 +299,7 @@ static void plan_all(peps_handle* h) {
     place(k.p, k.smem, budget, b);
   }
   // pair plan
-  budget = h->budget[2];
+  budget = part(2);
   {
     KPlan& k = h->kp[2];
     k.p.ci = ci;
@@ -300,7 +311,7 @@ static void plan_all(peps_handle* h) {
     place(k.p, k.smem, budget, b);
   }
   // sampler plan: union of the above
-  budget = h->budget[3];
+  budget = part(3);
   {
     KPlan& k = h->kp[3];
     k.p.ci = ci;
@@ -315,7 +326,7 @@ static void plan_all(peps_handle* h) {
         {B_RED, 40 * 8}, {B_SIG, (mX + 4) * E}, {B_SEL, 2 * mX * 4}, {B_S, (size_t)g.Lx * g.Ly}, {B_A, (size_t)g.sT * E}};
     std::vector<std::pair<int, size_t>> rowstep = {
         {B_E, (size_t)g.se * E}, {B_C, (size_t)n * chi * E}, {B_W, env_w_elems(chi, D, ci) * E},
-        {B_R, (size_t)n * n * E}, {B_Z, zsz * E}, {B_RHIST, (size_t)std::max(1, Ly - 1) * n * n * E}};
+        {B_ZS, (size_t)env_zs_elems(chi, D) * E}, {B_R, (size_t)n * n * E}, {B_Z, zsz * E}, {B_RHIST, (size_t)std::max(1, Ly - 1) * n * n * E}};
     std::vector<std::pair<int, size_t>> sandwich = {
         {B_A2, (size_t)g.sT * E}, {B_EU, (size_t)g.se * E}, {B_EL, (size_t)g.se * E}, {B_T1, tt * E},
         {B_T2, tt * E}, {B_LW, lw * E}, {B_LW2, lw * E}, {B_LP, lw * E}, {B_RP, (size_t)(Ly + 1) * lw * E}};
@@ -783,7 +794,7 @@ extern "C" peps_status peps_direct_prepare(peps_handle* h, int chi_double, void*
   k.p.cx = h->kp[0].p.cx;
   std::vector<std::pair<int, size_t>> b = {
       {B_RED, 40 * 8}, {B_SIG, (mX + 4) * E}, {B_SEL, 2 * mX * 4}, {B_A, (size_t)g.sT * E}, {B_E, (size_t)g.se * E},
-      {B_C, (size_t)n * chi * E}, {B_W, env_w_elems(chi, D, ci) * E}, {B_R, (size_t)n * n * E},
+      {B_C, (size_t)n * chi * E}, {B_W, env_w_elems(chi, D, ci) * E}, {B_ZS, (size_t)env_zs_elems(chi, D) * E}, {B_R, (size_t)n * n * E},
       {B_Z, env_z_elems(chi, D) * E}, {B_RHIST, (size_t)std::max(1, Ly - 1) * n * n * E}, {B_S, (size_t)Lx * Ly},
       {B_EU, (size_t)2 * Ly * g.se * E}, {B_LW2, (size_t)(g.d + 1) * rsz * E}, {B_RP, (size_t)(Ly + 1) * rsz * E},
       {B_LP, tsz * E}, {B_LW, tsz * E}, {B_T1, ksz * E}, {B_T2, ksz * E}};
@@ -1392,7 +1403,7 @@ static void plans_at(peps_handle* h, size_t budget, Plan* pe, Plan* pr, Plan* pq
   KPlan kb = h->kb;
   size_t bud[4] = {h->budget[0], h->budget[1], h->budget[2], h->budget[3]};
   h->budget[0] = h->budget[1] = h->budget[2] = budget;
-  plan_all(h);
+  plan_all(h, false);
   *pe = h->kp[0].p;
   *pr = h->kp[1].p;
   *pq = h->kp[2].p;

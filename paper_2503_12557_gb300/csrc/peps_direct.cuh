@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(NTHREADS) k_dl_env(G g, int chid, const T* __r
         w.Z[o] = acc;
       }
       __syncthreads();
-      qr_keep_r_smem(w.Z, mZ, nb, w.Rh + (size_t)k * nb * nb, taus, nb);
+      qr_keep_r_smem(w.Z, mZ, nb, w.Rh + (size_t)k * nb * nb, taus, nb, nb, nb, (T*)nullptr);
     }
     // ---- right pass
     blk_unit(w.C, nb * chid);
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(NTHREADS) k_dl_env(G g, int chid, const T* __r
         w.X[(size_t)i * LX + q] = acc;
       }
       __syncthreads();
-      const int sweeps = hestenes_rows<T, 0>(w.X, mX, Lr, LX, &flag, nullptr, red, sig);
+      const int sweeps = hestenes_rows(w.X, mX, Lr, LX, &flag, nullptr, red, sig, (T*)nullptr, 0);
       if (sweeps < 0 && tid == 0) st |= ST_NOCONV;
       // hestenes_rows left the singular values in sig
       // stable descending ranks (NaN below every number)

@@ -20,9 +20,18 @@ template <typename T> struct EnvBlocks {
 // instead of one) and, in FP64, 128 for n <= 32.  Measured, with one output per thread in the FP64
 // products (evaluation, one GB300, before -> after): 4x4, D = 2, chi = 4, 256 samples FP64
 // 3.52 -> 0.61 ms; n <= 32 flip chains 6x6, D = 3, chi = 9 FP64 18.6 -> 15.5 ms.
-inline int cta_threads(int esz_real, int n) {
+// In FP32 beyond n = 16 the samples of a large batch go to smaller CTAs, more of them per SM: the
+// serial parts of a truncation (a QR panel, the Jacobi on few rows) are one warp's work, and the other
+// warps of its CTA wait.  256 threads while the grid is at most three CTAs per SM, else 128 (the grid
+// follows from the plan's shared memory per CTA).  Measured, 256 -> 128 threads, at 4096 samples of 8x8,
+// D = 4, chi = 16: one-row kernel 15.4 -> 12.7 ms, environments 64.2 -> 61.3, row steps 44.0 -> 34.3;
+// 304 samples of 12x12 at chi = 24: environments 21.3 -> 14.2; but 100 samples of 7x9, D = 5, chi = 25,
+// less than two per SM: 5.9 -> 7.6.
+constexpr int N_SM = 152;
+inline int cta_threads(int esz_real, int n, int grid) {
   if (n <= 16) return 64;
-  return (n <= 32 && esz_real == 8) ? 128 : NTHREADS;
+  if (esz_real == 8) return n <= 32 ? 128 : NTHREADS;
+  return grid > 3 * N_SM ? 128 : NTHREADS;
 }
 
 // term record (ints): number of sites, the sites, window (first row, first column, width,

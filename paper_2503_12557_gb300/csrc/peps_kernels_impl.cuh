@@ -27,6 +27,7 @@ __device__ RowWork<T> carve_row(const Plan& p, char* smem, char* gbase) {
   w.E = (T*)buf_ptr(p, B_E, smem, gbase);
   w.A = (T*)buf_ptr(p, B_A, smem, gbase);
   w.Z = (T*)buf_ptr(p, B_Z, smem, gbase);
+  w.ZS = (T*)buf_ptr(p, B_ZS, smem, gbase);
   w.W = (T*)buf_ptr(p, B_W, smem, gbase);
   w.C = (T*)buf_ptr(p, B_C, smem, gbase);
   w.sig = (T*)buf_ptr(p, B_SIG, smem, gbase);
@@ -37,50 +38,41 @@ __device__ RowWork<T> carve_row(const Plan& p, char* smem, char* gbase) {
   return w;
 }
 
-// Upper environments E^u[-1..Lx-2] of configuration Ss into env (one sample's store).
+// One side of configuration Ss's environments into env (one sample's store): the upper ones
+// E^u[-1..Lx-2] (and the trivial E^l[Lx] that closes psi_top = E^u[Lx-2] . T_proj[Lx-1]) or the lower
+// ones E^l[1..Lx].  One row step for both sides: its code is large, and a second copy in a kernel whose
+// CTAs work on either side costs instruction fetches.
 template <typename T, typename G>
-__device__ void build_upper(const G& g, const T* Tpad, const uint8_t* Ss, T* env, double* logs,
-                            const RowWork<T>& w, int* st, int* flag) {
+__device__ __forceinline__ void build_side(const G& g, int lower, const T* Tpad, const uint8_t* Ss, T* env, double* logs,
+                                           const RowWork<T>& w, int* st, int* flag) {
   const size_t row = (size_t)g.Ly * g.se;
-  // trivial E^u[-1], and the trivial E^l[Lx] that closes psi_top = E^u[Lx-2] . T_proj[Lx-1]
-  T* trivial = env + (size_t)slot_up(g, -1) * row;
   T* trivial_lo = env + (size_t)slot_lo(g, g.Lx) * row;
   for (int k = 0; k < g.Ly; ++k) {
-    blk_unit(trivial + (size_t)k * g.se, g.se);
+    if (!lower) blk_unit(env + (size_t)slot_up(g, -1) * row + (size_t)k * g.se, g.se);
     blk_unit(trivial_lo + (size_t)k * g.se, g.se);
   }
-  if (threadIdx.x == 0) { logs[slot_up(g, -1)] = 0.0; logs[slot_lo(g, g.Lx)] = 0.0; }
+  if (threadIdx.x == 0) {
+    if (!lower) logs[slot_up(g, -1)] = 0.0;
+    logs[slot_lo(g, g.Lx)] = 0.0;
+  }
   __syncthreads();
-  Scaled f = env_first_row(g, env + (size_t)slot_up(g, 0) * row, Tpad, 0, Ss, false, w.A, w.Z, w.red, st);
   double lg = 0.0;
-  if (threadIdx.x == 0) logs[slot_up(g, 0)] = lg = sc_log(f);
-  for (int x = 1; x <= g.Lx - 2; ++x) {
-    f = env_row_step(g, env + (size_t)slot_up(g, x - 1) * row, env + (size_t)slot_up(g, x) * row, Tpad, x,
-                       Ss + (size_t)x * g.Ly, false, w, st, flag);
-    if (threadIdx.x == 0) logs[slot_up(g, x)] = lg += sc_log(f);
+  for (int i = 0; i < g.Lx - 1; ++i) {
+    const int x = lower ? g.Lx - 1 - i : i, slot = lower ? slot_lo(g, x) : slot_up(g, x);
+    const uint8_t* Srow = Ss + (size_t)x * g.Ly;
+    T* out = env + (size_t)slot * row;
+    Scaled f;
+    if (i == 0) f = env_first_row(g, out, Tpad, x, Srow, lower != 0, w.A, w.Z, w.red, st);
+    else f = env_row_step_inl(g, env + (size_t)(lower ? slot_lo(g, x + 1) : slot_up(g, x - 1)) * row, out, Tpad, x, Srow,
+                              lower != 0, w, st, flag);
+    if (threadIdx.x == 0) logs[slot] = lg += sc_log(f);
   }
   __syncthreads();
 }
-
-// Lower environments E^l[2..Lx] (and E^l[1] when full) of configuration Ss.
 template <typename T, typename G>
-__device__ void build_lower(const G& g, const T* Tpad, const uint8_t* Ss, T* env, double* logs,
-                            const RowWork<T>& w, int* st, int* flag, int xmin) {
-  const size_t row = (size_t)g.Ly * g.se;
-  T* trivial = env + (size_t)slot_lo(g, g.Lx) * row;
-  for (int k = 0; k < g.Ly; ++k) blk_unit(trivial + (size_t)k * g.se, g.se);
-  if (threadIdx.x == 0) logs[slot_lo(g, g.Lx)] = 0.0;
-  __syncthreads();
-  Scaled f = env_first_row(g, env + (size_t)slot_lo(g, g.Lx - 1) * row, Tpad, g.Lx - 1,
-                           Ss + (size_t)(g.Lx - 1) * g.Ly, true, w.A, w.Z, w.red, st);
-  double lg = 0.0;
-  if (threadIdx.x == 0) logs[slot_lo(g, g.Lx - 1)] = lg = sc_log(f);
-  for (int x = g.Lx - 2; x >= xmin; --x) {
-    f = env_row_step(g, env + (size_t)slot_lo(g, x + 1) * row, env + (size_t)slot_lo(g, x) * row, Tpad, x,
-                       Ss + (size_t)x * g.Ly, true, w, st, flag);
-    if (threadIdx.x == 0) logs[slot_lo(g, x)] = lg += sc_log(f);
-  }
-  __syncthreads();
+__device__ __noinline__ void build_side_call(const G g, int lower, const T* Tpad, const uint8_t* Ss, T* env, double* logs,
+                                             const RowWork<T> w, int* st, int* flag) {
+  build_side(g, lower, Tpad, Ss, env, logs, w, st, flag);
 }
 
 // One side (0 upper, 1 lower) of sample smp's environments, with the whole CTA.
@@ -95,8 +87,7 @@ __device__ __forceinline__ void env_item(const G g, const RowWork<T>& w, const T
   T* env = envs + (size_t)smp * env_sample_elems(g);
   double* lg = logs + (size_t)smp * 2 * g.Lx;
   const uint8_t* Ss = S + (size_t)smp * N;
-  if (side == 0) build_upper(g, Tpad, Ss, env, lg, w, &st, &flag);
-  else build_lower(g, Tpad, Ss, env, lg, w, &st, &flag, 1);
+  build_side(g, side, Tpad, Ss, env, lg, w, &st, &flag);
   if (threadIdx.x == 0) {
     if (st) atomicOr(status + smp, st);
   }
@@ -175,29 +166,33 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
   const T* EL = env + (size_t)slot_lo(g, x + 1) * rowsz;
   if (threadIdx.x == 0) st = 0;
   // right partials R[Ly] = unit, R[y] = R[y+1] absorbed over column y
-  blk_unit(RP + (size_t)Ly * se, se);
+  __shared__ int bu[MAX_LY + 1], bl[MAX_LY + 1], sl_[MAX_LY], sr_[MAX_LY];
+  mps_bonds(g, EU, bu, sl_, sr_);
+  mps_bonds(g, EL, bl, sl_, sr_);
+  const int D = g.D, chi = g.chi, cd = g.chi * g.D;
+  auto ext = [&](int y) { return BondExt{bu[y], bu[y + 1], bl[y], bl[y + 1]}; };
+  blk_unit(RP + (size_t)Ly * se, cd);
   if (threadIdx.x == 0) logR[Ly] = sc_one();
-  __syncthreads();
   for (int y = Ly - 1; y >= 0; --y) {
-    blk_copy(eu, EU + (size_t)y * se, se);
-    blk_copy(el, EL + (size_t)y * se, se);
+    blk_copy(eu, EU + (size_t)y * se, bu[y] * cd);
+    blk_copy(el, EL + (size_t)y * se, bl[y] * cd);
     load_A(A, Tpad, g, x * Ly + y, Ss[x * Ly + y], false);
     __syncthreads();
-    absorb1_right(g, RP + (size_t)(y + 1) * se, eu, A, el, t1, t2, RP + (size_t)y * se);
-    const double l = (double)blk_normalize(RP + (size_t)y * se, se, red, &st);
+    absorb1_right(g, ext(y), RP + (size_t)(y + 1) * se, eu, A, el, t1, t2, RP + (size_t)y * se);
+    const double l = (double)blk_normalize(RP + (size_t)y * se, bu[y] * D, chi, bl[y], red, &st);
     if (threadIdx.x == 0) logR[y] = sc_mul(logR[y + 1], l);
   }
   // left partials
-  blk_unit(LP, se);
+  blk_unit(LP, cd);
   if (threadIdx.x == 0) logL[0] = sc_one();
   __syncthreads();
   for (int y = 0; y < Ly; ++y) {
-    blk_copy(eu, EU + (size_t)y * se, se);
-    blk_copy(el, EL + (size_t)y * se, se);
+    blk_copy(eu, EU + (size_t)y * se, bu[y] * cd);
+    blk_copy(el, EL + (size_t)y * se, bl[y] * cd);
     load_A(A, Tpad, g, x * Ly + y, Ss[x * Ly + y], false);
     __syncthreads();
-    absorb1(g, LP + (size_t)y * se, eu, A, el, t1, t2, LP + (size_t)(y + 1) * se);
-    const double l = (double)blk_normalize(LP + (size_t)(y + 1) * se, se, red, &st);
+    absorb1(g, ext(y), LP + (size_t)y * se, eu, A, el, t1, t2, LP + (size_t)(y + 1) * se);
+    const double l = (double)blk_normalize(LP + (size_t)(y + 1) * se, bu[y + 1] * D, chi, bl[y + 1], red, &st);
     if (threadIdx.x == 0) logL[y + 1] = sc_mul(logL[y], l);
   }
   __syncthreads();
@@ -208,15 +203,19 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
   if (O != nullptr) {
     for (int y = 0; y < Ly; ++y) {
       const int site = x * Ly + y;
-      blk_copy(eu, EU + (size_t)y * se, se);
+      blk_copy(eu, EU + (size_t)y * se, bu[y] * cd);
       {
         // the lower environment site transposed, elT[z][b][d] = el[b][d][z] (into LW2)
         const T* ely = EL + (size_t)y * se;
-        const int cd = g.chi * g.D;
-        for (int o = threadIdx.x; o < se; o += blockDim.x) LW2[o] = ely[(size_t)(o % cd) * g.chi + o / cd];
+        const int nb = bl[y] * D;  // (b, d) for b below the bond
+        const FDiv fz = fdiv_of(bl[y + 1]);
+        for (int o = threadIdx.x; o < nb * fz.k; o += blockDim.x) {
+          const int bd = fdiv_q(o, fz), z = o - bd * fz.k;
+          LW2[z * cd + bd] = ely[(size_t)bd * chi + z];
+        }
       }
       __syncthreads();
-      site_env1(g, LP + (size_t)y * se, eu, LW2, RP + (size_t)(y + 1) * se, t1, t2, A);
+      site_env1(g, ext(y), LP + (size_t)y * se, eu, LW2, RP + (size_t)(y + 1) * se, t1, t2, A);
       if (threadIdx.x == 0) {
         const double sc = sc_ratio(sc_mul(logL[y], logR[y + 1]), logL[Ly]);
         fO = dz{ival.re * sc, ival.im * sc};
@@ -226,7 +225,6 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
       const int blk = Dl * Du * Dr * Dd;
       const int s_here = Ss[site];
       T* Orow = O + (size_t)smp * Np + site_off[site];
-      const int D = g.D;
       __syncthreads();
       const dz f = fO;
       for (int s = 0; s < g.d; ++s)
@@ -255,22 +253,22 @@ __device__ __forceinline__ void row_item(const G g, const Plan plan, char* smem,
         const double hr = tt.ent_h[2 * e], hi = tt.ent_h[2 * e + 1];
         if (b == a) { ere += hr; eim += hi; continue; }
         const int y0 = ti[TI_Y0], w = ti[TI_W];
-        blk_copy(LW, LP + (size_t)y0 * se, se);
+        const T* cur = LP + (size_t)y0 * se;
+        T* nxt = LW;
         Scaled lw = logL[y0];  // carried in thread 0
-        __syncthreads();
         for (int c = y0; c < y0 + w; ++c) {
           const int site = x * Ly + c;
-          blk_copy(eu, EU + (size_t)c * se, se);
-          blk_copy(el, EL + (size_t)c * se, se);
+          blk_copy(eu, EU + (size_t)c * se, bu[c] * cd);
+          blk_copy(el, EL + (size_t)c * se, bl[c] * cd);
           load_A(A, Tpad, g, site, state_after(ti, site, Ss, b, g.d), false);
           __syncthreads();
-          absorb1(g, LW, eu, A, el, t1, t2, LW2);
-          const double l = (double)blk_normalize(LW2, se, red, &st);
+          absorb1(g, ext(c), cur, eu, A, el, t1, t2, nxt);
+          const double l = (double)blk_normalize(nxt, bu[c + 1] * D, chi, bl[c + 1], red, &st);
           if (threadIdx.x == 0) lw = sc_mul(lw, l);
-          blk_copy(LW, LW2, se);
-          __syncthreads();
+          cur = nxt;
+          nxt = nxt == LW ? LW2 : LW;
         }
-        const T v = blk_dot(LW, RP + (size_t)(y0 + w) * se, se, red);
+        const T v = blk_dot(cur, RP + (size_t)(y0 + w) * se, bu[y0 + w] * D, chi, bl[y0 + w], red);
         if (threadIdx.x == 0) {
           const dz q = dz_mul(to_dz(v), ival);
           const double f = sc_ratio(sc_mul(lw, logR[y0 + w]), logL[Ly]);
@@ -342,31 +340,35 @@ __device__ __forceinline__ void pair_item(const G g, const Plan plan, char* smem
   const T* EU = env + (size_t)slot_up(g, x - 1) * rowsz;
   const T* EL = env + (size_t)slot_lo(g, x + 2) * rowsz;
   if (threadIdx.x == 0) st = 0;
-  blk_unit(RP + (size_t)Ly * s2, s2);
+  __shared__ int bu[MAX_LY + 1], bl[MAX_LY + 1], sl_[MAX_LY], sr_[MAX_LY];
+  mps_bonds(g, EU, bu, sl_, sr_);
+  mps_bonds(g, EL, bl, sl_, sr_);
+  const int D2 = g.D * g.D, chi = g.chi, cd = g.chi * g.D;
+  auto ext = [&](int y) { return BondExt{bu[y], bu[y + 1], bl[y], bl[y + 1]}; };
+  blk_unit(RP + (size_t)Ly * s2, D2 * chi);
   if (threadIdx.x == 0) logR[Ly] = sc_one();
-  __syncthreads();
   for (int y = Ly - 1; y >= 0; --y) {
-    blk_copy(eu, EU + (size_t)y * se, se);
-    blk_copy(el, EL + (size_t)y * se, se);
+    blk_copy(eu, EU + (size_t)y * se, bu[y] * cd);
+    blk_copy(el, EL + (size_t)y * se, bl[y] * cd);
     load_A(A1, Tpad, g, x * Ly + y, Ss[x * Ly + y], false);
     load_A(A2, Tpad, g, (x + 1) * Ly + y, Ss[(x + 1) * Ly + y], false);
     __syncthreads();
-    absorb2_right(g, RP + (size_t)(y + 1) * s2, eu, A1, A2, el, t1, t2, RP + (size_t)y * s2, plan.cx);
-    const double l = (double)blk_normalize(RP + (size_t)y * s2, s2, red, &st);
+    absorb2_right(g, ext(y), RP + (size_t)(y + 1) * s2, eu, A1, A2, el, t1, t2, RP + (size_t)y * s2, plan.cx);
+    const double l = (double)blk_normalize(RP + (size_t)y * s2, bu[y] * D2, chi, bl[y], red, &st);
     if (threadIdx.x == 0) logR[y] = sc_mul(logR[y + 1], l);
   }
-  blk_unit(LP, s2);
+  blk_unit(LP, D2 * chi);
   if (threadIdx.x == 0) logL[0] = sc_one();
   __syncthreads();
   // the left partials are only needed up to the last window start; build them all
   for (int y = 0; y < Ly; ++y) {
-    blk_copy(eu, EU + (size_t)y * se, se);
-    blk_copy(el, EL + (size_t)y * se, se);
+    blk_copy(eu, EU + (size_t)y * se, bu[y] * cd);
+    blk_copy(el, EL + (size_t)y * se, bl[y] * cd);
     load_A(A1, Tpad, g, x * Ly + y, Ss[x * Ly + y], false);
     load_A(A2, Tpad, g, (x + 1) * Ly + y, Ss[(x + 1) * Ly + y], false);
     __syncthreads();
-    absorb2(g, LP + (size_t)y * s2, eu, A1, A2, el, t1, t2, LP + (size_t)(y + 1) * s2, plan.cx);
-    const double l = (double)blk_normalize(LP + (size_t)(y + 1) * s2, s2, red, &st);
+    absorb2(g, ext(y), LP + (size_t)y * s2, eu, A1, A2, el, t1, t2, LP + (size_t)(y + 1) * s2, plan.cx);
+    const double l = (double)blk_normalize(LP + (size_t)(y + 1) * s2, bu[y + 1] * D2, chi, bl[y + 1], red, &st);
     if (threadIdx.x == 0) logL[y + 1] = sc_mul(logL[y], l);
   }
   __syncthreads();
@@ -382,22 +384,22 @@ __device__ __forceinline__ void pair_item(const G g, const Plan plan, char* smem
       const double hr = tt.ent_h[2 * e], hi = tt.ent_h[2 * e + 1];
       if (b == a) { ere += hr; eim += hi; continue; }
       const int y0 = ti[TI_Y0], w = ti[TI_W];
-      blk_copy(LW, LP + (size_t)y0 * s2, s2);
+      const T* cur = LP + (size_t)y0 * s2;
+      T* nxt = LW;
       Scaled lw = logL[y0];  // carried in thread 0
-      __syncthreads();
       for (int c = y0; c < y0 + w; ++c) {
-        blk_copy(eu, EU + (size_t)c * se, se);
-        blk_copy(el, EL + (size_t)c * se, se);
+        blk_copy(eu, EU + (size_t)c * se, bu[c] * cd);
+        blk_copy(el, EL + (size_t)c * se, bl[c] * cd);
         load_A(A1, Tpad, g, x * Ly + c, state_after(ti, x * Ly + c, Ss, b, g.d), false);
         load_A(A2, Tpad, g, (x + 1) * Ly + c, state_after(ti, (x + 1) * Ly + c, Ss, b, g.d), false);
         __syncthreads();
-        absorb2(g, LW, eu, A1, A2, el, t1, t2, LW2, plan.cx);
-        const double l = (double)blk_normalize(LW2, s2, red, &st);
+        absorb2(g, ext(c), cur, eu, A1, A2, el, t1, t2, nxt, plan.cx);
+        const double l = (double)blk_normalize(nxt, bu[c + 1] * D2, chi, bl[c + 1], red, &st);
         if (threadIdx.x == 0) lw = sc_mul(lw, l);
-        blk_copy(LW, LW2, s2);
-        __syncthreads();
+        cur = nxt;
+        nxt = nxt == LW ? LW2 : LW;
       }
-      const T v = blk_dot(LW, RP + (size_t)(y0 + w) * s2, s2, red);
+      const T v = blk_dot(cur, RP + (size_t)(y0 + w) * s2, bu[y0 + w] * D2, chi, bl[y0 + w], red);
       if (threadIdx.x == 0) {
         const dz q = dz_mul(to_dz(v), ival);
         const double f = sc_ratio(sc_mul(lw, logR[y0 + w]), logL[Ly]);
@@ -420,7 +422,7 @@ __device__ __forceinline__ void pair_item(const G g, const Plan plan, char* smem
 }
 
 template <typename T, typename G>
-__global__ void __launch_bounds__(NTHREADS) k_pair(G g, Plan plan, const T* __restrict__ Tpad,
+__global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_pair(G g, Plan plan, const T* __restrict__ Tpad,
                                                    const uint8_t* __restrict__ S, int Ns, const T* envs,
                                                    const double* logs, TermTab tt, double* pairout, int* status) {
   extern __shared__ __align__(16) char smem[];
@@ -561,12 +563,15 @@ __device__ inline unsigned sweep_slot0(const G& g, int x, int up, int move) {
 // psi_{xt,xt+1} = E^u[xt-1] . T[xt] . T[xt+1] . E^l[xt+2].  Slots from slot0 on; Sl (shared) is
 // updated in place; *acc counts the accepted moves (the same value in every thread).
 template <typename T, typename G>
-__device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, const T* Tpad, uint8_t* Sl,
+__device__ __noinline__ void row_moves(const G g, const Plan plan, const MoveBufs<T> b, const T* Tpad, uint8_t* Sl,
                           const T* env, int x, int up, int move, unsigned slot0, unsigned long long sweep_id, int c,
                           unsigned long long seed, long long* acc, int* st) {
   __shared__ Scaled logR[MAX_LY + 1];   // factors taken out of the partials
   __shared__ Scaled logLc, lcur;        // of the running left partial; |psi| of the configuration
   __shared__ int accept_flag;
+  __shared__ int bu[MAX_LY + 1], bl[MAX_LY + 1], sl_[MAX_LY], sr_[MAX_LY];
+  auto ext = [&](int y) { return BondExt{bu[y], bu[y + 1], bl[y], bl[y + 1]}; };
+  const int D = g.D, D2 = g.D * g.D, chi = g.chi, cd = g.chi * g.D;
   const int Ly = g.Ly, Lx = g.Lx, se = g.se, s2 = g.s2;
   const size_t rowsz = (size_t)Ly * se;
   const int nmv = (move == 0) ? Ly - 1 : Ly;
@@ -578,16 +583,17 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
   {
     const T* EU = env + (size_t)slot_up(g, x - 1) * rowsz;
     const T* EL = env + (size_t)slot_lo(g, x + 1) * rowsz;
-    blk_unit(RP + (size_t)Ly * se, se);
+    mps_bonds(g, EU, bu, sl_, sr_);
+    mps_bonds(g, EL, bl, sl_, sr_);
+    blk_unit(RP + (size_t)Ly * se, cd);
     if (threadIdx.x == 0) logR[Ly] = sc_one();
-    __syncthreads();
     for (int y = Ly - 1; y >= 0; --y) {
-      blk_copy(eu, EU + (size_t)y * se, se);
-      blk_copy(el, EL + (size_t)y * se, se);
+      blk_copy(eu, EU + (size_t)y * se, bu[y] * cd);
+      blk_copy(el, EL + (size_t)y * se, bl[y] * cd);
       load_A(A1, Tpad, g, x * Ly + y, Sl[x * Ly + y], false);
       __syncthreads();
-      absorb1_right(g, RP + (size_t)(y + 1) * se, eu, A1, el, t1, t2, RP + (size_t)y * se);
-      const double l = (double)blk_normalize(RP + (size_t)y * se, se, red, st);
+      absorb1_right(g, ext(y), RP + (size_t)(y + 1) * se, eu, A1, el, t1, t2, RP + (size_t)y * se);
+      const double l = (double)blk_normalize(RP + (size_t)y * se, bu[y] * D, chi, bl[y], red, st);
       if (threadIdx.x == 0) logR[y] = sc_mul(logR[y + 1], l);
     }
     __syncthreads();
@@ -595,7 +601,7 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
       lcur = sc_mul(logR[0], dz_abs(to_dz(RP[0])));
       logLc = sc_one();
     }
-    blk_unit(LC, se);
+    blk_unit(LC, cd);
     __syncthreads();
     for (int y = 0; y < nmv; ++y) {
       const unsigned my_slot = slot++;
@@ -613,22 +619,22 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
           int s_new;
           if (move == 0) s_new = (cc == 0) ? Sl[i1] : Sl[i0];
           else s_new = g.d - 1 - Sl[site];
-          blk_copy(eu, EU + (size_t)(y + cc) * se, se);
-          blk_copy(el, EL + (size_t)(y + cc) * se, se);
+          blk_copy(eu, EU + (size_t)(y + cc) * se, bu[y + cc] * cd);
+          blk_copy(el, EL + (size_t)(y + cc) * se, bl[y + cc] * cd);
           load_A(A1, Tpad, g, site, s_new, false);
           __syncthreads();
           if (cc == 0) {
-            absorb1(g, LC, eu, A1, el, t1, t2, LW2);
-            l0 = (double)blk_normalize(LW2, se, red, st);
+            absorb1(g, ext(y), LC, eu, A1, el, t1, t2, LW2);
+            l0 = (double)blk_normalize(LW2, bu[y + 1] * D, chi, bl[y + 1], red, st);
             if (threadIdx.x == 0) lw = sc_mul(logLc, l0);
           } else {
-            absorb1(g, LW2, eu, A1, el, t1, t2, LW);
-            const double l = (double)blk_normalize(LW, se, red, st);
+            absorb1(g, ext(y + 1), LW2, eu, A1, el, t1, t2, LW);
+            const double l = (double)blk_normalize(LW, bu[y + 2] * D, chi, bl[y + 2], red, st);
             if (threadIdx.x == 0) lw = sc_mul(lw, l);
           }
           __syncthreads();
         }
-        const T v = blk_dot(w_ == 2 ? LW : LW2, RP + (size_t)(y + w_) * se, se, red);
+        const T v = blk_dot(w_ == 2 ? LW : LW2, RP + (size_t)(y + w_) * se, bu[y + w_] * D, chi, bl[y + w_], red);
         if (threadIdx.x == 0) {
           const double u = uniform53(my_slot, (uint32_t)sweep_id, (uint32_t)c, 0u, seed);
           const Scaled l1 = sc_mul(sc_mul(lw, logR[y + w_]), dz_abs(to_dz(v)));
@@ -644,21 +650,23 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
         taken = accept_flag;
         if (taken) {
           // column y now holds the proposed state: the new LC is the window's first column
-          blk_copy(LC, LW2, se);
+          T* const tmp = LC;
+          LC = LW2;
+          LW2 = tmp;
           if (threadIdx.x == 0) logLc = sc_mul(logLc, l0);
-          __syncthreads();
         }
       }
       if (!taken) {
-        blk_copy(eu, EU + (size_t)y * se, se);
-        blk_copy(el, EL + (size_t)y * se, se);
+        blk_copy(eu, EU + (size_t)y * se, bu[y] * cd);
+        blk_copy(el, EL + (size_t)y * se, bl[y] * cd);
         load_A(A1, Tpad, g, x * Ly + y, Sl[x * Ly + y], false);
         __syncthreads();
-        absorb1(g, LC, eu, A1, el, t1, t2, LW2);
-        const double l = (double)blk_normalize(LW2, se, red, st);
-        blk_copy(LC, LW2, se);
+        absorb1(g, ext(y), LC, eu, A1, el, t1, t2, LW2);
+        const double l = (double)blk_normalize(LW2, bu[y + 1] * D, chi, bl[y + 1], red, st);
+        T* const tmp = LC;
+        LC = LW2;
+        LW2 = tmp;
         if (threadIdx.x == 0) logLc = sc_mul(logLc, l);
-        __syncthreads();
       }
     }
   }
@@ -667,17 +675,18 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
   if (move == 0 && xt >= 0 && xt < Lx - 1) {
     const T* EU = env + (size_t)slot_up(g, xt - 1) * rowsz;
     const T* EL2 = env + (size_t)slot_lo(g, xt + 2) * rowsz;
-    blk_unit(RP + (size_t)Ly * s2, s2);
+    mps_bonds(g, EU, bu, sl_, sr_);
+    mps_bonds(g, EL2, bl, sl_, sr_);
+    blk_unit(RP + (size_t)Ly * s2, D2 * chi);
     if (threadIdx.x == 0) logR[Ly] = sc_one();
-    __syncthreads();
     for (int y = Ly - 1; y >= 0; --y) {
-      blk_copy(eu, EU + (size_t)y * se, se);
-      blk_copy(el, EL2 + (size_t)y * se, se);
+      blk_copy(eu, EU + (size_t)y * se, bu[y] * cd);
+      blk_copy(el, EL2 + (size_t)y * se, bl[y] * cd);
       load_A(A1, Tpad, g, xt * Ly + y, Sl[xt * Ly + y], false);
       load_A(A2, Tpad, g, (xt + 1) * Ly + y, Sl[(xt + 1) * Ly + y], false);
       __syncthreads();
-      absorb2_right(g, RP + (size_t)(y + 1) * s2, eu, A1, A2, el, t1, t2, RP + (size_t)y * s2, plan.cx);
-      const double l = (double)blk_normalize(RP + (size_t)y * s2, s2, red, st);
+      absorb2_right(g, ext(y), RP + (size_t)(y + 1) * s2, eu, A1, A2, el, t1, t2, RP + (size_t)y * s2, plan.cx);
+      const double l = (double)blk_normalize(RP + (size_t)y * s2, bu[y] * D2, chi, bl[y], red, st);
       if (threadIdx.x == 0) logR[y] = sc_mul(logR[y + 1], l);
     }
     __syncthreads();
@@ -685,21 +694,21 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
       lcur = sc_mul(logR[0], dz_abs(to_dz(RP[0])));
       logLc = sc_one();
     }
-    blk_unit(LC, s2);
+    blk_unit(LC, D2 * chi);
     __syncthreads();
     for (int y = 0; y < Ly; ++y) {
       const unsigned my_slot = slot++;
       const int i0 = xt * Ly + y, i1 = (xt + 1) * Ly + y;
-      blk_copy(eu, EU + (size_t)y * se, se);
-      blk_copy(el, EL2 + (size_t)y * se, se);
+      blk_copy(eu, EU + (size_t)y * se, bu[y] * cd);
+      blk_copy(el, EL2 + (size_t)y * se, bl[y] * cd);
       int taken = 0;
       if (Sl[i0] != Sl[i1]) {
         load_A(A1, Tpad, g, i0, Sl[i1], false);
         load_A(A2, Tpad, g, i1, Sl[i0], false);
         __syncthreads();
-        absorb2(g, LC, eu, A1, A2, el, t1, t2, LW2, plan.cx);
-        const double l0 = (double)blk_normalize(LW2, s2, red, st);
-        const T v = blk_dot(LW2, RP + (size_t)(y + 1) * s2, s2, red);
+        absorb2(g, ext(y), LC, eu, A1, A2, el, t1, t2, LW2, plan.cx);
+        const double l0 = (double)blk_normalize(LW2, bu[y + 1] * D2, chi, bl[y + 1], red, st);
+        const T v = blk_dot(LW2, RP + (size_t)(y + 1) * s2, bu[y + 1] * D2, chi, bl[y + 1], red);
         if (threadIdx.x == 0) {
           const double u = uniform53(my_slot, (uint32_t)sweep_id, (uint32_t)c, 0u, seed);
           const Scaled l1 = sc_mul(sc_mul(sc_mul(logLc, l0), logR[y + 1]), dz_abs(to_dz(v)));
@@ -714,20 +723,22 @@ __device__ void row_moves(const G& g, const Plan& plan, const MoveBufs<T>& b, co
         taken = accept_flag;
         if (taken) {
           // the proposal's window is the new LC
-          blk_copy(LC, LW2, s2);
+          T* const tmp = LC;
+          LC = LW2;
+          LW2 = tmp;
           if (threadIdx.x == 0) logLc = sc_mul(logLc, l0);
-          __syncthreads();
         }
       }
       if (!taken) {
         load_A(A1, Tpad, g, i0, Sl[i0], false);
         load_A(A2, Tpad, g, i1, Sl[i1], false);
         __syncthreads();
-        absorb2(g, LC, eu, A1, A2, el, t1, t2, LW2, plan.cx);
-        const double l = (double)blk_normalize(LW2, s2, red, st);
-        blk_copy(LC, LW2, s2);
+        absorb2(g, ext(y), LC, eu, A1, A2, el, t1, t2, LW2, plan.cx);
+        const double l = (double)blk_normalize(LW2, bu[y + 1] * D2, chi, bl[y + 1], red, st);
+        T* const tmp = LC;
+        LC = LW2;
+        LW2 = tmp;
         if (threadIdx.x == 0) logLc = sc_mul(logLc, l);
-        __syncthreads();
       }
     }
   }
@@ -801,23 +812,16 @@ __global__ void __launch_bounds__(NTHREADS, EnvBlocks<T>::value) k_env_row(G g, 
     T* env = envs + (size_t)c * env_sample_elems(g);
     double* lg = logs + (size_t)c * 2 * g.Lx;
     const uint8_t* Ss = S + (size_t)c * N;
-    Scaled l;
+    const int slot = lower ? slot_lo(g, x) : slot_up(g, x), prev = lower ? slot_lo(g, x + 1) : slot_up(g, x - 1);
+    const bool first = lower ? x == g.Lx - 1 : x == 0;
     double l0 = 0.0;  // the row before's logarithm, in thread 0
-    int slot;
-    if (!lower) {
-      slot = slot_up(g, x);
-      if (threadIdx.x == 0 && x > 0) l0 = lg[slot_up(g, x - 1)];
-      if (x == 0) l = env_first_row(g, env + (size_t)slot * rowsz, Tpad, 0, Ss, false, w.A, w.Z, w.red, &st);
-      else l = env_row_step(g, env + (size_t)slot_up(g, x - 1) * rowsz, env + (size_t)slot * rowsz, Tpad, x,
-                            Ss + (size_t)x * g.Ly, false, w, &st, &flag);
-    } else {
-      slot = slot_lo(g, x);
-      if (threadIdx.x == 0 && x < g.Lx - 1) l0 = lg[slot_lo(g, x + 1)];
-      if (x == g.Lx - 1)
-        l = env_first_row(g, env + (size_t)slot * rowsz, Tpad, x, Ss + (size_t)x * g.Ly, true, w.A, w.Z, w.red, &st);
-      else l = env_row_step(g, env + (size_t)slot_lo(g, x + 1) * rowsz, env + (size_t)slot * rowsz, Tpad, x,
-                            Ss + (size_t)x * g.Ly, true, w, &st, &flag);
-    }
+    if (threadIdx.x == 0 && !first) l0 = lg[prev];
+    Scaled l;
+    if (first)
+      l = env_first_row(g, env + (size_t)slot * rowsz, Tpad, x, Ss + (size_t)x * g.Ly, lower != 0, w.A, w.Z, w.red, &st);
+    else
+      l = env_row_step_inl(g, env + (size_t)prev * rowsz, env + (size_t)slot * rowsz, Tpad, x, Ss + (size_t)x * g.Ly,
+                           lower != 0, w, &st, &flag);
     if (threadIdx.x == 0) {
       lg[slot] = l0 + sc_log(l);
       if (st) atomicOr(status + c, st);
@@ -859,7 +863,7 @@ __global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_sample(G g, P
       const unsigned long long sweep_id = sweep0 + (unsigned long long)t;
       const int up = (int)(sweep_id & 1ull);
       if (!up) {
-        build_lower(g, Tpad, Sl, env, lg, w, &st, &flag, 1);
+        build_side_call(g, 1, Tpad, Sl, env, lg, w, &st, &flag);
         sweep_trivial_row(g, env, lg, 0);
         __syncthreads();
         for (int x = 0; x < Lx; ++x) {
@@ -875,7 +879,7 @@ __global__ void __launch_bounds__(NTHREADS, MinBlocks<T>::value) k_sample(G g, P
           }
         }
       } else {
-        if (t == 0) build_upper(g, Tpad, Sl, env, lg, w, &st, &flag);
+        if (t == 0) build_side_call(g, 0, Tpad, Sl, env, lg, w, &st, &flag);
         sweep_trivial_row(g, env, lg, 1);
         __syncthreads();
         for (int x = Lx - 1; x >= 0; --x) {
@@ -1059,14 +1063,15 @@ static cudaError_t with_geo_for(const Geo& g, F&& f) {
 
 // Each translation unit defines PEPS_PART_ENV, PEPS_PART_ROW (k_row, k_pair, parameter padding)
 // or PEPS_PART_SAMPLE and instantiates its kernels with PEPS_INST_<part>(T).
-#define PEPS_KATTR(NAME, KERNEL)                                                                                   \
+// (the occupancy at the fewest threads a launch may take, which gives the most CTAs)
+#define PEPS_KATTR(NAME, KERNEL, MINT)                                                                             \
   template <typename T>                                                                                          \
   cudaError_t NAME(const Geo& g, size_t set_bytes, int* occ, size_t occ_smem) {                                  \
     return with_geo_for<T>(g, [&](auto gg) {                                                                            \
       using GG = decltype(gg);                                                                                   \
       cudaError_t e = cudaSuccess;                                                                               \
       if (set_bytes) e = cudaFuncSetAttribute(KERNEL<T, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)set_bytes); \
-      if (e == cudaSuccess && occ) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, KERNEL<T, GG>, cta_threads(sizeof(typename Scal<T>::R), g.n), occ_smem); \
+      if (e == cudaSuccess && occ) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, KERNEL<T, GG>, MINT, occ_smem); \
       return e;                                                                                                  \
     });                                                                                                          \
   }
@@ -1158,7 +1163,7 @@ template <typename T>
 cudaError_t launch_env(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
                        int sides, T* envs, double* logs, int* status, cudaStream_t s) {
   return with_geo_for<T>(g, [&](auto gg) {
-    k_env<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n), smem, s>>>(gg, p, Tpad, S, Ns, sides, envs, logs, status);
+    k_env<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n, grid), smem, s>>>(gg, p, Tpad, S, Ns, sides, envs, logs, status);
     return cudaGetLastError();
   });
 }
@@ -1166,13 +1171,13 @@ template <typename T>
 cudaError_t launch_env_row(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
                            int x, int lower, T* envs, double* logs, int* status, int* ustat, cudaStream_t s) {
   return with_geo_for<T>(g, [&](auto gg) {
-    k_env_row<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n), smem, s>>>(
+    k_env_row<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n, grid), smem, s>>>(
         gg, p, Tpad, S, Ns, x, lower, envs, logs, status, ustat);
     return cudaGetLastError();
   });
 }
-PEPS_KATTR(kattr_env_only, k_env)
-PEPS_KATTR(kattr_env_row, k_env_row)
+PEPS_KATTR(kattr_env_only, k_env, cta_threads(sizeof(typename Scal<T>::R), g.n, 1 << 30))
+PEPS_KATTR(kattr_env_row, k_env_row, cta_threads(sizeof(typename Scal<T>::R), g.n, 1 << 30))
 // k_env and, in FP32, the sampler's k_env_row, which runs on the same plan
 template <typename T>
 cudaError_t kattr_env(const Geo& g, size_t set_bytes, int* occ, size_t occ_smem) {
@@ -1196,7 +1201,7 @@ cudaError_t launch_row(const Geo& g, const Plan& p, int grid, size_t smem, const
                        int x_lo, int x_hi, const T* envs, const double* logs, T* O, const long long* site_off,
                        long long Np, const TermTab& tt, double* rowout, int* status, cudaStream_t s) {
   return with_geo_for<T>(g, [&](auto gg) {
-    k_row<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n), smem, s>>>(gg, p, Tpad, S, Ns, x_lo, x_hi, envs, logs, O, site_off, Np,
+    k_row<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n, grid), smem, s>>>(gg, p, Tpad, S, Ns, x_lo, x_hi, envs, logs, O, site_off, Np,
                                                         tt, rowout, status);
     return cudaGetLastError();
   });
@@ -1205,7 +1210,7 @@ template <typename T>
 cudaError_t launch_pair(const Geo& g, const Plan& p, int grid, size_t smem, const T* Tpad, const uint8_t* S, int Ns,
                         const T* envs, const double* logs, const TermTab& tt, double* pairout, int* status, cudaStream_t s) {
   return with_geo_for<T>(g, [&](auto gg) {
-    k_pair<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n), smem, s>>>(gg, p, Tpad, S, Ns, envs, logs, tt, pairout, status);
+    k_pair<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n, grid), smem, s>>>(gg, p, Tpad, S, Ns, envs, logs, tt, pairout, status);
     return cudaGetLastError();
   });
 }
@@ -1214,8 +1219,8 @@ cudaError_t launch_pad(const Geo& g, const double* theta, const long long* site_
   k_pad_theta<T><<<304, 256, 0, s>>>(g, theta, site_off, Tpad);
   return cudaGetLastError();
 }
-PEPS_KATTR(kattr_row, k_row)
-PEPS_KATTR(kattr_pair, k_pair)
+PEPS_KATTR(kattr_row, k_row, cta_threads(sizeof(typename Scal<T>::R), g.n, 1 << 30))
+PEPS_KATTR(kattr_pair, k_pair, cta_threads(sizeof(typename Scal<T>::R), g.n, 1 << 30))
 #define PEPS_INST_ROW(T)                                                                                          \
   template cudaError_t launch_row<T>(const Geo&, const Plan&, int, size_t, const T*, const uint8_t*, int, int, int, \
                                      const T*, const double*, T*, const long long*, long long, const TermTab&,    \
@@ -1228,6 +1233,14 @@ PEPS_KATTR(kattr_pair, k_pair)
 #endif
 
 #ifdef PEPS_PART_SAMPLE
+// The FP32 moves take 64 threads beyond six CTAs per SM: they are sandwiches of one sample after the
+// other, with a barrier per product (4096 chains, 8x8, D = 4, chi = 16: 41.6 -> 36.4 ms; the row step's
+// kernels lose, 61.3 -> 65.2 ms).
+template <typename T>
+static int sample_threads(int n, int grid) {
+  const int nt = cta_threads(sizeof(typename Scal<T>::R), n, grid);
+  return sizeof(T) == 4 && grid > 6 * N_SM ? 64 : nt;
+}
 // FP32 runs the sweep split by rows (k_env for the lower environments, then k_sweep_moves and
 // k_env_row per row; the environment plan pe / grid_e / smem_e for the row steps); the other
 // precisions run the single-launch k_sample.
@@ -1236,7 +1249,7 @@ cudaError_t launch_sample(const Geo& g, const Plan& p, int grid, size_t smem, co
                           size_t smem_e, const T* Tpad, uint8_t* S, int Ns, int move, int nsweeps,
                           unsigned long long seed, unsigned long long sweep0, T* envs, double* logs,
                           long long* accepted, int* status, int* ustat, cudaStream_t s) {
-  const int nt = cta_threads(sizeof(typename Scal<T>::R), g.n);
+  const int nt = sample_threads<T>(g.n, grid);
   return with_geo_for<T>(g, [&](auto gg) {
     using GG = decltype(gg);
     if constexpr (sizeof(T) == 4) {
@@ -1267,7 +1280,7 @@ cudaError_t launch_sample(const Geo& g, const Plan& p, int grid, size_t smem, co
 }
 template <typename T>
 cudaError_t kattr_sample(const Geo& g, size_t set_bytes, int* occ, size_t occ_smem) {
-  const int nt = cta_threads(sizeof(typename Scal<T>::R), g.n);
+  const int nt = sample_threads<T>(g.n, 1 << 30);
   return with_geo_for<T>(g, [&](auto gg) {
     using GG = decltype(gg);
     auto kernel = [&](auto* k) {
@@ -1293,12 +1306,12 @@ cudaError_t launch_bound(const Geo& g, const Plan& p, int grid, size_t smem, con
                          int cut, const T* envs, const double* logs, const TermTab& tt, double* bout, double* logabs,
                          double* phase, int* status, cudaStream_t s) {
   return with_geo_for<T>(g, [&](auto gg) {
-    k_bound<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n), smem, s>>>(gg, p, Tpad, S, Ns, cut, envs, logs, tt, bout, logabs, phase,
+    k_bound<T, decltype(gg)><<<grid, cta_threads(sizeof(typename Scal<T>::R), g.n, 1), smem, s>>>(gg, p, Tpad, S, Ns, cut, envs, logs, tt, bout, logabs, phase,
                                                           status);
     return cudaGetLastError();
   });
 }
-PEPS_KATTR(kattr_bound, k_bound)
+PEPS_KATTR(kattr_bound, k_bound, cta_threads(sizeof(typename Scal<T>::R), g.n, 1))
 #define PEPS_INST_BOUND(T)                                                                                        \
   template cudaError_t launch_bound<T>(const Geo&, const Plan&, int, size_t, const T*, const uint8_t*, int, int,  \
                                        const T*, const double*, const TermTab&, double*, double*, double*, int*,  \

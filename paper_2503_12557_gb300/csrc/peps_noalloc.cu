@@ -80,7 +80,7 @@ peps_status run(const peps_config& c, const double* theta, const uint8_t* S, int
   const std::pair<int, size_t> benv[] = {
       {B_RED, 40 * 8}, {B_SIG, (mX + 4) * E}, {B_SEL, 2 * (size_t)mX * 4}, {B_A, (size_t)g.sT * E},
       {B_E, (size_t)g.se * E}, {B_C, (size_t)n * chi * E}, {B_W, env_w_elems(chi, D, ci) * E},
-      {B_R, (size_t)n * n * E}, {B_Z, zsz * E}, {B_RHIST, (size_t)(Ly > 1 ? Ly - 1 : 1) * n * n * E}};
+      {B_ZS, (size_t)env_zs_elems(chi, D) * E}, {B_R, (size_t)n * n * E}, {B_Z, zsz * E}, {B_RHIST, (size_t)(Ly > 1 ? Ly - 1 : 1) * n * n * E}};
   const std::pair<int, size_t> brow[] = {
       {B_RED, 40 * 8}, {B_A, (size_t)g.sT * E}, {B_EU, (size_t)g.se * E}, {B_EL, (size_t)g.se * E},
       {B_T1, t1 * E}, {B_T2, t1 * E}, {B_LW, (size_t)g.se * E}, {B_LW2, (size_t)g.se * E},

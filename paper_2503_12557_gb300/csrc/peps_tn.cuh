@@ -157,9 +157,6 @@ struct GeoS {
                        s2 = CHI * DD * DD * CHI;
 };
 
-// Row length D chi of the truncation's Jacobi step when it is a compile-time constant, else 0.
-template <typename G> struct GeoLr { static constexpr int value = 0; };
-template <int CHI, int DD> struct GeoLr<GeoS<CHI, DD>> { static constexpr int value = CHI * DD; };
 // Row count chi D^2 of the left pass's QR when it is a compile-time constant, else 0.
 template <typename G> struct GeoMz { static constexpr int value = 0; };
 template <int CHI, int DD> struct GeoMz<GeoS<CHI, DD>> { static constexpr int value = CHI * DD * DD; };
@@ -169,7 +166,7 @@ template <int CHI, int DD> struct GeoMz<GeoS<CHI, DD>> { static constexpr int va
 // per-CTA slice of a global scratch arena, as the host planner decided.
 enum Buf : int {
   B_R = 0, B_E, B_A, B_A2, B_Z, B_W, B_C, B_SIG, B_SEL, B_RED,
-  B_RHIST, B_LP, B_RP, B_T1, B_T2, B_EU, B_EL, B_LW, B_LW2, B_S, B_NBUF
+  B_RHIST, B_ZS, B_LP, B_RP, B_T1, B_T2, B_EU, B_EL, B_LW, B_LW2, B_S, B_NBUF
 };
 
 struct Plan {
@@ -255,7 +252,7 @@ __device__ cplx<R> block_sum(cplx<R> v, double* red) {
 
 // 16 bytes at a time when both ends and the length allow it
 template <typename T>
-__device__ void blk_copy(T* dst, const T* src, int n) {
+__device__ __noinline__ void blk_copy(T* dst, const T* src, int n) {
   constexpr int V = 16 / sizeof(T) > 0 ? 16 / sizeof(T) : 1;
   if (V > 1 && n % V == 0 && (((uintptr_t)dst | (uintptr_t)src) & 15) == 0) {
     for (int o = threadIdx.x; o < n / V; o += blockDim.x)
@@ -270,7 +267,7 @@ __device__ void blk_fill(T* dst, T v, int n) {
 }
 // unit tensor: 1 at flat index 0, zeros elsewhere (trivial environments and partials)
 template <typename T>
-__device__ void blk_unit(T* dst, int n) {
+__device__ __noinline__ void blk_unit(T* dst, int n) {
   for (int o = threadIdx.x; o < n; o += blockDim.x) dst[o] = (o == 0) ? T(1) : T(0);
 }
 
@@ -311,15 +308,29 @@ __device__ __forceinline__ bool sc_accept(double u, const Scaled& a, const Scale
   return u * b.m * b.m < a.m * a.m * __longlong_as_double((long long)(k + 1023) << 52);
 }
 
+// Quotient m / k for 0 <= m < 2^22 and k >= 1 from a float reciprocal: (m + 1/2) / k lies at
+// least 1 / (2k) from every integer, and the two roundings (of 1 / k and of the product) move it
+// by at most (m + 1/2) 2^-23 / k < 1 / (2k), so truncation gives the exact quotient.  Cheaper
+// than an integer division when k is only known at run time.
+struct FDiv {
+  int k;
+  float r;
+};
+__device__ __forceinline__ FDiv fdiv_of(int k) { return FDiv{k, __frcp_rn((float)k)}; }
+__device__ __forceinline__ int fdiv_q(int m, FDiv d) { return __float2int_rz(((float)m + 0.5f) * d.r); }
+
 // Divide v[0..n) by its largest modulus (double: by the power of two below it, which changes no
 // mantissa and needs no division); returns what it was divided by (the same in every thread), or
 // 0 with ZERO_NORM / NONFINITE set in *st when the maximum is 0 or not finite.  Called with v
 // complete behind a barrier; ends with a barrier.
+// (nc columns of nrow rows of length ld)
 template <typename T>
-__device__ typename Scal<T>::R blk_normalize(T* v, int n, double* red, int* st) {
+__device__ __noinline__ typename Scal<T>::R blk_normalize(T* v, int nrow, int ld, int nc, double* red, int* st) {
   using R = typename Scal<T>::R;
+  const FDiv fc = fdiv_of(nc);
+  const int n = nrow * nc, skip = ld - nc;
   R m = 0;
-  for (int o = threadIdx.x; o < n; o += blockDim.x) m = max_(m, abs_(v[o]));
+  for (int o = threadIdx.x; o < n; o += blockDim.x) m = max_(m, abs_(v[o + fdiv_q(o, fc) * skip]));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max_(m, __shfl_xor_sync(0xffffffffu, m, o));
   const int nw = blockDim.x >> 5;
@@ -345,15 +356,19 @@ __device__ typename Scal<T>::R blk_normalize(T* v, int n, double* red, int* st) 
   } else {
     inv = R(1) / m;
   }
-  for (int o = threadIdx.x; o < n; o += blockDim.x) v[o] *= inv;
+  for (int o = threadIdx.x; o < n; o += blockDim.x) v[o + fdiv_q(o, fc) * skip] *= inv;
   __syncthreads();
   return m;
+}
+template <typename T>
+__device__ __forceinline__ typename Scal<T>::R blk_normalize(T* v, int n, double* red, int* st) {
+  return blk_normalize(v, 1, n, n, red, st);
 }
 
 // Projected PEPS tensor of site `site` with local state s, as A[l][u][r][d] (swap_ud: as
 // A[l][d][r][u], the lower-environment orientation).
 template <typename T, typename G>
-__device__ void load_A(T* As, const T* Tpad, const G& g, int site, int s, bool swap_ud) {
+__device__ __noinline__ void load_A(T* As, const T* Tpad, const G g, int site, int s, bool swap_ud) {
   if ((unsigned)s >= (unsigned)g.d) s = 0;  // a local state outside [0, d) is not valid input: read as 0
   const T* src = Tpad + ((size_t)site * g.d + s) * g.sT;
   const int D = g.D;
@@ -389,8 +404,23 @@ __device__ __forceinline__ void qr_apply_reflector(const T* zj, int j, T tau, T*
 // Blocked by panels of QB columns: warp 0 computes the panel's reflectors (applying each to
 // the rest of the panel), then every warp applies the panel's reflectors, in order, to the
 // trailing columns it owns.  Two block barriers per panel.  taus: at least nc entries.
+// R (and R2, may be null), row major with ld ldr: rows 0..kr-1, columns 0..kc-1; zero below the
+// diagonal and from column nc on.  Ends with a barrier.
 template <typename T>
-__device__ void qr_keep_r_smem(T* Z, int m, int nc, T* R, T* taus, int ldr) {
+__device__ __noinline__ void qr_store_r(const T* Z, int m, int nc, T* R, int ldr, int kr, int kc, T* R2) {
+  const FDiv fk = fdiv_of(kc);
+#pragma unroll 2
+  for (int o = threadIdx.x; o < kr * kc; o += blockDim.x) {
+    const int i = fdiv_q(o, fk), c = o - i * kc;
+    const T v = (c < nc && i <= c && i < m) ? Z[(size_t)c * m + i] : T(0);
+    R[(size_t)i * ldr + c] = v;
+    if (R2) R2[(size_t)i * ldr + c] = v;
+  }
+  __syncthreads();
+}
+
+template <typename T>
+__device__ void qr_keep_r_smem(T* Z, int m, int nc, T* R, T* taus, int ldr, int kr, int kc, T* R2) {
   constexpr int QB = 8;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int steps = (m < nc) ? m : nc;
@@ -435,11 +465,7 @@ __device__ void qr_keep_r_smem(T* Z, int m, int nc, T* R, T* taus, int ldr) {
     }
     __syncthreads();
   }
-  for (int o = tid; o < ldr * ldr; o += blockDim.x) {
-    const int i = o / ldr, c = o % ldr;
-    R[o] = (c < nc && i <= c && i < m) ? Z[(size_t)c * m + i] : T(0);
-  }
-  __syncthreads();
+  qr_store_r(Z, m, nc, R, ldr, kr, kc, R2);
 }
 
 // beta, tau and the scale 1 / (alpha - beta) of xLARFG's reflector for a real column with head
@@ -476,7 +502,10 @@ __device__ __forceinline__ void reflector(double alpha, double sigma, double& be
 
 // Panel of QB columns (j0 .. j0+pb-1) factored by one warp with the columns in registers
 // (element i = lane + 32 r, m <= 32 RPL): per column one warp reduction for the norm and one
-// independent reduction per remaining panel column, no shared-memory round trips.
+// independent reduction per remaining panel column, no shared-memory round trips.  The columns move
+// down one place after each step instead of the steps being unrolled, which took 30 to 60 KB of
+// instructions per row count: with CTAs in different phases on an SM, instruction fetches were 30 % of
+// the row step's stalls and made the others longer.
 template <typename T, int RPL, int QB>
 __device__ __forceinline__ void qr_panel_reg(T* Z, int m, int j0, int pb, T* taus, int lane) {
   T zp[QB][RPL];
@@ -487,64 +516,56 @@ __device__ __forceinline__ void qr_panel_reg(T* Z, int m, int j0, int pb, T* tau
       const int i = lane + 32 * r;
       zp[q][r] = (q < pb && i < m) ? Z[(size_t)(j0 + q) * m + i] : T(0);
     }
-#pragma unroll
-  for (int jj = 0; jj < QB; ++jj) {
-    if (jj < pb) {
-      const int j = j0 + jj;
-      T part = 0, aj = 0;
-#pragma unroll
-      for (int r = 0; r < RPL; ++r) {
-        const int i = lane + 32 * r;
-        if (i > j) part += zp[jj][r] * zp[jj][r];
-        if (r == (j >> 5)) aj = zp[jj][r];
-      }
-      const T sigma = warp_sum(part);
-      const T alpha = __shfl_sync(0xffffffffu, aj, j & 31);
-      T tau = 0, beta = alpha;
-      if (sigma != T(0)) {
-        T sc;
-        reflector(alpha, sigma, beta, tau, sc);
-#pragma unroll
-        for (int r = 0; r < RPL; ++r)
-          if (lane + 32 * r > j) zp[jj][r] *= sc;
-      }
-      if (tau != T(0)) {
-        // v = (1 at row j, the scaled column below it); column q <- column q - tau v (v . column q)
-        T v[RPL];
-#pragma unroll
-        for (int r = 0; r < RPL; ++r) {
-          const int i = lane + 32 * r;
-          v[r] = (i > j) ? zp[jj][r] : (i == j ? T(1) : T(0));
-        }
-        T d[QB];
-#pragma unroll
-        for (int q = jj + 1; q < QB; ++q) {
-          T s = 0;
-#pragma unroll
-          for (int r = 0; r < RPL; ++r) s += v[r] * zp[q][r];
-          d[q] = s;
-        }
-#pragma unroll
-        for (int q = jj + 1; q < QB; ++q) d[q] = tau * warp_sum(d[q]);
-#pragma unroll
-        for (int q = jj + 1; q < QB; ++q)
-          if (q < pb)
-#pragma unroll
-            for (int r = 0; r < RPL; ++r) zp[q][r] -= v[r] * d[q];
-      }
-#pragma unroll
-      for (int r = 0; r < RPL; ++r)
-        if (lane + 32 * r == j) zp[jj][r] = beta;
-      if (lane == 0) taus[j] = tau;
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < QB; ++q)
+#pragma unroll 1
+  for (int jj = 0; jj < pb; ++jj) {
+    const int j = j0 + jj;
+    T part = 0, aj = 0;
 #pragma unroll
     for (int r = 0; r < RPL; ++r) {
       const int i = lane + 32 * r;
-      if (q < pb && i < m) Z[(size_t)(j0 + q) * m + i] = zp[q][r];
+      if (i > j) part += zp[0][r] * zp[0][r];
+      if (r == (j >> 5)) aj = zp[0][r];
     }
+    const T sigma = warp_sum(part);
+    const T alpha = __shfl_sync(0xffffffffu, aj, j & 31);
+    T tau = 0, beta = alpha, sc = 0;
+    if (sigma != T(0)) reflector(alpha, sigma, beta, tau, sc);
+    if (tau != T(0)) {
+      // v = (1 at row j, the scaled column below it); column q <- column q - tau v (v . column q)
+      T v[RPL], d[QB];
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) {
+        const int i = lane + 32 * r;
+        v[r] = (i > j) ? zp[0][r] * sc : (i == j ? T(1) : T(0));
+        if (i > j) zp[0][r] = v[r];
+      }
+#pragma unroll
+      for (int q = 1; q < QB; ++q) {
+        T s = 0;
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) s += v[r] * zp[q][r];
+        d[q] = s;
+      }
+#pragma unroll
+      for (int q = 1; q < QB; ++q) d[q] = tau * warp_sum(d[q]);
+#pragma unroll
+      for (int q = 1; q < QB; ++q)
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) zp[q][r] -= v[r] * d[q];
+    }
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+      const int i = lane + 32 * r;
+      if (i < m) Z[(size_t)j * m + i] = i == j ? beta : zp[0][r];
+    }
+    if (lane == 0) taus[j] = tau;
+#pragma unroll
+    for (int q = 0; q + 1 < QB; ++q)
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) zp[q][r] = zp[q + 1][r];
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) zp[QB - 1][r] = T(0);
+  }
 }
 
 // Register form of the same blocked factorisation (m <= 32 RPL).
@@ -553,21 +574,24 @@ __device__ __forceinline__ void qr_panel_reg(T* Z, int m, int j0, int pb, T* tau
 //   panel column costs two warp reductions instead of one per remaining column.
 //   Trailing update (all warps): a warp loads CW trailing columns into registers (element
 //   i = lane + 32 r), applies the panel's reflectors to each in order and stores them once.
-template <typename T, int RPL>
-__device__ __noinline__ void qr_keep_r_reg(T* Z, int m, int nc, T* R, T* taus, int ldr) {
+//   SP: the panel is factored in memory instead of registers (whose sums run over other rows per lane).
+template <typename T, int RPL, bool SP = (sizeof(T) == 4 && RPL > 8)>
+__device__ __noinline__ void qr_keep_r_reg(T* Z, int m, int nc, T* R, T* taus, int ldr, int kr, int kc, T* R2) {
   // FP32 with 256 rows: panels of four columns, whose register panel (4 x 8 values a lane)
   // fits the environment kernels' 80 registers; eight columns spilled there
   // (FP64: two columns, since a warp alone has only its sub-partition's FP64 pipe, a quarter of the
   // SM's, and the trailing columns are spread over all four)
-  constexpr int QB = sizeof(T) == 8 ? 2 : (RPL == 8 ? 4 : 8);
+  constexpr int QB = sizeof(T) == 8 ? 2 : (RPL == 8 && !SP ? 4 : 8);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int steps = (m < nc) ? m : nc;
+#pragma unroll 1
   for (int j0 = 0; j0 < steps; j0 += QB) {
     const int pb = (steps - j0 < QB) ? steps - j0 : QB;
     if (warp == 0) {
-      if constexpr (RPL * QB * sizeof(T) <= (sizeof(T) == 8 ? 640 : 256)) {
+      if constexpr (!SP) {
         qr_panel_reg<T, RPL, QB>(Z, m, j0, pb, taus, lane);
       } else {
+#pragma unroll 1
         for (int jj = 0; jj < pb; ++jj) {
           const int j = j0 + jj;
           T* zj = Z + (size_t)j * m;
@@ -622,6 +646,7 @@ __device__ __noinline__ void qr_keep_r_reg(T* Z, int m, int nc, T* R, T* taus, i
     // CW trailing columns per warp at a time (c, c + nw, ...; the later ones may be absent), so
     // that their reductions overlap; one where the columns would not fit in registers
     constexpr int CW = (RPL <= 12) ? 2 : 1;
+#pragma unroll 1
     for (int c = j0 + pb + warp; c < nc; c += CW * nw) {
       T z[CW][RPL];
 #pragma unroll
@@ -633,6 +658,7 @@ __device__ __noinline__ void qr_keep_r_reg(T* Z, int m, int nc, T* R, T* taus, i
           z[w][r] = (cw < nc && i < m) ? Z[(size_t)cw * m + i] : T(0);
         }
       }
+#pragma unroll 1
       for (int jj = 0; jj < pb; ++jj) {
         const int j = j0 + jj;
         const T tau = taus[j];
@@ -668,36 +694,27 @@ __device__ __noinline__ void qr_keep_r_reg(T* Z, int m, int nc, T* R, T* taus, i
     }
     __syncthreads();
   }
-  for (int o = tid; o < ldr * ldr; o += blockDim.x) {
-    const int i = o / ldr, c = o % ldr;
-    R[o] = (c < nc && i <= c && i < m) ? Z[(size_t)c * m + i] : T(0);
-  }
-  __syncthreads();
+  qr_store_r(Z, m, nc, R, ldr, kr, kc, R2);
 }
 
-// Dispatch on the row count; MC > 0: a compile-time bound on m (m <= MC).  R is written as an
-// ldr x ldr row-major upper-triangular matrix (ldr >= nc; the columns from nc on are zero).
+// Dispatch on the row count (rows past m are zeros that change no sum).  R is written as qr_store_r
+// says: kr rows and kc columns of an upper-triangular matrix of ld ldr.
+// MC > 0: the compile-time most rows, whose panels decide how they are factored.
 template <typename T, int MC = 0>
-__device__ void qr_keep_r(T* Z, int m, int nc, T* R, T* taus, int ldr) {
+__device__ void qr_keep_r(T* Z, int m, int nc, T* R, T* taus, int ldr, int kr, int kc, T* R2) {
   if constexpr (Scal<T>::complex) {
-    qr_keep_r_smem(Z, m, nc, R, taus, ldr);
-  } else if constexpr (MC > 0) {
-    // the register form is compiled for up to MC rows and runs on the m <= MC rows given, the
-    // sites near the open edge on a shorter one (rows past m are zeros that change no sum)
-    constexpr int RPL = (MC + 31) / 32;
-    if constexpr (RPL <= 8) {
-      if (m <= 32) return qr_keep_r_reg<T, 1>(Z, m, nc, R, taus, ldr);
-      if (m <= 64) return qr_keep_r_reg<T, 2>(Z, m, nc, R, taus, ldr);
-    }
-    if constexpr (RPL <= 24) qr_keep_r_reg<T, RPL>(Z, m, nc, R, taus, ldr);
-    else qr_keep_r_smem(Z, m, nc, R, taus, ldr);
+    qr_keep_r_smem(Z, m, nc, R, taus, ldr, kr, kc, R2);
+  } else if constexpr (MC > 256) {
+    if (m <= 128) qr_keep_r_reg<T, 4, true>(Z, m, nc, R, taus, ldr, kr, kc, R2);
+    else if (m <= 256) qr_keep_r_reg<T, 8, true>(Z, m, nc, R, taus, ldr, kr, kc, R2);
+    else qr_keep_r_reg<T, (MC + 31) / 32, true>(Z, m, nc, R, taus, ldr, kr, kc, R2);
   } else {
-    if (m <= 32) qr_keep_r_reg<T, 1>(Z, m, nc, R, taus, ldr);
-    else if (m <= 64) qr_keep_r_reg<T, 2>(Z, m, nc, R, taus, ldr);
-    else if (m <= 128) qr_keep_r_reg<T, 4>(Z, m, nc, R, taus, ldr);
-    else if (m <= 256) qr_keep_r_reg<T, 8>(Z, m, nc, R, taus, ldr);
-    else if (m <= 768) qr_keep_r_reg<T, 24>(Z, m, nc, R, taus, ldr);
-    else qr_keep_r_smem(Z, m, nc, R, taus, ldr);
+    if (m <= 32) qr_keep_r_reg<T, 1>(Z, m, nc, R, taus, ldr, kr, kc, R2);
+    else if (m <= 64) qr_keep_r_reg<T, 2>(Z, m, nc, R, taus, ldr, kr, kc, R2);
+    else if (m <= 128) qr_keep_r_reg<T, 4>(Z, m, nc, R, taus, ldr, kr, kc, R2);
+    else if (m <= 256) qr_keep_r_reg<T, 8>(Z, m, nc, R, taus, ldr, kr, kc, R2);
+    else if (m <= 768) qr_keep_r_reg<T, 24>(Z, m, nc, R, taus, ldr, kr, kc, R2);
+    else qr_keep_r_smem(Z, m, nc, R, taus, ldr, kr, kc, R2);
   }
 }
 
@@ -791,13 +808,14 @@ __device__ int hestenes_rows_smem(T* X, int m, int L, int ldx, int* flag, unsign
         T* xp = X + (size_t)p * ldx;
         T* xq = X + (size_t)q * ldx;
         const R a = nrm[p], b = nrm[q];
+        if (!(a > tiny && b > tiny)) continue;  // (the eight lanes of a pair agree)
         T c = 0;
         for (int i = sub; i < L; i += 8) c = mad(c, xp[i], conj_(xq[i]));
         c += shfl_xor_(gmask, c, 4);
         c += shfl_xor_(gmask, c, 2);
         c += shfl_xor_(gmask, c, 1);
         const R ac = abs_(c);
-        if (ac != R(0) && a > tiny && b > tiny && ac > tol * sqrt(a * b)) {
+        if (ac != R(0) && ac > tol * sqrt(a * b)) {
           if (ac >= stop * sqrt(a * b)) big = 1;
           // with c = |c| e^{i phi}: rotate (x_p, e^{i phi} x_q), whose product is |c|;
           // zeta = (b - a) / (2|c|); t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)) is the smaller
@@ -903,9 +921,203 @@ __device__ __forceinline__ T grp_sum8(T v) {
   return v;
 }
 
+// The same sweeps when at most JFEW rows are above the zero threshold: one warp, the other rows left
+// out (no rotation touches them), the active rows copied to S in shared memory, without the 8-element
+// chunks that are zero in all of them (the new bond is mostly below chi).  The pairs are those that
+// hestenes_rows_grp looks at, in its order -- slot 0..2 for the pairs inside a block of four rows, then
+// four slots per super-round -- with pairs that share no row side by side (level: the first step after
+// both rows' earlier pairs), so that every rotation has the same operands and the results the same bits.
+// X = R Y of the early rows and of weakly entangled states has 4 to 10 active rows of 16 to 96,
+// where a sweep over all rows is 15 super-rounds (64 rows), most of them for nothing.
+constexpr int JFEW = 12;
+template <typename T>
+__device__ __noinline__ int hestenes_rows_few(T* X, int m, int L, int ldx, T tiny, const unsigned* mask,
+                                              unsigned long long* ctr, T* nrm, T* S, int lds) {
+  constexpr int NP = JFEW * (JFEW - 1) / 2;
+  __shared__ int act[JFEW], sweeps_s, live_s;
+  __shared__ unsigned plist[NP], psort[NP];
+  __shared__ T an[JFEW];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int g = lane >> 3, u = lane & 7;
+  int na = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (warp == 0 && (mask[k] >> lane & 1u)) act[na + __popc(mask[k] & ((1u << lane) - 1u))] = 32 * k + lane;
+    na += __popc(mask[k]);
+  }
+  if (threadIdx.x == 0) live_s = 0;
+  __syncthreads();
+  // chunks of eight columns with a nonzero entry
+#pragma unroll 1
+  for (int a = warp; a < na; a += nw) {
+    int lv = 0;
+#pragma unroll 2
+    for (int i = lane; i < L; i += 32) lv |= nonzero_(X[(size_t)act[a] * ldx + i]) << (i >> 3);
+    lv = (int)__reduce_or_sync(0xffffffffu, (unsigned)lv);
+    if (lane == 0) atomicOr(&live_s, lv);
+  }
+#pragma unroll 1
+  for (int p = threadIdx.x; p < m; p += blockDim.x) nrm[p] = T(0);
+  __syncthreads();
+  const unsigned live = (unsigned)live_s;
+#pragma unroll 1
+  for (int a = warp; a < na; a += nw)
+#pragma unroll 2
+    for (int i = lane; i < (L + 7) / 8 * 8; i += 32)
+      if (live >> (i >> 3) & 1u)
+        S[a * lds + 8 * __popc(live & ((1u << (i >> 3)) - 1u)) + u] = i < L ? X[(size_t)act[a] * ldx + i] : T(0);
+  const int nl = __popc(live);  // chunks kept
+  if (threadIdx.x < 32) {
+    const int np = na * (na - 1) / 2, NB = ((m + 7) / 8) * 2;
+#pragma unroll 1
+    for (int e = lane; e < np; e += 32) {
+      int i = 0, r = e;
+#pragma unroll 1
+      while (r >= na - 1 - i) { r -= na - 1 - i; ++i; }
+      int a = i, b = i + 1 + r;  // rows act[a] < act[b]
+      const int x = act[a] >> 2, y = act[b] >> 2;
+      int slot;
+      if (x == y) {
+        slot = ((act[a] ^ act[b]) & 3) - 1;
+      } else {
+        // blocks x < y meet in the super-round sr with x + y = 2 sr (mod NB - 1), block 0 and y in
+        // sr = y (mod NB - 1); the first of the pair is the block at the lower position
+        const int M = NB - 1;
+        int sr;
+        if (x == 0) {
+          sr = y == M ? 0 : y;
+        } else {
+          const int s2 = (x + y) >= M ? x + y - M : x + y;  // 2 sr mod M; x + y < 2 M
+          sr = (s2 & 1) ? (s2 + M) >> 1 : s2 >> 1;
+          int jx = x - sr;                                   // position of block x, in 1..M
+          if (jx < 1) jx += M;
+          if (jx >= NB / 2) { const int t = a; a = b; b = t; }
+        }
+        slot = 3 + 4 * sr + ((act[b] - act[a]) & 3);
+      }
+      plist[e] = (unsigned)a | (unsigned)b << 4 | (unsigned)slot << 8;
+    }
+    __syncwarp();
+    // in order of the slots
+#pragma unroll 1
+    for (int e = lane; e < np; e += 32) {
+      const unsigned me = plist[e];
+      int rank = 0;
+#pragma unroll 2
+      for (int k = 0; k < np; ++k) rank += plist[k] >> 8 < me >> 8 || (plist[k] >> 8 == me >> 8 && k < e);
+      psort[rank] = me & 255u;
+    }
+    __syncwarp();
+    // levels: lane a keeps the level after row a's pairs so far
+    {
+      int lv = 0;
+#pragma unroll 1
+      for (int k = 0; k < np; ++k) {
+        const unsigned e = psort[k];
+        const int p = (int)(e & 15u), q = (int)(e >> 4);
+        const int l = max(__shfl_sync(0xffffffffu, lv, p), __shfl_sync(0xffffffffu, lv, q));
+        if (lane == p || lane == q) lv = l + 1;
+        if (lane == 0) plist[k] = e | (unsigned)l << 8;
+      }
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int e = lane; e < np; e += 32) {
+      const unsigned me = plist[e];
+      int rank = 0;
+#pragma unroll 2
+      for (int k = 0; k < np; ++k) rank += plist[k] >> 8 < me >> 8 || (plist[k] >> 8 == me >> 8 && k < e);
+      psort[rank] = me;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const T tol = jacobi_tol_r<T>(L), stop = sqrt(tol);
+    const int np = na * (na - 1) / 2;
+    int sweep = 0, ret = -1;
+    unsigned long long nrot = 0;
+#pragma unroll 1
+    for (; sweep < JacobiTol<T>::sweeps && ret < 0; ++sweep) {
+#pragma unroll 1
+      for (int a0 = 0; a0 < na; a0 += 4) {
+        const int a = a0 + g < na ? a0 + g : 0;
+        T s = 0;
+#pragma unroll 2
+        for (int e = 0; e < nl; ++e) s += S[a * lds + 8 * e + u] * S[a * lds + 8 * e + u];
+        s = grp_sum8(s);
+        if (u == 0 && a0 + g < na) an[a] = s;
+      }
+      __syncwarp();
+      int big = 0;
+#pragma unroll 1
+      for (int pos = 0; pos < np;) {
+        const unsigned e0 = psort[pos], eg = psort[pos + g < np ? pos + g : pos];
+        const bool in = pos + g < np && eg >> 8 == e0 >> 8;
+        const unsigned e = in ? eg : e0;
+        T* xp = S + (e & 15u) * lds + u;
+        T* xq = S + (e >> 4 & 15u) * lds + u;
+        const T a = an[e & 15u], b = an[e >> 4 & 15u];
+        T c = 0;
+#pragma unroll 4
+        for (int k = 0; k < nl; ++k) c += xp[8 * k] * xq[8 * k];
+        c = grp_sum8(c);
+        T cs = 1, sn = 0, tc = 0;
+        int bg = 0;
+        jac_params(a, b, c, tol, tiny, stop, cs, sn, tc, bg);
+        if (in && sn != T(0)) {
+          big |= bg;
+#pragma unroll 4
+          for (int k = 0; k < nl; ++k) {
+            const T v = xp[8 * k], w = xq[8 * k];
+            xp[8 * k] = cs * v - sn * w;
+            xq[8 * k] = sn * v + cs * w;
+          }
+          if (u == 0) {
+            an[e & 15u] = fmax(T(0), a - tc);
+            an[e >> 4 & 15u] = b + tc;
+            ++nrot;
+          }
+        }
+        pos += __popc(__ballot_sync(0xffffffffu, in)) >> 3;
+        __syncwarp();
+      }
+      if (!__any_sync(0xffffffffu, big)) ret = sweep + 1;
+    }
+    if (ctr && nrot) atomicAdd(ctr + 1, nrot);
+    if (lane == 0) {
+      if (ctr) { atomicAdd(ctr + 0, (unsigned long long)sweep); atomicAdd(ctr + 2, 1ull); }
+      sweeps_s = ret;
+    }
+  }
+  __syncthreads();
+  // the rows back in place and their singular values; rows that ended below the threshold are zero
+#pragma unroll 1
+  for (int a = warp; a < na; a += nw) {
+    T* xa = X + (size_t)act[a] * ldx;
+    T s = 0;
+#pragma unroll 2
+    for (int i = lane; i < L; i += 32)
+      if (live >> (i >> 3) & 1u) {
+        const T v = S[a * lds + 8 * __popc(live & ((1u << (i >> 3)) - 1u)) + u];
+        xa[i] = v;
+        s += v * v;
+      }
+    s = warp_sum(s);
+    if (s <= tiny) {
+      s = 0;
+      for (int i = lane; i < L; i += 32) xa[i] = T(0);
+    }
+    if (lane == 0) nrm[act[a]] = sqrt(s);
+  }
+  __syncthreads();
+  return sweeps_s;
+}
+
+// S: scratch of scap elements in shared memory for the rows of hestenes_rows_few (may be empty).
+// Rows at or below the zero threshold are zero on return, or hold anything with nrm[p] = 0.
 template <typename T, int E8>
 __device__ __noinline__ int hestenes_rows_grp(T* X, int m, int L, int ldx, int* flag, unsigned long long* ctr,
-                                              double* red, T* nrm) {
+                                              double* red, T* nrm, T* S, int scap) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int g = lane >> 3, u = lane & 7;
   const T eps = JacobiTol<T>::eps;
@@ -916,11 +1128,28 @@ __device__ __noinline__ int hestenes_rows_grp(T* X, int m, int L, int ldx, int* 
   for (int p = warp; p < m; p += nw) {
     T s = 0;
     for (int i = lane; i < L; i += 32) s += X[(size_t)p * ldx + i] * X[(size_t)p * ldx + i];
-    nmax = fmax(nmax, warp_sum(s));
+    s = warp_sum(s);
+    nmax = fmax(nmax, s);
+    if (lane == 0) nrm[p] = s;
   }
   nmax = block_max(nmax, red);
   const T tiny = nmax * (T(L) * eps) * (T(L) * eps);
   const T stop = sqrt(tol);
+  // the active rows (above the zero threshold; NaN counts); m <= 128
+  __shared__ unsigned mask[4];
+  int na = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int p = 32 * k + lane;
+    const unsigned mk = __ballot_sync(0xffffffffu, p < m && !(nrm[p < m ? p : 0] <= tiny));
+    if (threadIdx.x == 0) mask[k] = mk;
+    na += __popc(mk);
+  }
+  __syncthreads();
+  {
+    const int lds = L + ((8 - L) % 32 + 32) % 32;  // 8 mod 32, as ldx
+    if (na <= JFEW && na * lds <= scap) return hestenes_rows_few(X, m, L, ldx, tiny, mask, ctr, nrm, S, lds);
+  }
   unsigned long long nrot = 0;
   for (int sweep = 0; sweep < JacobiTol<T>::sweeps; ++sweep) {
     if (threadIdx.x == 0) *flag = 0;
@@ -929,6 +1158,9 @@ __device__ __noinline__ int hestenes_rows_grp(T* X, int m, int L, int ldx, int* 
     for (int s = 0; s < NB - 1; ++s) {
       for (int bp = warp; bp < NB / 2; bp += nw) {
         const int bP = rr_player(bp, s, NB), bQ = rr_player(NB - 1 - bp, s, NB);
+        // blocks without an active row meet nobody
+        const bool aP = mask[bP >> 3] >> (4 * (bP & 7)) & 15u, aQ = mask[bQ >> 3] >> (4 * (bQ & 7)) & 15u;
+        if (s == 0 ? !(aP || aQ) : !(aP && aQ)) continue;
         const int rp = 4 * bP + g;
         int rq = 4 * bQ + g;
         T xp[E8], xq[E8];
@@ -946,7 +1178,7 @@ __device__ __noinline__ int hestenes_rows_grp(T* X, int m, int L, int ldx, int* 
           for (int e = 0; e < E8; ++e) { ap += xp[e] * xp[e]; aq += xq[e] * xq[e]; }
           np = grp_sum8(ap);
           nq = grp_sum8(aq);
-#pragma unroll
+#pragma unroll 1
           for (int k = 1; k < 4; ++k) {
             const bool lo = g < (g ^ k);
             T yp[E8], yq[E8];
@@ -979,7 +1211,7 @@ __device__ __noinline__ int hestenes_rows_grp(T* X, int m, int L, int ldx, int* 
           nq = (rq < m) ? nrm[rq] : T(0);
         }
         // the 16 cross pairs: in round t group g pairs P_g with Q_(g+t)%4
-#pragma unroll
+#pragma unroll 1
         for (int t = 0; t < 4; ++t) {
           T c = 0;
 #pragma unroll
@@ -1046,23 +1278,20 @@ __device__ __noinline__ int hestenes_rows_grp(T* X, int m, int L, int ldx, int* 
 
 // Dispatch: the 8-lane-group register form for rows of at most 128 elements (best with a row
 // stride ldx = 8 mod 32, so that the four groups' rows fall in different banks), else the
-// shared-memory form.  Same contract as hestenes_rows_smem.  LC > 0: the row length is the compile-time LC.
-template <typename T, int LC = 0>
+// shared-memory form.  Same contract as hestenes_rows_smem (m <= 128 where L is); S, scap as in
+// hestenes_rows_grp.
+template <typename T>
 __device__ int hestenes_rows(T* X, int m, int L, int ldx, int* flag, unsigned long long* ctr, double* red,
-                             typename Scal<T>::R* nrm) {
+                             typename Scal<T>::R* nrm, T* S, int scap) {
   if constexpr (Scal<T>::complex) {
     return hestenes_rows_smem(X, m, L, ldx, flag, ctr, red, nrm);
-  } else if constexpr (LC > 0) {
-    constexpr int E8 = (LC + 7) / 8;
-    if constexpr (E8 <= 16) return hestenes_rows_grp<T, E8>(X, m, LC, ldx, flag, ctr, red, nrm);
-    else return hestenes_rows_smem(X, m, LC, ldx, flag, ctr, red, nrm);
   } else {
     // (elements past L are zeros that change no sum: the smallest register form that holds a row)
-    if (L <= 8) return hestenes_rows_grp<T, 1>(X, m, L, ldx, flag, ctr, red, nrm);
-    if (L <= 16) return hestenes_rows_grp<T, 2>(X, m, L, ldx, flag, ctr, red, nrm);
-    if (L <= 32) return hestenes_rows_grp<T, 4>(X, m, L, ldx, flag, ctr, red, nrm);
-    if (L <= 64) return hestenes_rows_grp<T, 8>(X, m, L, ldx, flag, ctr, red, nrm);
-    if (L <= 128) return hestenes_rows_grp<T, 16>(X, m, L, ldx, flag, ctr, red, nrm);
+    if (L <= 8) return hestenes_rows_grp<T, 1>(X, m, L, ldx, flag, ctr, red, nrm, S, scap);
+    if (L <= 16) return hestenes_rows_grp<T, 2>(X, m, L, ldx, flag, ctr, red, nrm, S, scap);
+    if (L <= 32) return hestenes_rows_grp<T, 4>(X, m, L, ldx, flag, ctr, red, nrm, S, scap);
+    if (L <= 64) return hestenes_rows_grp<T, 8>(X, m, L, ldx, flag, ctr, red, nrm, S, scap);
+    if (L <= 128) return hestenes_rows_grp<T, 16>(X, m, L, ldx, flag, ctr, red, nrm, S, scap);
     return hestenes_rows_smem(X, m, L, ldx, flag, ctr, red, nrm);
   }
 }
@@ -1079,6 +1308,13 @@ __host__ __device__ inline size_t env_z_elems(int chi, int D) {
   const size_t zright = (size_t)chi * D * D * chi + n * LY + mX * LX + (size_t)chi * LY + n * chi + (size_t)chi * D * chi;
   return zleft > zright ? zleft : zright;
 }
+// Scratch for the row step's matrices where the bonds that are not zero make them small (R, Z, Y, X,
+// Vt): in shared memory under every plan, since what a warp writes to the arena the others read back
+// from L2.
+__host__ __device__ inline int env_zs_elems(int chi, int D) {
+  const size_t n = (size_t)chi * D, all = n * n + env_z_elems(chi, D);
+  return all < 4096 ? (int)all : 4096;
+}
 __host__ __device__ inline size_t env_w_elems(int chi, int D, int ci) { return (size_t)ci * ((size_t)D * D * chi + 1); }
 // Size of the one-row sandwich temporaries (the first holds rows padded to chi + 1).
 __host__ __device__ inline size_t sandwich1_t_elems(int chi, int D) { return (size_t)D * D * chi * (chi + 1); }
@@ -1087,7 +1323,7 @@ __host__ __device__ inline size_t sandwich1_t_elems(int chi, int D) { return (si
 // Per-CTA working set of one boundary-MPS row step.
 template <typename T>
 struct RowWork {
-  T *R, *Rhist, *E, *A, *Z, *W, *C, *sig;
+  T *R, *Rhist, *E, *A, *Z, *ZS, *W, *C, *sig;
   int* sel;
   double* red;
   int ci;
@@ -1103,10 +1339,11 @@ struct RowWork {
 struct Off2 {
   int a, c;
 };
-template <int RM, int RN, typename T, class FM, class FN>
+template <int RM, int RN, int U, typename T, class FM, class FN>
 __device__ __forceinline__ void blk_gemm_tile(const T* __restrict__ A, const T* __restrict__ B, T* __restrict__ C, int M,
                                          int N, int K1, int K2, int sa1, int sa2, int sb1, int sb2, FM fm, FN fn) {
   const int tm = (M + RM - 1) / RM, tn = (N + RN - 1) / RN;
+#pragma unroll 1
   for (int t = threadIdx.x; t < tm * tn; t += blockDim.x) {
     const int ti = t % tm, tj = t / tm;
     int ao[RM], co[RM], bo[RN], cn[RN];
@@ -1132,7 +1369,9 @@ __device__ __forceinline__ void blk_gemm_tile(const T* __restrict__ A, const T* 
     for (int i = 0; i < RM; ++i)
 #pragma unroll
       for (int j = 0; j < RN; ++j) acc[i][j] = T(0);
+#pragma unroll 1
     for (int k1 = 0; k1 < K1; ++k1) {
+#pragma unroll U
       for (int k2 = 0; k2 < K2; ++k2) {
         const int ka = k1 * sa1 + k2 * sa2, kb = k1 * sb1 + k2 * sb2;
         T a[RM], b[RN];
@@ -1154,23 +1393,64 @@ __device__ __forceinline__ void blk_gemm_tile(const T* __restrict__ A, const T* 
   }
   __syncthreads();
 }
+// The tiles are small (2 x 4): with the bonds cut to what is not zero a product has some 24 x 32
+// outputs, which larger tiles spread over a fraction of the threads, and the code is short.  U: steps
+// of the sum unrolled; two in the row step, whose code a CTA runs through once per site and fetches from
+// L2 each time (at four, environments 42.2 -> 47.6 ms at 8x8, 4096 samples), four in the sandwiches
+// (two-row kernel 18.3 -> 12.1 ms).
 // In FP64 one output per thread: a multiply-add holds its SM sub-partition for 64 cycles, so that
 // operand loads are free beside it and what counts is to have all four sub-partitions busy.
-template <int RM, int RN, typename T, class FM, class FN>
+template <int RM, int RN, int U = 4, typename T, class FM, class FN>
 __device__ __forceinline__ void blk_gemm(const T* __restrict__ A, const T* __restrict__ B, T* __restrict__ C, int M,
                                          int N, int K1, int K2, int sa1, int sa2, int sb1, int sb2, FM fm, FN fn) {
   constexpr bool f64 = sizeof(typename Scal<T>::R) == 8;
-  blk_gemm_tile<f64 ? 1 : RM, f64 ? 1 : RN>(A, B, C, M, N, K1, K2, sa1, sa2, sb1, sb2, fm, fn);
+  if (K2 == 1) { K2 = K1; sa2 = sa1; sb2 = sb1; K1 = 1; }  // the inner loop is the unrolled one
+  blk_gemm_tile<f64 ? 1 : RM, f64 ? 1 : RN, U>(A, B, C, M, N, K1, K2, sa1, sa2, sb1, sb2, fm, fn);
 }
 
 // ------------------------------------------------------------------------------------------
+// Bonds of a boundary MPS as far as they are not zero: bnd[k] (k = 0..Ly) = 1 + the largest index of
+// the bond between sites k-1 and k at which both have a nonzero entry (NaN and Inf count), at least
+// 1; 1 at the open ends.  The row step stores its bonds padded to chi, the kept singular values in
+// descending order and the zero ones last, so contractions can stop at these prefixes: what they
+// skip are exact zeros, and the others are added in the same order.  br, bl: Ly entries of scratch.
+// Ends with a barrier.
+template <typename T, typename G>
+__device__ __noinline__ void mps_bonds(const G g, const T* E, int* bnd, int* bl, int* br) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int chi = g.chi, rows = g.chi * g.D;
+  const int rpw = chi < 32 ? 32 / chi : 1, r0 = chi < 32 ? lane / chi : 0, b0 = chi < 32 ? lane - r0 * chi : lane;
+  for (int k = warp; k < g.Ly; k += nw) {
+    const T* Ek = E + (size_t)k * g.se;
+    unsigned row = 0, col = 0;
+    if (r0 < rpw) {
+#pragma unroll 4
+      for (int r = r0; r < rows; r += rpw)
+#pragma unroll 1
+        for (int b = b0; b < chi; b += 32)
+          if (nonzero_(Ek[(size_t)r * chi + b])) { row = r; col = max(col, (unsigned)b); }
+    }
+    row = __reduce_max_sync(0xffffffffu, row);
+    col = __reduce_max_sync(0xffffffffu, col);
+    if (lane == 0) {
+      bl[k] = (int)row / g.D + 1;
+      br[k] = (int)col + 1;
+    }
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k <= g.Ly; k += blockDim.x)
+    bnd[k] = (k == 0 || k == g.Ly) ? 1 : min(br[k - 1], bl[k]);
+  __syncthreads();
+}
+
 // One row step of the boundary MPS: Eout = normalise(truncate_chi(Eprev o T_proj[row])).
 //   Eprev, Eout: Ly environment sites (chi x D x chi each), may be global memory.
 //   Srow: the Ly local states of the applied row; lower: lower-environment orientation.
 // Returns the product of the Ly normalisation factors (in thread 0); *st collects status bits.
 template <typename T, typename G>
-__device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpad, int row,
-                               const uint8_t* Srow, bool lower, const RowWork<T>& w, int* st, int* flag) {
+__device__ __forceinline__ Scaled env_row_step_inl(const G& g, const T* Eprev, T* Eout, const T* Tpad, int row,
+                                                   const uint8_t* Srow, bool lower, const RowWork<T>& w, int* st,
+                                                   int* flag) {
   const int chi = g.chi, D = g.D, n = g.n, Ly = g.Ly;
   const int tid = threadIdx.x, NT = blockDim.x;
   const int Lr = D * chi;           // row length of X, Y (open leg x truncated bond)
@@ -1181,62 +1461,72 @@ __device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
   // rows, all of them first in its (i, d) row order.  The products and the QR run on those rows
   // alone (Z stored compactly with ld rk D); the dropped rows are exact zeros that would leave
   // every reflector, and so R, unchanged.
-  blk_unit(w.R, n);  // row 0; the later rows of R are read only where a QR wrote them
+  // All sums and outputs run over the bonds of Eprev that are not zero (mps_bonds): R_k has
+  // bnd[k+1] D columns, and the right pass's new bonds end at the nonzero singular values.
   __shared__ int rks_s[MAX_LY];  // rks_s[k]: nonzero rows of R_{k-1}
-  __syncthreads();
+  __shared__ int bnd[MAX_LY + 1], bl_s[MAX_LY], br_s[MAX_LY];
+  // R_{k-1} (ld bnd[k] D, its nonzero rows) and Z are in the scratch ZS where they fit together with R_k
+  const int zcap = env_zs_elems(chi, D);
+  T* R = w.ZS;
+  blk_unit(R, D);  // row 0 of R_{-1}
+  mps_bonds(g, Eprev, bnd, bl_s, br_s);
+  const int wcap = w.ci * (D * D * chi + 1);  // elements of W
   int rk = 1;
-  __shared__ int ncz_s, bx_s;
+  __shared__ int ncz_s, nz_s;
+#pragma unroll 1
   for (int k = 0; k + 1 < Ly; ++k) {
-    if (tid == 0) { ncz_s = 0; bx_s = 0; }
-    blk_copy(w.E, Eprev + (size_t)k * g.se, g.se);
+    const int ka = bnd[k], kb = bnd[k + 1];
+    const FDiv fkb = fdiv_of(kb);
+    if (tid == 0) ncz_s = 0;
+    blk_copy(w.E, Eprev + (size_t)k * g.se, ka * D * chi);
     load_A(w.A, Tpad, g, row * Ly + k, Srow[k], lower);
     __syncthreads();
-    const int mZ = rk * D;             // nonzero rows of Z; Z is stored column major (ld mZ)
-    const int WS = D * D * chi + 1;    // padded row stride of W (no bank conflicts across ii)
-    for (int i0 = 0; i0 < rk; i0 += w.ci) {
-      const int ci = (rk - i0 < w.ci) ? (rk - i0) : w.ci;
+    const int mZ = rk * D;           // nonzero rows of Z; Z is stored column major (ld mZ)
+    const int lR = ka * D, lR1 = kb * D, rn = mZ < lR1 ? mZ : lR1;
+    const int zo = max(rk * lR, rn * lR1);
+    T* const Z = R == w.ZS && zo + mZ * lR1 <= zcap ? w.ZS + zo : w.Z;
+    T* const R1 = Z != w.Z || rn * lR1 <= zcap ? w.ZS : w.R;
+    const int WS = D * D * kb + 1;   // padded row stride of W (no bank conflicts across ii)
+    const int cmax = min(rk, wcap / WS);
+#pragma unroll 1
+    for (int i0 = 0; i0 < rk; i0 += cmax) {
+      const int ci = (rk - i0 < cmax) ? (rk - i0) : cmax;
+      const FDiv fci = fdiv_of(ci);
       // W[ii][l][u][b] = sum_a R[i0+ii][(a,l)] E[a][u][b]   (m = (u, b), n = (ii, l), k = a)
-      blk_gemm<2, 8>(w.E, w.R + (size_t)i0 * n, w.W, D * chi, ci * D, chi, 1, D * chi, 0, D, 0,
-                     [=](int m) { return Off2{m, m}; },
-                     [=](int nn) { return Off2{(nn / D) * n + nn % D, (nn / D) * WS + (nn % D) * D * chi}; });
+      blk_gemm<2, 4, 2>(w.E, R + (size_t)i0 * lR, w.W, D * kb, ci * D, ka, 1, D * chi, 0, D, 0,
+                     [=](int m) {
+                       const int u = fdiv_q(m, fkb);
+                       return Off2{u * chi + m - u * kb, m};
+                     },
+                     [=](int nn) { return Off2{(nn / D) * lR + nn % D, (nn / D) * WS + (nn % D) * D * kb}; });
       // Z[(i0+ii, d)][(b, r)] = sum_{l,u} W[ii][l][u][b] A[l][u][r][d]   (m = (ii, b) with ii
       // fastest, n = (r, d), k = (l, u)); Z is column major with column (b, r)
-      blk_gemm<4, 4>(w.W, w.A, w.Z, ci * chi, D * D, D * D, 1, chi, 0, D * D, 0,
+      blk_gemm<2, 4, 2>(w.W, w.A, Z, ci * kb, D * D, D * D, 1, kb, 0, D * D, 0,
                      [=](int m) {
-                       const int ii = m % ci, b = m / ci;
+                       const int b = fdiv_q(m, fci), ii = m - b * ci;
                        return Off2{ii * WS + b, b * D * mZ + (i0 + ii) * D};
                      },
                      [=](int nn) { return Off2{nn, (nn / D) * mZ + nn % D}; });
     }
-    // the columns (b, r) of Z with b at or beyond the bond of E's site k are exact zeros (E's
-    // bonds are padded to chi with zeros; the first row has bond D, a truncation keeps at most
-    // chi): find the nonzero prefix and factor only it (a zero column leaves every reflector
-    // unchanged and is a zero column of R); R's rank, hence the next rk, is at most that width.
-    // The bond comes from E, so that only Z's columns from its last index down are looked at.
-    {
-      int bx = 0;
-      for (int o = tid; o < g.se; o += NT)
-        if (nonzero_(w.E[o])) bx = max(bx, o % chi + 1);
-      bx = (int)__reduce_max_sync(0xffffffffu, (unsigned)bx);
-      if ((tid & 31) == 0 && bx) atomicMax(&bx_s, bx);
-      __syncthreads();
-      for (int c1 = bx_s * D; c1 > 0; c1 -= D) {
-        int last = 0;
-        for (int o = (c1 - D) * mZ + tid; o < c1 * mZ; o += NT)
-          if (nonzero_(w.Z[o])) last = max(last, o / mZ + 1);
-        last = (int)__reduce_max_sync(0xffffffffu, (unsigned)last);
-        if ((tid & 31) == 0 && last) atomicMax(&ncz_s, last);
-        if (__syncthreads_or(last)) break;
-      }
+    // columns of Z that are exact zeros past its last nonzero one (a leg of A that is padded) are
+    // not factored: a zero column leaves every reflector unchanged and is a zero column of R; R's
+    // rank, hence the next rk, is at most that width
+#pragma unroll 1
+    for (int c1 = kb * D; c1 > 0; c1 -= D) {
+      int last = 0;
+#pragma unroll 2
+      for (int o = (c1 - D) * mZ + tid; o < c1 * mZ; o += NT)
+        if (nonzero_(Z[o])) last = max(last, o / mZ + 1);
+      last = (int)__reduce_max_sync(0xffffffffu, (unsigned)last);
+      if ((tid & 31) == 0 && last) atomicMax(&ncz_s, last);
+      if (__syncthreads_or(last)) break;
     }
     const int ncz = ncz_s;
-    qr_keep_r<T, GeoMz<G>::value>(w.Z, mZ, ncz, w.R, w.sig, n);
     if (tid == 0) rks_s[k] = rk;
     rk = (mZ < ncz) ? mZ : ncz;
-    if (rk > n) rk = n;
     if (rk < 1) rk = 1;
-    blk_copy(w.Rhist + (size_t)k * n * n, w.R, rk * n);
-    __syncthreads();
+    qr_keep_r<T, GeoMz<G>::value>(Z, mZ, ncz, R1, w.sig, lR1, rk, lR1, w.Rhist + (size_t)k * n * n);
+    R = R1;
   }
   if (tid == 0) rks_s[Ly - 1] = rk;  // the rows of R_{Ly-2}, the right pass's first cut
   __syncthreads();
@@ -1246,118 +1536,122 @@ __device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
   // groups (eight consecutive elements of four rows each) hit different banks
   const int LY = Lr + 1;
   const int LX = Lr + ((8 - Lr) % 32 + 32) % 32;
-  T* P = w.Z;                              // chi*D*D*chi
-  T* Y = P + (size_t)chi * D * D * chi;    // n x Lr   (ld LY)
-  T* X = Y + (size_t)n * LY;               // mX x Lr  (ld LX)
-  T* Vt = X + (size_t)mX * LX;             // chi x Lr (ld LY)
-  T* Bs = Vt + (size_t)chi * LY;           // chi x D x chi (the first site)
   // C_{Ly-1}[(b,r)][c] = delta_{(b,r),0} delta_{c,0}
-  blk_unit(w.C, n * chi);
+  for (int o = tid; o < D; o += NT) w.C[(size_t)o * chi] = o == 0 ? T(1) : T(0);
+  int cc = 1;  // columns of C that are not zero
   __syncthreads();
   Scaled lg = sc_one();
+#pragma unroll 1
   for (int k = Ly - 1; k >= 0; --k) {
-    blk_copy(w.E, Eprev + (size_t)k * g.se, g.se);
+    const int ka = bnd[k], kb = bnd[k + 1];
+    const FDiv fcc = fdiv_of(cc);
+    if (tid == 0) nz_s = 0;
+    blk_copy(w.E, Eprev + (size_t)k * g.se, ka * D * chi);
     load_A(w.A, Tpad, g, row * Ly + k, Srow[k], lower);
+    // R_{k-1} from the left pass: only its first rks_s[k] rows are nonzero
+    const int rkx = k > 0 ? rks_s[k] : 0, nR = ka * D;
+    const int mJ = min(rkx + (rkx & 1), mX);  // an even count, for the Jacobi
+    // the matrices of this site in the scratch where they fit (P in W, which the Jacobi takes later),
+    // else in their own buffers
+    const int nv = mJ < chi ? mJ : chi;
+    const bool zs = rkx * nR + nR * LY + mJ * LX + nv * LY <= zcap;
+    T* P = ka * D * D * chi <= wcap ? w.W : w.Z;                            // ka x D x D x chi
+    T* const Rx = zs ? w.ZS : w.R;                                          // rkx x nR
+    T* const Y = zs ? w.ZS + rkx * nR : w.Z + (size_t)chi * D * D * chi;    // nR x Lr (ld LY)
+    T* const X = Y + (size_t)(zs ? nR : n) * LY;                            // mJ x Lr (ld LX)
+    T* const Vt = X + (size_t)(zs ? mJ : mX) * LX;                          // nv x Lr (ld LY)
+    if (k > 0) {
+      const T* Rk = w.Rhist + (size_t)(k - 1) * n * n;
+#pragma unroll 4
+      for (int o = tid; o < rkx * nR; o += NT) {
+        Rx[o] = Rk[o];
+      }
+    }
     __syncthreads();
     // P[a][u][r][c] = sum_b E[a][u][b] C[(b,r)][c]   (m = (r, c), n = (a, u), k = b)
-    blk_gemm<2, 8>(w.C, w.E, P, D * chi, chi * D, chi, 1, D * chi, 0, 1, 0,
-                   [=](int m) { return Off2{m, m}; },
+    blk_gemm<2, 4, 2>(w.C, w.E, P, D * cc, ka * D, kb, 1, D * chi, 0, 1, 0,
+                   [=](int m) {
+                     const int r = fdiv_q(m, fcc), o = r * chi + m - r * cc;
+                     return Off2{o, o};
+                   },
                    [=](int nn) { return Off2{nn * chi, nn * D * chi}; });
     if (k == 0) {
       // first site: its left bond is trivial, keep only row (a,l) = (0,0) of Y = M_0 C_0
+#pragma unroll 1
       for (int o = tid; o < g.se; o += NT) {
         const int c = o % chi, dd = (o / chi) % D, a = o / (chi * D);
         T s = 0;
-        if (a == 0) {
+        if (a == 0 && c < cc) {
+#pragma unroll 1
           for (int u = 0; u < D; ++u)
             for (int r = 0; r < D; ++r) s += P[((0 * D + u) * D + r) * chi + c] * w.A[((0 * D + u) * D + r) * D + dd];
         }
-        Bs[o] = s;
+        w.R[o] = s;
       }
       __syncthreads();
-      const double f = (double)blk_normalize(Bs, g.se, w.red, st);
+      const double f = (double)blk_normalize(w.R, g.se, w.red, st);
       if (tid == 0) lg = sc_mul(lg, f);
-      blk_copy(Eout, Bs, g.se);
+      blk_copy(Eout, w.R, g.se);
       __syncthreads();
       break;
     }
     // Y[(a,l)][(d,c)] = sum_{u,r} P[a][u][r][c] A[l][u][r][d]   (m = (a, c), n = (l, d), k = (u, r))
-    blk_gemm<4, 4>(P, w.A, Y, chi * chi, D * D, D * D, 1, chi, 0, D, 0,
-                   [=](int m) { return Off2{(m / chi) * D * D * chi + m % chi, (m / chi) * D * LY + m % chi}; },
+    blk_gemm<2, 4, 2>(P, w.A, Y, ka * cc, D * D, D * D, 1, chi, 0, D, 0,
+                   [=](int m) {
+                     const int a = fdiv_q(m, fcc), c = m - a * cc;
+                     return Off2{a * D * D * chi + c, a * D * LY + c};
+                   },
                    [=](int nn) { return Off2{(nn / D) * D * D * D + nn % D, (nn / D) * LY + (nn % D) * chi}; });
-    // R_{k-1} from the left pass: only its first rks_s[k] rows are nonzero
-    const int rkx = rks_s[k] < n ? rks_s[k] : n;
-    blk_copy(w.R, w.Rhist + (size_t)(k - 1) * n * n, rkx * n);
-    __syncthreads();
-    // X = R_{k-1} Y (m = q, n = i, k = j), padded to mX rows, on the nonzero rows of R_{k-1}:
-    // a thread takes two columns q and a block of 8 rows i in [8b, 8b + 8), and since R is upper
-    // triangular (explicit zeros below the diagonal) its sums start at j = 8b: the terms skipped
-    // are exact zeros and the others are added in the same order as the full product.  Rows from
-    // rkx on are zero.
-    if constexpr (sizeof(typename Scal<T>::R) == 8) {
-      for (int o = tid; o < mX * Lr; o += NT) {  // one output per thread, as in blk_gemm
-        const int q = o % Lr, i = o / Lr;
-        T acc = T(0);
-        if (i < rkx)
-          for (int j = i; j < n; ++j) acc = mad(acc, Y[(size_t)j * LY + q], w.R[(size_t)i * n + j]);
-        X[(size_t)i * LX + q] = acc;
+    // X = R_{k-1} Y on the nonzero rows of R_{k-1}, the columns q = (d, c < cc) and j < nR.  A
+    // thread's sums start at the first row's diagonal (R is upper triangular with explicit zeros
+    // below): the terms skipped are exact zeros and the others are added in the same order.  The
+    // other entries of the first mJ rows (an even count, for the Jacobi) are zeros.
+    const int nq = D * cc;
+    constexpr int XI = sizeof(typename Scal<T>::R) == 8 ? 1 : 4;  // (FP64: one output per thread, as in blk_gemm)
+    for (int t = tid; t < nq * ((rkx + XI - 1) / XI); t += NT) {
+      const int b = t / nq, qq = t - b * nq, dd = fdiv_q(qq, fcc), q = dd * chi + qq - dd * cc;
+      T acc[XI];
+#pragma unroll
+      for (int ii = 0; ii < XI; ++ii) acc[ii] = T(0);
+#pragma unroll 2
+      for (int j = XI * b; j < nR; ++j) {
+        const T y = Y[(size_t)j * LY + q];
+#pragma unroll
+        for (int ii = 0; ii < XI; ++ii) acc[ii] = mad(acc[ii], y, Rx[min(XI * b + ii, rkx - 1) * nR + j]);
       }
-      __syncthreads();
-    } else {
-      const int nbk = (rkx + 7) / 8, tmq = (Lr + 1) / 2;
-      for (int t = tid; t < tmq * nbk; t += NT) {
-        const int ti = t % tmq, b = t / tmq;
-        const int q0 = ti, q1 = ti + tmq;
-        const bool v1 = q1 < Lr;
-        T acc0[8], acc1[8];
 #pragma unroll
-        for (int ii = 0; ii < 8; ++ii) { acc0[ii] = T(0); acc1[ii] = T(0); }
-        for (int j = 8 * b; j < n; ++j) {
-          const T a0 = Y[(size_t)j * LY + q0], a1 = v1 ? Y[(size_t)j * LY + q1] : T(0);
-#pragma unroll
-          for (int ii = 0; ii < 8; ++ii) {
-            const int i = 8 * b + ii;
-            const T r = (i < rkx) ? w.R[(size_t)i * n + j] : T(0);
-            acc0[ii] = mad(acc0[ii], a0, r);
-            acc1[ii] = mad(acc1[ii], a1, r);
-          }
-        }
-#pragma unroll
-        for (int ii = 0; ii < 8; ++ii) {
-          const int i = 8 * b + ii;
-          if (i < rkx) {
-            X[(size_t)i * LX + q0] = acc0[ii];
-            if (v1) X[(size_t)i * LX + q1] = acc1[ii];
-          }
-        }
-      }
-      for (int o = tid; o < (mX - rkx) * Lr; o += NT) X[(size_t)(rkx + o / Lr) * LX + o % Lr] = T(0);
-      __syncthreads();
+      for (int ii = 0; ii < XI; ++ii)
+        if (XI * b + ii < rkx) X[(size_t)(XI * b + ii) * LX + q] = acc[ii];
     }
+#pragma unroll 1
+    for (int o = tid; o < mJ * Lr; o += NT) {
+      const int i = o / Lr, q = o - i * Lr;
+      if (i >= rkx || q % chi >= cc) X[(size_t)i * LX + q] = T(0);
+    }
+    __syncthreads();
     // norms, singular values and the selection in the real type (the QR's taus, in the same
     // buffer, are no longer needed)
     using RT = typename Scal<T>::R;
     RT* sig = reinterpret_cast<RT*>(w.sig);
-    // only the first rks_s[k] rows of R_{k-1}, hence of X, are nonzero (found by the left
-    // pass): the Jacobi runs on those rows (an even count; the rest are exact zeros that no
-    // rotation would touch)
-    int mJ = rks_s[k] < n ? rks_s[k] : n;  // nonzero rows of R_{k-1} (k >= 1 here)
-    mJ += (mJ & 1);
-    if (mJ > mX) mJ = mX;
-    const int sweeps = hestenes_rows<T, GeoLr<G>::value>(X, mJ, Lr, LX, flag, w.ctr, w.red, sig);
+    // the Jacobi runs on the first mJ rows (the rest are exact zeros that no rotation would touch);
+    // W is free here
+    const int sweeps = hestenes_rows(X, mJ, Lr, LX, flag, w.ctr, w.red, sig, w.W, wcap);
     if (sweeps < 0 && tid == 0) *st |= ST_NOCONV;
     // singular values: hestenes_rows left those of its rows in sig, the other rows are zero
+#pragma unroll 1
     for (int p = mJ + tid; p < mX; p += NT) sig[p] = RT(0);
     __syncthreads();
     // stable descending rank; the first chi ranks are kept.  A NaN singular value (non-finite
     // input) ranks below every number, so that the ranks stay a permutation and every kept
     // index is valid; the sample is flagged.
     // Four threads count for a row.
+#pragma unroll 1
     for (int p0 = 0; p0 < mX; p0 += NT >> 2) {
       const int p = p0 + (tid >> 2);
       const RT sp = sig[p < mX ? p : 0];
       const auto kp = order_key(sp);
       int rk = 0;
+#pragma unroll 4
       for (int q = tid & 3; q < mX; q += 4) {
         const auto kq = order_key(sig[q]);
         rk += (kq > kp) || (kq == kp && q < p);
@@ -1368,6 +1662,7 @@ __device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
       if (!(sp == sp) || isinf(sp)) atomicOr(st, (int)ST_NONFINITE);
       w.sel[mX + p] = rk;          // rank of row p
       if (rk < chi) w.sel[rk] = p; // row holding rank rk
+      if (sp > RT(0)) atomicMax(&nz_s, rk + 1);
       if (rk == chi - 1) sig[mX + 0] = sp;  // sigma_(chi-1)
       if (rk == chi) sig[mX + 1] = sp;      // sigma_(chi)
       if (rk == 0) sig[mX + 2] = sp;        // sigma_(0)
@@ -1381,11 +1676,15 @@ __device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
       __shared__ int kc_s;
       if (tid == 0) kc_s = mX;
       double part = 0.0;
+#pragma unroll 1
       for (int p = tid; p < mX; p += NT) part += (double)sig[p] * (double)sig[p];
       const double tot_s = block_sum(part, w.red);  // ends with a barrier
       const double thr = g.cut * tot_s;
+#pragma unroll 1
       for (int r = tid + 1; r < mX; r += NT) {
         double tail = 0.0;
+        
+#pragma unroll 1
         for (int p = 0; p < mX; ++p)
           if (w.sel[mX + p] >= r) tail += (double)sig[p] * (double)sig[p];
         if (tail <= thr) atomicMin(&kc_s, r);
@@ -1395,10 +1694,13 @@ __device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
       if (tot_s > 0.0 && kc < nkeep) {
         if (tid == 0) {
           // a boundary weight within 1e-9 of the cutoff: the choice is not stable under rounding
+#pragma unroll 1
           for (int k = kc - 1; k <= kc; ++k) {
             if (k < 1) continue;
             double tail = 0.0;
-            for (int p = 0; p < mX; ++p)
+            
+#pragma unroll 1
+        for (int p = 0; p < mX; ++p)
               if (w.sel[mX + p] >= k) tail += (double)sig[p] * (double)sig[p];
             if (fabs(tail - thr) <= 1e-9 * thr) *st |= ST_NEAR_DEGENERATE;
           }
@@ -1418,17 +1720,16 @@ __device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
         if (s0 > RT(0) && (sk - sd) < RT(1e-8) * s0 && sd > RT(1e-12) * s0) *st |= ST_NEAR_DEGENERATE;
       }
     }
-    // Vt[c'][q] = X[sel(c')][q] / sigma  (the rows of V^H); rows from nkeep on are zero.  Its
-    // largest modulus normalises the new site B[c'][d][c] = Vt[c'][(d, c)] on the way out.
+    // Vt[c'][q] = X[sel(c')][q] / sigma (the rows of V^H) for the kept singular values that are not
+    // zero, q = (d, c < cc); the others are zero.  Its largest modulus normalises the new site
+    // B[c'][d][c] = Vt[c'][(d, c)] on the way out.
+    const int nk = min(nkeep, nz_s);
     RT vm = 0;
-    for (int o = tid; o < chi * Lr; o += NT) {
-      const int q = o % Lr, cp = o / Lr;
-      T v = 0;
-      if (cp < nkeep) {
-        const int p = w.sel[cp];
-        const RT s = sig[p];
-        if (s > RT(0)) v = X[(size_t)p * LX + q] * (RT(1) / s);
-      }
+#pragma unroll 2
+    for (int o = tid; o < nk * Lr; o += NT) {
+      const int cp = o / Lr, q = o - cp * Lr;
+      const int p = w.sel[cp];
+      const T v = X[(size_t)p * LX + q] * (RT(1) / sig[p]);
       Vt[(size_t)cp * LY + q] = v;
       vm = max_(vm, abs_(v));
     }
@@ -1447,31 +1748,48 @@ __device__ Scaled env_row_step(const G& g, const T* Eprev, T* Eout, const T* Tpa
       if (tid == 0) lg = sc_mul(lg, (double)vm);
     }
     T* Ek = Eout + (size_t)k * g.se;
-    for (int o = tid; o < g.se; o += NT) Ek[o] = Vt[(size_t)(o / Lr) * LY + o % Lr] * inv;
+#pragma unroll 2
+    for (int o = tid; o < g.se; o += NT) {
+      const int cp = o / Lr, q = o - cp * Lr;
+      Ek[o] = cp < nk ? Vt[(size_t)cp * LY + q] * inv : T(0);
+    }
     // C_{k-1} = Y V: C[j][c'] = sum_q Y[j][q] conj(Vt[c'][q])   (C_k was last read by P)
     if constexpr (Scal<T>::complex) {
-      for (int o = tid; o < n * chi; o += NT) {
-        const int cp = o % chi, j = o / chi;
+      for (int o = tid; o < ka * D * nk; o += NT) {
+        const int j = o / nk, cp = o - j * nk;
         const T* Yr = Y + (size_t)j * LY;
         const T* Vr = Vt + (size_t)cp * LY;
         T s = 0;
-        for (int q = 0; q < Lr; ++q) s = mad(s, Yr[q], conj_(Vr[q]));
-        w.C[o] = s;
+        for (int d = 0; d < D; ++d)
+          for (int c = 0; c < cc; ++c) s = mad(s, Yr[d * chi + c], conj_(Vr[d * chi + c]));
+        w.C[j * chi + cp] = s;
       }
       __syncthreads();
     } else {
-      blk_gemm<2, 2>(Y, Vt, w.C, n, chi, Lr, 1, 1, 0, 1, 0, [=](int m) { return Off2{m * LY, m * chi}; },
+      blk_gemm<2, 2, 2>(Y, Vt, w.C, ka * D, nk, D, cc, chi, 1, chi, 1, [=](int m) { return Off2{m * LY, m * chi}; },
                      [=](int nn) { return Off2{nn * LY, nn}; });
+    }
+    cc = nk > 0 ? nk : 1;
+    if (nk == 0) {  // nothing left (flagged above): the remaining sites are zero
+      for (int o = tid; o < ka * D; o += NT) w.C[(size_t)o * chi] = T(0);
+      __syncthreads();
     }
   }
   return lg;
+}
+
+// The row step as a call, for kernels that take it in several places.
+template <typename T, typename G>
+__device__ __noinline__ Scaled env_row_step(const G g, const T* Eprev, T* Eout, const T* Tpad, int row,
+                                            const uint8_t* Srow, bool lower, const RowWork<T> w, int* st, int* flag) {
+  return env_row_step_inl(g, Eprev, Eout, Tpad, row, Srow, lower, w, st, flag);
 }
 
 // First environment row: row 0 read as an MPS (upper side, e[a=l][p=d][b=r] = A[l][0][r][d])
 // or row Lx-1 (lower side, e[l][u][r] = A[l][u][r][0]); every site normalised.  Returns the product
 // of the factors (in thread 0).
 template <typename T, typename G>
-__device__ Scaled env_first_row(const G& g, T* Eout, const T* Tpad, int row, const uint8_t* Srow,
+__device__ __noinline__ Scaled env_first_row(const G g, T* Eout, const T* Tpad, int row, const uint8_t* Srow,
                                 bool lower, T* Abuf, T* Bs, double* red, int* st) {
   const int chi = g.chi, D = g.D;
   Scaled lg = sc_one();
@@ -1493,67 +1811,14 @@ __device__ Scaled env_first_row(const G& g, T* Eout, const T* Tpad, int row, con
 }
 
 // ------------------------------------------------------------------------------------------
-// Quotient m / k for 0 <= m < 2^22 and k >= 1 from a float reciprocal: (m + 1/2) / k lies at
-// least 1 / (2k) from every integer, and the two roundings (of 1 / k and of the product) move it
-// by at most (m + 1/2) 2^-23 / k < 1 / (2k), so truncation gives the exact quotient.  Cheaper
-// than an integer division when k is only known at run time.
-struct FDiv {
-  int k;
-  float r;
-};
-__device__ __forceinline__ FDiv fdiv_of(int k) { return FDiv{k, __frcp_rn((float)k)}; }
-__device__ __forceinline__ int fdiv_q(int m, FDiv d) { return __float2int_rz(((float)m + 0.5f) * d.r); }
-
-// Nonzero prefixes of the bond legs of an upper environment site eu[a][u][x] and a lower one
-// el[b][d][z] (chi x D x chi each): a = 1 + the largest left-bond index with a nonzero entry of
-// eu, x the same for its right bond, b and z for el (each at least 1).  Near the open edges
-// and in the first rows the boundary MPS's bonds are smaller than chi and the row step stores
-// them zero-padded (its kept singular values come in descending order, the zero ones last), so
-// a contraction over such a bond can stop at the prefix: the skipped terms are exact zeros and
-// the kept ones are summed in the same order, which leaves every result unchanged.  NaN and Inf
-// entries count as nonzero.  Ends with a barrier; every thread gets the same extents.
+// Bonds of one column of a sandwich between an upper boundary MPS (sites eu[a][u][x]) and a lower
+// one (el[b][d][z]), as far as they are not zero (mps_bonds of both): a, x of the upper one's left
+// and right bond, b, z of the lower one's.  Contractions, normalisations and copies stop there:
+// partials keep their full layouts, entries past the bonds are neither computed nor read, and what
+// is left out of a sum are exact zeros, the rest added in the same order.
 struct BondExt {
   int a, x, b, z;
 };
-template <typename T, typename G>
-__device__ BondExt bond_ext(const G& g, const T* eu, const T* el) {
-  __shared__ int ext_w[32][4];
-  const int chi = g.chi, Dc = g.D * g.chi;
-  int ea = 0, ex = 0, eb = 0, ez = 0;
-  for (int o = threadIdx.x; o < g.se; o += blockDim.x) {
-    const int a = o / Dc + 1, x = o % chi + 1;
-    if (nonzero_(eu[o])) { ea = max(ea, a); ex = max(ex, x); }
-    if (nonzero_(el[o])) { eb = max(eb, a); ez = max(ez, x); }
-  }
-  const unsigned full = 0xffffffffu;
-  ea = (int)__reduce_max_sync(full, (unsigned)ea);
-  ex = (int)__reduce_max_sync(full, (unsigned)ex);
-  eb = (int)__reduce_max_sync(full, (unsigned)eb);
-  ez = (int)__reduce_max_sync(full, (unsigned)ez);
-  if ((threadIdx.x & 31) == 0) {
-    int* w = ext_w[threadIdx.x >> 5];
-    w[0] = ea; w[1] = ex; w[2] = eb; w[3] = ez;
-  }
-  __syncthreads();
-  BondExt e{1, 1, 1, 1};
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
-    e.a = max(e.a, ext_w[i][0]);
-    e.x = max(e.x, ext_w[i][1]);
-    e.b = max(e.b, ext_w[i][2]);
-    e.z = max(e.z, ext_w[i][3]);
-  }
-  return e;
-}
-
-// Zero v[p][q][r] (P x Q x R, row major) outside p < kp, r < kr.  Ends with a barrier.
-template <typename T>
-__device__ void zero_outside(T* v, int P, int Q, int R, int kp, int kr) {
-  if (kp >= P && kr >= R) return;
-  const int QR = Q * R;
-  for (int o = threadIdx.x; o < P * QR; o += blockDim.x)
-    if (o / QR >= kp || o % R >= kr) v[o] = T(0);
-  __syncthreads();
-}
 
 // ------------------------------------------------------------------------------------------
 // One-row sandwich partials.  L[a][l][b] -> L'[x][r][z] over one column with eu[a][u][x],
@@ -1561,18 +1826,16 @@ __device__ void zero_outside(T* v, int P, int Q, int R, int kp, int kr) {
 // intermediates are laid out so that the index that varies across threads is contiguous in the
 // operand it is read from; t2's (x, r) rows are padded to D (chi + 1), so that the two column
 // groups a warp reads in the last product (16 rows per group at chi = 16) fall in different
-// shared-memory banks.  The bond indices run over the nonzero prefixes of bond_ext (a < ka,
-// b < kb, x < kx, z < kz): the intermediates keep their full layouts, entries outside the
-// prefixes are neither computed nor read, and L' is zero outside x < kx, z < kz.
+// shared-memory banks.  L' is written for x < e.x, z < e.z.
 template <typename T, typename G>
-__device__ void absorb1(const G& g, const T* L, const T* eu, const T* A, const T* el, T* t1, T* t2, T* out) {
+__device__ __noinline__ void absorb1(const G g, const BondExt e, const T* L, const T* eu, const T* A, const T* el, T* t1, T* t2,
+                        T* out) {
   const int chi = g.chi, D = g.D;
   const int PS = D * chi + D;  // padded (x, r) row stride of t2
-  const BondExt e = bond_ext(g, eu, el);
   const int kb = e.b, kx = e.x;
   const FDiv fb = fdiv_of(kb), fx = fdiv_of(kx);
   // t1[u][l][x][b] = sum_a L[a][l][b] eu[a][u][x]        (m = (l, b), n = (u, x), k = a)
-  blk_gemm<2, 8>(L, eu, t1, D * kb, D * kx, e.a, 1, D * chi, 0, D * chi, 0,
+  blk_gemm<2, 4>(L, eu, t1, D * kb, D * kx, e.a, 1, D * chi, 0, D * chi, 0,
                  [=](int m) {
                    const int l = fdiv_q(m, fb), b = m - l * kb;
                    return Off2{l * chi + b, l * chi * chi + b};
@@ -1582,7 +1845,7 @@ __device__ void absorb1(const G& g, const T* L, const T* eu, const T* A, const T
                    return Off2{u * chi + x, u * D * chi * chi + x * chi};
                  });
   // t2[x][r][d][b] = sum_{l,u} t1[u][l][x][b] A[l][u][r][d]   (m = (x, b), n = (r, d), k = (l, u))
-  blk_gemm<4, 4>(t1, A, t2, kx * kb, D * D, D, D, chi * chi, D * chi * chi, D * D * D, D * D,
+  blk_gemm<2, 4>(t1, A, t2, kx * kb, D * D, D, D, chi * chi, D * chi * chi, D * D * D, D * D,
                  [=](int m) {
                    const int x = fdiv_q(m, fb), b = m - x * kb;
                    return Off2{x * chi + b, x * D * PS + b};
@@ -1592,27 +1855,26 @@ __device__ void absorb1(const G& g, const T* L, const T* eu, const T* A, const T
   blk_gemm<1, 4>(el, t2, out, e.z, kx * D, kb, D, D * chi, chi, 1, chi,
                  [=](int m) { return Off2{m, m}; },
                  [=](int n) { return Off2{n * PS, n * chi}; });
-  zero_outside(out, chi, D, chi, kx, e.z);
 }
 
 // R[x][r][z] -> R'[a][l][b] = sum eu[a][u][x] A[l][u][r][d] el[b][d][z] R[x][r][z].
-// t1: D^2 chi (chi+1) elements (its rows padded to chi+1), t2: chi^2 D^2.  Bond indices over
-// the nonzero prefixes of bond_ext, as in absorb1; R' is zero outside a < ka, b < kb.
+// t1: D^2 chi (chi+1) elements (its rows padded to chi+1), t2: chi^2 D^2.  R' is written for
+// a < e.a, b < e.b.
 template <typename T, typename G>
-__device__ void absorb1_right(const G& g, const T* R, const T* eu, const T* A, const T* el, T* t1, T* t2, T* out) {
+__device__ __noinline__ void absorb1_right(const G g, const BondExt e, const T* R, const T* eu, const T* A, const T* el, T* t1,
+                              T* t2, T* out) {
   const int chi = g.chi, D = g.D, P = chi + 1;
-  const BondExt e = bond_ext(g, eu, el);
   const int ka = e.a, kz = e.z;
   const FDiv fz = fdiv_of(kz), fa = fdiv_of(ka);
   // t1[u][r][z][a] (rows of a padded to P) = sum_x R[x][r][z] eu[a][u][x]   (m = (r, z), n = (a, u))
-  blk_gemm<2, 8>(R, eu, t1, D * kz, ka * D, e.x, 1, D * chi, 0, 1, 0,
+  blk_gemm<2, 4>(R, eu, t1, D * kz, ka * D, e.x, 1, D * chi, 0, 1, 0,
                  [=](int m) {
                    const int r = fdiv_q(m, fz), z = m - r * kz;
                    return Off2{r * chi + z, (r * chi + z) * P};
                  },
                  [=](int n) { return Off2{n * chi, (n % D) * D * chi * P + n / D}; });
   // t2[z][d][a][l] = sum_{u,r} t1[u][r][z][a] A[l][u][r][d]   (m = (z, a), n = (l, d), k = (u, r))
-  blk_gemm<4, 4>(t1, A, t2, kz * ka, D * D, D, D, D * chi * P, chi * P, D * D, D,
+  blk_gemm<2, 4>(t1, A, t2, kz * ka, D * D, D, D, D * chi * P, chi * P, D * D, D,
                  [=](int m) {
                    const int z = fdiv_q(m, fa), a = m - z * ka;
                    return Off2{z * P + a, z * D * chi * D + a * D};
@@ -1622,7 +1884,6 @@ __device__ void absorb1_right(const G& g, const T* R, const T* eu, const T* A, c
   blk_gemm<2, 2>(t2, el, out, ka * D, e.b, kz, D, D * chi * D, chi * D, 1, chi,
                  [=](int m) { return Off2{m, m * chi}; },
                  [=](int n) { return Off2{n * D * chi, n}; });
-  zero_outside(out, chi, D, chi, ka, e.b);
 }
 
 // Site environment of the one-row sandwich: env[l][u][r][d] = sum L[a][l][b] eu[a][u][x]
@@ -1630,35 +1891,48 @@ __device__ void absorb1_right(const G& g, const T* R, const T* eu, const T* A, c
 // environment site read transposed, so that the contraction over z has a contiguous operand).
 // t1: D^2 chi (chi+1), its (u, l) rows padded to chi (chi + 1); t2: chi^2 D^2.
 template <typename T, typename G>
-__device__ void site_env1(const G& g, const T* L, const T* eu, const T* elT, const T* R, T* t1, T* t2, T* env) {
+__device__ __noinline__ void site_env1(const G g, const BondExt e, const T* L, const T* eu, const T* elT, const T* R, T* t1, T* t2,
+                          T* env) {
   const int chi = g.chi, D = g.D;
   const int S1 = chi * chi + chi;  // padded (u, l) row stride of t1
+  const int kb = e.b, kx = e.x;
+  const FDiv fb = fdiv_of(kb), fx = fdiv_of(kx);
   // t1[u][l][x][b] = sum_a L[a][l][b] eu[a][u][x]   (as in absorb1, rows padded)
-  blk_gemm<2, 8>(L, eu, t1, D * chi, D * chi, chi, 1, D * chi, 0, D * chi, 0,
-                 [=](int m) { return Off2{m, (m / chi) * S1 + m % chi}; },
-                 [=](int n) { return Off2{n, (n / chi) * D * S1 + (n % chi) * chi}; });
+  blk_gemm<2, 4>(L, eu, t1, D * kb, D * kx, e.a, 1, D * chi, 0, D * chi, 0,
+                 [=](int m) {
+                   const int l = fdiv_q(m, fb), b = m - l * kb;
+                   return Off2{l * chi + b, l * S1 + b};
+                 },
+                 [=](int n) {
+                   const int u = fdiv_q(n, fx), x = n - u * kx;
+                   return Off2{u * chi + x, u * D * S1 + x * chi};
+                 });
   // t4[b][x][r][d] = sum_z elT[z][b][d] R[x][r][z]   (m = (b, d), n = (x, r), k = z)
-  blk_gemm<2, 8>(elT, R, t2, chi * D, chi * D, chi, 1, chi * D, 0, 1, 0,
+  blk_gemm<2, 4>(elT, R, t2, kb * D, kx * D, e.z, 1, chi * D, 0, 1, 0,
                  [=](int m) { return Off2{m, (m / D) * chi * D * D + m % D}; },
                  [=](int n) { return Off2{n * chi, n * D}; });
   // env[l][u][r][d] = sum_{b,x} t4[b][x][r][d] t1[u][l][x][b]   (m = (r, d), n = (u, l) with l
   // fastest, so that the two column groups of a warp read t1 rows one padded stride apart)
-  blk_gemm<1, 1>(t2, t1, env, D * D, D * D, chi, chi, chi * D * D, D * D, 1, chi,
+  blk_gemm<1, 1>(t2, t1, env, D * D, D * D, kb, kx, chi * D * D, D * D, 1, chi,
                  [=](int m) { return Off2{m, m}; },
                  [=](int n) { return Off2{(n / D) * D * S1 + (n % D) * S1, ((n % D) * D + n / D) * D * D}; });
 }
 
 // sum_i a_i b_i, summed as 256 threads do it whatever the CTA's size (a smaller CTA's threads stand
-// in for several), so that the result does not depend on the launch shape.
+// in for several), so that the result does not depend on the launch shape.  The terms are those of
+// rows < nrow and columns < nc of the rows of length ld (the others are zeros).
 template <typename T>
-__device__ T blk_dot(const T* a, const T* b, int n, double* red) {
+__device__ __noinline__ T blk_dot(const T* a, const T* b, int nrow, int ld, int nc, double* red) {
+  const int n = nrow * ld;
   const int l = threadIdx.x & 31;
   T* r = reinterpret_cast<T*>(red);
   __syncthreads();
+#pragma unroll 1
   for (int w = threadIdx.x >> 5; w < 8; w += blockDim.x >> 5) {
     T s = 0;
     if (w * 32 < n) {
-      for (int o = w * 32 + l; o < n; o += 256) s += a[o] * b[o];
+      for (int o = w * 32 + l; o < n; o += 256)
+        if (o % ld < nc) s += a[o] * b[o];
       s = warp_sum(s);
     }
     if (l == 0) r[w] = s;
@@ -1712,13 +1986,11 @@ __device__ T mps_overlap(const G& g, const T* EU, const T* EL, T* Lb, T* Lb2, T*
 // first temporary holds chi more).  Intermediates are laid out so that the index that varies
 // across threads is contiguous in the operand it is read from.
 // L2[a][i][j][b] -> out[x][r1][r2][z] with eu[a][u][x], A1[i][u][r1][v], A2[j][v][r2][d], el[b][d][z].
-// Bond indices over the nonzero prefixes of bond_ext, as in absorb1 (the chunks cover x < kx);
-// out is zero outside x < kx, z < kz.
+// out is written for x < e.x (which the chunks cover), z < e.z.
 template <typename T, typename G>
-__device__ void absorb2(const G& g, const T* L2, const T* eu, const T* A1, const T* A2, const T* el,
+__device__ __noinline__ void absorb2(const G g, const BondExt e, const T* L2, const T* eu, const T* A1, const T* A2, const T* el,
                         T* t1, T* t2, T* out, int cx) {
   const int chi = g.chi, D = g.D;
-  const BondExt e = bond_ext(g, eu, el);
   const int kb = e.b, kx = e.x;
   const FDiv fb = fdiv_of(kb);
   for (int x0 = 0; x0 < kx; x0 += cx) {
@@ -1726,21 +1998,21 @@ __device__ void absorb2(const G& g, const T* L2, const T* eu, const T* A1, const
     const int cc = chi * c;
     const FDiv fbc = fdiv_of(kb * c);
     // t1[i][u][j][b][xx] = sum_a L2[a][i][j][b] eu[a][u][x0+xx]      (m = (i, j, b), n = (u, xx))
-    blk_gemm<4, 4>(L2, eu + x0, t1, D * D * kb, D * c, e.a, 1, D * D * chi, 0, D * chi, 0,
+    blk_gemm<2, 4>(L2, eu + x0, t1, D * D * kb, D * c, e.a, 1, D * D * chi, 0, D * chi, 0,
                    [=](int m) {
                      const int ij = fdiv_q(m, fb), b = m - ij * kb;
                      return Off2{ij * chi + b, (ij / D) * D * D * cc + ((ij % D) * chi + b) * c};
                    },
                    [=](int n) { return Off2{(n / c) * chi + n % c, (n / c) * D * cc + n % c}; });
     // t2[j][v][b][xx][r1] = sum_{i,u} t1[i][u][j][b][xx] A1[i][u][r1][v]   (m = (j, b, xx), n = (r1, v))
-    blk_gemm<4, 4>(t1, A1, t2, D * kb * c, D * D, D, D, D * D * cc, D * cc, D * D * D, D * D,
+    blk_gemm<2, 4>(t1, A1, t2, D * kb * c, D * D, D, D, D * D * cc, D * cc, D * D * D, D * D,
                    [=](int m) {
                      const int j = fdiv_q(m, fbc), rem = m - j * kb * c;
                      return Off2{j * cc + rem, j * D * D * cc + rem * D};
                    },
                    [=](int n) { return Off2{n, (n % D) * cc * D + n / D}; });
     // t3[r2][d][b][xx][r1] = sum_{j,v} t2[j][v][b][xx][r1] A2[j][v][r2][d]   (into t1; m = (b, xx, r1), n = (r2, d))
-    blk_gemm<4, 4>(t2, A2, t1, kb * c * D, D * D, D, D, D * cc * D, cc * D, D * D * D, D * D,
+    blk_gemm<2, 4>(t2, A2, t1, kb * c * D, D * D, D, D, D * cc * D, cc * D, D * D * D, D * D,
                    [=](int m) { return Off2{m, m}; },
                    [=](int n) { return Off2{n, n * cc * D}; });
     // out[x0+xx][r1][r2][z] = sum_{b,d} el[b][d][z] t3[r2][d][b][xx][r1]   (m = z, n = (xx, r2, r1)
@@ -1752,17 +2024,14 @@ __device__ void absorb2(const G& g, const T* L2, const T* eu, const T* A1, const
                      return Off2{r2 * D * cc * D + xx * D + r1, (((x0 + xx) * D + r1) * D + r2) * chi};
                    });
   }
-  zero_outside(out, chi, D * D, chi, kx, e.z);
 }
 
 // R2[x][r1][r2][z] -> out[a][i][j][b] = sum eu[a][u][x] A1[i][u][r1][v] A2[j][v][r2][d] el[b][d][z] R2[x][r1][r2][z].
-// Bond indices over the nonzero prefixes of bond_ext (the chunks cover a < ka); out is zero
-// outside a < ka, b < kb.
+// out is written for a < e.a (which the chunks cover), b < e.b.
 template <typename T, typename G>
-__device__ void absorb2_right(const G& g, const T* R2, const T* eu, const T* A1, const T* A2, const T* el,
+__device__ __noinline__ void absorb2_right(const G g, const BondExt e, const T* R2, const T* eu, const T* A1, const T* A2, const T* el,
                               T* t1, T* t2, T* out, int ca) {
   const int chi = g.chi, D = g.D;
-  const BondExt e = bond_ext(g, eu, el);
   const int ka = e.a, kz = e.z;
   const FDiv fz = fdiv_of(kz);
   for (int a0 = 0; a0 < ka; a0 += ca) {
@@ -1770,21 +2039,21 @@ __device__ void absorb2_right(const G& g, const T* R2, const T* eu, const T* A1,
     const int cdx = c * D * chi;             // one (u, r1) block of t1, one (v, r2) block of t2
     const int Sz = D * c * D * D + 1;        // z stride of t3 (odd: consecutive z in different banks)
     // t1[u][r1][aa][r2][z] = sum_x R2[x][r1][r2][z] eu[a0+aa][u][x]   (m = (r1, r2, z), n = (aa, u))
-    blk_gemm<4, 4>(R2, eu + (size_t)a0 * D * chi, t1, D * D * kz, c * D, e.x, 1, D * D * chi, 0, 1, 0,
+    blk_gemm<2, 4>(R2, eu + (size_t)a0 * D * chi, t1, D * D * kz, c * D, e.x, 1, D * D * chi, 0, 1, 0,
                    [=](int m) {
                      const int q = fdiv_q(m, fz), z = m - q * kz;  // q = (r1, r2)
                      return Off2{q * chi + z, (q / D) * cdx + (q % D) * chi + z};
                    },
                    [=](int n) { return Off2{n * chi, (n % D) * D * cdx + (n / D) * D * chi}; });
     // t2[v][r2][aa][i][z] = sum_{u,r1} t1[u][r1][aa][r2][z] A1[i][u][r1][v]   (m = (aa, r2, z), n = (i, v))
-    blk_gemm<4, 4>(t1, A1, t2, c * D * kz, D * D, D, D, D * cdx, cdx, D * D, D,
+    blk_gemm<2, 4>(t1, A1, t2, c * D * kz, D * D, D, D, D * cdx, cdx, D * D, D,
                    [=](int m) {
                      const int q = fdiv_q(m, fz), z = m - q * kz;  // q = (aa, r2)
                      return Off2{q * chi + z, (q % D) * cdx + (q / D) * D * chi + z};
                    },
                    [=](int n) { return Off2{(n / D) * D * D * D + n % D, (n % D) * D * cdx + (n / D) * chi}; });
     // t3[z][d][aa][i][j] (z stride Sz) = sum_{v,r2} t2[v][r2][aa][i][z] A2[j][v][r2][d]   (into t1)
-    blk_gemm<4, 4>(t2, A2, t1, c * D * kz, D * D, D, D, D * cdx, cdx, D * D, D,
+    blk_gemm<2, 4>(t2, A2, t1, c * D * kz, D * D, D, D, D * cdx, cdx, D * D, D,
                    [=](int m) {
                      const int q = fdiv_q(m, fz), z = m - q * kz;  // q = (aa, i)
                      return Off2{q * chi + z, z * Sz + q * D};
@@ -1795,7 +2064,6 @@ __device__ void absorb2_right(const G& g, const T* R2, const T* eu, const T* A1,
                    [=](int m) { return Off2{m, (a0 * D * D + m) * chi}; },
                    [=](int n) { return Off2{n * D * chi, n}; });
   }
-  zero_outside(out, chi, D * D, chi, ka, e.b);
 }
 
 // ------------------------------------------------------------------------------------------
