@@ -839,7 +839,7 @@ extern "C" peps_status peps_direct_prepare(peps_handle* h, int chi_double, void*
     return launch_dl_env<T>(g, chi_double, (const T*)h->Tpad, (T*)h->DL, w, h->dl_status, s);
   });
   if (e != cudaSuccess) return cuda_fail(h, e, "double-layer kernel");
-  tstop(h, ts, s);
+  tstop(h, ts, s, 2LL * (Lx - 1));
   return PEPS_OK;
 }
 

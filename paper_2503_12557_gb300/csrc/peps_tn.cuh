@@ -391,19 +391,19 @@ template <typename T>
 __device__ __forceinline__ void qr_apply_reflector(const T* zj, int j, T tau, T* zc, int m, int lane) {
   // zc <- (I - conj(tau) v v^H) zc with v = (1, zj[j+1..m))  (H^H of H = I - tau v v^H; real:
   // I - tau v v^T)
+  constexpr int U = Scal<T>::complex ? 2 : 8;
   T s = 0;
+#pragma unroll U
   for (int i = j + 1 + lane; i < m; i += 32) s = mad(s, conj_(zj[i]), zc[i]);
   s = warp_sum(s);
   const T w = (s + zc[j]) * conj_(tau);
   __syncwarp();
   if (lane == 0) zc[j] -= w;
+#pragma unroll U
   for (int i = j + 1 + lane; i < m; i += 32) zc[i] -= zj[i] * w;
   __syncwarp();
 }
 
-// Blocked by panels of QB columns: warp 0 computes the panel's reflectors (applying each to
-// the rest of the panel), then every warp applies the panel's reflectors, in order, to the
-// trailing columns it owns.  Two block barriers per panel.  taus: at least nc entries.
 // R (and R2, may be null), row major with ld ldr: rows 0..kr-1, columns 0..kc-1; zero below the
 // diagonal and from column nc on.  Ends with a barrier.
 template <typename T>
@@ -419,52 +419,50 @@ __device__ __noinline__ void qr_store_r(const T* Z, int m, int nc, T* R, int ldr
   __syncthreads();
 }
 
+// Column by column, in memory: after the barrier of step j every warp applies reflector j to its
+// columns (c mod nw); the warp that owns column j + 1 takes that one first and forms reflector j + 1.
+// (A panel of eight columns on one warp, the others waiting, was most of the double layer's time: its
+// 1024 x 64 factorisations, 8x8, D = 4, chi_d = 4.)  taus: at least nc entries.
 template <typename T>
-__device__ void qr_keep_r_smem(T* Z, int m, int nc, T* R, T* taus, int ldr, int kr, int kc, T* R2) {
-  constexpr int QB = 8;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+__device__ __noinline__ void qr_keep_r_smem(T* Z, int m, int nc, T* R, T* taus, int ldr, int kr, int kc, T* R2) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int steps = (m < nc) ? m : nc;
-  for (int j0 = 0; j0 < steps; j0 += QB) {
-    const int pb = (steps - j0 < QB) ? steps - j0 : QB;
-    if (warp == 0) {
-      for (int jj = 0; jj < pb; ++jj) {
-        const int j = j0 + jj;
-        T* zj = Z + (size_t)j * m;
-        typename Scal<T>::R part = 0;
-        for (int i = j + 1 + lane; i < m; i += 32) part += abs2_(zj[i]);
-        const typename Scal<T>::R sigma = warp_sum(part);
-        const T alpha = zj[j];
-        T tau = 0, beta = alpha;
-        if (sigma != 0) {
-          // LAPACK's xLARFG: beta = -sign(Re alpha) sqrt(|alpha|^2 + sigma) (real),
-          // tau = (beta - alpha) / beta, v = x / (alpha - beta)
-          const typename Scal<T>::R nrm = sqrt(abs2_(alpha) + sigma);
-          const typename Scal<T>::R bt = (re_(alpha) >= 0) ? -nrm : nrm;
-          beta = T(bt);
-          tau = (beta - alpha) * (typename Scal<T>::R(1) / bt);
-          const T sc = inv_(alpha - beta);
-          for (int i = j + 1 + lane; i < m; i += 32) zj[i] *= sc;
-        }
-        __syncwarp();
-        if (tau != T(0))
-          for (int c = j + 1; c < j0 + pb; ++c) qr_apply_reflector(zj, j, tau, Z + (size_t)c * m, m, lane);
-        if (lane == 0) {
-          taus[j] = tau;
-          zj[j] = beta;
-        }
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-    for (int c = j0 + pb + warp; c < nc; c += nw) {
+#pragma unroll 1
+  for (int j = -1; j < steps; ++j) {
+    if (j >= 0) __syncthreads();
+    const T tau = j >= 0 ? taus[j] : T(0);
+    const int jn = j + 1;
+#pragma unroll 1
+    for (int c = jn + (warp - jn % nw + nw) % nw; c < nc; c += nw) {  // (column c belongs to warp c mod nw)
       T* zc = Z + (size_t)c * m;
-      for (int jj = 0; jj < pb; ++jj) {
-        const T tau = taus[j0 + jj];
-        if (tau != T(0)) qr_apply_reflector(Z + (size_t)(j0 + jj) * m, j0 + jj, tau, zc, m, lane);
+      if (tau != T(0)) qr_apply_reflector(Z + (size_t)j * m, j, tau, zc, m, lane);
+      if (c != jn || jn >= steps) continue;
+      typename Scal<T>::R part = 0;
+#pragma unroll 4
+      for (int i = jn + 1 + lane; i < m; i += 32) part += abs2_(zc[i]);
+      const typename Scal<T>::R sigma = warp_sum(part);
+      const T alpha = zc[jn];
+      T tn = 0, beta = alpha;
+      if (sigma != 0) {
+        // LAPACK's xLARFG: beta = -sign(Re alpha) sqrt(|alpha|^2 + sigma) (real),
+        // tau = (beta - alpha) / beta, v = x / (alpha - beta)
+        const typename Scal<T>::R nrm = sqrt(abs2_(alpha) + sigma);
+        const typename Scal<T>::R bt = (re_(alpha) >= 0) ? -nrm : nrm;
+        beta = T(bt);
+        tn = (beta - alpha) * (typename Scal<T>::R(1) / bt);
+        const T sc = inv_(alpha - beta);
+#pragma unroll 4
+        for (int i = jn + 1 + lane; i < m; i += 32) zc[i] *= sc;
       }
+      __syncwarp();
+      if (lane == 0) {
+        taus[jn] = tn;
+        zc[jn] = beta;
+      }
+      __syncwarp();
     }
-    __syncthreads();
   }
+  __syncthreads();
   qr_store_r(Z, m, nc, R, ldr, kr, kc, R2);
 }
 
