@@ -246,11 +246,38 @@ template cudaError_t launch_center_global<float>(const float*, const double*, co
 // one; rotation parameters are recomputed from the old diagonal blocks (classical two-sided
 // Jacobi, Golub & Van Loan sym.schur2: tau = (a_qq - a_pp) / (2 a_pq), t = sign(tau) /
 // (|tau| + sqrt(1 + tau^2)), c = 1/sqrt(1+t^2), s = t c; B = J^T A J with J = [[c, s], [-s, c]]).
+// sqrt(x)^-1 and x^-1 from single-precision starts and two Newton steps (x within the float range):
+// a few dependent FP64 operations where sqrt and a division are some twenty each, and a round's
+// parameters are one such chain that the whole grid waits for (333 rows: 43.0 -> 36.9 ms with the
+// 32-bit indices of the apply phase; one CTA of 512 threads per SM instead of 256: 37.3).
+__device__ __forceinline__ double rsqrt_nr(double x) {
+  double y = (double)rsqrtf((float)x);
+  const double h = -0.5 * x;
+  y = y * fma(h, y * y, 1.5);
+  return y * fma(h, y * y, 1.5);
+}
+__device__ __forceinline__ double rcp_nr(double x) {
+  double r = (double)__frcp_rn((float)x);
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+}
 __device__ __forceinline__ void jac_params(const double* A, int n, int p, int q, double* c, double* s) {
   const double apq = A[(size_t)p * n + q];
   const double app = A[(size_t)p * n + p], aqq = A[(size_t)q * n + q];
-  if (apq == 0.0 || fabs(apq) <= 1e-15 * sqrt(fabs(app * aqq))) { *c = 1.0; *s = 0.0; return; }
-  const double tau = (aqq - app) / (2.0 * apq);
+  *c = 1.0;
+  *s = 0.0;
+  // t = sign(tau) / (|tau| + sqrt(1 + tau^2)) = 2 a_pq sign(d) / (|d| + sqrt(d^2 + 4 a_pq^2)), d = a_qq - a_pp
+  const double d = aqq - app, x = 2.0 * apq, n2 = fma(d, d, x * x), ab = fabs(app * aqq), o2 = apq * apq;
+  if (n2 > 1e-30 && n2 < 1e30 && o2 > 1e-250 && ab > 1e-250) {
+    if (o2 <= 1e-30 * ab) return;
+    const double h = n2 * rsqrt_nr(n2);
+    const double t = (d < 0.0 ? -x : x) * rcp_nr(fabs(d) + h);
+    *c = rsqrt_nr(fma(t, t, 1.0));
+    *s = t * (*c);
+    return;
+  }
+  if (apq == 0.0 || fabs(apq) <= 1e-15 * sqrt(ab)) return;
+  const double tau = d / x;
   double t;
   if (fabs(tau) > 1e150) t = 0.5 / tau;
   else t = copysign(1.0, tau) / (fabs(tau) + sqrt(1.0 + tau * tau));
@@ -276,15 +303,16 @@ __device__ __forceinline__ void jacobi_round_params(const double* __restrict__ A
   }
 }
 
+// (IX: 32-bit indices where they suffice, whose divisions are a fifth of the 64-bit ones)
+template <typename IX>
 __device__ __forceinline__ void jacobi_round_apply(const double* __restrict__ A, double* __restrict__ An, double* V,
-                                                   const double* __restrict__ cs, int n, int r, long long t0,
-                                                   long long tstride) {
+                                                   const double* __restrict__ cs, int n, int r, IX t0, IX tstride) {
   const int h = n / 2;
-  const long long nblk = (long long)h * h;
-  const long long nv = (long long)n * h;
-  for (long long o = t0; o < nblk + nv; o += tstride) {
+  const IX nblk = (IX)h * (IX)h;
+  const IX nv = (IX)n * (IX)h;
+  for (IX o = t0; o < nblk + nv; o += tstride) {
     if (o < nblk) {
-      const int I = (int)(o / h), J = (int)(o % h);
+      const int I = (int)(o / (IX)h), J = (int)(o - (IX)I * (IX)h);
       const int pI = rr_player(I, r, n), qI = rr_player(n - 1 - I, r, n);
       const int pJ = rr_player(J, r, n), qJ = rr_player(n - 1 - J, r, n);
       const double cI = cs[2 * I], sI = cs[2 * I + 1], cJ = cs[2 * J], sJ = cs[2 * J + 1];
@@ -302,8 +330,8 @@ __device__ __forceinline__ void jacobi_round_apply(const double* __restrict__ A,
       An[(size_t)qI * n + pJ] = d10;
       An[(size_t)qI * n + qJ] = d11;
     } else {
-      const long long v = o - nblk;
-      const int i = (int)(v / h), J = (int)(v % h);
+      const IX v = o - nblk;
+      const int i = (int)(v / (IX)h), J = (int)(v - (IX)i * (IX)h);
       const double c = cs[2 * J], s = cs[2 * J + 1];
       if (s != 0.0) {
         const int pJ = rr_player(J, r, n), qJ = rr_player(n - 1 - J, r, n);
@@ -339,7 +367,8 @@ __global__ void __launch_bounds__(256) k_jacobi_coop(double* A, double* B, doubl
     for (int r = 0; r < n - 1; ++r) {
       jacobi_round_params(cur, cs, n, r, c, t0, ts);
       grid.sync();
-      jacobi_round_apply(cur, nxt, V, cs, n, r, t0, ts);
+      if (n < 32768) jacobi_round_apply<unsigned>(cur, nxt, V, cs, n, r, (unsigned)t0, (unsigned)ts);
+      else jacobi_round_apply<unsigned long long>(cur, nxt, V, cs, n, r, (unsigned long long)t0, (unsigned long long)ts);
       grid.sync();
       double* t = cur; cur = nxt; nxt = t;
     }

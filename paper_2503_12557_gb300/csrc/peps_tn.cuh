@@ -720,7 +720,8 @@ __device__ void qr_keep_r(T* Z, int m, int nc, T* R, T* taus, int ldr, int kr, i
 // round r.  Every round pairs position j with position m-1-j; the pairs of one round are
 // disjoint and every pair meets once per m-1 rounds.
 __device__ __forceinline__ int rr_player(int j, int r, int m) {
-  return (j == 0) ? 0 : ((j - 1 + r) % (m - 1)) + 1;
+  const int v = j - 1 + r;  // below 2 (m - 1): r < m - 1
+  return (j == 0) ? 0 : (v >= m - 1 ? v - (m - 1) : v) + 1;
 }
 
 template <typename T> struct JacobiTol;
