@@ -1814,7 +1814,9 @@ __device__ __noinline__ Scaled env_first_row(const G g, T* Eout, const T* Tpad, 
 // one (el[b][d][z]), as far as they are not zero (mps_bonds of both): a, x of the upper one's left
 // and right bond, b, z of the lower one's.  Contractions, normalisations and copies stop there:
 // partials keep their full layouts, entries past the bonds are neither computed nor read, and what
-// is left out of a sum are exact zeros, the rest added in the same order.
+// is left out of a sum are exact zeros, the rest added in the same order.  The two intermediates t1 and
+// t2 are packed to the bonds, and t2 lies behind t1 where both fit in t1's buffer, which the plans
+// keep in shared memory longest.
 struct BondExt {
   int a, x, b, z;
 };
@@ -1830,28 +1832,30 @@ template <typename T, typename G>
 __device__ __noinline__ void absorb1(const G g, const BondExt e, const T* L, const T* eu, const T* A, const T* el, T* t1, T* t2,
                         T* out) {
   const int chi = g.chi, D = g.D;
-  const int PS = D * chi + D;  // padded (x, r) row stride of t2
   const int kb = e.b, kx = e.x;
   const FDiv fb = fdiv_of(kb), fx = fdiv_of(kx);
+  const int PS = D * kb + D;  // padded (x, r) row stride of t2
+  const int xb = kx * kb, ts = D * kx * PS;
+  if (2 * ts <= (int)sandwich1_t_elems(chi, D)) t2 = t1 + ts;
   // t1[u][l][x][b] = sum_a L[a][l][b] eu[a][u][x]        (m = (l, b), n = (u, x), k = a)
   blk_gemm<2, 4>(L, eu, t1, D * kb, D * kx, e.a, 1, D * chi, 0, D * chi, 0,
                  [=](int m) {
                    const int l = fdiv_q(m, fb), b = m - l * kb;
-                   return Off2{l * chi + b, l * chi * chi + b};
+                   return Off2{l * chi + b, l * xb + b};
                  },
                  [=](int n) {
                    const int u = fdiv_q(n, fx), x = n - u * kx;
-                   return Off2{u * chi + x, u * D * chi * chi + x * chi};
+                   return Off2{u * chi + x, u * D * xb + x * kb};
                  });
   // t2[x][r][d][b] = sum_{l,u} t1[u][l][x][b] A[l][u][r][d]   (m = (x, b), n = (r, d), k = (l, u))
-  blk_gemm<2, 4>(t1, A, t2, kx * kb, D * D, D, D, chi * chi, D * chi * chi, D * D * D, D * D,
+  blk_gemm<2, 4>(t1, A, t2, kx * kb, D * D, D, D, xb, D * xb, D * D * D, D * D,
                  [=](int m) {
                    const int x = fdiv_q(m, fb), b = m - x * kb;
-                   return Off2{x * chi + b, x * D * PS + b};
+                   return Off2{m, x * D * PS + b};
                  },
-                 [=](int n) { return Off2{n, (n / D) * PS + (n % D) * chi}; });
+                 [=](int n) { return Off2{n, (n / D) * PS + (n % D) * kb}; });
   // out[x][r][z] = sum_{b,d} el[b][d][z] t2[x][r][d][b]      (m = z, n = (x, r), k = (b, d))
-  blk_gemm<1, 4>(el, t2, out, e.z, kx * D, kb, D, D * chi, chi, 1, chi,
+  blk_gemm<1, 4>(el, t2, out, e.z, kx * D, kb, D, D * chi, chi, 1, kb,
                  [=](int m) { return Off2{m, m}; },
                  [=](int n) { return Off2{n * PS, n * chi}; });
 }
@@ -1862,25 +1866,27 @@ __device__ __noinline__ void absorb1(const G g, const BondExt e, const T* L, con
 template <typename T, typename G>
 __device__ __noinline__ void absorb1_right(const G g, const BondExt e, const T* R, const T* eu, const T* A, const T* el, T* t1,
                               T* t2, T* out) {
-  const int chi = g.chi, D = g.D, P = chi + 1;
+  const int chi = g.chi, D = g.D;
   const int ka = e.a, kz = e.z;
   const FDiv fz = fdiv_of(kz), fa = fdiv_of(ka);
+  const int P = ka + 1, zP = kz * P, ts = D * D * zP;
+  if (2 * ts <= (int)sandwich1_t_elems(chi, D)) t2 = t1 + ts;
   // t1[u][r][z][a] (rows of a padded to P) = sum_x R[x][r][z] eu[a][u][x]   (m = (r, z), n = (a, u))
   blk_gemm<2, 4>(R, eu, t1, D * kz, ka * D, e.x, 1, D * chi, 0, 1, 0,
                  [=](int m) {
                    const int r = fdiv_q(m, fz), z = m - r * kz;
-                   return Off2{r * chi + z, (r * chi + z) * P};
+                   return Off2{r * chi + z, m * P};
                  },
-                 [=](int n) { return Off2{n * chi, (n % D) * D * chi * P + n / D}; });
+                 [=](int n) { return Off2{n * chi, (n % D) * D * zP + n / D}; });
   // t2[z][d][a][l] = sum_{u,r} t1[u][r][z][a] A[l][u][r][d]   (m = (z, a), n = (l, d), k = (u, r))
-  blk_gemm<2, 4>(t1, A, t2, kz * ka, D * D, D, D, D * chi * P, chi * P, D * D, D,
+  blk_gemm<2, 4>(t1, A, t2, kz * ka, D * D, D, D, D * zP, zP, D * D, D,
                  [=](int m) {
                    const int z = fdiv_q(m, fa), a = m - z * ka;
-                   return Off2{z * P + a, z * D * chi * D + a * D};
+                   return Off2{z * P + a, z * D * ka * D + a * D};
                  },
-                 [=](int n) { return Off2{(n / D) * D * D * D + n % D, (n % D) * chi * D + n / D}; });
+                 [=](int n) { return Off2{(n / D) * D * D * D + n % D, (n % D) * ka * D + n / D}; });
   // out[a][l][b] = sum_{z,d} t2[z][d][a][l] el[b][d][z]   (m = (a, l), n = b, k = (z, d))
-  blk_gemm<2, 2>(t2, el, out, ka * D, e.b, kz, D, D * chi * D, chi * D, 1, chi,
+  blk_gemm<2, 2>(t2, el, out, ka * D, e.b, kz, D, D * ka * D, ka * D, 1, chi,
                  [=](int m) { return Off2{m, m * chi}; },
                  [=](int n) { return Off2{n * D * chi, n}; });
 }
@@ -1893,9 +1899,11 @@ template <typename T, typename G>
 __device__ __noinline__ void site_env1(const G g, const BondExt e, const T* L, const T* eu, const T* elT, const T* R, T* t1, T* t2,
                           T* env) {
   const int chi = g.chi, D = g.D;
-  const int S1 = chi * chi + chi;  // padded (u, l) row stride of t1
   const int kb = e.b, kx = e.x;
   const FDiv fb = fdiv_of(kb), fx = fdiv_of(kx);
+  const int S1 = kx * kb + kb;  // padded (u, l) row stride of t1
+  const int ts = D * D * S1;
+  if (2 * ts <= (int)sandwich1_t_elems(chi, D)) t2 = t1 + ts;
   // t1[u][l][x][b] = sum_a L[a][l][b] eu[a][u][x]   (as in absorb1, rows padded)
   blk_gemm<2, 4>(L, eu, t1, D * kb, D * kx, e.a, 1, D * chi, 0, D * chi, 0,
                  [=](int m) {
@@ -1904,15 +1912,15 @@ __device__ __noinline__ void site_env1(const G g, const BondExt e, const T* L, c
                  },
                  [=](int n) {
                    const int u = fdiv_q(n, fx), x = n - u * kx;
-                   return Off2{u * chi + x, u * D * S1 + x * chi};
+                   return Off2{u * chi + x, u * D * S1 + x * kb};
                  });
   // t4[b][x][r][d] = sum_z elT[z][b][d] R[x][r][z]   (m = (b, d), n = (x, r), k = z)
   blk_gemm<2, 4>(elT, R, t2, kb * D, kx * D, e.z, 1, chi * D, 0, 1, 0,
-                 [=](int m) { return Off2{m, (m / D) * chi * D * D + m % D}; },
+                 [=](int m) { return Off2{m, (m / D) * kx * D * D + m % D}; },
                  [=](int n) { return Off2{n * chi, n * D}; });
   // env[l][u][r][d] = sum_{b,x} t4[b][x][r][d] t1[u][l][x][b]   (m = (r, d), n = (u, l) with l
   // fastest, so that the two column groups of a warp read t1 rows one padded stride apart)
-  blk_gemm<1, 1>(t2, t1, env, D * D, D * D, kb, kx, chi * D * D, D * D, 1, chi,
+  blk_gemm<1, 1>(t2, t1, env, D * D, D * D, kb, kx, kx * D * D, D * D, 1, kb,
                  [=](int m) { return Off2{m, m}; },
                  [=](int n) { return Off2{(n / D) * D * S1 + (n % D) * S1, ((n % D) * D + n / D) * D * D}; });
 }
@@ -1994,20 +2002,21 @@ __device__ __noinline__ void absorb2(const G g, const BondExt e, const T* L2, co
   const FDiv fb = fdiv_of(kb);
   for (int x0 = 0; x0 < kx; x0 += cx) {
     const int c = (kx - x0 < cx) ? kx - x0 : cx;
-    const int cc = chi * c;
-    const FDiv fbc = fdiv_of(kb * c);
+    const int cc = kb * c, ts = D * D * D * cc;
+    const FDiv fbc = fdiv_of(cc);
+    if (2 * ts <= D * D * D * chi * cx) t2 = t1 + ts;
     // t1[i][u][j][b][xx] = sum_a L2[a][i][j][b] eu[a][u][x0+xx]      (m = (i, j, b), n = (u, xx))
     blk_gemm<2, 4>(L2, eu + x0, t1, D * D * kb, D * c, e.a, 1, D * D * chi, 0, D * chi, 0,
                    [=](int m) {
                      const int ij = fdiv_q(m, fb), b = m - ij * kb;
-                     return Off2{ij * chi + b, (ij / D) * D * D * cc + ((ij % D) * chi + b) * c};
+                     return Off2{ij * chi + b, (ij / D) * D * D * cc + ((ij % D) * kb + b) * c};
                    },
                    [=](int n) { return Off2{(n / c) * chi + n % c, (n / c) * D * cc + n % c}; });
     // t2[j][v][b][xx][r1] = sum_{i,u} t1[i][u][j][b][xx] A1[i][u][r1][v]   (m = (j, b, xx), n = (r1, v))
     blk_gemm<2, 4>(t1, A1, t2, D * kb * c, D * D, D, D, D * D * cc, D * cc, D * D * D, D * D,
                    [=](int m) {
-                     const int j = fdiv_q(m, fbc), rem = m - j * kb * c;
-                     return Off2{j * cc + rem, j * D * D * cc + rem * D};
+                     const int j = fdiv_q(m, fbc), rem = m - j * cc;
+                     return Off2{m, j * D * D * cc + rem * D};
                    },
                    [=](int n) { return Off2{n, (n % D) * cc * D + n / D}; });
     // t3[r2][d][b][xx][r1] = sum_{j,v} t2[j][v][b][xx][r1] A2[j][v][r2][d]   (into t1; m = (b, xx, r1), n = (r2, d))
@@ -2035,27 +2044,29 @@ __device__ __noinline__ void absorb2_right(const G g, const BondExt e, const T* 
   const FDiv fz = fdiv_of(kz);
   for (int a0 = 0; a0 < ka; a0 += ca) {
     const int c = (ka - a0 < ca) ? ka - a0 : ca;
-    const int cdx = c * D * chi;             // one (u, r1) block of t1, one (v, r2) block of t2
+    const int cdx = c * D * kz;              // one (u, r1) block of t1, one (v, r2) block of t2
     const int Sz = D * c * D * D + 1;        // z stride of t3 (odd: consecutive z in different banks)
+    const int ts = kz * Sz;
+    if (2 * ts <= D * D * D * chi * ca) t2 = t1 + ts;
     // t1[u][r1][aa][r2][z] = sum_x R2[x][r1][r2][z] eu[a0+aa][u][x]   (m = (r1, r2, z), n = (aa, u))
     blk_gemm<2, 4>(R2, eu + (size_t)a0 * D * chi, t1, D * D * kz, c * D, e.x, 1, D * D * chi, 0, 1, 0,
                    [=](int m) {
                      const int q = fdiv_q(m, fz), z = m - q * kz;  // q = (r1, r2)
-                     return Off2{q * chi + z, (q / D) * cdx + (q % D) * chi + z};
+                     return Off2{q * chi + z, (q / D) * cdx + (q % D) * kz + z};
                    },
-                   [=](int n) { return Off2{n * chi, (n % D) * D * cdx + (n / D) * D * chi}; });
+                   [=](int n) { return Off2{n * chi, (n % D) * D * cdx + (n / D) * D * kz}; });
     // t2[v][r2][aa][i][z] = sum_{u,r1} t1[u][r1][aa][r2][z] A1[i][u][r1][v]   (m = (aa, r2, z), n = (i, v))
     blk_gemm<2, 4>(t1, A1, t2, c * D * kz, D * D, D, D, D * cdx, cdx, D * D, D,
                    [=](int m) {
                      const int q = fdiv_q(m, fz), z = m - q * kz;  // q = (aa, r2)
-                     return Off2{q * chi + z, (q % D) * cdx + (q / D) * D * chi + z};
+                     return Off2{m, (q % D) * cdx + (q / D) * D * kz + z};
                    },
-                   [=](int n) { return Off2{(n / D) * D * D * D + n % D, (n % D) * D * cdx + (n / D) * chi}; });
+                   [=](int n) { return Off2{(n / D) * D * D * D + n % D, (n % D) * D * cdx + (n / D) * kz}; });
     // t3[z][d][aa][i][j] (z stride Sz) = sum_{v,r2} t2[v][r2][aa][i][z] A2[j][v][r2][d]   (into t1)
     blk_gemm<2, 4>(t2, A2, t1, c * D * kz, D * D, D, D, D * cdx, cdx, D * D, D,
                    [=](int m) {
                      const int q = fdiv_q(m, fz), z = m - q * kz;  // q = (aa, i)
-                     return Off2{q * chi + z, z * Sz + q * D};
+                     return Off2{m, z * Sz + q * D};
                    },
                    [=](int n) { return Off2{(n / D) * D * D * D + n % D, (n % D) * c * D * D + n / D}; });
     // out[a0+aa][i][j][b] = sum_{z,d} t3[z][d][aa][i][j] el[b][d][z]   (m = (aa, i, j), n = b)
