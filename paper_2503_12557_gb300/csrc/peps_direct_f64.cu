@@ -1,4 +1,4 @@
-// double instantiation of the direct-sampling kernels (k_dl_env, k_direct).
+// double instantiation of the direct-sampling kernels (k_dl_prod, k_dl_row, k_direct).
 #include "peps_direct.cuh"
 
 namespace peps {

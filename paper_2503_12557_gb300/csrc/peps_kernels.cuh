@@ -176,7 +176,7 @@ __host__ __device__ inline DlDims dl_dims(int D, int chid) {
   d.mX = d.nb + (d.nb & 1);
   return d;
 }
-// element counts of the global work buffers of k_dl_env, in the order B, Rh, Z, Y, X, Vt, C, Cn
+// element counts of the global work buffers of k_dl_prod and k_dl_row, in the order B, Rh, Z, Y, X, Vt, C, Cn
 __host__ __device__ inline void dl_work_elems(int Ly, int D, int chid, size_t* n8) {
   const DlDims d = dl_dims(D, chid);
   n8[0] = (size_t)Ly * d.nb * d.P * d.nb;
@@ -188,7 +188,7 @@ __host__ __device__ inline void dl_work_elems(int Ly, int D, int chid, size_t* n
   n8[6] = (size_t)d.nb * chid;
   n8[7] = (size_t)d.nb * chid;
 }
-// dynamic shared memory of k_dl_env: reduction scratch, singular values, ranks, Householder taus
+// dynamic shared memory of k_dl_row: reduction scratch, singular values, ranks, Householder taus
 __host__ __device__ inline size_t dl_smem_bytes(int D, int chid, size_t esz, size_t rsz) {
   const DlDims d = dl_dims(D, chid);
   size_t b = 40 * 8;
