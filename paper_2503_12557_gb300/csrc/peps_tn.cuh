@@ -767,7 +767,8 @@ __device__ void zero_tiny_rows(T* X, int m, int L, int ldx, typename Scal<T>::R 
 // the first sweep in which no pair had a relative dot product of sqrt(tol) or more: by the
 // quadratic convergence of cyclic Jacobi, that sweep's rotations leave dot products of order tol,
 // so the next sweep would rotate nothing.  On return the rows are sigma_i v_i^T with v_i the
-// right singular vectors of the input, and nrm[p] = sigma_p (zero for the rows set to zero).
+// right singular vectors of the input, and nrm[p] = sigma_p (zero for the rows set to zero), in FP64
+// up to one power of two for all rows (rescale_rows).
 //   Each warp treats four pairs at once (eight lanes per pair).  The squared row norms live in
 //   nrm[] (m entries): exact at the start of every sweep, and within a sweep updated after a
 //   rotation by Rutishauser's formulas a' = a - t g, b' = b + t g (g the pair's dot product), so
@@ -869,7 +870,8 @@ __device__ int hestenes_rows_smem(T* X, int m, int L, int ldx, int* flag, unsign
 __device__ __forceinline__ void jac_params(double a, double b, double c, double tol, double tiny, double stop,
                                            double& cs, double& sn, double& tc, int& big) {
   // |c| > tol sqrt(a b) as c^2 > tol^2 a b: most pairs fail it, and a square root is a dozen FP64
-  // instructions of 64 cycles each (a, b > tiny keep the squares of what matters in range)
+  // instructions of 64 cycles each (a, b > tiny keep the squares of what matters in range: the largest
+  // squared norm is within [1e-100, 1e100], see rescale_rows, and tiny is at least 1e-32 of it)
   const double ab = a * b, c2 = c * c;
   if (c2 > tol * tol * ab && a > tiny && b > tiny) {
     if (c2 >= stop * stop * ab) big = 1;
@@ -1112,6 +1114,36 @@ __device__ __noinline__ int hestenes_rows_few(T* X, int m, int L, int ldx, T tin
   return sweeps_s;
 }
 
+// X times the power of two that takes its largest modulus to 1 (X is not normalised: R multiplies the
+// site tensors of a row, so that X scales as their product).  The pair test compares c^2 with a b: with
+// the largest squared norm outside [1e-100, 1e100] those products leave the double range, the test reads
+// 0 > 0 and the sweeps would stop on rows that are not orthogonal.  Power of two, so that no mantissa
+// changes; the caller uses the singular values only relative to each other and for v = x / sigma.  Writes
+// the new squared norms to nrm and returns the largest (nmax as it was when X is zero or not finite).
+template <typename T>
+__device__ __noinline__ T rescale_rows(T* X, int m, int L, int ldx, T nmax, double* red, T* nrm) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  T am = 0;
+  for (int p = warp; p < m; p += nw)
+    for (int i = lane; i < L; i += 32) am = max_(am, abs_(X[(size_t)p * ldx + i]));
+  am = block_max(am, red);
+  if (!(am > T(0) && am < INFINITY)) return nmax;
+  const int e = -ilogb(am);
+  nmax = 0;
+  for (int p = warp; p < m; p += nw) {
+    T s = 0;
+    for (int i = lane; i < L; i += 32) {
+      const T v = scalbn(X[(size_t)p * ldx + i], e);
+      X[(size_t)p * ldx + i] = v;
+      s += v * v;
+    }
+    s = warp_sum(s);
+    nmax = fmax(nmax, s);
+    if (lane == 0) nrm[p] = s;
+  }
+  return block_max(nmax, red);
+}
+
 // S: scratch of scap elements in shared memory for the rows of hestenes_rows_few (may be empty).
 // Rows at or below the zero threshold are zero on return, or hold anything with nrm[p] = 0.
 template <typename T, int E8>
@@ -1132,6 +1164,9 @@ __device__ __noinline__ int hestenes_rows_grp(T* X, int m, int L, int ldx, int* 
     if (lane == 0) nrm[p] = s;
   }
   nmax = block_max(nmax, red);
+  if constexpr (sizeof(T) == 8) {
+    if (!(nmax >= T(1e-100) && nmax <= T(1e100))) nmax = rescale_rows(X, m, L, ldx, nmax, red, nrm);
+  }
   const T tiny = nmax * (T(L) * eps) * (T(L) * eps);
   const T stop = sqrt(tol);
   // the active rows (above the zero threshold; NaN counts); m <= 128
