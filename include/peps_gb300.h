@@ -95,7 +95,10 @@ typedef struct {
     int max_samples; /* largest Ns any later call may pass (sizes the environment store)     */
     int gram;     /* MinSR Gram matrix: 0 or 2 = FP64 accuracy (each row of Obar as seven signed
                      8-bit digits of a fixed-point number, the digit products exact on the
-                     tcgen05 tensor cores and summed in 64-bit integers); 1 = split BF16 on the
+                     tcgen05 tensor cores and summed in 64-bit integers; the error of T_ij over
+                     |Obar_i||Obar_j| is that of an FP64 multiply-add sum or less: about 1e-16 for
+                     rows of entries alike, up to 5e-15 at 2 10^4 columns where single entries
+                     outweigh the rest of their rows); 1 = split BF16 on the
                      tcgen05 tensor cores (Obar = hi + lo, T ~ hi hi^T + hi lo^T + lo hi^T, FP32
                      accumulation; about 1e-5 relative error per entry)                     */
     int solve;    /* MinSR solve when rcond == 0: 0 = FP64 Cholesky; 1 = FP32 Cholesky of

@@ -4,8 +4,8 @@
 // multiplication", 2012): GB300's FP64 pipes run at 1/64 of the FP32 rate, its BF16 tensor
 // cores at 2000 times the FP64 rate.
 //
-// Slices.  Row i of Obar is scaled by a power of two 2^-e_i (2^e_i above its largest modulus) and
-// written in fixed point with NS = 7 signed 8-bit digits,
+// Slices.  Row i of Obar is scaled by a power of two 2^-e_i, above its largest modulus and such that
+// its squared norm is below 2^8, and written in fixed point with NS = 7 signed 8-bit digits,
 //   x = 2^e_i sum_p d_p 2^(-7 - 8 p) + err,   |d_p| <= 128,   |err| <= 2^(e_i - 56),
 // each digit an integer that BF16 holds exactly.  T_ij = 2^(e_i + e_j) sum_d 2^(-14 - 8 d) v_d with
 // v_d = sum_{p + q = d} sum_k d_p(i, k) d_q(j, k); the terms with d >= NS (below 2^-56) are dropped.
@@ -14,15 +14,24 @@
 // FP32 accumulators in tensor memory ever hold is an integer below 2^24, so the products and sums
 // are exact.  After every chunk the epilogue warps read the seven v_d, turn them into integers
 // (one FP32 add of 1.5 * 2^23 puts the integer in the low mantissa bits) and add them to 64-bit
-// fixed-point sums in registers with lsb 2^-f, f chosen from the largest scaled row norm so that
-// |T_ij| 2^(f - e_i - e_j) < 2^62 by Cauchy-Schwarz.  Only the digits below that lsb round (half
-// up and half down on alternate chunks).  Integer addition is associative: the partial sums of
-// tiles that are split over several CTAs along K are added with 64-bit integer atomics and give
-// the same bits in any order.
+// fixed-point sums in registers with lsb 2^-54 of the scaled rows; |T_ij| 2^(54 - e_i - e_j) < 2^62 by
+// Cauchy-Schwarz.  Only the digits below that lsb round, once a chunk (half up and half down on alternate
+// chunks of the columns).  Integer addition is associative: the partial sums of tiles that are split
+// over several CTAs along K, or of panels of columns, are added with 64-bit integer atomics and give the
+// same bits in any order and for any split.
+//
+// Scale.  With one lsb for the whole matrix taken from the largest row norm, a row of equal entries
+// beside rows with one large entry (norms 300 times apart at 80 000 columns) left those rows' products
+// 37 bits.  Now the norms are at most 16 to 32 apart (one large entry is at least 1/2): what is lost is the
+// low end of a flat row's digits, 2^-56 of its scale.  Rows of norm 8 to 16 also keep the dropped products
+// (1e-15 at 21 632 columns for a norm of 1) below the rounding of the result.  Largest error over |a||b| of
+// 16 x 16 entries against long double at 21 632 columns, before -> now: one flat row among spiky ones
+// 2.4e-13 -> 5.1e-15, spiky rows 8.4e-15 -> 5.1e-15, Gaussian rows 0.9e-16 -> 1.2e-16, the rounding of the
+// result (an FP64 multiply-add sum in order: 8.2e-15, 8.2e-15, 1.1e-14).
 //
 // Measured on the whole MinSR step (one GB300): 4096 x 21 632 from 118.4 ms with the float-float
 // FP32 Gram (85.2 ms of it) to 44.2 ms, 1000 x 3528 from 8.28 ms with the FP64 FMA Gram (3.9 ms)
-// to 4.71 ms; dtheta against 64-bit linear algebra 3.0e-13 -> 3.0e-15 and 4.8e-15 -> 1.7e-15.
+// to 4.71 ms (the Gram matrix itself 10.9 and 0.18 ms); dtheta against 64-bit linear algebra 3.0e-13 -> 3.0e-15 and 4.8e-15 -> 1.7e-15.
 // tests/test_gpu_gram_slices.py holds the error bound against an extended-precision sum.
 #include <cuda_bf16.h>
 
@@ -32,27 +41,23 @@
 namespace peps {
 namespace {
 
-constexpr int F_MAX = 52, F_MIN = 38;        // range of f
+constexpr int FL = 54;  // fixed-point sums: lsb 2^-FL of the scaled rows (that of d = 4, 5)
+constexpr int NL = 8;   // squared norms of the scaled rows are below 2^NL: |T_ij| 2^FL < 2^62
 
-// f and the extra row exponent t (t > 0 only when the largest scaled squared row norm exceeds
-// 2^23, i.e. beyond 8 million columns) from nmax, the largest sum_k (x_k / 2^e)^2 of any row.
-struct SliceScale {
-  int f, t;
-};
-__device__ __forceinline__ SliceScale slice_scale(float nmax) {
-  int ex = 0;
-  frexpf(nmax, &ex);  // nmax < 2^ex
-  SliceScale r;
-  r.t = ex > 61 - F_MIN ? (ex - (61 - F_MIN) + 1) / 2 : 0;
-  const int f = 61 - (ex - 2 * r.t);
-  r.f = f > F_MAX ? F_MAX : f;
-  return r;
+// a += w 2^32 and a += w m, one instruction each (written as 64-bit shifts and sums the 64 sums of a
+// thread spill: 11.8 -> 15.9 ms for the Gram matrix of 4096 x 21 632)
+static_assert(FL == 54, "the weights of the digit products");
+__device__ __forceinline__ void add_high(long long& a, int w) {
+  asm("{\n .reg .b32 l, h;\n mov.b64 {l, h}, %0;\n add.s32 h, h, %1;\n mov.b64 %0, {l, h};\n}\n" : "+l"(a) : "r"(w));
+}
+__device__ __forceinline__ void mad_wide(long long& a, int w, int m) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a) : "r"(w), "r"(m));
 }
 
 // Row scales: rowE[r] = the largest biased exponent of the row (at least 1: the exponent of a
-// subnormal), or ROW_NONFINITE when an entry is Inf or NaN; *nmax (zeroed before) = an upper bound
-// of the largest scaled squared row norm.  One CTA per row; the second pass finds the row in L2.
-__global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ A, long long K, int* rowE, int* nmax) {
+// subnormal), raised until the scaled squared norm is below 2^NL, or ROW_NONFINITE when an entry is Inf
+// or NaN.  One CTA per row; the second pass finds the row in L2.
+__global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ A, long long K, int* rowE) {
   __shared__ int sE[8];
   __shared__ float sN[8];
   const unsigned long long* x = reinterpret_cast<const unsigned long long*>(A) + (size_t)blockIdx.x * K;
@@ -81,8 +86,9 @@ __global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ A
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 8; ++w) n += sN[w];
-    rowE[blockIdx.x] = e < 2047 ? e : ROW_NONFINITE;
-    if (e < 2047) atomicMax(nmax, __float_as_int(n * 1.001f + 1e-30f));
+    int ex = 0;
+    frexpf(n * 1.001f, &ex);  // the squared norm is below 2^ex (1.001: the truncated mantissas and the sum's rounding)
+    rowE[blockIdx.x] = e < 2047 ? e + (ex > NL ? (ex - NL + 1) / 2 : 0) : ROW_NONFINITE;
   }
 }
 
@@ -91,11 +97,10 @@ __global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ A
 // the doubles (the FP64 pipes would be the limit), one 16-byte store per digit.
 __global__ void __launch_bounds__(256) k_slice_digits(const double* __restrict__ A, int Ns, long long K, long long k0,
                                                       int kw, int Npad, int Kpad, const int* __restrict__ rowE,
-                                                      const int* __restrict__ nmax, __nv_bfloat16* __restrict__ D) {
+                                                      __nv_bfloat16* __restrict__ D) {
   const int nv = Kpad / 8;
   const long long total = (long long)Npad * nv;
   const size_t plane = (size_t)Npad * Kpad;
-  const int t = slice_scale(__int_as_float(*nmax)).t;
   for (long long o = blockIdx.x * 256ll + threadIdx.x; o < total; o += gridDim.x * 256ll) {
     const int r = (int)(o / nv), kb = (int)(o - (long long)r * nv) * 8;
     const int E = r < Ns ? rowE[r] : ROW_NONFINITE;
@@ -104,7 +109,7 @@ __global__ void __launch_bounds__(256) k_slice_digits(const double* __restrict__
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const unsigned long long b = (E >= 0 && kb + j < kw) ? x[j] : 0ull;
-      put_digits(fixed_point(b, E + t), j, w);
+      put_digits(fixed_point(b, E), j, w);
     }
 #pragma unroll
     for (int p = 0; p < NS; ++p)
@@ -121,9 +126,10 @@ __global__ void __launch_bounds__(256) k_slice_digits(const double* __restrict__
 //   The MMAs of a chunk take 56 x 64 = 3584 tensor cycles and its epilogue about 22 instructions
 // per element = 2800 issue cycles on the four schedulers: the tile shape balances the two, and
 // shared memory feeds both operands of a 128 x 128 x 16 MMA at its full 128 bytes per cycle.
+// cb: the chunk of the matrix's columns that the map's first one is.
 __global__ void __launch_bounds__(SL_THREADS, 1) k_gram_sl(const __grid_constant__ CUtensorMap map, int full, int ks,
-                                                           int nchunk, int Ns, const int* __restrict__ nmax,
-                                                           unsigned long long* Tm, int ld, int* err) {
+                                                           int nchunk, int cb, int Ns, unsigned long long* Tm, int ld,
+                                                           int* err) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* ring = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t full_bar[SSTAGES], empty_bar[SSTAGES], ufull[2], uempty[2];
@@ -203,15 +209,13 @@ __global__ void __launch_bounds__(SL_THREADS, 1) k_gram_sl(const __grid_constant
       }
     }
   } else {
-    const SliceScale sc = slice_scale(__int_as_float(*nmax));
-    const int m01 = 1 << (sc.f - 22), m23 = 1 << (sc.f - 38), r45 = 54 - sc.f, r6 = 62 - sc.f;
     const uint32_t tw = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (warp >> 2) * 64;
     long long acc[64];
 #pragma unroll
     for (int j = 0; j < 64; ++j) acc[j] = 0;
     bool ok = true;
     for (int c = 0; c < nc; ++c) {
-      const int h45 = (1 << (r45 - 1)) - (c & 1), h6 = (1 << (r6 - 1)) - (c & 1);
+      const int half = (1 << (61 - FL)) - ((cb + c0 + c) & 1);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const uint32_t slot = u & 1, par = (2 * c + (u >> 1)) & 1;
@@ -227,14 +231,14 @@ __global__ void __launch_bounds__(SL_THREADS, 1) k_gram_sl(const __grid_constant
           tmem_wait();
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const int a = f2i_exact(va[j]);
+            const int a = f2i_exact(va[j]);  // of weight 2^(-14 - 16 u)
             if (u < 3) {
               const int w = a * 256 + f2i_exact(vb[j]);  // |w| < 2^31
-              if (u == 0) acc[cc + j] += (long long)w * m01;
-              if (u == 1) acc[cc + j] += (long long)w * m23;
-              if (u == 2) acc[cc + j] += (w + h45) >> r45;
+              if (u == 0) add_high(acc[cc + j], w);
+              if (u == 1) mad_wide(acc[cc + j], w, 1 << (FL - 38));
+              if (u == 2) mad_wide(acc[cc + j], w, 1);
             } else {
-              acc[cc + j] += (a + h6) >> r6;
+              mad_wide(acc[cc + j], (a + half) >> (62 - FL), 1);
             }
           }
         }
@@ -262,11 +266,10 @@ __global__ void __launch_bounds__(SL_THREADS, 1) k_gram_sl(const __grid_constant
   }
 }
 
-// The fixed-point sums of the lower triangle, in place, to T_ij = sum 2^(e_i + e_j - f) in double,
+// The fixed-point sums of the lower triangle, in place, to T_ij = sum 2^(e_i + e_j - FL) in double,
 // and the upper triangle mirrored from it (32 x 32 tiles through shared memory).  Rows with a
 // non-finite entry give NaN.
-__global__ void __launch_bounds__(256) k_slice_finish(double* T, int Ns, int ld, const int* __restrict__ rowE,
-                                                      const int* __restrict__ nmax) {
+__global__ void __launch_bounds__(256) k_slice_finish(double* T, int Ns, int ld, const int* __restrict__ rowE) {
   __shared__ double tile[32][33];
   int t = blockIdx.x, bi = 0;
   bi = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
@@ -274,7 +277,6 @@ __global__ void __launch_bounds__(256) k_slice_finish(double* T, int Ns, int ld,
   while ((long long)bi * (bi + 1) / 2 > t) --bi;
   const int bj = t - (int)((long long)bi * (bi + 1) / 2);
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const SliceScale sc = slice_scale(__int_as_float(*nmax));
   const int c = bj * 32 + tx;
   const int ec = c < Ns ? rowE[c] : 0;
   for (int k = ty; k < 32; k += 8) {
@@ -282,7 +284,7 @@ __global__ void __launch_bounds__(256) k_slice_finish(double* T, int Ns, int ld,
     double v = 0.0;
     if (r < Ns && c <= r) {
       const int er = rowE[r];
-      v = scalbn((double)__double_as_longlong(T[(size_t)r * ld + c]), er + ec + 2 * sc.t - sc.f - 2044);
+      v = scalbn((double)__double_as_longlong(T[(size_t)r * ld + c]), er + ec - FL - 2044);
       if (er < 0 || ec < 0) v = __longlong_as_double(0x7ff8000000000000ll);
       T[(size_t)r * ld + c] = v;
     }
@@ -305,7 +307,7 @@ constexpr size_t SLICE_CAP = 2ull << 30;
 }  // namespace
 
 size_t gram_sl_bytes(int Ns, long long K) {
-  const size_t rows = (size_t)round_up(Ns, SM_), head = (size_t)round_up(4ll * Ns + 256, 1024);
+  const size_t rows = (size_t)round_up(Ns, SM_), head = (size_t)round_up(4ll * Ns, 1024);
   const size_t all = rows * (size_t)round_up(K > 0 ? K : 1, CK) * 2 * NS;
   const size_t least = rows * CK * 2 * NS;
   return head + (all < SLICE_CAP ? all : (SLICE_CAP > least ? SLICE_CAP : least));
@@ -316,9 +318,8 @@ cudaError_t launch_gram_sl(const double* A, int Ns, long long K, void* ws, size_
   EncodeTiled enc = get_encode();
   if (!enc) return cudaErrorNotSupported;
   const int Npad = (int)round_up(Ns, SM_);
-  const size_t head = (size_t)round_up(4ll * Ns + 256, 1024);
-  int* nmax = (int*)ws;
-  int* rowE = nmax + 64;
+  const size_t head = (size_t)round_up(4ll * Ns, 1024);
+  int* rowE = (int*)ws;
   __nv_bfloat16* D = (__nv_bfloat16*)((char*)ws + head);
   const long long fit = (long long)((ws_bytes - head) / ((size_t)Npad * 2 * NS)) / CK * CK;  // columns of a panel
   if (fit < CK) return cudaErrorInvalidValue;
@@ -326,8 +327,7 @@ cudaError_t launch_gram_sl(const double* A, int Ns, long long K, void* ws, size_
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(nmax, 0, 4, s)) != cudaSuccess) return e;
-  k_slice_rows<<<Ns, 256, 0, s>>>(A, K, rowE, nmax);
+  k_slice_rows<<<Ns, 256, 0, s>>>(A, K, rowE);
   const size_t smem = (size_t)SSTAGES * SSTAGE + 1024;
   if ((e = cudaFuncSetAttribute(k_gram_sl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
   const int nt = Npad / SM_, tiles = nt * (nt + 1) / 2;
@@ -336,7 +336,7 @@ cudaError_t launch_gram_sl(const double* A, int Ns, long long K, void* ws, size_
     const int kw = (int)(K - k0 < fit ? K - k0 : fit), Kpad = (int)round_up(kw, CK), nchunk = Kpad / CK;
     const long long vecs = (long long)Npad * (Kpad / 8);
     k_slice_digits<<<(int)(vecs / 256 < 16 * nsm ? vecs / 256 + 1 : 16 * nsm), 256, 0, s>>>(A, Ns, K, k0, kw, Npad, Kpad,
-                                                                                        rowE, nmax, D);
+                                                                                        rowE, D);
     CUtensorMap map;
     const cuuint64_t dims[3] = {(cuuint64_t)Kpad, (cuuint64_t)Npad, NS};
     const cuuint64_t strides[2] = {(cuuint64_t)Kpad * 2, (cuuint64_t)Kpad * 2 * Npad};
@@ -357,11 +357,12 @@ cudaError_t launch_gram_sl(const double* A, int Ns, long long K, void* ws, size_
         if (waves < best) { best = waves; ks = q; }
       }
     }
-    k_gram_sl<<<full + rest * ks, SL_THREADS, smem, s>>>(map, full, ks, nchunk, Ns, nmax, (unsigned long long*)Tm, ld, err);
+    k_gram_sl<<<full + rest * ks, SL_THREADS, smem, s>>>(map, full, ks, nchunk, (int)(k0 / CK), Ns,
+                                                         (unsigned long long*)Tm, ld, err);
     nl += 2;
   }
   const long long nb = (Ns + 31) / 32;
-  k_slice_finish<<<(int)(nb * (nb + 1) / 2), 256, 0, s>>>(Tm, Ns, ld, rowE, nmax);
+  k_slice_finish<<<(int)(nb * (nb + 1) / 2), 256, 0, s>>>(Tm, Ns, ld, rowE);
   *launches = nl + 1;
   return cudaGetLastError();
 }

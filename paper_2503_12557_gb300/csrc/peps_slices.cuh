@@ -20,13 +20,14 @@ constexpr int SL_THREADS = (EPI_WARPS + 2) * 32;
 constexpr int ROW_NONFINITE = -1;
 
 // Fixed-point integer (below 2^55) of the double with bits b in a row whose largest biased
-// exponent is E: x 2^(1077 - E), rounded half up in magnitude.
+// exponent is E: x 2^(1077 - E), rounded half to even (ties are half of the entries that lose one bit:
+// half up in magnitude, the diagonal of a Gram matrix came out 1e-16 too large).
 __device__ __forceinline__ long long fixed_point(unsigned long long b, int E) {
   const int ex = (int)(b >> 52) & 0x7ff;
   const int sh = E - max(ex, 1);
   unsigned long long m = (b & 0xfffffffffffffull) | (ex ? 0x10000000000000ull : 0ull);
   m <<= 2;
-  if (sh > 0) m = sh < 60 ? (m + (1ull << (sh - 1))) >> sh : 0ull;
+  if (sh > 0) m = sh < 60 ? (m + (1ull << (sh - 1)) - 1 + ((m >> sh) & 1)) >> sh : 0ull;
   return (b >> 63) ? -(long long)m : (long long)m;
 }
 // The NS signed digits of q, as BF16, into position j of eight packed per digit
