@@ -598,7 +598,7 @@ __device__ __noinline__ void row_moves(const G g, const Plan plan, const MoveBuf
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      lcur = sc_mul(logR[0], dz_abs(to_dz(RP[0])));
+      lcur = sc_amplitude(logR[0], dz_abs(to_dz(RP[0])));
       logLc = sc_one();
     }
     blk_unit(LC, cd);
@@ -691,7 +691,7 @@ __device__ __noinline__ void row_moves(const G g, const Plan plan, const MoveBuf
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      lcur = sc_mul(logR[0], dz_abs(to_dz(RP[0])));
+      lcur = sc_amplitude(logR[0], dz_abs(to_dz(RP[0])));
       logLc = sc_one();
     }
     blk_unit(LC, D2 * chi);

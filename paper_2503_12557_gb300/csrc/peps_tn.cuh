@@ -293,6 +293,10 @@ __device__ __forceinline__ Scaled sc_norm(double m, int e) {
 }
 __device__ __forceinline__ Scaled sc_mul(const Scaled& a, double f) { return sc_norm(a.m * f, a.e); }
 __device__ __forceinline__ Scaled sc_mul(const Scaled& a, const Scaled& b) { return sc_norm(a.m * b.m, a.e + b.e); }
+// |psi| = a v of a chain's configuration; NaN where v is not finite, which no proposal's u < (a / b)^2 passes
+__device__ __forceinline__ Scaled sc_amplitude(const Scaled& a, double v) {
+  return v < INFINITY ? sc_mul(a, v) : Scaled{__longlong_as_double(0x7ff8000000000000ll), 0};
+}
 // (not inlined: the environments a sampler leaves behind and those of an evaluation have to get the
 // same bits from every kernel that takes the logarithm)
 static __device__ __noinline__ double sc_log(Scaled a) {
@@ -300,7 +304,8 @@ static __device__ __noinline__ double sc_log(Scaled a) {
 }
 // a / b (inf or NaN when b is 0)
 __device__ __forceinline__ double sc_ratio(const Scaled& a, const Scaled& b) { return scalbn(a.m / b.m, a.e - b.e); }
-// u < (a / b)^2 for a finite, nonzero a (b = 0: true), without division or transcendentals
+// u < (a / b)^2 for a finite, nonzero a (b = 0: true; b NaN: false), without division or
+// transcendentals
 __device__ __forceinline__ bool sc_accept(double u, const Scaled& a, const Scaled& b) {
   if (!(a.m > 0.0)) return false;
   int k = 2 * (a.e - b.e);
