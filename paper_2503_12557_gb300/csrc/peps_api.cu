@@ -995,14 +995,27 @@ extern "C" peps_status peps_sample(peps_handle* h, int move, uint8_t* S_dev, int
 // record of the tridiagonal eigen route (about n^2 doubles, relatively more for tiny n) fits
 static size_t rec_doubles(int n) { return std::max((size_t)n * n, (size_t)4096); }
 
+// Frees the MinSR workspace; the handle then has none (a later call allocates it anew).
+static void free_minsr(peps_handle* h) {
+  h->ms_cap = 0;
+  h->ms_np = 0;
+  h->g_bytes = 0;
+  void** bufs[] = {(void**)&h->Obar, (void**)&h->Tm, (void**)&h->Vm, (void**)&h->Hm, (void**)&h->mean, (void**)&h->ebar,
+                   (void**)&h->yv, (void**)&h->xv, (void**)&h->cnt, (void**)&h->td, &h->cw, &h->g_hi, &h->g_lo};
+  for (void** b : bufs)
+    if (*b) { h_free(h, *b); *b = nullptr; }
+}
+
 // MinSR workspace for Ns rows of Np real columns (a complex handle passes its real embedding:
 // 2 Ns x 2 Np)
 static peps_status ensure_minsr(peps_handle* h, int Ns, long long Np) {
   const int n = Ns + (Ns & 1);
   if (h->ms_cap >= n && h->ms_np >= Np) return PEPS_OK;
-  double** bufs[] = {&h->Obar, &h->Tm, &h->Vm, &h->Hm, &h->mean, &h->ebar, &h->yv, &h->xv, &h->cnt, &h->td};
-  for (double** b : bufs)
-    if (*b) { h_free(h, *b); *b = nullptr; }
+  free_minsr(h);
+  auto refused = [&](const char* what) {  // what was had before is given back: no half of a workspace stays
+    free_minsr(h);
+    return fail(h, PEPS_E_WORKSPACE, what);
+  };
   const size_t nn = (size_t)n * n;
   const size_t nr = rec_doubles(n);  // V and H: also the tridiagonal route's rotation record
   // Obar holds n rows (the capacity): a later call with an even Ns up to n reuses it
@@ -1013,20 +1026,15 @@ static peps_status ensure_minsr(peps_handle* h, int Ns, long long Np) {
       h_malloc(h, (void**)&h->mean, sizeof(double) * (size_t)Np) != cudaSuccess ||
       h_malloc(h, (void**)&h->ebar, sizeof(double) * n) != cudaSuccess || h_malloc(h, (void**)&h->yv, sizeof(double) * n) != cudaSuccess ||
       h_malloc(h, (void**)&h->xv, sizeof(double) * n) != cudaSuccess || h_malloc(h, (void**)&h->cnt, sizeof(double) * 16) != cudaSuccess)
-    return fail(h, PEPS_E_WORKSPACE, "MinSR workspace allocation failed");
-  if (h->cw) { h_free(h, h->cw); h->cw = nullptr; }
-  if (h_malloc(h, &h->cw, chol64_ws_bytes(n)) != cudaSuccess)
-    return fail(h, PEPS_E_WORKSPACE, "MinSR workspace allocation failed");
-  if (h->g_hi) { h_free(h, h->g_hi); h->g_hi = nullptr; }
-  if (h->g_lo) { h_free(h, h->g_lo); h->g_lo = nullptr; }
+    return refused("MinSR workspace allocation failed");
+  if (h_malloc(h, &h->cw, chol64_ws_bytes(n)) != cudaSuccess) return refused("MinSR workspace allocation failed");
   if (h->cfg.gram == 1) {
     const size_t e = (size_t)gram_tc_pad_rows(Ns) * (size_t)gram_tc_pad_k(h->Np) * 2;
     if (h_malloc(h, (void**)&h->g_hi, e) != cudaSuccess || h_malloc(h, (void**)&h->g_lo, e) != cudaSuccess)
-      return fail(h, PEPS_E_WORKSPACE, "Gram workspace allocation failed");
+      return refused("Gram workspace allocation failed");
   } else {
     h->g_bytes = gram_sl_bytes(n, Np);  // the capacity, n rows
-    if (h_malloc(h, (void**)&h->g_hi, h->g_bytes) != cudaSuccess)
-      return fail(h, PEPS_E_WORKSPACE, "Gram workspace allocation failed");
+    if (h_malloc(h, (void**)&h->g_hi, h->g_bytes) != cudaSuccess) return refused("Gram workspace allocation failed");
   }
   h->ms_cap = n;
   h->ms_np = Np;

@@ -1,0 +1,65 @@
+"""Device memory at its limits, through the caller's allocator: refused allocations, smaller workspaces, and
+calls after a failure."""
+import ctypes as C
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2503_12557_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+class Limited:
+    """Caller's allocator over torch's that refuses what `refuse(nbytes)` says."""
+
+    def __init__(self, P, monkeypatch):
+        self.sizes, self.refuse = [], lambda n: False
+
+        def alloc(ctx, n):
+            if self.refuse(int(n)):
+                return None
+            self.sizes.append(int(n))
+            return P._torch_alloc(ctx, n)
+
+        self.ref = P._Allocator(P._ALLOC_FN(alloc), P._FREE_FN(P._torch_free), None)
+        monkeypatch.setattr(P, "_TORCH_ALLOCATOR", self.ref)
+
+
+@pytest.fixture
+def P():
+    from paper_2503_12557_gb300 import build, peps
+    build.build()
+    return peps
+
+
+def _minsr(P, h, ns, seed=3):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    O = torch.randn(ns, h.Np, generator=g, device="cuda", dtype=h.odtype)
+    e = torch.zeros(ns, 2, device="cuda", dtype=torch.float64)
+    e[:, 0] = torch.randn(ns, generator=g, device="cuda", dtype=torch.float64)
+    return h.minsr_step(O, e, lam=1e-3)[0].clone()
+
+
+@pytest.mark.parametrize("gram", [0, 1])
+def test_a_refused_growth_leaves_no_half_of_a_workspace(P, monkeypatch, gram):
+    # the larger workspace fails at its k-th allocation; the smaller call that follows allocates anew
+    lim = Limited(P, monkeypatch)
+    h = P.PEPS(4, 4, 2, 2, 4, prec=0, max_samples=1, gram=gram)
+    first = _minsr(P, h, 40)
+    for k in range(14):
+        calls = []
+
+        def nth(n):
+            calls.append(n)
+            return len(calls) == k + 1
+
+        lim.refuse = nth
+        try:
+            _minsr(P, h, 100)
+        except RuntimeError as e:
+            assert "PEPS_E_WORKSPACE" in str(e)
+        lim.refuse = lambda n: False
+        assert torch.equal(_minsr(P, h, 40), first)
+    h.close()
