@@ -1029,7 +1029,7 @@ static peps_status ensure_minsr(peps_handle* h, int Ns, long long Np) {
     return refused("MinSR workspace allocation failed");
   if (h_malloc(h, &h->cw, chol64_ws_bytes(n)) != cudaSuccess) return refused("MinSR workspace allocation failed");
   if (h->cfg.gram == 1) {
-    const size_t e = (size_t)gram_tc_pad_rows(Ns) * (size_t)gram_tc_pad_k(h->Np) * 2;
+    const size_t e = (size_t)gram_tc_pad_rows(n) * (size_t)gram_tc_pad_k(Np) * 2;
     if (h_malloc(h, (void**)&h->g_hi, e) != cudaSuccess || h_malloc(h, (void**)&h->g_lo, e) != cudaSuccess)
       return refused("Gram workspace allocation failed");
   } else {

@@ -63,3 +63,17 @@ def test_a_refused_growth_leaves_no_half_of_a_workspace(P, monkeypatch, gram):
         lim.refuse = lambda n: False
         assert torch.equal(_minsr(P, h, 40), first)
     h.close()
+
+
+def test_split_bf16_gram_of_more_columns_than_parameters(P):
+    # minsr_gram takes any K: its operands are sized for the K of the call
+    h = P.PEPS(2, 2, 2, 2, 2, max_samples=1, gram=1)
+    A = torch.randn(130, 40 * h.Np + 3, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda",
+                    dtype=torch.float64)
+    T = h.minsr_gram(A)
+    assert h.last_status() == 0
+    n = A.norm(dim=1)
+    # two BF16 parts of 8 bits each: 2^-16 of |a||b| dropped, FP32 sums of K terms
+    bound = (2.0 ** -15 + A.shape[1] * 2.0 ** -23) * n[:, None] * n[None, :]
+    assert torch.all((T - A @ A.T).abs() <= bound)
+    h.close()
