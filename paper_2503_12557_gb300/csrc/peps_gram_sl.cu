@@ -205,7 +205,8 @@ __global__ void __launch_bounds__(SL_THREADS, 1) k_gram_sl(const __grid_constant
           }
           mma_commit(&ufull[slot]);
         }
-        if (ok) mma_commit(&empty_bar[s]);
+        // (only where the loader waits for it: nothing may arrive on a barrier after the CTA has left)
+        if (ok && c + SSTAGES < nc) mma_commit(&empty_bar[s]);
       }
     }
   } else {

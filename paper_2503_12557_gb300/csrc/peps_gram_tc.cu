@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(128, 1) k_gram_tc(const __grid_constant__ CUte
   const int r0 = ti * TM, c0 = tj * TN;
   if (warp == 0 && lane == 0) {
     // TMA producer
+    int issued = 0;
     for (int kt = 0; kt < nk; ++kt) {
       const int s = kt % STAGES;
       if (kt >= STAGES && !mbar_wait(&empty_bar[s], ((kt / STAGES) - 1) & 1)) { atomicExch(&failed, 1); break; }
@@ -89,7 +90,11 @@ __global__ void __launch_bounds__(128, 1) k_gram_tc(const __grid_constant__ CUte
       tma_load_2d(st + 1 * TILE_BYTES, &map_lo, kt * TK, r0, &full_bar[s]);
       tma_load_2d(st + 2 * TILE_BYTES, &map_hi, kt * TK, c0, &full_bar[s]);
       tma_load_2d(st + 3 * TILE_BYTES, &map_lo, kt * TK, c0, &full_bar[s]);
+      issued = kt + 1;
     }
+    // the loads of the last stages have landed before the CTA may leave (bounded)
+    for (int kt = issued > STAGES ? issued - STAGES : 0; kt < issued; ++kt)
+      for (int i = 0; i < (1 << 16) && !mbar_try(&full_bar[kt % STAGES], (kt / STAGES) & 1); ++i) {}
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
     for (int kt = 0; kt < nk; ++kt) {
@@ -107,7 +112,8 @@ __global__ void __launch_bounds__(128, 1) k_gram_tc(const __grid_constant__ CUte
         mma_bf16(tmem, ahi + off, blo + off, 1u);
         mma_bf16(tmem, alo + off, bhi + off, 1u);
       }
-      mma_commit(&empty_bar[s]);
+      // (only where the loader waits for it: nothing may arrive on a barrier after the CTA has left)
+      if (kt + STAGES < nk) mma_commit(&empty_bar[s]);
     }
     mma_commit(&done_bar);
   }
