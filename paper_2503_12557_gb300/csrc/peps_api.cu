@@ -347,7 +347,8 @@ static peps_status finish_plans(peps_handle* h) {
   cudaError_t e = cudaSuccess;
   {
     std::lock_guard<std::mutex> lk(g_attr_mu);
-    const int variant = (h->g.chi == 16 && h->g.D == 4) ? 1 : (h->g.chi == 24 && h->g.D == 4) ? 2 : 0;
+    // (complex handles run the runtime-shape kernels whatever their shape)
+    const int variant = h->cfg.cplx ? 0 : (h->g.chi == 16 && h->g.D == 4) ? 1 : (h->g.chi == 24 && h->g.D == 4) ? 2 : 0;
     int dev = 0;
     cudaGetDevice(&dev);
     size_t& cur = g_attr_max[{h->elem * 64 + dev, variant}];  // per kernel scalar type
