@@ -424,12 +424,12 @@ peps_status peps_sample_learned(peps_handle* h, int C, int wprec, const void* w_
  * device-memory budget fixed before this library is used).  This entry point has no
  * counterpart in the paper; it exists for those callers only.
  *   It needs no handle and calls no allocation routine: every intermediate lives in one
- *   32 MiB device array that the library reserves on every GPU it is loaded on until the
+ *   device array of 32 MiB and 32 KiB that the library reserves on every GPU it is loaded on until the
  *   process exits.  cfg gives the lattice, chi and precision (max_samples is ignored);
  *   theta_dev: N_p doubles; S_dev: Ns x (Lx*Ly) uint8; logabs_dev, phase_dev: Ns doubles;
  *   status_dev: Ns int32 or NULL.  All device memory owned by the caller.
  *   Returns PEPS_E_CAPACITY, before any launch, when the parameters, environments and one CTA's
- *   work buffers of this lattice and Ns do not fit in the 32 MiB (about 8 KiB per sample at
+ *   work buffers of this lattice and Ns do not fit in the array (about 8 KiB per sample at
  *   4x4, D=2, chi=4 in FP64; larger problems need a handle).  Where two CTAs per SM do not fit,
  *   fewer CTAs share the samples: the same results, less concurrency.
  *   Every call made outside a stream capture looks up the array's device address with the

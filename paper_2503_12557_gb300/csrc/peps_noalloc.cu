@@ -6,7 +6,7 @@
 // down, or code in a process whose device memory budget is fixed up front.  For them this
 // entry point keeps every intermediate (padded parameter copy, boundary-MPS environments,
 // per-CTA work buffers, per-sample bookkeeping) in one file-scope device array of
-// kNoAllocBytes (32 MiB) that the library reserves on every GPU it is loaded on, for the life
+// kNoAllocBytes (32 MiB and 32 KiB) that the library reserves on every GPU it is loaded on, for the life
 // of the process.  The caller passes only its inputs and outputs.
 //
 // Every call made outside a stream capture looks up that device's address of the array (with
@@ -24,7 +24,8 @@
 
 namespace {
 
-constexpr size_t kNoAllocBytes = 32ull << 20;
+// (the 32 KiB are one CTA's row-step scratch, env_zs_elems: what fitted without it still does)
+constexpr size_t kNoAllocBytes = (32ull << 20) + (32ull << 10);
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 constexpr int kMaxDevices = 64;

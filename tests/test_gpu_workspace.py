@@ -77,3 +77,20 @@ def test_split_bf16_gram_of_more_columns_than_parameters(P):
     bound = (2.0 ** -15 + A.shape[1] * 2.0 ** -23) * n[:, None] * n[None, :]
     assert torch.all((T - A @ A.T).abs() <= bound)
     h.close()
+
+
+def test_noalloc_takes_what_fits_32_mib_without_the_scratch():
+    # 536 samples of 4x4, D = 3, chi = 9 in FP64: parameters, environments and one CTA's buffers apart
+    # from the row step's scratch are within 32 MiB
+    from test_zz_no_alloc import _call, _noalloc_fn
+    peps, f = _noalloc_fn()
+    lat = I.Lattice(4, 4, 2, 3)
+    theta = torch.as_tensor(I.peps_random(lat, 1, scale=0.5, bias=1.0)).cuda()
+    S = torch.as_tensor(I.configs_uniform_sz0(lat, 536, 2)).cuda()
+    rc, la, _, st = _call(peps, f, lat, 9, 0, theta, S)
+    assert rc == 0
+    h = peps.PEPS(4, 4, 2, 3, 9, prec=0, max_samples=536)
+    h.set_params(theta)
+    ref = h.amplitudes(S)
+    assert float((la - ref[0]).abs().max()) <= 1e-10
+    h.close()
