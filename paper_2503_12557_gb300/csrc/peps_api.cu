@@ -80,7 +80,7 @@ struct peps_handle {
   long long ms_np = 0;
   double *Obar = nullptr, *Tm = nullptr, *Vm = nullptr, *Hm = nullptr, *mean = nullptr, *ebar = nullptr,
          *yv = nullptr, *xv = nullptr, *cnt = nullptr;
-  void* cw = nullptr;    // FP64 Cholesky: digits, inverted diagonal blocks (chol64_ws_bytes)
+  void* cw = nullptr;    // FP64 Cholesky: digits, inverted diagonal blocks (chol64_ws_bytes); NULL: in Hm
   double* td = nullptr;  // tridiagonal eigen route: vectors and partial sums (td_workspace_doubles)
   // timing: event pairs per kernel class, recorded on the call's stream when enabled
   bool timing = false;
@@ -92,7 +92,7 @@ struct peps_handle {
   // learned-proposal workspace (allocated on first use)
   uint8_t* lp_Sp = nullptr;
   double *lp_l0 = nullptr, *lp_l1 = nullptr, *lp_aux = nullptr;
-  // operands of the tensor-core Gram: split BF16 (gram = 1), or the digits (g_hi, g_bytes)
+  // operands of the tensor-core Gram: split BF16 (gram = 1), or the digits (g_hi, g_bytes; NULL: in Hm)
   void *g_hi = nullptr, *g_lo = nullptr;
   size_t g_bytes = 0;
   // status word (device): OR of the per-sample status bits and the MinSR flags since the last
@@ -106,7 +106,11 @@ struct peps_handle {
 
 static cudaError_t h_malloc(peps_handle* h, void** p, size_t bytes) {
   *p = nullptr;
-  if (!h->has_alloc) return cudaMalloc(p, bytes);
+  if (!h->has_alloc) {
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();  // (a smaller request may follow: no launch may report this one)
+    return e;
+  }
   void* q = h->alloc.alloc(h->alloc.ctx, bytes ? bytes : 1);
   if (!q) return cudaErrorMemoryAllocation;
   *p = q;
@@ -996,6 +1000,10 @@ extern "C" peps_status peps_sample(peps_handle* h, int move, uint8_t* S_dev, int
 // record of the tridiagonal eigen route (about n^2 doubles, relatively more for tiny n) fits
 static size_t rec_doubles(int n) { return std::max((size_t)n * n, (size_t)4096); }
 
+// bytes at the start of Hm that the solves use: the residual norms' partial sums and one vector
+static size_t hm_head(int n) { return al(2 * sizeof(double) * (size_t)n); }
+static void* chol_ws(peps_handle* h, int n) { return h->cw ? h->cw : (char*)h->Hm + hm_head(n); }
+
 // Frees the MinSR workspace; the handle then has none (a later call allocates it anew).
 static void free_minsr(peps_handle* h) {
   h->ms_cap = 0;
@@ -1028,14 +1036,24 @@ static peps_status ensure_minsr(peps_handle* h, int Ns, long long Np) {
       h_malloc(h, (void**)&h->ebar, sizeof(double) * n) != cudaSuccess || h_malloc(h, (void**)&h->yv, sizeof(double) * n) != cudaSuccess ||
       h_malloc(h, (void**)&h->xv, sizeof(double) * n) != cudaSuccess || h_malloc(h, (void**)&h->cnt, sizeof(double) * 16) != cudaSuccess)
     return refused("MinSR workspace allocation failed");
-  if (h_malloc(h, &h->cw, chol64_ws_bytes(n)) != cudaSuccess) return refused("MinSR workspace allocation failed");
+  // where the factor's workspace or the digits are refused they are in Hm, which neither the Gram nor
+  // the solve needs whole: up to 85 to 180 rows Hm is too small (255 KB is then the most that is needed)
+  const size_t hm = nr * sizeof(double);
+  if (h_malloc(h, &h->cw, chol64_ws_bytes(n)) != cudaSuccess && hm_head(n) + chol64_ws_bytes(n) > hm)
+    return refused("MinSR workspace allocation failed");
   if (h->cfg.gram == 1) {
     const size_t e = (size_t)gram_tc_pad_rows(n) * (size_t)gram_tc_pad_k(Np) * 2;
     if (h_malloc(h, (void**)&h->g_hi, e) != cudaSuccess || h_malloc(h, (void**)&h->g_lo, e) != cudaSuccess)
       return refused("Gram workspace allocation failed");
   } else {
     h->g_bytes = gram_sl_bytes(n, Np);  // the capacity, n rows
-    if (h_malloc(h, (void**)&h->g_hi, h->g_bytes) != cudaSuccess) return refused("Gram workspace allocation failed");
+    if (h_malloc(h, (void**)&h->g_hi, h->g_bytes) != cudaSuccess) {
+      h->g_bytes = hm;  // (fewer columns of digits at a time; the same sums)
+      if (gram_sl_bytes(n, 1) > hm) {
+        h->g_bytes = gram_sl_bytes(n, 1);
+        if (h_malloc(h, (void**)&h->g_hi, h->g_bytes) != cudaSuccess) return refused("Gram workspace allocation failed");
+      }
+    }
   }
   h->ms_cap = n;
   h->ms_np = Np;
@@ -1056,7 +1074,7 @@ static peps_status minsr_gram_into(peps_handle* h, const double* A, int Ns, long
     tstop(h, ts, s, mirror ? 3 : 2);
   } else {
     long long nl = 0;
-    CK(launch_gram_sl(A, Ns, K, h->g_hi, h->g_bytes, T, ld, gerr, s, &nl), "Gram");
+    CK(launch_gram_sl(A, Ns, K, h->g_hi ? h->g_hi : (void*)h->Hm, h->g_bytes, T, ld, gerr, s, &nl), "Gram");
     tstop(h, ts, s, nl);
   }
   return PEPS_OK;
@@ -1103,13 +1121,13 @@ static peps_status minsr_solve_core(peps_handle* h, int Ns, double lambda, doubl
         nl = 1 + chol_solve_mixed(h->Tm, (float*)h->Vm, n, Ns, lambda, h->ebar, h->xv, h->yv, h->cnt + 6, h->Hm, 4,
                                   (int*)h->cnt, info_dev, need64, h->Hm + n, s, &e);
         if (e != cudaSuccess) return cuda_fail(h, e, "Cholesky");
-        nl += chol_solve(h->Tm, n, Ns, lambda, h->ebar, h->xv, (int*)h->cnt, info_dev, need64, h->yv, h->cw, s, &e);
+        nl += chol_solve(h->Tm, n, Ns, lambda, h->ebar, h->xv, (int*)h->cnt, info_dev, need64, h->yv, chol_ws(h, n), s, &e);
       } else {
         nl = 1 + chol_solve_refined(h->Tm, h->Vm, n, Ns, lambda, h->ebar, h->xv, h->yv, h->cnt + 6, h->Hm, 2,
-                                    (int*)h->cnt, info_dev, h->Hm + n, h->cw, s, &e);
+                                    (int*)h->cnt, info_dev, h->Hm + n, chol_ws(h, n), s, &e);
       }
     } else {
-      nl = chol_solve(h->Tm, n, Ns, lambda, h->ebar, h->xv, (int*)h->cnt, info_dev, nullptr, h->yv, h->cw, s, &e);
+      nl = chol_solve(h->Tm, n, Ns, lambda, h->ebar, h->xv, (int*)h->cnt, info_dev, nullptr, h->yv, chol_ws(h, n), s, &e);
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "Cholesky");
     tstop(h, ts, s, nl);

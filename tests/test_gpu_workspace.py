@@ -94,3 +94,24 @@ def test_noalloc_takes_what_fits_32_mib_without_the_scratch():
     ref = h.amplitudes(S)
     assert float((la - ref[0]).abs().max()) <= 1e-10
     h.close()
+
+
+@pytest.mark.parametrize("gram,solve,prec", [(0, 0, 0), (2, 2, 1), (0, 1, 1)])
+def test_minsr_without_the_digit_and_factor_workspaces(P, monkeypatch, gram, solve, prec):
+    # 600 rows: where neither workspace can be had, the n x n buffers that the solve leaves free hold them
+    ns = 600
+    n, K = ns, I.num_params(I.Lattice(6, 6, 2, 3))
+    up = lambda x, a: (x + a - 1) // a * a  # noqa: E731
+    digits = up(4 * n, 1024) + up(n, 128) * up(K, 32) * 14
+    factor = up(14 * n * 64, 256) + (n + 63) // 64 * 64 * 65 * 8 + 4 * n + 256
+    lim = Limited(P, monkeypatch)
+    h = P.PEPS(6, 6, 2, 3, 9, prec=prec, max_samples=1, gram=gram, solve=solve)
+    full = _minsr(P, h, ns)
+    assert digits in lim.sizes and factor in lim.sizes
+    rest = set(lim.sizes) - {digits, factor}
+    h.close()
+    lim.refuse = lambda b: b not in rest
+    h = P.PEPS(6, 6, 2, 3, 9, prec=prec, max_samples=1, gram=gram, solve=solve)
+    d = _minsr(P, h, ns)
+    h.close()
+    assert torch.equal(d, full)
