@@ -37,7 +37,8 @@ struct peps_handle {
   double* pairout = nullptr;
   int* status_tmp = nullptr;
   char* gscratch = nullptr;
-  size_t gscratch_bytes = 0;
+  size_t gscratch_bytes = 0, gscratch_asked = 0;
+  bool plans_ok = false;  // the plans point into gscratch and their grids fit it
   KPlan kp[4];  // env, row, pair, sample
   KPlan kb;     // variational-bound estimator (row-step buffers of the env budget)
   double* bout = nullptr;  // k_bound's per-(sample, term) sums
@@ -51,7 +52,7 @@ struct peps_handle {
   int* dl_status = nullptr;
   KPlan kd;
   char* dscratch = nullptr;
-  size_t dscratch_bytes = 0;
+  size_t dscratch_bytes = 0, dscratch_asked = 0;
   // reuse of the sampler's upper environments by the next evaluation (opt-in): the last
   // sampled batch (pointer, size, parameter generation) and the upper row steps' status bits
   int env_reuse = 0;
@@ -345,7 +346,30 @@ static void plan_all(peps_handle* h, bool split = true) {
 static std::mutex g_attr_mu;
 static std::map<std::pair<int, int>, size_t> g_attr_max;
 
+// An arena of at least `want` bytes in *p (*have bytes): where it is refused, half, a quarter, .. of it, down
+// to `least`.  *asked: the most that was asked for (not asked for again while what was had will do).  False,
+// and no arena, when even `least` is refused.
+static bool grow_arena(peps_handle* h, char** p, size_t* have, size_t* asked, size_t want, size_t least) {
+  if (want <= *have || (want <= *asked && least <= *have)) return true;
+  *asked = want;
+  if (*p) h_free(h, *p);
+  *p = nullptr;
+  *have = 0;
+  for (;; want = std::max(want / 2, least)) {
+    if (h_malloc(h, (void**)p, want) == cudaSuccess) {
+      *have = want;
+      return true;
+    }
+    if (want <= least) return false;
+  }
+}
+// as many CTAs as an arena has slices for: they share the samples, with the same results
+static void cap_grid(KPlan& k, size_t arena) {
+  if (k.p.gstride > 0) k.grid = (int)std::min<size_t>(k.grid, arena / k.p.gstride);
+}
+
 static peps_status finish_plans(peps_handle* h) {
+  h->plans_ok = false;  // (until every plan points into an arena that holds it)
   size_t maxsmem = h->kb.smem;
   for (auto& k : h->kp) maxsmem = std::max(maxsmem, k.smem);
   cudaError_t e = cudaSuccess;
@@ -362,13 +386,14 @@ static peps_status finish_plans(peps_handle* h) {
     }
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaFuncSetAttribute");
-  size_t gmax = 0;
+  size_t gmax = 0, gmin = 0;  // of the arena: a slice for every CTA, for one CTA
   for (int i = 0; i < 4; ++i) {
     KPlan& k = h->kp[i];
     int occ = dispatch_elem(h, [&](auto z) { return occupancy<decltype(z)>(h->g, i, k.smem); });
     if (occ < 1) return fail(h, PEPS_E_SHAPE, "kernel does not fit on an SM");
     k.grid = h->nsm * occ;
     gmax = std::max(gmax, (size_t)k.grid * (size_t)k.p.gstride);
+    gmin = std::max(gmin, (size_t)k.p.gstride);
   }
   {
     KPlan& k = h->kb;
@@ -376,15 +401,11 @@ static peps_status finish_plans(peps_handle* h) {
     if (occ < 1) return fail(h, PEPS_E_SHAPE, "bound kernel does not fit on an SM");
     k.grid = h->nsm * occ;
     gmax = std::max(gmax, (size_t)k.grid * (size_t)k.p.gstride);
+    gmin = std::max(gmin, (size_t)k.p.gstride);
   }
-  if (gmax > h->gscratch_bytes) {
-    if (h->gscratch) h_free(h, h->gscratch);
-    h->gscratch = nullptr;
-    h->gscratch_bytes = 0;
-    e = h_malloc(h, (void**)&h->gscratch, gmax);
-    if (e != cudaSuccess) return fail(h, PEPS_E_WORKSPACE, "scratch allocation failed");
-    h->gscratch_bytes = gmax;
-  }
+  if (!grow_arena(h, &h->gscratch, &h->gscratch_bytes, &h->gscratch_asked, gmax, gmin)) return fail(h, PEPS_E_WORKSPACE, "scratch allocation failed");
+  for (auto& k : h->kp) cap_grid(k, h->gscratch_bytes);
+  cap_grid(h->kb, h->gscratch_bytes);
   if (!h->ctr) {
     if (h_malloc(h, (void**)&h->ctr, 8 * sizeof(unsigned long long)) != cudaSuccess)
       return fail(h, PEPS_E_WORKSPACE, "counter allocation failed");
@@ -396,6 +417,7 @@ static peps_status finish_plans(peps_handle* h) {
   }
   h->kb.p.gbase = h->gscratch;
   h->kb.p.ctr = h->ctr;
+  h->plans_ok = true;
   return PEPS_OK;
 }
 
@@ -719,6 +741,7 @@ static peps_status check_eval(peps_handle* h, const uint8_t* S, int Ns) {
   if (!h) return PEPS_E_ARG;
   if (Ns < 0 || (Ns > 0 && !S)) return fail(h, PEPS_E_ARG, "bad configuration batch");
   if (Ns > h->cfg.max_samples) return fail(h, PEPS_E_SHAPE, "Ns exceeds max_samples");
+  if (!h->plans_ok) return fail(h, PEPS_E_WORKSPACE, "no scratch arena");
   return PEPS_OK;
 }
 
@@ -762,6 +785,7 @@ extern "C" peps_status peps_direct_prepare(peps_handle* h, int chi_double, void*
   const Geo& g = h->g;
   const int D = g.D, Ly = g.Ly, Lx = g.Lx;
   if (chi_double < 1 || chi_double * D * D > 1024) return fail(h, PEPS_E_ARG, "chi_double outside 1 .. 1024 / D^2");
+  h->dl_chid = 0;  // (peps_direct_sample refuses until this call has succeeded)
   cudaStream_t s = (cudaStream_t)stream;
   const size_t E = h->esz;
   const DlDims dd = dl_dims(D, chi_double);
@@ -820,14 +844,9 @@ extern "C" peps_status peps_direct_prepare(peps_handle* h, int chi_double, void*
   e = dispatch_elem(h, [&](auto z) { return kattr_direct<decltype(z)>(g, 0, &occ, k.smem); });
   if (e != cudaSuccess || occ < 1) return fail(h, PEPS_E_SHAPE, "direct-sampling kernel does not fit on an SM");
   k.grid = h->nsm * occ;
-  const size_t ab = (size_t)k.grid * k.p.gstride;
-  if (ab > h->dscratch_bytes) {
-    if (h->dscratch) h_free(h, h->dscratch);
-    h->dscratch = nullptr;
-    h->dscratch_bytes = 0;
-    if (h_malloc(h, (void**)&h->dscratch, ab) != cudaSuccess) return fail(h, PEPS_E_WORKSPACE, "direct-sampling arena");
-    h->dscratch_bytes = ab;
-  }
+  if (!grow_arena(h, &h->dscratch, &h->dscratch_bytes, &h->dscratch_asked, (size_t)k.grid * k.p.gstride, (size_t)k.p.gstride))
+    return fail(h, PEPS_E_WORKSPACE, "direct-sampling arena");
+  cap_grid(k, h->dscratch_bytes);
   k.p.gbase = h->dscratch;
   k.p.ctr = h->ctr;
   h->dl_chid = chi_double;

@@ -115,3 +115,54 @@ def test_minsr_without_the_digit_and_factor_workspaces(P, monkeypatch, gram, sol
     d = _minsr(P, h, ns)
     h.close()
     assert torch.equal(d, full)
+
+
+def test_a_smaller_scratch_arena_gives_the_same_results(P, monkeypatch):
+    lat = I.Lattice(6, 6, 2, 4)
+    theta = torch.as_tensor(I.peps_random(lat, 1, scale=0.5, bias=1.0, alpha=1.5)).cuda()
+    S = torch.as_tensor(I.configs_uniform_sz0(lat, 600, 2)).cuda()
+    H = I.heisenberg(lat)
+    store = 600 * 2 * 36 * 24 * 4 * 24 * 4
+    lim = Limited(P, monkeypatch)
+    h = P.PEPS(6, 6, 2, 4, 24, prec=1, max_samples=600)
+    h.set_params(theta)
+    full = h.evaluate(H, S)
+    a = h.sample(S.clone(), P.MOVE_EXCHANGE, 1, seed=3, sweep0=0)[0].clone()
+    h.close()
+    arena = max(n for n in lim.sizes if n != store)
+    lim.refuse = lambda n: n > arena // 3 and n != store
+    h = P.PEPS(6, 6, 2, 4, 24, prec=1, max_samples=600)
+    h.set_params(theta)
+    r = h.evaluate(H, S)
+    for k in ("logabs", "eloc", "O"):
+        assert torch.equal(r[k], full[k])
+    assert torch.equal(h.sample(S.clone(), P.MOVE_EXCHANGE, 1, seed=3, sweep0=0)[0], a)
+    h.close()
+
+
+def test_direct_sampling_after_a_refused_prepare(P, monkeypatch):
+    lat = I.Lattice(4, 4, 2, 2)
+    theta = torch.as_tensor(I.peps_random(lat, 1, scale=0.5, bias=1.0)).cuda()
+    lim = Limited(P, monkeypatch)
+    for k in range(4):
+        h = P.PEPS(4, 4, 2, 2, 4, prec=0, max_samples=8)
+        h.set_params(theta)
+        h.direct_prepare(2)
+        first = h.direct_sample(8, seed=1)[0].clone()
+        calls = []
+
+        def from_kth(n):
+            calls.append(n)
+            return len(calls) > k
+
+        lim.refuse = from_kth
+        try:
+            h.direct_prepare(8)
+        except RuntimeError as e:
+            assert "PEPS_E_WORKSPACE" in str(e)
+            with pytest.raises(RuntimeError, match="PEPS_E_ARG"):
+                h.direct_sample(8, seed=1)
+        lim.refuse = lambda n: False
+        h.direct_prepare(2)
+        assert torch.equal(h.direct_sample(8, seed=1)[0], first)
+        h.close()
