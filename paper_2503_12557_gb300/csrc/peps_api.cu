@@ -226,15 +226,29 @@ static void place_overlay(Plan& p, size_t& smem, size_t budget, const std::vecto
   p.gstride = gl;
 }
 
+// Product bond D min(chi, D^(Ly/2)) of the row step where a state fills its bonds.
+static int full_bond(const Geo& g) {
+  long long b = 1;
+  for (int k = 0; k < g.Ly / 2 && b < g.chi; ++k) b *= g.D;
+  return g.D * (int)std::min<long long>(b, g.chi);
+}
 // Default shared-memory budget per CTA of 256 threads and kernel class (0 env, 1 row, 2 pair, 3
 // sampler); what does not fit is in the L2-resident arena.  FP64: one CTA of 256 threads per SM (the
 // FP64 pipe is the limit; smaller CTAs share the SM's memory); FP32 three CTAs per SM (72 KB each) for
 // the environment, one-row and sampler kernels (the sampler's moves and row steps run as separate
 // launches in FP32), two for the two-row kernel; complex FP32 two for every kernel.
+//   Shared memory is taken from the L1 cache that the arena is read through: the kernels that run the row
+// step take less where its matrices outgrow the scratch and are in the arena.  Measured, one GB300, states
+// that fill their bonds: environments (FP32), 72 -> 36 KB: 4x4, D = 8, chi = 32, 40 samples 15.5 -> 7.0 ms,
+// 6x6, D = 4, chi = 32, 152 samples 8.0 -> 5.9 (8x8, chi = 16 and 24: 13.5 -> 13.7 and 32.5 -> 32.1, and
+// 2.59 -> 2.71 where the bonds are small).
 static size_t default_budget(const peps_handle* h, int cls) {
   const bool f64 = h->cfg.prec == PEPS_PREC_FP64;
   if (f64) return (210 * 1024) / (NTHREADS / cta_threads(8, h->g.n, 1));
-  return (cls == 2 || h->cfg.cplx) ? 110 * 1024 : 72 * 1024;
+  const int nb = full_bond(h->g);
+  if (h->cfg.cplx) return 110 * 1024;
+  if (cls == 0 && nb > 96) return 36 * 1024;
+  return cls == 2 ? 110 * 1024 : 72 * 1024;
 }
 // Parts a budget is shared in: FP32 beyond n = 16, where the handle's batch gives more than three items
 // per SM, two CTAs of half the size and threads (cta_threads), the moves of more than six chains per SM
