@@ -241,12 +241,13 @@ static int full_bond(const Geo& g) {
 // step take less where its matrices outgrow the scratch and are in the arena.  Measured, one GB300, states
 // that fill their bonds: environments (FP32), 72 -> 36 KB: 4x4, D = 8, chi = 32, 40 samples 15.5 -> 7.0 ms,
 // 6x6, D = 4, chi = 32, 152 samples 8.0 -> 5.9 (8x8, chi = 16 and 24: 13.5 -> 13.7 and 32.5 -> 32.1, and
-// 2.59 -> 2.71 where the bonds are small).
+// 2.59 -> 2.71 where the bonds are small); complex FP32 chains, 110 -> 72 KB: 5x5, D = 4, chi = 16, 304
+// chains 27.2 -> 11.4 ms, chi = 10 9.5 -> 7.2 (D = 3, chi = 9, whose matrices fit, 608 chains 6.06 -> 6.94).
 static size_t default_budget(const peps_handle* h, int cls) {
   const bool f64 = h->cfg.prec == PEPS_PREC_FP64;
   if (f64) return (210 * 1024) / (NTHREADS / cta_threads(8, h->g.n, 1));
   const int nb = full_bond(h->g);
-  if (h->cfg.cplx) return 110 * 1024;
+  if (h->cfg.cplx) return cls == 3 && nb * h->g.D * nb > env_zs_elems(h->g.chi, h->g.D) ? 72 * 1024 : 110 * 1024;
   if (cls == 0 && nb > 96) return 36 * 1024;
   return cls == 2 ? 110 * 1024 : 72 * 1024;
 }
