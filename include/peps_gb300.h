@@ -442,8 +442,11 @@ peps_status peps_amplitudes_noalloc(const peps_config* cfg, const double* theta_
 
 /* Autotuner (no counterpart in the paper).  For each kernel class (environments, one-row
  * sandwiches, two-row sandwiches, sampler) the shared-memory budget per CTA decides which work
- * buffers stay on chip and how many CTAs share an SM.  The call plans every candidate budget
- * (FP32: 72, 110, 220 KB; FP64: 100, 210 KB), runs peps_evaluate (with H when non-NULL) and
+ * buffers stay on chip and how many CTAs share an SM.  A budget is that of a CTA of 256 threads;
+ * where smaller CTAs take its place they share it (FP64: two for chi D <= 32, four for chi D <=
+ * 16; FP32 beyond chi D = 16: two, or four for the sampler's moves, on a handle for more than
+ * three, or six, samples per SM).  The call plans every candidate budget
+ * (FP32: 72, 110, 220 KB; FP64 and complex: 100, 210 KB; and the default), runs peps_evaluate (with H when non-NULL) and
  * one sampler sweep of kind `move` on a copy of S_dev, times each class with CUDA events and
  * keeps the fastest budget per class for all later calls.  Results do not depend on the budget
  * (same arithmetic in the same order).  budget_kb_host: 4 ints written (may be NULL).  Allocates

@@ -234,7 +234,7 @@ static int full_bond(const Geo& g) {
 }
 // Default shared-memory budget per CTA of 256 threads and kernel class (0 env, 1 row, 2 pair, 3
 // sampler); what does not fit is in the L2-resident arena.  FP64: one CTA of 256 threads per SM (the
-// FP64 pipe is the limit; smaller CTAs share the SM's memory); FP32 three CTAs per SM (72 KB each) for
+// FP64 pipe is the limit); FP32 three CTAs per SM (72 KB each) for
 // the environment, one-row and sampler kernels (the sampler's moves and row steps run as separate
 // launches in FP32), two for the two-row kernel; complex FP32 two for every kernel.
 //   Shared memory is taken from the L1 cache that the arena is read through: the kernels that run the row
@@ -244,20 +244,20 @@ static int full_bond(const Geo& g) {
 // 2.59 -> 2.71 where the bonds are small); complex FP32 chains, 110 -> 72 KB: 5x5, D = 4, chi = 16, 304
 // chains 27.2 -> 11.4 ms, chi = 10 9.5 -> 7.2 (D = 3, chi = 9, whose matrices fit, 608 chains 6.06 -> 6.94).
 static size_t default_budget(const peps_handle* h, int cls) {
-  const bool f64 = h->cfg.prec == PEPS_PREC_FP64;
-  if (f64) return (210 * 1024) / (NTHREADS / cta_threads(8, h->g.n, 1));
+  if (h->cfg.prec == PEPS_PREC_FP64) return 210 * 1024;
   const int nb = full_bond(h->g);
   if (h->cfg.cplx) return cls == 3 && nb * h->g.D * nb > env_zs_elems(h->g.chi, h->g.D) ? 72 * 1024 : 110 * 1024;
   if (cls == 0 && nb > 96) return 36 * 1024;
   return cls == 2 ? 110 * 1024 : 72 * 1024;
 }
-// Parts a budget is shared in: FP32 beyond n = 16, where the handle's batch gives more than three items
-// per SM, two CTAs of half the size and threads (cta_threads), the moves of more than six chains per SM
-// four of a quarter.
+// Parts a budget is shared in.  FP64: the CTAs of fewer threads that take the place of one (cta_threads).
+// FP32 beyond n = 16, where the handle's batch gives more than three items per SM: two CTAs of half the
+// size and threads, the moves of more than six chains per SM four of a quarter.
 static size_t budget_parts(const peps_handle* h, int cls) {
+  if (h->cfg.prec == PEPS_PREC_FP64) return NTHREADS / cta_threads(8, h->g.n, 1);
   const long long per[4] = {2, h->g.Lx, h->g.Lx - 1, 1};
   const long long items = (long long)h->cfg.max_samples * per[cls];
-  if (h->cfg.prec == PEPS_PREC_FP64 || h->g.n <= 16 || items <= 3 * N_SM) return 1;
+  if (h->g.n <= 16 || items <= 3 * N_SM) return 1;
   return cls == 3 && !h->cfg.cplx && items > 6 * N_SM ? 4 : 2;
 }
 // budget of the bound and direct-sampling plans (compiled for two CTAs per SM in FP32)
@@ -1368,9 +1368,12 @@ extern "C" peps_status peps_autotune(peps_handle* h, const peps_hamiltonian* H, 
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  std::vector<size_t> cand = (h->esz >= 8) ? std::vector<size_t>{100 * 1024, 210 * 1024}
-                                           : std::vector<size_t>{72 * 1024, 110 * 1024, 220 * 1024};
-  for (auto& b : cand) b = std::min(b, (size_t)optin - 2048);
+  const std::vector<size_t> sizes = (h->esz >= 8) ? std::vector<size_t>{100 * 1024, 210 * 1024}
+                                                  : std::vector<size_t>{72 * 1024, 110 * 1024, 220 * 1024};
+  const size_t ncand = sizes.size() + 1;
+  auto cand = [&](int cls, size_t ci) {  // the last one: the class's default, where it is none of the sizes
+    return std::min(ci < sizes.size() ? sizes[ci] : default_budget(h, cls), (size_t)optin - 2048);
+  };
   // scratch outputs and a copy of the configurations for the sampler trial
   const size_t N = (size_t)h->g.Lx * h->g.Ly;
   double *la = nullptr, *ph = nullptr, *el = nullptr;
@@ -1393,10 +1396,12 @@ extern "C" peps_status peps_autotune(peps_handle* h, const peps_hamiltonian* H, 
   }
   const bool was_timing = h->timing;
   const int cls[4] = {TC_ENV, TC_ROW, TC_PAIR, TC_SAMPLE};
-  std::vector<std::vector<float>> ms(4, std::vector<float>(cand.size(), 1e30f));
+  std::vector<std::vector<float>> ms(4, std::vector<float>(ncand, 1e30f));
   peps_status st = PEPS_OK;
-  for (size_t ci = 0; ci < cand.size() && st == PEPS_OK; ++ci) {
-    for (int i = 0; i < 4; ++i) h->budget[i] = cand[ci];
+  bool other = false;
+  for (int i = 0; i < 4; ++i) other = other || std::find(sizes.begin(), sizes.end(), default_budget(h, i)) == sizes.end();
+  for (size_t ci = 0; ci < sizes.size() + (other ? 1 : 0) && st == PEPS_OK; ++ci) {
+    for (int i = 0; i < 4; ++i) h->budget[i] = cand(i, ci);
     plan_all(h);
     st = finish_plans(h);
     if (st != PEPS_OK) break;
@@ -1425,11 +1430,11 @@ extern "C" peps_status peps_autotune(peps_handle* h, const peps_hamiltonian* H, 
   }
   for (int i = 0; i < 4; ++i) {
     size_t best = 0;
-    for (size_t ci = 1; ci < cand.size(); ++ci)
+    for (size_t ci = 1; ci < ncand; ++ci)
       if (ms[i][ci] < ms[i][best]) best = ci;
     if (i == 2 && !(H && h->n_pair_terms > 0)) best = 0;  // the pair kernel did not run: keep the smallest
-    h->budget[i] = cand[best];
-    if (budget_kb_host) budget_kb_host[i] = (int)(cand[best] / 1024);
+    h->budget[i] = cand(i, best);
+    if (budget_kb_host) budget_kb_host[i] = (int)(h->budget[i] / 1024);
   }
   plan_all(h);
   return finish_plans(h);
