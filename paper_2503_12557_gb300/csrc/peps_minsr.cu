@@ -246,21 +246,10 @@ template cudaError_t launch_center_global<float>(const float*, const double*, co
 // one; rotation parameters are recomputed from the old diagonal blocks (classical two-sided
 // Jacobi, Golub & Van Loan sym.schur2: tau = (a_qq - a_pp) / (2 a_pq), t = sign(tau) /
 // (|tau| + sqrt(1 + tau^2)), c = 1/sqrt(1+t^2), s = t c; B = J^T A J with J = [[c, s], [-s, c]]).
-// sqrt(x)^-1 and x^-1 from single-precision starts and two Newton steps (x within the float range):
-// a few dependent FP64 operations where sqrt and a division are some twenty each, and a round's
-// parameters are one such chain that the whole grid waits for (333 rows: 43.0 -> 36.9 ms with the
-// 32-bit indices of the apply phase; one CTA of 512 threads per SM instead of 256: 37.3).
-__device__ __forceinline__ double rsqrt_nr(double x) {
-  double y = (double)rsqrtf((float)x);
-  const double h = -0.5 * x;
-  y = y * fma(h, y * y, 1.5);
-  return y * fma(h, y * y, 1.5);
-}
-__device__ __forceinline__ double rcp_nr(double x) {
-  double r = (double)__frcp_rn((float)x);
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
-}
+// The reciprocals and roots by Newton steps (peps_newton.cuh): a few dependent FP64 operations where sqrt
+// and a division are some twenty each, and a round's parameters are one such chain that the whole grid
+// waits for (333 rows: 43.0 -> 36.9 ms with the 32-bit indices of the apply phase; one CTA of 512 threads
+// per SM instead of 256: 37.3).
 __device__ __forceinline__ void jac_params(const double* A, int n, int p, int q, double* c, double* s) {
   const double apq = A[(size_t)p * n + q];
   const double app = A[(size_t)p * n + p], aqq = A[(size_t)q * n + q];

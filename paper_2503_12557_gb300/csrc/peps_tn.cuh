@@ -27,6 +27,8 @@
 #include <stdint.h>
 #include <math.h>
 
+#include "peps_newton.cuh"
+
 namespace peps {
 
 // ------------------------------------------------------------------------------------------
@@ -472,9 +474,9 @@ __device__ __noinline__ void qr_keep_r_smem(T* Z, int m, int nc, T* R, T* taus, 
 }
 
 // beta, tau and the scale 1 / (alpha - beta) of xLARFG's reflector for a real column with head
-// alpha and squared tail norm sigma > 0.  Double: one reciprocal square root and one reciprocal,
-// each a single-precision start and two Newton steps, where sqrt and two divisions would be
-// about 70 instructions of 64 cycles on the FP64 pipes (tau = 1 + |alpha| / norm).
+// alpha and squared tail norm sigma > 0.  Double: one reciprocal square root and one reciprocal by
+// Newton steps, where sqrt and two divisions would be about 70 instructions of 64 cycles on the FP64
+// pipes (tau = 1 + |alpha| / norm); no less accurate (peps_newton.cuh).
 __device__ __forceinline__ void reflector(float alpha, float sigma, float& beta, float& tau, float& sc) {
   const float nrm = sqrt(alpha * alpha + sigma);
   beta = (alpha >= 0.f) ? -nrm : nrm;
@@ -484,15 +486,8 @@ __device__ __forceinline__ void reflector(float alpha, float sigma, float& beta,
 __device__ __forceinline__ void reflector(double alpha, double sigma, double& beta, double& tau, double& sc) {
   const double n2 = fma(alpha, alpha, sigma);
   if (n2 > 1e-30 && n2 < 1e30) {
-    double y = (double)rsqrtf((float)n2);
-    const double h = -0.5 * n2;
-    y = y * fma(h, y * y, 1.5);
-    y = y * fma(h, y * y, 1.5);
-    const double nrm = n2 * y, aa = fabs(alpha), d = aa + nrm;
+    const double y = rsqrt_nr(n2), nrm = sqrt_nr(n2, y), aa = fabs(alpha), r = rcp_nr(aa + nrm);
     tau = fma(aa, y, 1.0);
-    double r = (double)__frcp_rn((float)d);
-    r = fma(r, fma(-d, r, 1.0), r);
-    r = fma(r, fma(-d, r, 1.0), r);
     beta = (alpha >= 0.0) ? -nrm : nrm;
     sc = (alpha >= 0.0) ? r : -r;
   } else {
