@@ -208,12 +208,11 @@ def _peaks():
 
 
 # DRAM bytes (read + write) of one sampler call of 2 sweeps in FP32 (the 31 kernel launches of the
-# split sweep), from one ncu capture of such a call at 304 chains, scaled by the chains processed
+# split sweep), from one ncu capture of such a call at 1024 chains, scaled by the chains processed
 # (each chain's environment rows and partials are its own traffic); None until such a capture of
-# the current kernels exists.  profiles/sampler_split_heis8x8_D4_chi16_ns304.md: 1.192 GB per call
-# of 2 sweeps over 304 chains (k_env one-side pass 0.223 GB, 16 k_sweep_moves 0.700 GB, 14
-# k_env_row 0.269 GB).
-_SAMPLER_CAPTURE = {"bytes": 1.1915e9, "chains": 304, "sweeps": 2}
+# the current kernels exists.  profiles/sampler_split_heis8x8_D4_chi16_ns1024.md: 3.738 GB per call of
+# 2 sweeps over 1024 chains (k_env one-side pass 0.364 GB, 16 k_sweep_moves 2.837 GB, 14 k_env_row 0.537 GB).
+_SAMPLER_CAPTURE = {"bytes": 3.738e9, "chains": 1024, "sweeps": 2}
 
 
 def _measured_traffic(kernel, ns, sweeps, prec):
@@ -224,6 +223,20 @@ def _measured_traffic(kernel, ns, sweeps, prec):
     if c and kernel == "sample" and prec == P.PREC_FP32 and sweeps == c["sweeps"]:
         return c["bytes"] * ns / c["chains"]
     return None
+
+
+def _dtheta_fp64(O, eloc, w, lam, tau):
+    """The MinSR update of O, E_loc and the weights w in FP64 (torch's products, numpy's solve)."""
+    import torch
+    w = w / w.sum()
+    Ob = O.double()
+    Ob -= w @ Ob
+    Ob *= w.sqrt()[:, None]
+    eb = w.sqrt() * (eloc[:, 0] - w @ eloc[:, 0])
+    T = Ob @ Ob.T
+    T.diagonal().add_(lam)
+    x = np.linalg.solve(T.cpu().numpy(), eb.cpu().numpy())
+    return -tau * (Ob.T @ torch.as_tensor(x, device=Ob.device))
 
 
 def _tau_chains(E, c=5.0):
@@ -354,15 +367,13 @@ def run_gpu(a):
     e_site = [float(E[k][ok[k]].mean()) / lat.nsites for k in range(a.steps)]
     lo_b, hi_b = HEIS_BOUNDS[0] * nbonds / lat.nsites, HEIS_BOUNDS[1] * nbonds / lat.nsites
     tau = _tau_chains(E)
-    # the last timed step's MinSR update against an FP64 Gram of the same O and E_loc
+    # the last timed step's MinSR update against FP64 linear algebra on the same O and E_loc
     dtheta_check = None
-    if gram != 0 and world == 1:
+    if w["rcond"] == 0.0 and world == 1:
         wl = h.status_weights(r["status"], mask)
         dth_last = h.minsr_step(r["O"], r["eloc"], w=wl, lam=w["lam"], rcond=w["rcond"], tau=w["tau"])[0].clone()
-        h64g = P.PEPS(lat.Lx, lat.Ly, lat.d, lat.D, w["chi"], prec=prec, max_samples=2, gram=0, solve=0)
-        dth64 = h64g.minsr_step(r["O"], r["eloc"], w=wl, lam=w["lam"], rcond=w["rcond"], tau=w["tau"])[0]
+        dth64 = _dtheta_fp64(r["O"], r["eloc"], wl, w["lam"], w["tau"])
         dtheta_check = float((dth_last - dth64).norm() / dth64.norm())
-        h64g.close()
     ms_step = ms_total / a.steps
     if world > 1:
         t = torch.tensor([ms_step], device="cuda")
@@ -404,7 +415,9 @@ def run_gpu(a):
                     "k_sweep_moves and k_env_row per row)" if prec == P.PREC_FP32 else "k_sample")
     roof = {"kernel": {"env": "k_env", "sample": sampler_name, "row": "k_row", "pair": "k_pair",
                        "minsr_gram": "k_gram_sl"}[dom],
-            "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+            # (the contraction kernels execute a part of the arithmetic that is counted: no fraction of a peak)
+            "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": achieved / peak if dom == "minsr_gram" else None, "dense_equivalent": dom != "minsr_gram",
             # per launch, as achieved: the call's bytes spread over the launches the call made
             "traffic": (None if _measured_traffic(dom, ns, a.sweeps, prec) is None else
                         _measured_traffic(dom, ns, a.sweeps, prec) * a.steps / max(1, launches[dom])),
@@ -413,9 +426,9 @@ def run_gpu(a):
                             "measured: peps_probe_fma FP64" if peak == fp64_peak else "MEASURED_PEAKS bf16_tflops"),
             "algorithmic_tflop_per_launch": flops[dom] / max(1, launches[dom]) / 1e12,
             "launch_ms": dom_launch_ms,
-            "counting": ("the loop nests' flops at the full bond chi (products, QR, sandwiches) plus the Jacobi "
-                         "rotations and sweeps the library counted; the kernels skip the exact-zero rows and "
-                         "columns near the open edge, so the executed flops are fewer")}
+            "counting": ("the loop nests' flops with every bond at chi (products, QR, sandwiches) plus the Jacobi "
+                         "rotations and sweeps the library counted; the kernels stop at the nonzero bonds and rows "
+                         "and execute far fewer, so achieved is a dense-equivalent rate")}
     # library launches per step: the classes' counts plus the memsets of evaluate / minsr
     gpu_launches = int(sum(launches.values())) + 4 * a.steps
     line = {"metric": METRIC, "value": value, "unit": "samples/s", "n_gpus": world, "steps": a.steps,

@@ -1,6 +1,9 @@
-"""Counted arithmetic of the kernels as written (flops = 2 per multiply-add), used for the
-roofline figures.  Each formula follows the loop nests of the kernel it names; the one-sided
-Jacobi part uses the sweep / rotation counts the library records (peps_timing_read counters).
+"""Counted arithmetic of the contractions with every bond at its largest (flops = 2 per
+multiply-add): the loop nests of the kernels it names at full chi, which they run on states that fill
+their bonds; elsewhere they stop at the nonzero bonds, rows and columns, and the figures are
+dense-equivalent.  The one-sided Jacobi part uses the sweep / rotation counts the library records
+(peps_timing_read counters) and counts the checks of every pair of rows, active or not.  The Gram's
+counts are what its kernels execute.
 
 Notation: chi = boundary bond D_c, D = PEPS bond, n = chi*D (exact product bond),
 Lr = D*chi (row length of the truncation matrix X), mX = n rounded up to even.

@@ -12,7 +12,8 @@
 // Measured (one GB300, whole MinSR step): 4096 x 21 632 with refinement (solve = 2) 44.2 -> 27.8 ms
 // against a float-float factor on the FP32 pipes, 1000 x 3528 (solve = 0) 4.71 -> 2.68 ms against
 // FP64 FMA tiles; dtheta's error against 64-bit linear algebra is unchanged (3.0e-15, 1.7e-15).
-// The diagonal blocks, at about 97 us each, are now the longest part: one SM's FP64 pipes.
+// The diagonal blocks are now the longest part, 38 % of a 4096-row solve (100 us each, cold, under a
+// profiler): one SM's FP64 pipes, barriers and instruction fetches.
 #include "peps_kernels.cuh"
 #include "peps_slices.cuh"
 

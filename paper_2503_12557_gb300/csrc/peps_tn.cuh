@@ -1343,8 +1343,8 @@ __host__ __device__ inline size_t env_z_elems(int chi, int D) {
   return zleft > zright ? zleft : zright;
 }
 // Scratch for the row step's matrices where the bonds that are not zero make them small (R, Z, Y, X,
-// Vt): in shared memory under every plan, since what a warp writes to the arena the others read back
-// from L2.
+// Vt).  The plans place it before R and Z: in shared memory, where what a warp writes the others need not
+// read back from L2, as far as the budget goes (it is in the arena for chi >= 20 at D = 4 under half of 72 KB).
 __host__ __device__ inline int env_zs_elems(int chi, int D) {
   const size_t n = (size_t)chi * D, all = n * n + env_z_elems(chi, D);
   return all < 4096 ? (int)all : 4096;
@@ -1432,6 +1432,9 @@ __device__ __forceinline__ void blk_gemm_tile(const T* __restrict__ A, const T* 
 // of the sum unrolled; two in the row step, whose code a CTA runs through once per site and fetches from
 // L2 each time (at four, environments 42.2 -> 47.6 ms at 8x8, 4096 samples), four in the sandwiches
 // (two-row kernel 18.3 -> 12.1 ms).
+// On states that fill their bonds 4 x 4 tiles for products of 16 outputs per thread and more would gain
+// (8x8, chi = 16: evaluation 31.9 -> 30.8 ms, amplitudes 13.5 -> 13.4, where 2 x 8 and 4 x 4 tiles
+// everywhere took 35.2 and 13.1), but their code costs the sweeps of small bonds 8 % (78.1 -> 84.3 ms).
 // In FP64 one output per thread: a multiply-add holds its SM sub-partition for 64 cycles, so that
 // operand loads are free beside it and what counts is to have all four sub-partitions busy.
 template <int RM, int RN, int U = 4, typename T, class FM, class FN>
